@@ -1,0 +1,600 @@
+// Spectral Born operator of the line geometry on the folded table index.
+//
+// The operator (eqs. DMV and M read forward) is F(p, q) = s_f sum_j g_p g_q Vhat(p - q) over the
+// depths j, with g_n = g(|k_n|, z_j) even in n and Vhat(-m) = conj Vhat(m) for a real model.  The
+// N^2 entries of a frequency plane therefore come from the pairs k >= l of the table index
+// 0..H, H = N/2, eight entries to a pair.  With a = g_k g_l and the real sums' shorthand
+//   P = sum a Re Vhat(k - l),  Q = sum a Im Vhat(k - l)   (complex times real: 4 multiply-adds)
+//   P2, Q2 the same with Vhat(k + l),
+//   F(k, l) = F(-l, -k) = s_f (P + iQ),      F(l, k) = F(-k, -l) = s_f (P - iQ),
+//   F(k, -l) = F(l, -k) = s_f (P2 + iQ2),    F(-k, l) = F(-l, k) = s_f (P2 - iQ2),
+// so a pair and depth take 12 multiply-adds where the eight entries one by one take 64 (complex
+// a times complex Vhat each).  A pair with k = H has -k = k and needs P and Q only (edge
+// kernels); l = 0 and k = l name some entries twice, with the same value.
+//
+// Three arithmetics of the same tile (32 x 32 pairs, 2 x 2 per thread, depths staged in shared
+// memory 8 at a time):
+//   F32   the misfit's residual (the FP32 table sqrt|s_f| g);
+//   F64   the forward model of the FP64 path, bound by the FP64 unit;
+//   DF    the forward model of the mixed path, FP64 table and sums carried as float pairs on
+//         the FP32 pipes (an FP64 multiply-add costs 64 FP32 ones here).  Table and Vhat rows
+//         are scaled by powers of two to at most 1, so a sum of nz products stays below nz and
+//         is accumulated on a bias C = 4 nz (rounded up to a power of two): s stays within a
+//         binade or two of C, the rounding error of s' = fma(a, v, s) is then exactly
+//         fma(a, v, s - s'), and one multiply-add of pairs takes 6 FP32 operations instead of
+//         the 12 of an unordered TwoSum.  The result is rounded to FP32 once.
+//
+// Measured at N = 512, 128 frequencies, 256 depths (GB300): the forward contraction 3.55 ms in
+// DF, where the 512^2 entries one by one in FP64 took 153 ms (FP64-bound); the operation count
+// (86 FP32 operations per pair and depth) allows 2.3 ms.  Against a 64-bit restatement the
+// data are 1.6e-7 off either way: the FP32 transforms behind it set the error.
+//
+// The gradients read the residual plane R2 (or the data plane) only through the sums over the
+// entries of a class, so the residual kernel leaves, per pair, the folded values
+//   E[k][l] = (S, S'),  S = R(k, l) + R(-l, -k),   S' = R(l, k) + R(-k, -l),
+//   T[k][l] = (T, T'),  T = R(k, -l) + R(l, -k),   T' = R(-k, l) + R(-l, k),
+// times conj(s_f)/|s_f|, for every ordered (k, l) (E[l][k] = (S', S), T[l][k] = (T, T')).
+#include "edt_internal.h"
+#include "cplx.cuh"
+#include "dfloat.cuh"
+
+namespace edt {
+
+namespace {
+
+constexpr int BT = 32, BZ = 8;              // pairs per tile side, depths per staged chunk
+constexpr int BKS = BT + 1, BVS = 2 * BT + 1;   // odd rows: the transposing stores spread over banks
+constexpr int BTHREADS = 256;
+
+// ---- arithmetics -------------------------------------------------------------------------
+struct ArF32 {
+  using E = float2;
+  float s[8];
+  __device__ __forceinline__ void init(float) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s[i] = 0.f;
+  }
+  __device__ __forceinline__ void mac(E k, E l, E v, E w) {
+    const E a = k * l;
+    s[0] = fmaf(a.x, v.x, s[0]); s[1] = fmaf(a.y, v.x, s[1]);
+    s[2] = fmaf(a.x, v.y, s[2]); s[3] = fmaf(a.y, v.y, s[3]);
+    s[4] = fmaf(a.x, w.x, s[4]); s[5] = fmaf(a.y, w.x, s[5]);
+    s[6] = fmaf(a.x, w.y, s[6]); s[7] = fmaf(a.y, w.y, s[7]);
+  }
+};
+
+struct ArF64 {
+  using E = double2;
+  double s[8];
+  __device__ __forceinline__ void init(float) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) s[i] = 0.0;
+  }
+  __device__ __forceinline__ void mac(E k, E l, E v, E w) {
+    const E a = k * l;
+    s[0] = fma(a.x, v.x, s[0]); s[1] = fma(a.y, v.x, s[1]);
+    s[2] = fma(a.x, v.y, s[2]); s[3] = fma(a.y, v.y, s[3]);
+    s[4] = fma(a.x, w.x, s[4]); s[5] = fma(a.y, w.x, s[5]);
+    s[6] = fma(a.x, w.y, s[6]); s[7] = fma(a.y, w.y, s[7]);
+  }
+};
+
+// complex pairs (re hi, im hi, re lo, im lo), |re|, |im| <= 1
+struct ArDF {
+  using E = float4;
+  float s[8], lo[8];
+  __device__ __forceinline__ void init(float bias) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) { s[i] = bias; lo[i] = 0.f; }
+  }
+  __device__ __forceinline__ void acc(int i, float ah, float al, float vh, float vl) {
+    const float t = fmaf(ah, vh, s[i]);
+    const float e = fmaf(ah, vh, __fsub_rn(s[i], t));      // the rounding error of t, exactly
+    s[i] = t;
+    lo[i] = fmaf(al, vh, fmaf(ah, vl, __fadd_rn(lo[i], e)));
+  }
+  __device__ __forceinline__ void mac(E k, E l, E v, E w) {
+    float2 ah, al;
+    cmul_df(make_float2(k.x, k.y), make_float2(k.z, k.w), make_float2(l.x, l.y), make_float2(l.z, l.w), ah, al);
+    acc(0, ah.x, al.x, v.x, v.z); acc(1, ah.y, al.y, v.x, v.z);
+    acc(2, ah.x, al.x, v.y, v.w); acc(3, ah.y, al.y, v.y, v.w);
+    acc(4, ah.x, al.x, w.x, w.z); acc(5, ah.y, al.y, w.x, w.z);
+    acc(6, ah.x, al.x, w.y, w.w); acc(7, ah.y, al.y, w.y, w.w);
+  }
+};
+
+template <class E> __device__ __forceinline__ E zero_of();
+template <> __device__ __forceinline__ float2 zero_of<float2>() { return make_float2(0.f, 0.f); }
+template <> __device__ __forceinline__ double2 zero_of<double2>() { return make_double2(0.0, 0.0); }
+template <> __device__ __forceinline__ float4 zero_of<float4>() { return make_float4(0.f, 0.f, 0.f, 0.f); }
+
+// tile pair (tk >= tl) of the lower triangle, row-major
+__device__ __forceinline__ void tile_of(int t, int& tk, int& tl) {
+  tk = int((sqrtf(8.0f * t + 1.0f) - 1.0f) * 0.5f);
+  while (tk * (tk + 1) / 2 > t) --tk;
+  while ((tk + 1) * (tk + 2) / 2 <= t) ++tk;
+  tl = t - tk * (tk + 1) / 2;
+}
+inline int tile_count(int H) { const int T = (H + BT - 1) / BT; return T * (T + 1) / 2; }
+
+// A warp covers 8 x 4 pairs, so that each of its shared reads touches at most 11 consecutive
+// elements; pair (a, b) of a thread is k = tx + 16 a, l = ty + 16 b.
+__device__ __forceinline__ void thread_xy(int& tx, int& ty) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  tx = (w & 1) * 8 + (lane & 7);
+  ty = (w >> 1) * 4 + (lane >> 3);
+}
+
+template <class E> constexpr size_t tile_smem() { return size_t(BZ) * (2 * BKS + 2 * BVS) * sizeof(E); }
+
+// Sums of the tile's pairs over the depths.  g: table row n at g + n gs; v: Vhat row m at
+// v + m vs.  Rows k, l >= H are not part of the tile (their pairs are not used).
+template <class Ar>
+__device__ __forceinline__ void fold_tile(const typename Ar::E* g, size_t gs, const typename Ar::E* v, size_t vs,
+                                          int nz, int N, int k0, int l0, typename Ar::E* sm, Ar (&acc)[2][2]) {
+  using E = typename Ar::E;
+  E* sk = sm;                       // [BZ][BKS] rows k0 + i
+  E* sl = sk + BZ * BKS;            // [BZ][BKS] rows l0 + i
+  E* s1 = sl + BZ * BKS;            // [BZ][BVS] rows k0 - l0 - 31 + i
+  E* s2 = s1 + BZ * BVS;            // [BZ][BVS] rows k0 + l0 + i
+  const int H = N / 2, msk = N - 1;
+  int tx, ty;
+  thread_xy(tx, ty);
+  const bool diag = k0 == l0;
+  for (int z0 = 0; z0 < nz; z0 += BZ) {
+    for (int e = threadIdx.x; e < BT * BZ; e += BTHREADS) {
+      const int i = e / BZ, zz = e - i * BZ;
+      const bool in = z0 + zz < nz;
+      sk[zz * BKS + i] = in && k0 + i < H ? g[size_t(k0 + i) * gs + z0 + zz] : zero_of<E>();
+      sl[zz * BKS + i] = in && l0 + i < H ? g[size_t(l0 + i) * gs + z0 + zz] : zero_of<E>();
+    }
+    for (int e = threadIdx.x; e < 2 * BT * BZ; e += BTHREADS) {
+      const int i = e / BZ, zz = e - i * BZ;
+      const bool in = z0 + zz < nz;
+      s1[zz * BVS + i] = in ? v[size_t((k0 - l0 - (BT - 1) + i) & msk) * vs + z0 + zz] : zero_of<E>();
+      s2[zz * BVS + i] = in ? v[size_t((k0 + l0 + i) & msk) * vs + z0 + zz] : zero_of<E>();
+    }
+    __syncthreads();
+#pragma unroll 2
+    for (int zz = 0; zz < BZ; ++zz) {
+      E gk[2], gl[2], v1[3], v2[3];
+#pragma unroll
+      for (int a = 0; a < 2; ++a) {
+        gk[a] = sk[zz * BKS + tx + 16 * a];
+        gl[a] = sl[zz * BKS + ty + 16 * a];
+      }
+#pragma unroll
+      for (int t = 0; t < 3; ++t) {
+        v1[t] = s1[zz * BVS + tx - ty + 16 * (t - 1) + BT - 1];
+        v2[t] = s2[zz * BVS + tx + ty + 16 * t];
+      }
+#pragma unroll
+      for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b)
+          if (!(diag && a < b)) acc[a][b].mac(gk[a], gl[b], v1[a - b + 1], v2[a + b]);   // a < b: k < l
+    }
+    __syncthreads();
+  }
+}
+
+// ---- preparation of the double-float forward model ---------------------------------------
+__device__ __forceinline__ float block_max(float m, float* red) {
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
+  __syncthreads();
+  m = red[0];
+  for (int w = 1; w < int(blockDim.x >> 5); ++w) m = fmaxf(m, red[w]);
+  return m;
+}
+
+// One row of nz <= 512 FP64 complex values per CTA, replaced in place by float pairs of
+// value * c * 2^-e with the largest component just under 1; e goes to exps[row].  c is
+// sqrt(s_f) = omega~ sqrt(dz/dx) for the Green's table (so the products carry s_f) and 1 for Vhat.
+constexpr int PREP_THREADS = 128, PREP_Q = 4;
+__global__ void __launch_bounds__(PREP_THREADS) born_prep_kernel(Dev d, double2* rows, int per_f, int* exps) {
+  __shared__ float red[PREP_THREADS / 32];
+  const size_t row = blockIdx.x;
+  double2 c = make_double2(1.0, 0.0);
+  if (per_f) {
+    const FreqConst fc = d.fc[row / per_f];
+    const double q = sqrt(d.dz / d.dx);
+    c = make_double2(q * fc.om_re, q * fc.om_im);
+  }
+  double2* r = rows + row * d.nz;
+  double2 v[PREP_Q];
+  float m = 0.f;
+#pragma unroll
+  for (int i = 0; i < PREP_Q; ++i) {
+    const int z = threadIdx.x + PREP_THREADS * i;
+    v[i] = z < d.nz ? r[z] : make_double2(0.0, 0.0);
+    if (per_f) v[i] = c * v[i];
+    m = fmaxf(m, fmaxf(fabsf(float(v[i].x)), fabsf(float(v[i].y))));
+  }
+  m = block_max(m, red);
+  int e = 0;
+  if (m > 0.f && isfinite(m)) frexpf(m, &e);
+  e = max(-126, min(126, e));
+  const double sc = __longlong_as_double((long long)(1023 - e) << 52);      // 2^-e
+#pragma unroll
+  for (int i = 0; i < PREP_Q; ++i) {
+    const int z = threadIdx.x + PREP_THREADS * i;
+    if (z >= d.nz) continue;
+    const double x = v[i].x * sc, y = v[i].y * sc;
+    const float xh = float(x), yh = float(y);
+    reinterpret_cast<float4*>(r)[z] = make_float4(xh, yh, float(x - double(xh)), float(y - double(yh)));
+  }
+  if (threadIdx.x == 0) exps[row] = e;
+}
+
+// Vhat rows rounded to FP32 in place (row m's float2 values at the start of its FP64 row)
+__global__ void __launch_bounds__(PREP_THREADS) born_v32_kernel(Dev d) {
+  double2* r = d.vfull + size_t(blockIdx.x) * d.nz;
+  double2 v[PREP_Q];
+#pragma unroll
+  for (int i = 0; i < PREP_Q; ++i) {
+    const int z = threadIdx.x + PREP_THREADS * i;
+    v[i] = z < d.nz ? r[z] : make_double2(0.0, 0.0);
+  }
+  __syncthreads();
+#pragma unroll
+  for (int i = 0; i < PREP_Q; ++i) {
+    const int z = threadIdx.x + PREP_THREADS * i;
+    if (z < d.nz) reinterpret_cast<float2*>(r)[z] = make_float2(float(v[i].x), float(v[i].y));
+  }
+}
+
+// ---- forward model -----------------------------------------------------------------------
+__host__ __device__ inline float df_bias(int nz) {
+  float c = 4.f;
+  for (int n = 1; n < nz; n <<= 1) c *= 2.f;
+  return c;
+}
+
+// one rounding of (xh + xl) + sg (yh + yl), scaled by 2^e
+__device__ __forceinline__ float df_comb(float xh, float xl, float yh, float yl, float sg, int e) {
+  const float2 t = two_sum(xh, sg * yh);
+  return ldexpf(t.x + (t.y + (xl + sg * yl)), e);
+}
+// f1 = A + iB, f2 = A - iB for A = (s[o], s[o+1]), B = (s[o+2], s[o+3])
+__device__ __forceinline__ void df_result(const ArDF& a, int o, float bias, int e, float2& f1, float2& f2) {
+  const float a0 = a.s[o] - bias, a1 = a.s[o + 1] - bias, b0 = a.s[o + 2] - bias, b1 = a.s[o + 3] - bias;
+  f1 = make_float2(df_comb(a0, a.lo[o], b1, a.lo[o + 3], -1.f, e), df_comb(a1, a.lo[o + 1], b0, a.lo[o + 2], 1.f, e));
+  f2 = make_float2(df_comb(a0, a.lo[o], b1, a.lo[o + 3], 1.f, e), df_comb(a1, a.lo[o + 1], b0, a.lo[o + 2], -1.f, e));
+}
+
+// X[fi][q][p] = F(p, q) for the pairs of one tile (mixed path: FP32 planes)
+__global__ void __launch_bounds__(BTHREADS, 2) born_fwd_df_kernel(Dev d, int f0) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int N = d.N, H = N / 2, msk = N - 1, fi = blockIdx.y, f = f0 + fi;
+  int tk, tl;
+  tile_of(blockIdx.x, tk, tl);
+  const int k0 = tk * BT, l0 = tl * BT;
+  const float bias = df_bias(d.nz);
+  ArDF acc[2][2];
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int b = 0; b < 2; ++b) acc[a][b].init(bias);
+  fold_tile<ArDF>(reinterpret_cast<const float4*>(d.g64) + size_t(f) * d.nk * d.nz, d.nz,
+                  reinterpret_cast<const float4*>(d.vfull), d.nz, d.nz, N, k0, l0,
+                  reinterpret_cast<float4*>(smem_raw), acc);
+  int tx, ty;
+  thread_xy(tx, ty);
+  float2* X = reinterpret_cast<float2*>(d.X) + size_t(fi) * N * N;
+  const int* eg = d.born_exp + size_t(f) * d.nk;
+  const int* ev = d.born_exp + size_t(d.nf) * d.nk;
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const int k = k0 + tx + 16 * a, l = l0 + ty + 16 * b;
+      if (k >= H || l > k) continue;
+      const int e = eg[k] + eg[l], nk_ = (N - k) & msk, nl_ = (N - l) & msk;
+      float2 f1, f2, h1, h2;
+      df_result(acc[a][b], 0, bias, e + ev[(k - l) & msk], f1, f2);
+      df_result(acc[a][b], 4, bias, e + ev[(k + l) & msk], h1, h2);
+      X[size_t(l) * N + k] = f1;
+      X[size_t(nk_) * N + nl_] = f1;
+      X[size_t(k) * N + l] = f2;
+      X[size_t(nl_) * N + nk_] = f2;
+      X[size_t(nl_) * N + k] = h1;
+      X[size_t(nk_) * N + l] = h1;
+      X[size_t(l) * N + nk_] = h2;
+      X[size_t(k) * N + nl_] = h2;
+    }
+}
+
+__global__ void __launch_bounds__(BTHREADS, 2) born_fwd_f64_kernel(Dev d, int f0) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int N = d.N, H = N / 2, msk = N - 1, fi = blockIdx.y, f = f0 + fi;
+  int tk, tl;
+  tile_of(blockIdx.x, tk, tl);
+  const int k0 = tk * BT, l0 = tl * BT;
+  ArF64 acc[2][2];
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int b = 0; b < 2; ++b) acc[a][b].init(0.f);
+  fold_tile<ArF64>(d.g64 + size_t(f) * d.nk * d.nz, d.nz, d.vfull, d.nz, d.nz, N, k0, l0,
+                   reinterpret_cast<double2*>(smem_raw), acc);
+  int tx, ty;
+  thread_xy(tx, ty);
+  double2* X = reinterpret_cast<double2*>(d.X) + size_t(fi) * N * N;
+  const FreqConst fc = d.fc[f];
+  const double2 om = make_double2(fc.om_re, fc.om_im), sf = (d.dz / d.dx) * (om * om);
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const int k = k0 + tx + 16 * a, l = l0 + ty + 16 * b;
+      if (k >= H || l > k) continue;
+      const int nk_ = (N - k) & msk, nl_ = (N - l) & msk;
+      const double* s = acc[a][b].s;
+      const double2 f1 = sf * make_double2(s[0] - s[3], s[1] + s[2]), f2 = sf * make_double2(s[0] + s[3], s[1] - s[2]);
+      const double2 h1 = sf * make_double2(s[4] - s[7], s[5] + s[6]), h2 = sf * make_double2(s[4] + s[7], s[5] - s[6]);
+      X[size_t(l) * N + k] = f1;
+      X[size_t(nk_) * N + nl_] = f1;
+      X[size_t(k) * N + l] = f2;
+      X[size_t(nl_) * N + nk_] = f2;
+      X[size_t(nl_) * N + k] = h1;
+      X[size_t(nk_) * N + l] = h1;
+      X[size_t(l) * N + nk_] = h2;
+      X[size_t(k) * N + nl_] = h2;
+    }
+}
+
+// Pairs (H, l), l = 0..H: one warp per (plane, l), lanes over the depths.
+// F(H, l) = F(-l, H) = s_f (P + iQ), F(l, H) = F(H, -l) = s_f (P - iQ).
+template <typename T> struct EdgeSum;
+template <> struct EdgeSum<float> {                       // double-float partial sums
+  float2 s[4];
+  __device__ __forceinline__ void init() {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) s[i] = make_float2(0.f, 0.f);
+  }
+  __device__ __forceinline__ void mac(float4 k, float4 l, float4 v) {
+    float2 ah, al;
+    cmul_df(make_float2(k.x, k.y), make_float2(k.z, k.w), make_float2(l.x, l.y), make_float2(l.z, l.w), ah, al);
+    const float2 ar = make_float2(ah.x, al.x), ai = make_float2(ah.y, al.y);
+    df_acc(s[0], ar, make_float2(v.x, v.z)); df_acc(s[1], ai, make_float2(v.x, v.z));
+    df_acc(s[2], ar, make_float2(v.y, v.w)); df_acc(s[3], ai, make_float2(v.y, v.w));
+  }
+  __device__ __forceinline__ void warp_sum() {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      s[i] = df_norm(s[i]);
+      for (int o = 16; o > 0; o >>= 1)
+        s[i] = df_add(s[i], make_float2(__shfl_xor_sync(0xffffffffu, s[i].x, o), __shfl_xor_sync(0xffffffffu, s[i].y, o)));
+    }
+  }
+};
+
+__global__ void __launch_bounds__(256) born_fwd_edge_df_kernel(Dev d, int f0) {
+  const int N = d.N, H = N / 2, msk = N - 1, lane = threadIdx.x & 31;
+  const int l = blockIdx.x * 8 + (threadIdx.x >> 5), fi = blockIdx.y, f = f0 + fi;
+  if (l > H) return;
+  const float4* g = reinterpret_cast<const float4*>(d.g64) + size_t(f) * d.nk * d.nz;
+  const float4* v = reinterpret_cast<const float4*>(d.vfull) + size_t(H - l) * d.nz;
+  EdgeSum<float> a;
+  a.init();
+  for (int z = lane; z < d.nz; z += 32) a.mac(g[size_t(H) * d.nz + z], g[size_t(l) * d.nz + z], v[z]);
+  a.warp_sum();
+  if (lane != 0) return;
+  const int e = d.born_exp[size_t(f) * d.nk + H] + d.born_exp[size_t(f) * d.nk + l] +
+                d.born_exp[size_t(d.nf) * d.nk + (H - l)];
+  auto out = [&](float2 x, float2 y, float sg) { return df_comb(x.x, x.y, y.x, y.y, sg, e); };
+  const float2 f1 = make_float2(out(a.s[0], a.s[3], -1.f), out(a.s[1], a.s[2], 1.f));
+  const float2 f2 = make_float2(out(a.s[0], a.s[3], 1.f), out(a.s[1], a.s[2], -1.f));
+  float2* X = reinterpret_cast<float2*>(d.X) + size_t(fi) * N * N;
+  const int nl_ = (N - l) & msk;
+  X[size_t(l) * N + H] = f1;
+  X[size_t(H) * N + nl_] = f1;
+  X[size_t(H) * N + l] = f2;
+  X[size_t(nl_) * N + H] = f2;
+}
+
+__global__ void __launch_bounds__(256) born_fwd_edge_f64_kernel(Dev d, int f0) {
+  const int N = d.N, H = N / 2, msk = N - 1, lane = threadIdx.x & 31;
+  const int l = blockIdx.x * 8 + (threadIdx.x >> 5), fi = blockIdx.y, f = f0 + fi;
+  if (l > H) return;
+  const double2* g = d.g64 + size_t(f) * d.nk * d.nz;
+  const double2* v = d.vfull + size_t(H - l) * d.nz;
+  double2 p = make_double2(0.0, 0.0), q = p;
+  for (int z = lane; z < d.nz; z += 32) {
+    const double2 a = g[size_t(H) * d.nz + z] * g[size_t(l) * d.nz + z];
+    p = p + v[z].x * a;
+    q = q + v[z].y * a;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    p.x += __shfl_xor_sync(0xffffffffu, p.x, o); p.y += __shfl_xor_sync(0xffffffffu, p.y, o);
+    q.x += __shfl_xor_sync(0xffffffffu, q.x, o); q.y += __shfl_xor_sync(0xffffffffu, q.y, o);
+  }
+  if (lane != 0) return;
+  const FreqConst fc = d.fc[f];
+  const double2 om = make_double2(fc.om_re, fc.om_im), sf = (d.dz / d.dx) * (om * om);
+  const double2 f1 = sf * make_double2(p.x - q.y, p.y + q.x), f2 = sf * make_double2(p.x + q.y, p.y - q.x);
+  double2* X = reinterpret_cast<double2*>(d.X) + size_t(fi) * N * N;
+  const int nl_ = (N - l) & msk;
+  X[size_t(l) * N + H] = f1;
+  X[size_t(H) * N + nl_] = f1;
+  X[size_t(H) * N + l] = f2;
+  X[size_t(nl_) * N + H] = f2;
+}
+
+// ---- residual and folding ----------------------------------------------------------------
+__device__ __forceinline__ float4 pack2(float2 a, float2 b) { return make_float4(a.x, a.y, b.x, b.y); }
+
+__device__ __forceinline__ void add_sq(float2& acc, float2 r, float w) {
+  df_acc(acc, make_float2(w * r.x, 0.f), make_float2(r.x, 0.f));     // w a power of two
+  df_acc(acc, make_float2(w * r.y, 0.f), make_float2(r.y, 0.f));
+}
+
+__device__ __forceinline__ double block_sum(double v, double* red) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if ((threadIdx.x & 31) == 0) red[w] = v;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x == 0)
+    for (int i = 0; i < nw; ++i) t += red[i];
+  return t;
+}
+
+// RES: R = F - D2 with the FP32 table and Vhat, sum |R|^2 into gacc[0] and R folded;
+// else R = D2 (the adjoint operator).  X[fi][q][p] = D2(p, q) is only read.
+template <bool RES>
+__global__ void __launch_bounds__(BTHREADS, 3) born_resid_kernel(Dev d, int f0) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double red[BTHREADS / 32];
+  const int N = d.N, H = N / 2, msk = N - 1, nk = d.nk, fi = blockIdx.y, f = f0 + fi;
+  int tk, tl;
+  tile_of(blockIdx.x, tk, tl);
+  const int k0 = tk * BT, l0 = tl * BT;
+  ArF32 acc[2][2];
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int b = 0; b < 2; ++b) acc[a][b].init(0.f);
+  if (RES)
+    fold_tile<ArF32>(d.g32 + size_t(f) * nk * d.nzs, d.nzs, reinterpret_cast<const float2*>(d.vfull),
+                     2 * size_t(d.nz), d.nz, N, k0, l0, reinterpret_cast<float2*>(smem_raw), acc);
+  int tx, ty;
+  thread_xy(tx, ty);
+  const float2* X = reinterpret_cast<const float2*>(d.X) + size_t(fi) * N * N;
+  float4* E = d.born_fold + size_t(fi) * 2 * nk * nk;
+  float4* T = E + size_t(nk) * nk;
+  const FreqConst fc = d.fc[f];
+  const float2 rot = make_float2(float(fc.rot_re), float(fc.rot_im));   // conj(s_f) / |s_f|
+  float2 jp = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const int k = k0 + tx + 16 * a, l = l0 + ty + 16 * b;
+      if (k >= H || l > k) continue;
+      const int nk_ = (N - k) & msk, nl_ = (N - l) & msk;
+      float2 r[8] = {X[size_t(l) * N + k],   X[size_t(nk_) * N + nl_], X[size_t(k) * N + l],   X[size_t(nl_) * N + nk_],
+                     X[size_t(nl_) * N + k], X[size_t(nk_) * N + l],   X[size_t(l) * N + nk_], X[size_t(k) * N + nl_]};
+      if (RES) {
+        const float2 ph = cconj(rot);
+        const float* s = acc[a][b].s;
+        const float2 f1 = ph * make_float2(s[0] - s[3], s[1] + s[2]), f2 = ph * make_float2(s[0] + s[3], s[1] - s[2]);
+        const float2 h1 = ph * make_float2(s[4] - s[7], s[5] + s[6]), h2 = ph * make_float2(s[4] + s[7], s[5] - s[6]);
+        r[0] = f1 - r[0]; r[1] = f1 - r[1]; r[2] = f2 - r[2]; r[3] = f2 - r[3];
+        r[4] = h1 - r[4]; r[5] = h1 - r[5]; r[6] = h2 - r[6]; r[7] = h2 - r[7];
+        // every distinct entry once: l = 0 names its entries twice, k = l the two of each kind
+        const float w1 = k == l ? (l == 0 ? 0.25f : 0.5f) : 1.f, w2 = l == 0 ? 0.f : w1;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) { add_sq(jp, r[i], w1); add_sq(jp, r[4 + i], w2); }
+      }
+      const float2 S = rot * (r[0] + r[1]), S2 = rot * (r[2] + r[3]);
+      const float2 U = rot * (r[4] + r[5]), U2 = rot * (r[6] + r[7]);
+      E[size_t(k) * nk + l] = pack2(S, S2);
+      E[size_t(l) * nk + k] = pack2(S2, S);
+      T[size_t(k) * nk + l] = pack2(U, U2);
+      T[size_t(l) * nk + k] = pack2(U, U2);
+    }
+  if (RES) {
+    const double t = block_sum(df_val(jp), red);
+    if (threadIdx.x == 0) atomicAdd(d.gacc, t);
+  }
+}
+
+// the pairs (H, l): E[H][l], E[l][H] and T[H][l] = E[l][H] (the entries of -l against H = -H)
+template <bool RES>
+__global__ void __launch_bounds__(256) born_resid_edge_kernel(Dev d, int f0) {
+  __shared__ double red[8];
+  const int N = d.N, H = N / 2, msk = N - 1, nk = d.nk, lane = threadIdx.x & 31;
+  const int l = blockIdx.x * 8 + (threadIdx.x >> 5), fi = blockIdx.y, f = f0 + fi;
+  double jp = 0.0;
+  if (l <= H) {
+    float2 p = make_float2(0.f, 0.f), q = p;
+    if (RES) {
+      const float2* g = d.g32 + size_t(f) * nk * d.nzs;
+      const float2* v = reinterpret_cast<const float2*>(d.vfull) + size_t(H - l) * 2 * d.nz;
+      for (int z = lane; z < d.nz; z += 32) {
+        const float2 a = g[size_t(H) * d.nzs + z] * g[size_t(l) * d.nzs + z], b = v[z];
+        p.x = fmaf(a.x, b.x, p.x); p.y = fmaf(a.y, b.x, p.y);
+        q.x = fmaf(a.x, b.y, q.x); q.y = fmaf(a.y, b.y, q.y);
+      }
+      for (int o = 16; o > 0; o >>= 1) {
+        p.x += __shfl_xor_sync(0xffffffffu, p.x, o); p.y += __shfl_xor_sync(0xffffffffu, p.y, o);
+        q.x += __shfl_xor_sync(0xffffffffu, q.x, o); q.y += __shfl_xor_sync(0xffffffffu, q.y, o);
+      }
+    }
+    if (lane == 0) {
+      const float2* X = reinterpret_cast<const float2*>(d.X) + size_t(fi) * N * N;
+      const FreqConst fc = d.fc[f];
+      const float2 rot = make_float2(float(fc.rot_re), float(fc.rot_im));
+      const int nl_ = (N - l) & msk;
+      float2 r[4] = {X[size_t(l) * N + H], X[size_t(H) * N + nl_], X[size_t(H) * N + l], X[size_t(nl_) * N + H]};
+      if (RES) {
+        const float2 ph = cconj(rot);
+        const float2 f1 = ph * make_float2(p.x - q.y, p.y + q.x), f2 = ph * make_float2(p.x + q.y, p.y - q.x);
+        r[0] = f1 - r[0]; r[1] = f1 - r[1]; r[2] = f2 - r[2]; r[3] = f2 - r[3];
+        float2 j2 = make_float2(0.f, 0.f);
+        const float w = l == 0 ? 0.5f : (l == H ? 0.25f : 1.f);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) add_sq(j2, r[i], w);
+        jp = df_val(j2);
+      }
+      float4* E = d.born_fold + size_t(fi) * 2 * nk * nk;
+      float4* T = E + size_t(nk) * nk;
+      const float2 S = rot * (r[0] + r[1]), S2 = rot * (r[2] + r[3]);
+      E[size_t(H) * nk + l] = pack2(S, S2);
+      E[size_t(l) * nk + H] = pack2(S2, S);
+      T[size_t(H) * nk + l] = pack2(S2, S);
+    }
+  }
+  if (RES) {
+    const double t = block_sum(jp, red);
+    if (threadIdx.x == 0) atomicAdd(d.gacc, t);
+  }
+}
+
+}  // namespace
+
+cudaError_t prepare_born() {
+  const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e = cudaFuncSetAttribute(born_fwd_df_kernel, attr, int(tile_smem<float4>()));
+  if (e != cudaSuccess) return e;
+  return cudaFuncSetAttribute(born_fwd_f64_kernel, attr, int(tile_smem<double2>()));
+}
+
+cudaError_t launch_born_prep(const Dev& d, cudaStream_t s) {
+  born_prep_kernel<<<unsigned(size_t(d.nf) * d.nk), PREP_THREADS, 0, s>>>(d, d.g64, d.nk, d.born_exp);
+  born_prep_kernel<<<d.N, PREP_THREADS, 0, s>>>(d, d.vfull, 0, d.born_exp + size_t(d.nf) * d.nk);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_born_v32(const Dev& d, cudaStream_t s) {
+  born_v32_kernel<<<d.N, PREP_THREADS, 0, s>>>(d);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_born_forward(const Dev& d, int f0, int nfc, cudaStream_t s) {
+  const dim3 g(tile_count(d.N / 2), nfc), ge((d.nk + 7) / 8, nfc);
+  if (d.precision == EDT_FP64) {
+    born_fwd_f64_kernel<<<g, BTHREADS, tile_smem<double2>(), s>>>(d, f0);
+    born_fwd_edge_f64_kernel<<<ge, 256, 0, s>>>(d, f0);
+  } else {
+    born_fwd_df_kernel<<<g, BTHREADS, tile_smem<float4>(), s>>>(d, f0);
+    born_fwd_edge_df_kernel<<<ge, 256, 0, s>>>(d, f0);
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_born_residual(const Dev& d, int f0, int nfc, bool model, cudaStream_t s) {
+  const dim3 g(tile_count(d.N / 2), nfc), ge((d.nk + 7) / 8, nfc);
+  if (model) {
+    born_resid_kernel<true><<<g, BTHREADS, tile_smem<float2>(), s>>>(d, f0);
+    born_resid_edge_kernel<true><<<ge, 256, 0, s>>>(d, f0);
+  } else {
+    born_resid_kernel<false><<<g, BTHREADS, 0, s>>>(d, f0);
+    born_resid_edge_kernel<false><<<ge, 256, 0, s>>>(d, f0);
+  }
+  return cudaGetLastError();
+}
+
+}  // namespace edt

@@ -46,6 +46,27 @@ __device__ __forceinline__ float2 shfl_df(float2 v, int src) {
   return make_float2(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
 }
 
+// exact product of two hi parts split as (rounded product, its error)
+__device__ __forceinline__ float two_prod_err(float a, float b, float p) { return fmaf(a, b, -p); }
+
+// a_h + a_l = (ph + pl)(qh + ql) for one complex depth value, to ~2^-44 relative
+__device__ __forceinline__ void cmul_df(float2 ph, float2 pl, float2 qh, float2 ql, float2& ah, float2& al) {
+  const float p1 = __fmul_rn(ph.x, qh.x), p2 = __fmul_rn(ph.y, qh.y);
+  const float e1 = two_prod_err(ph.x, qh.x, p1), e2 = two_prod_err(ph.y, qh.y, p2);
+  const float sr = __fsub_rn(p1, p2);
+  const float br = __fsub_rn(sr, p1);
+  const float er = __fadd_rn(__fsub_rn(p1, __fsub_rn(sr, br)), __fsub_rn(-p2, br));
+  const float cr = fmaf(ph.x, ql.x, fmaf(pl.x, qh.x, -fmaf(ph.y, ql.y, __fmul_rn(pl.y, qh.y))));
+  const float p3 = __fmul_rn(ph.x, qh.y), p4 = __fmul_rn(ph.y, qh.x);
+  const float e3 = two_prod_err(ph.x, qh.y, p3), e4 = two_prod_err(ph.y, qh.x, p4);
+  const float si = __fadd_rn(p3, p4);
+  const float bi = __fsub_rn(si, p3);
+  const float ei = __fadd_rn(__fsub_rn(p3, __fsub_rn(si, bi)), __fsub_rn(p4, bi));
+  const float ci = fmaf(ph.x, ql.y, fmaf(pl.x, qh.y, fmaf(ph.y, ql.x, __fmul_rn(pl.y, qh.x))));
+  ah = make_float2(sr, si);
+  al = make_float2(((e1 - e2) + er) + cr, ((e3 + e4) + ei) + ci);
+}
+
 // 1 / sqrt(a) for a double-float a > 0: the FP32 estimate y0 and one Newton step,
 // y = y0 - y0 e / 2 with e = a y0^2 - 1 formed by fused multiply-adds on the exact square
 // y0^2 = ph + pl (each fma rounds a quantity of order 2^-22 once, so e carries ~2^-46 absolute

@@ -104,7 +104,7 @@ struct edt_ctx {
   void* ws = nullptr;
   Region r_fc, r_ltop, r_lvel, r_zl, r_zo, r_rows, r_roff, r_roffmf, r_band, r_bcol, r_cpre, r_kval, r_pairm, r_fjoff, r_fjent, r_jact, r_jmap, r_Gs, r_U, r_Dw, r_A32, r_tw64, r_tw32, r_segm, r_segr0,
       r_segn, r_ctas, r_mslot, r_zo32, r_fc32, r_coef, r_coef32, r_g64, r_g32, r_g32lo, r_rowmax, r_gscale, r_X, r_Dst, r_Vst, r_rhs, r_gent, r_gpart, r_G,
-      r_dinv, r_L32, r_dinv32, r_b, r_tr, r_tpart, r_x, r_r, r_rpart, r_rowc, r_xmu, r_gam, r_tref, r_treoff, r_vhat, r_vfull, r_gscr, r_adj, r_gacc, r_gcpart, r_status, r_flags,
+      r_dinv, r_L32, r_dinv32, r_b, r_tr, r_tpart, r_x, r_r, r_rpart, r_rowc, r_xmu, r_gam, r_tref, r_treoff, r_vhat, r_vfull, r_gscr, r_adj, r_gacc, r_gcpart, r_bexp, r_bfold, r_status, r_flags,
       r_kzP, r_kzp, r_kzgoff, r_kzvoff, r_kzG, r_kzT, r_kzb, r_kzx;
   Dev dev{};
   cudaStream_t last_stream = nullptr;
@@ -690,12 +690,13 @@ void layout(edt_ctx* c) {
                        ? ns * size_t(refine_stride(c->rows_max_sub)) * nz * 2 * sizeof(double) : 0);
   take(c->r_vhat, ns * nz * sizeof(double2));
   take(c->r_vfull, (c->win ? nxy : N) * nz * sizeof(double2));
-  // misfit gradients: line geometry, mixed path (their dJ/dg buffer aliases r_g64, which
-  // holds nf (N/2 + 1) nz complex doubles >= nf N nz complex floats)
+  // misfit gradients: line geometry, mixed path (their dJ/dg buffer aliases r_g64)
   const bool grad = !c->win && mixed && c->nlayer <= GRAD_MAX_LAYERS && N >= 64;
   take(c->r_gscr, grad ? nf * size_t(c->nlayer) * 8 * nk * sizeof(double2) : 0);
   take(c->r_adj, grad ? size_t(N) * nz * sizeof(double2) : 0);
   take(c->r_gacc, grad ? size_t(1 + c->nlayer) * sizeof(double) : 0);
+  take(c->r_bexp, mixed && !c->win ? (nf * nk + N) * sizeof(int) : 0);
+  take(c->r_bfold, grad ? size_t(c->fchunk) * 2 * nk * nk * sizeof(float4) : 0);
   take(c->r_gcpart, grad ? size_t(nf) * ((nk + 127) / 128) * 4 * c->nlayer * sizeof(double) : 0);
   const bool rg = ref_grad_planned(c);
   take(c->r_rowc, rg ? std::max<size_t>(R, 1) * 2 * sizeof(float4) : 0);
@@ -803,6 +804,8 @@ void bind(edt_ctx* c) {
   d.adj = c->r_adj.bytes ? at<double2*>(c, c->r_adj) : nullptr;
   d.gacc = c->r_gacc.bytes ? at<double*>(c, c->r_gacc) : nullptr;
   d.gcpart = c->r_gcpart.bytes ? at<double*>(c, c->r_gcpart) : nullptr;
+  d.born_exp = c->r_bexp.bytes ? at<int*>(c, c->r_bexp) : nullptr;
+  d.born_fold = c->r_bfold.bytes ? at<float4*>(c, c->r_bfold) : nullptr;
   d.gbar = c->r_gscr.bytes ? reinterpret_cast<float2*>(d.g64) : nullptr;
   d.rowc = c->r_rowc.bytes ? at<float4*>(c, c->r_rowc) : nullptr;
   d.xmu = c->r_xmu.bytes ? at<float4*>(c, c->r_xmu) : nullptr;
@@ -1047,7 +1050,7 @@ int edt_set_workspace(edt_ctx* c, void* ws, size_t bytes) {
   }
   if (c->variant) EDT_TRY(prepare_variants(c->nz));
   EDT_TRY(prepare_fft(c->dev));
-  EDT_TRY(prepare_grad(c->dev));
+  EDT_TRY(prepare_born());
   EDT_TRY(prepare_chol(c->dev));
   if (c->cfg.precision == EDT_MIXED) EDT_TRY(prepare_gram_tc(c->dev));
   if (c->band_mode) EDT_TRY(prepare_band(c->dev));
@@ -1533,10 +1536,11 @@ int edt_get_stats(edt_ctx* c, edt_stats* o) {
                              (c->ny > 1 ? 4 : 3);
   }
   o->freq_chunk = c->band_mode ? c->band_maxplanes : c->fchunk;
-  // misfit gradient: green (3), zero, lateral DFT, per chunk transform (2) and three
-  // contractions, depth march forward / field / reversed (3), inverse lateral DFT, finalize
+  // misfit gradient: green (3), zero, lateral DFT and its FP32 copy, per chunk transform (2), the
+  // residual (2) and two contractions, depth march forward / field / reversed (3), inverse
+  // lateral DFT, finalize
   o->launches_per_grad = grad_supported(c->dev) && c->fchunk > 0
-                             ? 3 + 2 + 5 * ((c->nf + c->fchunk - 1) / c->fchunk) + 5 : 0;
+                             ? 3 + 3 + 6 * ((c->nf + c->fchunk - 1) / c->fchunk) + 5 : 0;
   o->gram_rows_padded = 0;
   for (long long n : c->seg_nrow) o->gram_rows_padded += (n + TC_KC - 1) / TC_KC * TC_KC;
   if (c->ws) {

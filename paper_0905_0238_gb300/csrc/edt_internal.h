@@ -159,7 +159,11 @@ struct Dev {
   double2* adj;                 // [N][nz] Ahat = F^H R2 summed over frequencies
   double* gacc;                 // [1 + nlayer] sum |R2|^2
   double* gcpart;               // [warps of the reverse march][nlayer] partial dJ/dc_l
-  float2* gbar;                 // [nf][N][nz] dJ/dg per full lateral index (aliases g64)
+  float2* gbar;                 // [nf][nk][nz] dJ/dg per table row (aliases g64)
+  // spectral Born operator on the folded table index (csrc/born.cu)
+  int* born_exp;                // [nf * nk + N] power-of-two exponents of the forward model's
+                                //   scaled Green's-table rows and Vhat rows
+  float4* born_fold;            // [fchunk][2][nk][nk] folded residual (or data) planes E, T
   // dL/dc through the damped solve (line geometry, mixed path)
   float4* rowc;                 // [rows_solved][2] per row (u_+, u_-) = d - A x, (v_+, v_-) = -A mu
   float4* xmu;                  // [nsub][nz] (x_+, x_-, mu_+, mu_-) in FP32
@@ -257,6 +261,15 @@ cudaError_t launch_refine(const Dev& d, cudaStream_t s);
 int refine_stride(long long rows_max_sub);                      // refinement CTAs per subproblem, at most
 cudaError_t launch_refine_update(const Dev& d, cudaStream_t s);   // x += (LL^T)^-1 (r - lam x)
 cudaError_t launch_inverse(const Dev& d, void* V, int V_dtype, cudaStream_t s);
+// Spectral Born operator (csrc/born.cu): the chunk's planes X[fi][q][p] = F(p, q) from the FP64
+// table and vfull (mixed path: after launch_born_prep, which scales and splits both in place);
+// the folded planes of R2 = F - X (model; vfull as FP32 by launch_born_v32, sum |R2|^2 added to
+// gacc[0]) or of X itself.
+cudaError_t prepare_born();
+cudaError_t launch_born_prep(const Dev& d, cudaStream_t s);
+cudaError_t launch_born_v32(const Dev& d, cudaStream_t s);
+cudaError_t launch_born_forward(const Dev& d, int f0, int nfc, cudaStream_t s);
+cudaError_t launch_born_residual(const Dev& d, int f0, int nfc, bool model, cudaStream_t s);
 cudaError_t launch_forward(const Dev& d, const void* V, int V_dtype, void* D, int D_dtype,
                            cudaStream_t s);
 // vfull[m][z] = sum_x V[x][z] e^{-i k_m x} (FP64)
@@ -316,7 +329,6 @@ cudaError_t launch_solve_variant(const Dev& d, cudaStream_t s);
 cudaError_t prepare_fft(const Dev& d);
 cudaError_t prepare_chol(const Dev& d);
 cudaError_t prepare_gram_tc(const Dev& d);
-cudaError_t prepare_grad(const Dev& d);
 
 // Tensor-core Gram tiling (shared by host planning and the kernel).
 constexpr int TC_M = 128;              // MMA rows (depth unknowns per M tile)

@@ -12,8 +12,7 @@
 // completed by Vhat(-k_m) = conj Vhat(k_m) (eq. VSym), then
 // V(x, z) = (1/N) sum_m Vhat(k_m, z) e^{+i k_m x}, real part.
 //
-// Forward model (eqs. DMV/M read forward): D2(p, q) = s_f sum_j g(k_p,z_j) g(k_q,z_j)
-// Vhat(k_p - k_q, z_j), then the inverse of the data transform.
+// Forward model: the spectral Born operator (csrc/born.cu), then the inverse of the data transform.
 #include "edt_internal.h"
 #include "cplx.cuh"
 #include "wfft.cuh"
@@ -153,8 +152,8 @@ constexpr int WR_WARPS = 8;   // rows per block in the row kernel
 
 template <int P>
 __global__ void __launch_bounds__(WR_WARPS * 32) wfft_rows_kernel(Dev d, const void* in, int in_dtype,
-                                                                 float2* out, long long nrows, int sign,
-                                                                 float scale) {
+                                                                 void* out, int out_dtype, long long nrows,
+                                                                 int sign, float scale) {
   constexpr int N = 32 * P;
   __shared__ float2 sm[WR_WARPS][N + N / 16];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -168,11 +167,10 @@ __global__ void __launch_bounds__(WR_WARPS * 32) wfft_rows_kernel(Dev d, const v
 #pragma unroll
   for (int k1 = 0; k1 < P; ++k1) sm[warp][pd(k1 + brl)] = r[k1];
   __syncwarp();
-  float2* o = out + size_t(row) * N;
 #pragma unroll
   for (int j = 0; j < P; ++j) {
     const float2 v = sm[warp][pd(32 * j + lane)];
-    o[32 * j + lane] = make_float2(v.x * scale, v.y * scale);
+    store_c<float2>(out, out_dtype, size_t(row) * N + 32 * j + lane, make_float2(v.x * scale, v.y * scale));
   }
 }
 
@@ -207,10 +205,10 @@ __global__ void __launch_bounds__(WC * 32) wfft_cols_kernel(Dev d, float2* X, in
 }
 
 template <int P>
-cudaError_t wfft_rows_launch(const Dev& d, const void* in, int in_dtype, float2* out, long long nrows,
-                             int sign, float scale, cudaStream_t st) {
+cudaError_t wfft_rows_launch(const Dev& d, const void* in, int in_dtype, void* out, int out_dtype,
+                             long long nrows, int sign, float scale, cudaStream_t st) {
   const long long nb = (nrows + WR_WARPS - 1) / WR_WARPS;
-  wfft_rows_kernel<P><<<unsigned(nb), WR_WARPS * 32, 0, st>>>(d, in, in_dtype, out, nrows, sign, scale);
+  wfft_rows_kernel<P><<<unsigned(nb), WR_WARPS * 32, 0, st>>>(d, in, in_dtype, out, out_dtype, nrows, sign, scale);
   return cudaGetLastError();
 }
 
@@ -231,15 +229,15 @@ cudaError_t wfft_cols_prepare() {
 }
 
 // FP32 row / column transforms for N >= 32 (warp FFT); false if N is outside that range
-bool wfft_rows(const Dev& d, const void* in, int in_dtype, float2* out, long long nrows, int sign,
+bool wfft_rows(const Dev& d, const void* in, int in_dtype, void* out, int out_dtype, long long nrows, int sign,
                float scale, cudaStream_t st, cudaError_t* e) {
   switch (d.N) {
-    case 32: *e = wfft_rows_launch<1>(d, in, in_dtype, out, nrows, sign, scale, st); return true;
-    case 64: *e = wfft_rows_launch<2>(d, in, in_dtype, out, nrows, sign, scale, st); return true;
-    case 128: *e = wfft_rows_launch<4>(d, in, in_dtype, out, nrows, sign, scale, st); return true;
-    case 256: *e = wfft_rows_launch<8>(d, in, in_dtype, out, nrows, sign, scale, st); return true;
-    case 512: *e = wfft_rows_launch<16>(d, in, in_dtype, out, nrows, sign, scale, st); return true;
-    case 1024: *e = wfft_rows_launch<32>(d, in, in_dtype, out, nrows, sign, scale, st); return true;
+    case 32: *e = wfft_rows_launch<1>(d, in, in_dtype, out, out_dtype, nrows, sign, scale, st); return true;
+    case 64: *e = wfft_rows_launch<2>(d, in, in_dtype, out, out_dtype, nrows, sign, scale, st); return true;
+    case 128: *e = wfft_rows_launch<4>(d, in, in_dtype, out, out_dtype, nrows, sign, scale, st); return true;
+    case 256: *e = wfft_rows_launch<8>(d, in, in_dtype, out, out_dtype, nrows, sign, scale, st); return true;
+    case 512: *e = wfft_rows_launch<16>(d, in, in_dtype, out, out_dtype, nrows, sign, scale, st); return true;
+    case 1024: *e = wfft_rows_launch<32>(d, in, in_dtype, out, out_dtype, nrows, sign, scale, st); return true;
     default: return false;
   }
 }
@@ -344,44 +342,6 @@ __global__ void lateral_dft_kernel(Dev d, const void* V, int V_dtype) {
   }
 }
 
-// D2[f][q][p] = s_f sum_j g(|p'|, j) g(|q'|, j) Vhat((p - q) mod N, j): 16 x 16 (p, q) tile
-// per block, depth in chunks of 32 staged in shared memory.
-template <typename T>
-__global__ void born_spectral_kernel(Dev d, cplx_t<T>* X, int f0) {
-  using T2 = cplx_t<T>;
-  constexpr int TP = 16, ZC = 32;
-  __shared__ double2 gp[TP][ZC], gq[TP][ZC], vh[2 * TP][ZC];
-  const int N = d.N, f = f0 + blockIdx.z;   // X holds the chunk's planes only
-  const int p0 = blockIdx.x * TP, q0 = blockIdx.y * TP;
-  const int tp = threadIdx.x & (TP - 1), tq = threadIdx.x / TP;
-  double2 acc = make_double2(0.0, 0.0);
-  const double2* g = d.g64 + size_t(f) * d.nk * d.nz;
-  for (int zc = 0; zc < d.nz; zc += ZC) {
-    for (int e = threadIdx.x; e < TP * ZC; e += blockDim.x) {
-      int i = e / ZC, j = e - i * ZC, z = zc + j;
-      int pa = p0 + i, qa = q0 + i;
-      int np = pa <= N / 2 ? pa : N - pa, nq = qa <= N / 2 ? qa : N - qa;
-      gp[i][j] = z < d.nz ? g[size_t(np) * d.nz + z] : make_double2(0.0, 0.0);
-      gq[i][j] = z < d.nz ? g[size_t(nq) * d.nz + z] : make_double2(0.0, 0.0);
-    }
-    for (int e = threadIdx.x; e < 2 * TP * ZC; e += blockDim.x) {
-      int i = e / ZC, j = e - i * ZC, z = zc + j;
-      int m = (p0 - q0 - (TP - 1) + i) & (N - 1);     // m = p - q covers [p0-q0-15, p0-q0+15]
-      vh[i][j] = z < d.nz ? d.vfull[size_t(m) * d.nz + z] : make_double2(0.0, 0.0);
-    }
-    __syncthreads();
-    const int mi = tp - tq + (TP - 1);
-#pragma unroll 4
-    for (int j = 0; j < ZC; ++j) acc = acc + gp[tp][j] * gq[tq][j] * vh[mi][j];
-    __syncthreads();
-  }
-  const FreqConst fc = d.fc[f];
-  double2 om = make_double2(fc.om_re, fc.om_im);
-  double2 sf = (d.dz / d.dx) * (om * om);
-  acc = sf * acc;
-  X[size_t(blockIdx.z) * N * N + size_t(q0 + tq) * N + p0 + tp] = cmk(T(acc.x), T(acc.y));
-}
-
 // out[x][z] = scale Re sum_m in[m][z] e^{+i k_m x}: one block per z tile, every m given.
 __global__ void lateral_idft_kernel(Dev d, const double2* in, double scale, void* out, int out_dtype) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -414,7 +374,7 @@ cudaError_t launch_transform(const Dev& d, const void* D, int D_dtype, int f0, i
   const void* Dc = static_cast<const char*>(D) + size_t(f0) * d.N * d.N * esz;
   const long long nrows = (long long)nfc * d.N;
   cudaError_t e = cudaSuccess;
-  if (sizeof(T) == 4 && wfft_rows(d, Dc, D_dtype, reinterpret_cast<float2*>(d.X), nrows, -1, 1.f, s, &e)) {
+  if (sizeof(T) == 4 && wfft_rows(d, Dc, D_dtype, d.X, EDT_C64, nrows, -1, 1.f, s, &e)) {
     if (e != cudaSuccess) return e;
     wfft_cols(d, reinterpret_cast<float2*>(d.X), nfc, +1, 1.f, s, &e);
     return e;
@@ -480,29 +440,35 @@ cudaError_t launch_lateral_idft_real(const Dev& d, const double2* in, double sca
   return cudaGetLastError();
 }
 
+// Columns (sign -) then rows (sign +) of the chunk's planes X[fi][q][p] into D[f0 + fi], each
+// transform times `scale`: the data transform undone (scale 1/N) or its adjoint (scale 1).
 template <typename T>
-cudaError_t forward_chunk(const Dev& d, void* D, int D_dtype, int f0, int nfc, cudaStream_t s) {
+static cudaError_t transform_back(const Dev& d, void* D, int D_dtype, int f0, int nfc, T scale, cudaStream_t s) {
   using T2 = cplx_t<T>;
   const int xdtype = sizeof(T) == 4 ? EDT_C64 : EDT_C128;
   const size_t esz = D_dtype == EDT_C64 ? sizeof(float2) : sizeof(double2);
   void* Dc = static_cast<char*>(D) + size_t(f0) * d.N * d.N * esz;
-  dim3 g(d.N / 16, d.N / 16, nfc);
-  born_spectral_kernel<T><<<g, 256, 0, s>>>(d, reinterpret_cast<T2*>(d.X), f0);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  // inverse of the data transform: undo pass 2 (sign -, 1/N), then pass 1 (sign +, 1/N)
-  if ((e = cols_fft<T>(d, reinterpret_cast<T2*>(d.X), nfc, -1, T(1) / T(d.N), s)) != cudaSuccess) return e;
-  return rows_fft<T>(d, d.X, xdtype, Dc, D_dtype, (long long)nfc * d.N, +1, T(1) / T(d.N), s);
+  const long long nrows = (long long)nfc * d.N;
+  cudaError_t e = cudaSuccess;
+  if (sizeof(T) == 4 && wfft_cols(d, reinterpret_cast<float2*>(d.X), nfc, -1, float(scale), s, &e)) {
+    if (e != cudaSuccess) return e;
+    wfft_rows(d, d.X, EDT_C64, Dc, D_dtype, nrows, +1, float(scale), s, &e);
+    return e;
+  }
+  if ((e = cols_fft<T>(d, reinterpret_cast<T2*>(d.X), nfc, -1, scale, s)) != cudaSuccess) return e;
+  return rows_fft<T>(d, d.X, xdtype, Dc, D_dtype, nrows, +1, scale, s);
 }
 
-// Adjoint of the data transform on the chunk's planes X[fi][q][p] (FP32): the conjugate
-// transpose of pass 2 (sign -, unscaled) then of pass 1 (sign +, unscaled) into D[f0 + fi].
-cudaError_t launch_transform_adjoint(const Dev& d, void* D, int D_dtype, int f0, int nfc, cudaStream_t s) {
-  const size_t esz = D_dtype == EDT_C64 ? sizeof(float2) : sizeof(double2);
-  void* Dc = static_cast<char*>(D) + size_t(f0) * d.N * d.N * esz;
-  cudaError_t e = cols_fft<float>(d, reinterpret_cast<float2*>(d.X), nfc, -1, 1.f, s);
+template <typename T>
+cudaError_t forward_chunk(const Dev& d, void* D, int D_dtype, int f0, int nfc, cudaStream_t s) {
+  const cudaError_t e = launch_born_forward(d, f0, nfc, s);
   if (e != cudaSuccess) return e;
-  return rows_fft<float>(d, d.X, EDT_C64, Dc, D_dtype, (long long)nfc * d.N, +1, 1.f, s);
+  return transform_back<T>(d, D, D_dtype, f0, nfc, T(1) / T(d.N), s);
+}
+
+// Adjoint of the data transform on the chunk's planes X[fi][q][p] (FP32) into D[f0 + fi].
+cudaError_t launch_transform_adjoint(const Dev& d, void* D, int D_dtype, int f0, int nfc, cudaStream_t s) {
+  return transform_back<float>(d, D, D_dtype, f0, nfc, 1.f, s);
 }
 
 // Adjoint of the spectral Born model on one chunk of FP64 planes X[fi][q][p] = D2(p, q):
@@ -550,6 +516,7 @@ cudaError_t launch_forward(const Dev& d, const void* V, int V_dtype, void* D, in
   lateral_dft_kernel<<<(d.nz + INV_ZT - 1) / INV_ZT, 256, smem, s>>>(d, V, V_dtype);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
+  if (d.precision != EDT_FP64 && (e = launch_born_prep(d, s)) != cudaSuccess) return e;
   // the spectrum X holds one chunk of frequency planes at a time
   for (int f0 = 0; f0 < d.nf; f0 += d.fchunk) {
     const int nfc = std::min(d.fchunk, d.nf - f0);

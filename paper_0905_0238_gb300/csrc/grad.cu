@@ -21,15 +21,12 @@
 // The FP32 table of the mixed path holds sqrt|s_f| g, so s_f g_p g_q = ph_f g32_p g32_q with
 // ph_f = s_f/|s_f|, and dJ/dg = sqrt|s_f| dJ/dg32 -> the factor 2 c_J ph_f sqrt|s_f| below.
 //
-// Kernels per chunk of frequency planes (X holds D2, then R2 in place):
-//   grad_residual  (p, q) tiles of 64 x 64, 4 x 4 per thread, depth in chunks of 32 in
-//                  shared memory: R2 and the partial sums of |R2|^2;
-//   grad_vhat      (m, j) outputs, 8 consecutive m per thread and one j per lane; the
-//                  thread walks p, so its 8 legs q = p - m slide by one per step and stay
-//                  in registers: Ahat accumulated across frequencies in FP64;
-//   grad_gbar      (n, j) outputs, 8 consecutive n per thread walking m (legs q = n - m
-//                  slide the same way): S1 and S2 together (the same legs and Vhat) into
-//                  the gbar buffer;
+// Kernels per chunk of frequency planes (X holds D2):
+//   born_resid     (csrc/born.cu) R2, sum |R2|^2 and the folded planes: one value per class of
+//                  entries that share a kernel row product;
+//   grad_vhat      (m, j) outputs: Ahat(m) + conj Ahat(-m), m = 0..N/2, accumulated across
+//                  frequencies in FP64;
+//   grad_gbar      (n, j) outputs on the table index n = 0..N/2: S1 and S2 of both signs;
 // then once, in FP64: grad_march (per (f, k): the recursion forward), grad_field (per
 // (f, k, layer): the field's depths of that layer, reversed), grad_reverse (per (f, k): the
 // two recursions reversed, then the per-layer sums); the inverse lateral DFT of Ahat and a
@@ -51,32 +48,6 @@ __device__ __forceinline__ double2 crcp(double2 b) {
   return cmk(b.x * r, -b.y * r);
 }
 
-// acc += a * b (complex)
-__device__ __forceinline__ void cmac(float2& acc, float2 a, float2 b) {
-  acc.x = fmaf(a.x, b.x, acc.x);
-  acc.x = fmaf(-a.y, b.y, acc.x);
-  acc.y = fmaf(a.x, b.y, acc.y);
-  acc.y = fmaf(a.y, b.x, acc.y);
-}
-// acc += conj(a) * b
-__device__ __forceinline__ void cmac_conj(float2& acc, float2 a, float2 b) {
-  acc.x = fmaf(a.x, b.x, acc.x);
-  acc.x = fmaf(a.y, b.y, acc.x);
-  acc.y = fmaf(a.x, b.y, acc.y);
-  acc.y = fmaf(-a.y, b.x, acc.y);
-}
-
-__device__ __forceinline__ double block_sum(double v, double* red) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-  if (lane == 0) red[w] = v;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int i = 0; i < nw; ++i) t += red[i];
-  return t;
-}
-
 __global__ void grad_zero_kernel(Dev d) {
   const size_t n = size_t(d.N) * d.nz;
   for (size_t i = size_t(blockIdx.x) * blockDim.x + threadIdx.x; i < n; i += size_t(gridDim.x) * blockDim.x)
@@ -85,221 +56,185 @@ __global__ void grad_zero_kernel(Dev d) {
     for (int i = threadIdx.x; i <= d.nlayer; i += blockDim.x) d.gacc[i] = 0.0;
 }
 
-// ---- residual R2 = ph_f sum_j g32_p g32_q Vhat(p - q) - D2, and sum |R2|^2 ------------------
-constexpr int RT = 64, RJC = 32, RTM = 2 * RT - 1;
-constexpr size_t RES_SMEM = (size_t(2) * RJC * (RT + 1) + size_t(RJC) * (RTM + 2)) * sizeof(float2);
-
-__global__ void __launch_bounds__(256, 3) grad_residual_kernel(Dev d, int f0) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2 (*gp)[RT + 1] = reinterpret_cast<float2 (*)[RT + 1]>(smem_raw);
-  float2 (*gq)[RT + 1] = reinterpret_cast<float2 (*)[RT + 1]>(smem_raw + size_t(RJC) * (RT + 1) * sizeof(float2));
-  float2 (*vh)[RTM + 2] = reinterpret_cast<float2 (*)[RTM + 2]>(smem_raw + size_t(2) * RJC * (RT + 1) * sizeof(float2));
-  __shared__ double red[8];
-  const int N = d.N, fi = blockIdx.z, f = f0 + fi;
-  const int p0 = blockIdx.x * RT, q0 = blockIdx.y * RT;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-  const float2* g = d.g32 + size_t(f) * d.nk * d.nzs;
-  float2 acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = make_float2(0.f, 0.f);
-  for (int j0 = 0; j0 < d.nz; j0 += RJC) {
-    for (int e = threadIdx.x; e < RT * RJC; e += blockDim.x) {
-      const int i = e / RJC, jj = e - i * RJC, j = j0 + jj;
-      const bool in = j < d.nz;
-      gp[jj][i] = in ? g[size_t(tab_index(p0 + i, N)) * d.nzs + j] : make_float2(0.f, 0.f);
-      gq[jj][i] = in ? g[size_t(tab_index(q0 + i, N)) * d.nzs + j] : make_float2(0.f, 0.f);
-    }
-    for (int e = threadIdx.x; e < RTM * RJC; e += blockDim.x) {
-      const int i = e / RJC, jj = e - i * RJC, j = j0 + jj;
-      const int m = (p0 - q0 - (RT - 1) + i) & (N - 1);
-      const double2 v = j < d.nz ? d.vfull[size_t(m) * d.nz + j] : make_double2(0.0, 0.0);
-      vh[jj][i] = make_float2(float(v.x), float(v.y));
-    }
-    __syncthreads();
-#pragma unroll 2
-    for (int jj = 0; jj < RJC; ++jj) {
-      float2 ga[4], gb[4], v[7];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) ga[a] = gp[jj][tx + 16 * a];
-#pragma unroll
-      for (int b = 0; b < 4; ++b) gb[b] = gq[jj][ty + 16 * b];
-      // p - q = tx - ty + 16 (a - b); slot p - q + RT - 1
-#pragma unroll
-      for (int t = 0; t < 7; ++t) v[t] = vh[jj][tx - ty + 16 * (t - 3) + RT - 1];
-#pragma unroll
-      for (int a = 0; a < 4; ++a)
-#pragma unroll
-        for (int b = 0; b < 4; ++b) cmac(acc[a][b], ga[a] * gb[b], v[a - b + 3]);
-    }
-    __syncthreads();
-  }
-  const FreqConst fc = d.fc[f];
-  const float2 ph = make_float2(float(fc.rot_re), float(-fc.rot_im));     // s_f / |s_f|
-  float2* X = reinterpret_cast<float2*>(d.X) + size_t(fi) * N * N;
-  double jp = 0.0;
-#pragma unroll
-  for (int b = 0; b < 4; ++b)
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      const size_t o = size_t(q0 + ty + 16 * b) * N + p0 + tx + 16 * a;   // X[q][p] = D2(p, q)
-      const float2 r = ph * acc[a][b] - X[o];
-      X[o] = r;
-      jp += double(r.x) * r.x + double(r.y) * r.y;
-    }
-  const double t = block_sum(jp, red);
-  if (threadIdx.x == 0) atomicAdd(d.gacc, t);
-}
-
-// ---- Ahat(m, j) += conj(ph_f) sum_p conj(g32_p g32_{p-m}) R2(p, p - m) -----------------------
-constexpr int VM = 64, VPC = 32, VQR = VPC + VM - 1, VLT = VQR + 2;   // VLT odd
-constexpr size_t VHAT_SMEM = (size_t(VPC) * 33 + size_t(VQR) * 33 + size_t(VPC) * VLT + 1) * sizeof(float2);
-static_assert(VLT % 2 == 1, "odd row length: each step's 8 residuals start 16-byte aligned");
+// ---- B(m, j) += sum over the classes of m of Re(a) U + Im(a) W ------------------------------
+// Every entry (p, q) of the plane appears once: the classes {(p, q), (-q, -p)} of m = p - q and
+// their mirror images {(q, p), (-p, -q)} of -m share a = g32_p g32_q, and V = Re sum Ahat(m)
+// e^{ikx} needs only B(m) = Ahat(m) + conj Ahat(-m) = conj(a) S + a conj(S'), m = 0..N/2, i.e.
+// U = S + conj S', W = -i (S - conj S') with four multiply-adds per class and depth.  For
+// m = 2 j or 2 j + 1 the classes are p = t + j (+ 1), q = t - j, t = 0..N/2 (t < N/2 for odd m),
+// so the legs of a thread's four j slide by one per step of t and stay in registers; the ends
+// t = 0, N/2 of even m are their own partners, and m = 0, N/2 their own mirror images.
+constexpr int VJ = 32, VTC = 16;           // j per CTA (4 per warp), t per staged chunk
 
 __global__ void __launch_bounds__(256, 3) grad_vhat_kernel(Dev d, int f0) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  float2 (*gps)[33] = reinterpret_cast<float2 (*)[33]>(smem_raw);
-  float2 (*gqs)[33] = reinterpret_cast<float2 (*)[33]>(smem_raw + size_t(VPC) * 33 * sizeof(float2));
-  // residual tile transposed, rsT[pl * VLT + qi] = R2(p0 + pl, q(qi)): at step pl a thread's 8
-  // legs are the run qi = pl - 8w + 56 .. pl - 8w + 63, whose start pl (VLT + 1) - 8w + 56 is
-  // even, so the run is read with four 16-byte broadcast loads
-  constexpr size_t RS_OFF = (size_t(VPC + VQR) * 33 + 1) & ~size_t(1);   // even: 16-byte aligned
-  float2* rsT = reinterpret_cast<float2*>(smem_raw + RS_OFF * sizeof(float2));
-  const int N = d.N, fi = blockIdx.z, f = f0 + fi;
-  const int m0 = blockIdx.x * VM, j0 = blockIdx.y * 32;
+  __shared__ float2 gps[VTC + VJ][32];     // rows p = t0 + j0 + i
+  __shared__ float2 gqs[VTC + VJ - 1][32]; // rows q = t0 - j0 - (VJ - 1) + i
+  __shared__ float4 cf[VTC][2 * VJ];       // (U, W) of (t, m)
+  const int N = d.N, H = N / 2, msk = N - 1, nk = d.nk, fi = blockIdx.z, f = f0 + fi;
+  const int jt = blockIdx.x * VJ, z0 = blockIdx.y * 32;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int j = j0 + lane;
-  const float2* g = d.g32 + size_t(f) * d.nk * d.nzs;
-  const float2* X = reinterpret_cast<const float2*>(d.X) + size_t(fi) * N * N;
+  const int z = z0 + lane;
+  const float2* g = d.g32 + size_t(f) * nk * d.nzs;
+  const float4* E = d.born_fold + size_t(fi) * 2 * nk * nk;
+  const float4* T = E + size_t(nk) * nk;
+  const bool live = 2 * (jt + 4 * w) <= H;                 // the same in the whole warp
   float2 acc[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) acc[k] = make_float2(0.f, 0.f);
-  for (int p0 = 0; p0 < N; p0 += VPC) {
-    // rows qi <-> q = p0 - m0 - (VM - 1) + qi (mod N)
-    for (int e = threadIdx.x; e < VQR * 32; e += blockDim.x) {
-      const int qi = e >> 5, jl = e & 31, jj = j0 + jl;
-      const int q = (p0 - m0 - (VM - 1) + qi) & (N - 1);
-      gqs[qi][jl] = jj < d.nz ? g[size_t(tab_index(q, N)) * d.nzs + jj] : make_float2(0.f, 0.f);
+  for (int t0 = 0; t0 <= H; t0 += VTC) {
+    for (int e = threadIdx.x; e < (VTC + VJ) * 32; e += blockDim.x) {
+      const int i = e >> 5, zz = z0 + (e & 31);
+      gps[i][e & 31] = zz < d.nz ? g[size_t(tab_index((t0 + jt + i) & msk, N)) * d.nzs + zz] : make_float2(0.f, 0.f);
+      if (i < VTC + VJ - 1)
+        gqs[i][e & 31] = zz < d.nz ? g[size_t(tab_index((t0 - jt - (VJ - 1) + i) & msk, N)) * d.nzs + zz]
+                                   : make_float2(0.f, 0.f);
     }
-    for (int e = threadIdx.x; e < VPC * 32; e += blockDim.x) {
-      const int pl = e >> 5, jl = e & 31, jj = j0 + jl;
-      gps[pl][jl] = jj < d.nz ? g[size_t(tab_index(p0 + pl, N)) * d.nzs + jj] : make_float2(0.f, 0.f);
-    }
-    for (int e = threadIdx.x; e < VQR * VPC; e += blockDim.x) {
-      const int qi = e / VPC, pl = e - qi * VPC;
-      const int q = (p0 - m0 - (VM - 1) + qi) & (N - 1);
-      rsT[pl * VLT + qi] = X[size_t(q) * N + p0 + pl];
+    for (int e = threadIdx.x; e < VTC * 2 * VJ; e += blockDim.x) {
+      const int tt = e / (2 * VJ), mi = e - tt * (2 * VJ);
+      const int t = t0 + tt, m = 2 * jt + mi, odd = m & 1, j = m >> 1;
+      float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (m <= H && t <= H - odd) {
+        int p = t + j + odd, q = t - j;
+        if (p > H) p -= N;                                  // signed indices, never both negative
+        const float4 c = p >= 0 && q >= 0 ? E[size_t(p) * nk + q]
+                                          : T[size_t(p >= 0 ? p : -p) * nk + (q >= 0 ? q : -q)];
+        float2 S = make_float2(c.x, c.y), S2 = make_float2(c.z, c.w);
+        if (p < 0) { const float2 x = S; S = S2; S2 = x; }
+        float wt = !odd && (t == 0 || t == H) ? 0.5f : 1.f;
+        if (m == 0 || m == H) wt *= 0.5f;
+        o = make_float4(wt * (S.x + S2.x), wt * (S.y - S2.y), wt * (S.y + S2.y), wt * (S2.x - S.x));
+      }
+      cf[tt][mi] = o;
     }
     __syncthreads();
-    // thread's m_k = m0 + 8 w + k; at p = p0 + pl its leg q_k = p - m_k sits in row
-    // qi = pl - 8 w - k + VM - 1, one row further per step of p: a sliding window
-    float2 win[8];
+    if (live) {
+      float2 P[5], Q[4];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) win[k] = gqs[VM - 1 - 8 * w - k][lane];
+      for (int i = 0; i < 5; ++i) P[i] = gps[4 * w + i][lane];
 #pragma unroll
-    for (int pl = 0; pl < VPC; ++pl) {
-      if (pl > 0) {
+      for (int i = 0; i < 4; ++i) Q[i] = gqs[VJ - 1 - 4 * w - i][lane];
 #pragma unroll
-        for (int k = 7; k > 0; --k) win[k] = win[k - 1];
-        win[0] = gqs[pl + VM - 1 - 8 * w][lane];
-      }
-      const float2 gpv = gps[pl][lane];
-      const float4* r4 = reinterpret_cast<const float4*>(rsT + pl * VLT + pl + VM - 8 - 8 * w);
+      for (int tt = 0; tt < VTC; ++tt) {
+        if (tt > 0) {
+          if (t0 + tt > H) break;
 #pragma unroll
-      for (int h = 0; h < 4; ++h) {                      // legs k = 7 - 2h (.xy) and 6 - 2h (.zw)
-        const float4 rr = r4[h];
-        cmac_conj(acc[7 - 2 * h], gpv * win[7 - 2 * h], make_float2(rr.x, rr.y));
-        cmac_conj(acc[6 - 2 * h], gpv * win[6 - 2 * h], make_float2(rr.z, rr.w));
+          for (int i = 0; i < 4; ++i) P[i] = P[i + 1];
+          P[4] = gps[tt + 4 * w + 4][lane];
+#pragma unroll
+          for (int i = 3; i > 0; --i) Q[i] = Q[i - 1];
+          Q[0] = gqs[tt + VJ - 1 - 4 * w][lane];
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int o = 0; o < 2; ++o) {
+            const float4 c = cf[tt][8 * w + 2 * i + o];
+            const float2 a = P[i + o] * Q[i];
+            float2& s = acc[2 * i + o];
+            s.x = fmaf(a.x, c.x, fmaf(a.y, c.z, s.x));
+            s.y = fmaf(a.x, c.y, fmaf(a.y, c.w, s.y));
+          }
       }
     }
     __syncthreads();
   }
-  if (j < d.nz) {
-    const FreqConst fc = d.fc[f];
-    const double2 cph = make_double2(fc.rot_re, fc.rot_im);               // conj(s_f)/|s_f|
+  if (z < d.nz) {
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
-      const double2 v = cph * make_double2(double(acc[k].x), double(acc[k].y));
-      double* o = reinterpret_cast<double*>(d.adj + size_t(m0 + 8 * w + k) * d.nz + j);
-      atomicAdd(o, v.x);
-      atomicAdd(o + 1, v.y);
+      const int m = 2 * (jt + 4 * w) + k;
+      if (m > H) continue;
+      double* o = reinterpret_cast<double*>(d.adj + size_t(m) * d.nz + z);
+      atomicAdd(o, double(acc[k].x));
+      atomicAdd(o + 1, double(acc[k].y));
     }
   }
 }
 
-// ---- S1 + S2 at (n, j): sum_m [conj(R2(n, n - m)) Vhat(m) + conj(R2(n - m, n)) conj(Vhat(m))]
-//      g32_{n-m}; gbar_f(n, j) = 2 c_J ph_f sqrt|s_f| (S1 + S2) ----------------------------------
+// ---- gbar_f(n, j), n = 0..N/2 -----------------------------------------------------------------
+// The entries whose row a holds g_n are, for every signed q, the class of (n, q) and its mirror
+// image: dJ/dg32_n = 2 c_J sum_q g32_q [C1 Re Vhat(n - q) + C2 Im Vhat(n - q)] with
+// C1 = conj(S + S'), C2 = i conj(S - S') (the folded values carry conj(s_f)/|s_f|); n = 0 and
+// N/2 meet every class twice.  8 consecutive n per thread walking m = n - q, one depth per lane:
+// the legs q = n - m slide by one per step, Vhat(m) is common to the eight.
 constexpr int GA = 64, GMC = 16, GQR = GA + GMC - 1;
-constexpr size_t GBAR_SMEM = (size_t(2) * GMC * GA + size_t(GQR) * 33 + size_t(GMC) * 33) * sizeof(float2);
 
 __global__ void __launch_bounds__(256, 3) grad_gbar_kernel(Dev d, int f0) {
-  extern __shared__ __align__(16) unsigned char smem_raw[];
-  // bs[2][GMC][GA] first (16-byte aligned rows for the float4 reads): [0] R2(n, q), [1] R2(q, n)
-  float2 (*bs)[GMC][GA] = reinterpret_cast<float2 (*)[GMC][GA]>(smem_raw);
-  float2 (*gqs)[33] = reinterpret_cast<float2 (*)[33]>(smem_raw + size_t(2) * GMC * GA * sizeof(float2));
-  float2 (*ws)[33] = reinterpret_cast<float2 (*)[33]>(smem_raw + (size_t(2) * GMC * GA + size_t(GQR) * 33) * sizeof(float2));
-  const int N = d.N, fi = blockIdx.z, f = f0 + fi;
+  __shared__ float4 cf[GMC][GA + 1];
+  __shared__ float2 gqs[GQR][32];
+  __shared__ float2 ws[GMC][32];
+  const int N = d.N, H = N / 2, msk = N - 1, nk = d.nk, fi = blockIdx.z, f = f0 + fi;
   const int a0 = blockIdx.x * GA, j0 = blockIdx.y * 32;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int j = j0 + lane;
-  const float2* g = d.g32 + size_t(f) * d.nk * d.nzs;
-  const float2* X = reinterpret_cast<const float2*>(d.X) + size_t(fi) * N * N;
-  float2 acc[8];
+  const float2* g = d.g32 + size_t(f) * nk * d.nzs;
+  const float2* vh = reinterpret_cast<const float2*>(d.vfull);     // row m at 2 nz m
+  const float4* E = d.born_fold + size_t(fi) * 2 * nk * nk;
+  const float4* T = E + size_t(nk) * nk;
+  const bool live = a0 + 8 * w <= H;                       // the same in the whole warp
+  float2 tot[8];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) acc[k] = make_float2(0.f, 0.f);
+  for (int k = 0; k < 8; ++k) tot[k] = make_float2(0.f, 0.f);
   for (int mc = 0; mc < N; mc += GMC) {
     // rows qi <-> q = a0 - mc - (GMC - 1) + qi (mod N)
     for (int e = threadIdx.x; e < GQR * 32; e += blockDim.x) {
-      const int qi = e >> 5, jl = e & 31, jj = j0 + jl;
-      const int q = (a0 - mc - (GMC - 1) + qi) & (N - 1);
-      gqs[qi][jl] = jj < d.nz ? g[size_t(tab_index(q, N)) * d.nzs + jj] : make_float2(0.f, 0.f);
+      const int qi = e >> 5, jj = j0 + (e & 31);
+      const int q = (a0 - mc - (GMC - 1) + qi) & msk;
+      gqs[qi][e & 31] = jj < d.nz ? g[size_t(tab_index(q, N)) * d.nzs + jj] : make_float2(0.f, 0.f);
     }
     for (int e = threadIdx.x; e < GMC * 32; e += blockDim.x) {
-      const int mi = e >> 5, jl = e & 31, jj = j0 + jl;
-      const double2 v = jj < d.nz ? d.vfull[size_t(mc + mi) * d.nz + jj] : make_double2(0.0, 0.0);
-      ws[mi][jl] = make_float2(float(v.x), float(v.y));
+      const int mi = e >> 5, jj = j0 + (e & 31);
+      ws[mi][e & 31] = jj < d.nz ? vh[size_t(mc + mi) * 2 * d.nz + jj] : make_float2(0.f, 0.f);
     }
     for (int e = threadIdx.x; e < GMC * GA; e += blockDim.x) {
-      const int mi = e / GA, al = e - mi * GA;
-      const int a = a0 + al, q = (a - mc - mi) & (N - 1);
-      bs[0][mi][al] = X[size_t(q) * N + a];           // R2(a, q) = X[q][a]
-      bs[1][mi][al] = X[size_t(a) * N + q];           // R2(q, a) = X[a][q]
+      const int al = e / GMC, mi = e - al * GMC, n = a0 + al;
+      float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (n <= H) {
+        int q = (n - mc - mi) & msk;
+        if (q > H) q -= N;
+        const float4 c = q >= 0 ? E[size_t(n) * nk + q] : T[size_t(n) * nk - q];
+        const float wt = n == 0 || n == H ? 0.5f : 1.f;
+        o = make_float4(wt * (c.x + c.z), -wt * (c.y + c.w), wt * (c.y - c.w), wt * (c.x - c.z));
+      }
+      cf[mi][al] = o;
     }
     __syncthreads();
-    // thread's n_k = a0 + 8 w + k; at m = mc + mi its leg q_k = n_k - m sits in row
-    // qi = 8 w + k - mi + GMC - 1, one row lower per step of m
-    float2 win[8];
+    if (live) {
+      // thread's n_k = a0 + 8 w + k; at m = mc + mi its leg q_k = n_k - m sits in row
+      // qi = 8 w + k - mi + GMC - 1, one row lower per step of m
+      float2 win[8], acc[8];
 #pragma unroll
-    for (int k = 0; k < 8; ++k) win[k] = gqs[8 * w + k + GMC - 1][lane];
+      for (int k = 0; k < 8; ++k) acc[k] = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int mi = 0; mi < GMC; ++mi) {
-      if (mi > 0) {
+      for (int k = 0; k < 8; ++k) win[k] = gqs[8 * w + k + GMC - 1][lane];
 #pragma unroll
-        for (int k = 7; k > 0; --k) win[k] = win[k - 1];
-        win[0] = gqs[8 * w - mi + GMC - 1][lane];
+      for (int mi = 0; mi < GMC; ++mi) {
+        if (mi > 0) {
+#pragma unroll
+          for (int k = 7; k > 0; --k) win[k] = win[k - 1];
+          win[0] = gqs[8 * w - mi + GMC - 1][lane];
+        }
+        const float2 v = ws[mi][lane];
+#pragma unroll
+        for (int k = 0; k < 8; ++k) {
+          const float4 c = cf[mi][8 * w + k];
+          const float tx = fmaf(c.x, v.x, c.z * v.y), ty = fmaf(c.y, v.x, c.w * v.y);
+          acc[k].x = fmaf(win[k].x, tx, fmaf(-win[k].y, ty, acc[k].x));
+          acc[k].y = fmaf(win[k].x, ty, fmaf(win[k].y, tx, acc[k].y));
+        }
       }
-      const float2 wv = ws[mi][lane], wc = make_float2(wv.x, -wv.y);
-      const float4* b0 = reinterpret_cast<const float4*>(&bs[0][mi][8 * w]);
-      const float4* b1 = reinterpret_cast<const float4*>(&bs[1][mi][8 * w]);
 #pragma unroll
-      for (int h = 0; h < 4; ++h) {
-        const float4 x0 = b0[h], x1 = b1[h];
-        cmac_conj(acc[2 * h], make_float2(x0.x, x0.y), win[2 * h] * wv);
-        cmac_conj(acc[2 * h], make_float2(x1.x, x1.y), win[2 * h] * wc);
-        cmac_conj(acc[2 * h + 1], make_float2(x0.z, x0.w), win[2 * h + 1] * wv);
-        cmac_conj(acc[2 * h + 1], make_float2(x1.z, x1.w), win[2 * h + 1] * wc);
-      }
+      for (int k = 0; k < 8; ++k) tot[k] = tot[k] + acc[k];
     }
     __syncthreads();
   }
   if (j < d.nz) {
-    const FreqConst fc = d.fc[f];
-    const double sc = 2.0 / (double(N) * N) * sqrt(fc.s_abs);
-    const float2 scale = make_float2(float(sc * fc.rot_re), float(-sc * fc.rot_im));
-    float2* G = d.gbar + size_t(f) * N * d.nz;
+    const float sc = float(2.0 / (double(N) * N) * sqrt(d.fc[f].s_abs));
+    float2* G = d.gbar + size_t(f) * nk * d.nz;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) G[size_t(a0 + 8 * w + k) * d.nz + j] = scale * acc[k];
+    for (int k = 0; k < 8; ++k) {
+      const int n = a0 + 8 * w + k;
+      if (n <= H) G[size_t(n) * d.nz + j] = make_float2(sc * tot[k].x, sc * tot[k].y);
+    }
   }
 }
 
@@ -386,7 +321,6 @@ __global__ void __launch_bounds__(128) grad_field_kernel(Dev d, const double2* g
   const int j0 = lower(l), j1 = lower(l + 1);
   double2 bA = cmk(0.0, 0.0), bRho = bA, bK = bA;
   if (j0 < j1) {
-    const int N = d.N;
     const double2 kl = gs_at(d, f, l, GS_KAP, k), Al = gs_at(d, f, l, GS_A, k);
     const bool last = l == J - 1;
     const double h = last ? 0.0 : d.layer_top[l + 1] - d.layer_top[l];
@@ -397,16 +331,14 @@ __global__ void __launch_bounds__(128) grad_field_kernel(Dev d, const double2* g
     double dd = d.z_off[j0];
     double2 P = cexp(cmk(-kl.y * dd, kl.x * dd));
     double2 Q = last ? cmk(0.0, 0.0) : cexp(cmk(-kl.y * (2.0 * h - dd), kl.x * (2.0 * h - dd)));
-    const float2* G = d.gbar + size_t(f) * N * d.nz;
-    const bool two = k > 0 && k < N / 2;
+    const float2* G = d.gbar + (size_t(f) * d.nk + k) * d.nz;
     for (int j = j0; j < j1; ++j) {
       dd = d.z_off[j];
       double2 gbar;
       if (gb64) {
         gbar = gb64[(size_t(f) * d.nk + k) * d.nz + j];
       } else {
-        float2 gb = G[size_t(k) * d.nz + j];
-        if (two) gb = gb + G[size_t(N - k) * d.nz + j];
+        const float2 gb = G[j];
         gbar = cmk(double(gb.x), double(gb.y));
       }
       const double2 gA = gbar * Al;
@@ -794,12 +726,8 @@ cudaError_t launch_invert_vjp(const Dev& d0, const void* Vbar, int Vbar_dtype, v
   return cudaSuccess;
 }
 
-cudaError_t prepare_grad(const Dev&) {
-  cudaError_t e = cudaFuncSetAttribute(grad_residual_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(RES_SMEM));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(grad_vhat_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(VHAT_SMEM));
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(grad_gbar_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(GBAR_SMEM));
+static dim3 vhat_grid(const Dev& d, int nfc) {          // m = 0..N/2, two per j
+  return dim3((d.N / 4 + 1 + VJ - 1) / VJ, (d.nz + 31) / 32, nfc);
 }
 
 bool grad_supported(const Dev& d) {
@@ -830,7 +758,8 @@ cudaError_t launch_adjoint(const Dev& d, const void* D, int D_dtype, void* V, in
   for (int f0 = 0; f0 < d.nf; f0 += d.fchunk) {
     const int nfc = std::min(d.fchunk, d.nf - f0);
     if ((e = launch_transform<float>(d, D, D_dtype, f0, nfc, s)) != cudaSuccess) return e;
-    grad_vhat_kernel<<<dim3(N / VM, (d.nz + 31) / 32, nfc), 256, VHAT_SMEM, s>>>(d, f0);
+    if ((e = launch_born_residual(d, f0, nfc, false, s)) != cudaSuccess) return e;
+    grad_vhat_kernel<<<vhat_grid(d, nfc), 256, 0, s>>>(d, f0);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return launch_lateral_idft_real(d, d.adj, scale, V, V_dtype, s);
@@ -842,14 +771,14 @@ cudaError_t launch_misfit_grad(const Dev& d, const void* V, int V_dtype, const v
   grad_zero_kernel<<<152, 256, 0, s>>>(d);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = launch_lateral_dft(d, V, V_dtype, s)) != cudaSuccess) return e;
+  if ((e = launch_born_v32(d, s)) != cudaSuccess) return e;
   const int N = d.N;
   for (int f0 = 0; f0 < d.nf; f0 += d.fchunk) {
     const int nfc = std::min(d.fchunk, d.nf - f0);
     if ((e = launch_transform<float>(d, D, D_dtype, f0, nfc, s)) != cudaSuccess) return e;
-    grad_residual_kernel<<<dim3(N / RT, N / RT, nfc), 256, RES_SMEM, s>>>(d, f0);
-    const dim3 gj(N / VM, (d.nz + 31) / 32, nfc);
-    grad_vhat_kernel<<<gj, 256, VHAT_SMEM, s>>>(d, f0);
-    grad_gbar_kernel<<<gj, 256, GBAR_SMEM, s>>>(d, f0);
+    if ((e = launch_born_residual(d, f0, nfc, true, s)) != cudaSuccess) return e;
+    grad_vhat_kernel<<<vhat_grid(d, nfc), 256, 0, s>>>(d, f0);
+    grad_gbar_kernel<<<dim3((d.nk + GA - 1) / GA, (d.nz + 31) / 32, nfc), 256, 0, s>>>(d, f0);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   const dim3 gk((d.nk + 127) / 128, d.nf);

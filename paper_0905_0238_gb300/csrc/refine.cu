@@ -15,6 +15,7 @@
 // refinement corrects the Gram's rounding.
 #include "edt_internal.h"
 #include "cplx.cuh"
+#include "dfloat.cuh"
 
 #include <algorithm>
 
@@ -149,27 +150,6 @@ __global__ void __launch_bounds__(RF_WARPS * 32) refine_kernel(Dev d) {
 //     and the a_l u go to a low-order FP32 sum; the lane sums are combined in FP64 across
 //     warps and blocks.
 // The error-free steps use the _rn intrinsics so that no multiply-add is contracted.
-
-// exact product of two hi parts split as (rounded product, its error)
-__device__ __forceinline__ float two_prod_err(float a, float b, float p) { return fmaf(a, b, -p); }
-
-// a_h + a_l = (ph + pl)(qh + ql) for one complex depth value, to ~2^-44 relative
-__device__ __forceinline__ void cmul_df(float2 ph, float2 pl, float2 qh, float2 ql, float2& ah, float2& al) {
-  const float p1 = __fmul_rn(ph.x, qh.x), p2 = __fmul_rn(ph.y, qh.y);
-  const float e1 = two_prod_err(ph.x, qh.x, p1), e2 = two_prod_err(ph.y, qh.y, p2);
-  const float sr = __fsub_rn(p1, p2);
-  const float br = __fsub_rn(sr, p1);
-  const float er = __fadd_rn(__fsub_rn(p1, __fsub_rn(sr, br)), __fsub_rn(-p2, br));
-  const float cr = fmaf(ph.x, ql.x, fmaf(pl.x, qh.x, -fmaf(ph.y, ql.y, __fmul_rn(pl.y, qh.y))));
-  const float p3 = __fmul_rn(ph.x, qh.y), p4 = __fmul_rn(ph.y, qh.x);
-  const float e3 = two_prod_err(ph.x, qh.y, p3), e4 = two_prod_err(ph.y, qh.x, p4);
-  const float si = __fadd_rn(p3, p4);
-  const float bi = __fsub_rn(si, p3);
-  const float ei = __fadd_rn(__fsub_rn(p3, __fsub_rn(si, bi)), __fsub_rn(p4, bi));
-  const float ci = fmaf(ph.x, ql.y, fmaf(pl.x, qh.y, fmaf(ph.y, ql.x, __fmul_rn(pl.y, qh.x))));
-  ah = make_float2(sr, si);
-  al = make_float2(((e1 - e2) + er) + cr, ((e3 + e4) + ei) + ci);
-}
 
 // TwoSum step: s + (the returned rounding error) = s_old + x exactly
 __device__ __forceinline__ float two_sum_acc(float& s, float x) {

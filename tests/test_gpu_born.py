@@ -1,0 +1,62 @@
+"""The spectral Born operator on the folded table index (forward model, misfit and its
+gradients) at the sizes where its tiles, edge pairs and depth chunks begin and end, against the
+oracle.
+
+Every entry of a frequency plane comes from a pair of the table index 0..N/2 (eight entries to a
+pair, four with the edge N/2, fewer distinct ones at 0 and on the diagonal): N = 16 leaves part of
+a 32-wide tile empty, N = 64 fills one, N = 128 takes off-diagonal tiles.  Depths come in chunks
+of 8 in the forward model and 32 to 128 in the gradients.
+
+Tolerances: the mixed forward model carries its sums in about 48 bits and rounds once, so its
+error is that of the two FP32 transforms, at most about 3 u per radix-2 stage (u = 2^-24) in the
+2-norm, 2 * 7 * 3 u = 2.5e-6 for N = 128; FP64 1e-11 as elsewhere.  The misfit's sums are FP32
+over the depths and one lateral axis: 1e-5 as in test_gpu_grad."""
+import numpy as np
+import pytest
+
+import synth
+from oracle import edt2d, grad2d
+from tests.gpu_helpers import rel_l2, small_workload, dev
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+LAYERS = (np.array([0.0, 60.0, 150.0, 250.0]), np.array([1500.0, 1800.0, 2300.0, 2900.0]))
+
+
+def _workload(nx, nz, nf):
+    return small_workload(nx=nx, nz=nz, nf=nf, fmin=8.0, fmax=35.0, cutoff=0.0, layers=LAYERS, alpha=1e-3)
+
+
+def _solver(wl, precision):
+    from paper_0905_0238_gb300 import Config, Solver
+    return Solver(Config.from_workload(wl, precision=precision))
+
+
+def _model(wl, salt):
+    # every wavenumber present, so that every entry of the planes counts
+    return 1e-8 * synth.rng_for(7, salt=salt).standard_normal((wl.nx, wl.nz))
+
+
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-11), ("mixed", 2.5e-6)])
+@pytest.mark.parametrize("nx,nz,nf", [(16, 1, 2), (16, 9, 3), (32, 8, 2), (64, 33, 2), (128, 17, 2), (128, 70, 1)])
+def test_forward_edges(precision, tol, nx, nz, nf):
+    from paper_0905_0238_gb300 import EDT_FP64, EDT_MIXED
+    wl = _workload(nx, nz, nf)
+    V = _model(wl, 1)
+    s = _solver(wl, EDT_FP64 if precision == "fp64" else EDT_MIXED)
+    D = s.forward(dev(V)).cpu().numpy()
+    assert rel_l2(D, edt2d.forward(wl, V)) < tol
+
+
+@pytest.mark.parametrize("nx,nz,nf", [(64, 1, 2), (64, 65, 1), (64, 129, 1), (128, 7, 2), (256, 34, 1)])
+def test_gradient_edges(nx, nz, nf):
+    from paper_0905_0238_gb300 import EDT_MIXED
+    wl = _workload(nx, nz, nf)
+    V, D = _model(wl, 2), edt2d.forward(wl, _model(wl, 3))
+    J, gV, gc = _solver(wl, EDT_MIXED).misfit_grad(dev(V), dev(D))
+    assert abs(float(J.cpu()) / grad2d.misfit(wl, V, D) - 1) < 1e-5
+    assert rel_l2(gV.cpu().numpy(), grad2d.grad_V(wl, V, D)) < 1e-5
+    assert rel_l2(gc.cpu().numpy(), grad2d.grad_c(wl, V, D)) < 1e-5
+    Vt = _solver(wl, EDT_MIXED).adjoint(dev(D)).cpu().numpy()
+    assert rel_l2(Vt, edt2d.adjoint(wl, D)) < 1e-5

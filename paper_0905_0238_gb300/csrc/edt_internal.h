@@ -329,6 +329,7 @@ cudaError_t launch_solve_variant(const Dev& d, cudaStream_t s);
 cudaError_t prepare_fft(const Dev& d);
 cudaError_t prepare_chol(const Dev& d);
 cudaError_t prepare_gram_tc(const Dev& d);
+cudaError_t prepare_grad();
 
 // Tensor-core Gram tiling (shared by host planning and the kernel).
 constexpr int TC_M = 128;              // MMA rows (depth unknowns per M tile)

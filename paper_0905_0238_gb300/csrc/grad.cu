@@ -56,40 +56,80 @@ __global__ void grad_zero_kernel(Dev d) {
     for (int i = threadIdx.x; i <= d.nlayer; i += blockDim.x) d.gacc[i] = 0.0;
 }
 
+// Both contractions below stage their operands in shared memory and keep the sliding legs in
+// registers.  A 16-byte shared read costs four cycles of the SM's shared-memory port even when
+// it is a broadcast, so a thread has to reuse each coefficient over several depths and each leg
+// over several outputs: ZP pairs of depths per lane (64 ZP per CTA) and GN = 8 / ZP outputs per
+// thread, 128 multiply-adds per 128 to 160 bytes read.  One depth and eight outputs per thread
+// read 144 bytes per 64 multiply-adds and ran at the port's rate: at N = 512, 128 frequencies, 256
+// depths, 1.43 ms (vhat) and 2.60 ms (gbar); the whole gradient went from 7.97 to 7.19 ms.
+template <int ZP> struct Row {                              // a lane's depths of one table row
+  float4 v[ZP];
+  __device__ __forceinline__ float2 at(int i) const {
+    return i & 1 ? make_float2(v[i >> 1].z, v[i >> 1].w) : make_float2(v[i >> 1].x, v[i >> 1].y);
+  }
+};
+// row r of a shared array of rows of 64 ZP depths: depth pair 32 h + lane
+template <int ZP>
+__device__ __forceinline__ Row<ZP> row_of(const float2* s, int r, int lane) {
+  Row<ZP> o;
+  const float4* p = reinterpret_cast<const float4*>(s + size_t(r) * (64 * ZP)) + lane;
+#pragma unroll
+  for (int h = 0; h < ZP; ++h) o.v[h] = p[32 * h];
+  return o;
+}
+// depth of a lane's element i (two consecutive depths per pair)
+__device__ __forceinline__ int lane_z(int i, int lane) { return 64 * (i >> 1) + 2 * lane + (i & 1); }
+
+constexpr int CT = 16;                     // steps per staged chunk
+
 // ---- B(m, j) += sum over the classes of m of Re(a) U + Im(a) W ------------------------------
 // Every entry (p, q) of the plane appears once: the classes {(p, q), (-q, -p)} of m = p - q and
 // their mirror images {(q, p), (-p, -q)} of -m share a = g32_p g32_q, and V = Re sum Ahat(m)
 // e^{ikx} needs only B(m) = Ahat(m) + conj Ahat(-m) = conj(a) S + a conj(S'), m = 0..N/2, i.e.
 // U = S + conj S', W = -i (S - conj S') with four multiply-adds per class and depth.  For
 // m = 2 j or 2 j + 1 the classes are p = t + j (+ 1), q = t - j, t = 0..N/2 (t < N/2 for odd m),
-// so the legs of a thread's four j slide by one per step of t and stay in registers; the ends
-// t = 0, N/2 of even m are their own partners, and m = 0, N/2 their own mirror images.
-constexpr int VJ = 32, VTC = 16;           // j per CTA (4 per warp), t per staged chunk
+// so the legs of a thread's JT consecutive j slide by one per step of t; the ends t = 0, N/2 of
+// even m are their own partners, and m = 0, N/2 their own mirror images.  Consecutive chunks of
+// t share all but CT of their rows, which stay where they are (circular buffers).
+template <int ZP> struct VhatShape {
+  static constexpr int JT = 4 / ZP, VJ = 8 * JT;           // j per thread and per CTA (two m each)
+  static constexpr int R = CT + VJ;                        // rows buffered of either leg
+  static constexpr int SMEM = (2 * R * 64 * ZP) * int(sizeof(float2)) + CT * 2 * VJ * int(sizeof(float4));
+};
 
-__global__ void __launch_bounds__(256, 3) grad_vhat_kernel(Dev d, int f0) {
-  __shared__ float2 gps[VTC + VJ][32];     // rows p = t0 + j0 + i
-  __shared__ float2 gqs[VTC + VJ - 1][32]; // rows q = t0 - j0 - (VJ - 1) + i
-  __shared__ float4 cf[VTC][2 * VJ];       // (U, W) of (t, m)
+template <int ZP>
+__global__ void __launch_bounds__(256, 2) grad_vhat_kernel(Dev d, int f0) {
+  using S = VhatShape<ZP>;
+  constexpr int JT = S::JT, VJ = S::VJ, R = S::R, ZC = 64 * ZP;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float4 (*cf)[2 * VJ] = reinterpret_cast<float4 (*)[2 * VJ]>(smem_raw);    // [CT] (U, W) of (t, m)
+  float2* gps = reinterpret_cast<float2*>(cf + CT);        // row jt + u, u = t + ..., in slot u mod R
+  float2* gqs = gps + R * ZC;                              // row u - jt, u = t - ..., in slot (u + VJ) mod R
   const int N = d.N, H = N / 2, msk = N - 1, nk = d.nk, fi = blockIdx.z, f = f0 + fi;
-  const int jt = blockIdx.x * VJ, z0 = blockIdx.y * 32;
+  const int jt = blockIdx.x * VJ, z0 = blockIdx.y * ZC;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int z = z0 + lane;
   const float2* g = d.g32 + size_t(f) * nk * d.nzs;
   const float4* E = d.born_fold + size_t(fi) * 2 * nk * nk;
   const float4* T = E + size_t(nk) * nk;
-  const bool live = 2 * (jt + 4 * w) <= H;                 // the same in the whole warp
-  float2 acc[8];
+  const bool live = 2 * (jt + JT * w) <= H;                // the same in the whole warp
+  float2 acc[2 * JT][2 * ZP];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) acc[k] = make_float2(0.f, 0.f);
-  for (int t0 = 0; t0 <= H; t0 += VTC) {
-    for (int e = threadIdx.x; e < (VTC + VJ) * 32; e += blockDim.x) {
-      const int i = e >> 5, zz = z0 + (e & 31);
-      gps[i][e & 31] = zz < d.nz ? g[size_t(tab_index((t0 + jt + i) & msk, N)) * d.nzs + zz] : make_float2(0.f, 0.f);
-      if (i < VTC + VJ - 1)
-        gqs[i][e & 31] = zz < d.nz ? g[size_t(tab_index((t0 - jt - (VJ - 1) + i) & msk, N)) * d.nzs + zz]
-                                   : make_float2(0.f, 0.f);
+  for (int k = 0; k < 2 * JT; ++k)
+#pragma unroll
+    for (int i = 0; i < 2 * ZP; ++i) acc[k][i] = make_float2(0.f, 0.f);
+  // rows [lo, hi) of u: gps gets jt + u, gqs (u - VJ + 1) - jt
+  auto load_rows = [&](int lo, int hi) {
+    for (int e = threadIdx.x; e < (hi - lo) * ZC; e += 256) {
+      const int u = lo + e / ZC, zz = e % ZC, z = z0 + zz, sl = (u % R) * ZC + zz;
+      const bool in = z < d.nz;
+      gps[sl] = in ? g[size_t(tab_index((jt + u) & msk, N)) * d.nzs + z] : make_float2(0.f, 0.f);
+      gqs[sl] = in ? g[size_t(tab_index((u - VJ + 1 - jt) & msk, N)) * d.nzs + z] : make_float2(0.f, 0.f);
     }
-    for (int e = threadIdx.x; e < VTC * 2 * VJ; e += blockDim.x) {
+  };
+  for (int t0 = 0; t0 <= H; t0 += CT) {
+    load_rows(t0 == 0 ? 0 : t0 + VJ, t0 + VJ + CT);
+    for (int e = threadIdx.x; e < CT * 2 * VJ; e += 256) {
       const int tt = e / (2 * VJ), mi = e - tt * (2 * VJ);
       const int t = t0 + tt, m = 2 * jt + mi, odd = m & 1, j = m >> 1;
       float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -98,54 +138,65 @@ __global__ void __launch_bounds__(256, 3) grad_vhat_kernel(Dev d, int f0) {
         if (p > H) p -= N;                                  // signed indices, never both negative
         const float4 c = p >= 0 && q >= 0 ? E[size_t(p) * nk + q]
                                           : T[size_t(p >= 0 ? p : -p) * nk + (q >= 0 ? q : -q)];
-        float2 S = make_float2(c.x, c.y), S2 = make_float2(c.z, c.w);
-        if (p < 0) { const float2 x = S; S = S2; S2 = x; }
+        float2 S1 = make_float2(c.x, c.y), S2 = make_float2(c.z, c.w);
+        if (p < 0) { const float2 x = S1; S1 = S2; S2 = x; }
         float wt = !odd && (t == 0 || t == H) ? 0.5f : 1.f;
         if (m == 0 || m == H) wt *= 0.5f;
-        o = make_float4(wt * (S.x + S2.x), wt * (S.y - S2.y), wt * (S.y + S2.y), wt * (S2.x - S.x));
+        o = make_float4(wt * (S1.x + S2.x), wt * (S1.y - S2.y), wt * (S1.y + S2.y), wt * (S2.x - S1.x));
       }
       cf[tt][mi] = o;
     }
     __syncthreads();
     if (live) {
-      float2 P[5], Q[4];
+      // at t = t0 + tt: P[i] = row p of j = jt + JT w + i (u = t + JT w + i), Q[i] = its row q
+      // (u = t + VJ - 1 - JT w - i)
+      Row<ZP> P[JT + 1], Q[JT];
 #pragma unroll
-      for (int i = 0; i < 5; ++i) P[i] = gps[4 * w + i][lane];
+      for (int i = 0; i <= JT; ++i) P[i] = row_of<ZP>(gps, (t0 + JT * w + i) % R, lane);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) Q[i] = gqs[VJ - 1 - 4 * w - i][lane];
+      for (int i = 0; i < JT; ++i) Q[i] = row_of<ZP>(gqs, (t0 + VJ - 1 - JT * w - i) % R, lane);
+      int sp = (t0 + JT * w + JT) % R, sq = (t0 + VJ - 1 - JT * w) % R;
 #pragma unroll
-      for (int tt = 0; tt < VTC; ++tt) {
+      for (int tt = 0; tt < CT; ++tt) {
         if (tt > 0) {
           if (t0 + tt > H) break;
+          sp = sp + 1 == R ? 0 : sp + 1;
+          sq = sq + 1 == R ? 0 : sq + 1;
 #pragma unroll
-          for (int i = 0; i < 4; ++i) P[i] = P[i + 1];
-          P[4] = gps[tt + 4 * w + 4][lane];
+          for (int i = 0; i < JT; ++i) P[i] = P[i + 1];
+          P[JT] = row_of<ZP>(gps, sp, lane);
 #pragma unroll
-          for (int i = 3; i > 0; --i) Q[i] = Q[i - 1];
-          Q[0] = gqs[tt + VJ - 1 - 4 * w][lane];
+          for (int i = JT - 1; i > 0; --i) Q[i] = Q[i - 1];
+          Q[0] = row_of<ZP>(gqs, sq, lane);
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+        for (int i = 0; i < JT; ++i)
 #pragma unroll
           for (int o = 0; o < 2; ++o) {
-            const float4 c = cf[tt][8 * w + 2 * i + o];
-            const float2 a = P[i + o] * Q[i];
-            float2& s = acc[2 * i + o];
-            s.x = fmaf(a.x, c.x, fmaf(a.y, c.z, s.x));
-            s.y = fmaf(a.x, c.y, fmaf(a.y, c.w, s.y));
+            const float4 c = cf[tt][2 * (JT * w + i) + o];
+#pragma unroll
+            for (int x = 0; x < 2 * ZP; ++x) {
+              const float2 a = P[i + o].at(x) * Q[i].at(x);
+              float2& s = acc[2 * i + o][x];
+              s.x = fmaf(a.x, c.x, fmaf(a.y, c.z, s.x));
+              s.y = fmaf(a.x, c.y, fmaf(a.y, c.w, s.y));
+            }
           }
       }
     }
     __syncthreads();
   }
-  if (z < d.nz) {
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int m = 2 * (jt + 4 * w) + k;
-      if (m > H) continue;
+  for (int k = 0; k < 2 * JT; ++k) {
+    const int m = 2 * (jt + JT * w) + k;
+    if (m > H) continue;
+#pragma unroll
+    for (int x = 0; x < 2 * ZP; ++x) {
+      const int z = z0 + lane_z(x, lane);
+      if (z >= d.nz) continue;
       double* o = reinterpret_cast<double*>(d.adj + size_t(m) * d.nz + z);
-      atomicAdd(o, double(acc[k].x));
-      atomicAdd(o + 1, double(acc[k].y));
+      atomicAdd(o, double(acc[k][x].x));
+      atomicAdd(o + 1, double(acc[k][x].y));
     }
   }
 }
@@ -154,39 +205,51 @@ __global__ void __launch_bounds__(256, 3) grad_vhat_kernel(Dev d, int f0) {
 // The entries whose row a holds g_n are, for every signed q, the class of (n, q) and its mirror
 // image: dJ/dg32_n = 2 c_J sum_q g32_q [C1 Re Vhat(n - q) + C2 Im Vhat(n - q)] with
 // C1 = conj(S + S'), C2 = i conj(S - S') (the folded values carry conj(s_f)/|s_f|); n = 0 and
-// N/2 meet every class twice.  8 consecutive n per thread walking m = n - q, one depth per lane:
-// the legs q = n - m slide by one per step, Vhat(m) is common to the eight.
-constexpr int GA = 64, GMC = 16, GQR = GA + GMC - 1;
+// N/2 meet every class twice.  GN consecutive n per thread walking m = n - q: the legs q = n - m
+// slide by one per step, Vhat(m) is common to them.  dJ/dc_l sums gbar over near-critical
+// wavenumbers with much cancellation, so the FP32 sum over m is taken in two levels (CT terms,
+// then the chunks).
+template <int ZP> struct GbarShape {
+  static constexpr int GN = 8 / ZP, GA = 8 * GN;           // n per thread and per CTA
+  static constexpr int R = GA + CT;                        // rows buffered
+  static constexpr int SMEM = (R + CT) * 64 * ZP * int(sizeof(float2)) + CT * (GA + 1) * int(sizeof(float4));
+};
 
-__global__ void __launch_bounds__(256, 3) grad_gbar_kernel(Dev d, int f0) {
-  __shared__ float4 cf[GMC][GA + 1];
-  __shared__ float2 gqs[GQR][32];
-  __shared__ float2 ws[GMC][32];
+template <int ZP>
+__global__ void __launch_bounds__(256, 2) grad_gbar_kernel(Dev d, int f0) {
+  using S = GbarShape<ZP>;
+  constexpr int GN = S::GN, GA = S::GA, R = S::R, ZC = 64 * ZP;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float4 (*cf)[GA + 1] = reinterpret_cast<float4 (*)[GA + 1]>(smem_raw);    // [CT] (C1, C2) of (m, n)
+  float2* ws = reinterpret_cast<float2*>(cf + CT);         // [CT] Vhat rows
+  float2* gqs = ws + CT * ZC;                              // row a0 + GA - 1 - u in slot u mod R
   const int N = d.N, H = N / 2, msk = N - 1, nk = d.nk, fi = blockIdx.z, f = f0 + fi;
-  const int a0 = blockIdx.x * GA, j0 = blockIdx.y * 32;
+  const int a0 = blockIdx.x * GA, z0 = blockIdx.y * ZC;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int j = j0 + lane;
   const float2* g = d.g32 + size_t(f) * nk * d.nzs;
   const float2* vh = reinterpret_cast<const float2*>(d.vfull);     // row m at 2 nz m
   const float4* E = d.born_fold + size_t(fi) * 2 * nk * nk;
   const float4* T = E + size_t(nk) * nk;
-  const bool live = a0 + 8 * w <= H;                       // the same in the whole warp
-  float2 tot[8];
+  const bool live = a0 + GN * w <= H;                      // the same in the whole warp
+  float2 tot[GN][2 * ZP];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) tot[k] = make_float2(0.f, 0.f);
-  for (int mc = 0; mc < N; mc += GMC) {
-    // rows qi <-> q = a0 - mc - (GMC - 1) + qi (mod N)
-    for (int e = threadIdx.x; e < GQR * 32; e += blockDim.x) {
-      const int qi = e >> 5, jj = j0 + (e & 31);
-      const int q = (a0 - mc - (GMC - 1) + qi) & msk;
-      gqs[qi][e & 31] = jj < d.nz ? g[size_t(tab_index(q, N)) * d.nzs + jj] : make_float2(0.f, 0.f);
+  for (int k = 0; k < GN; ++k)
+#pragma unroll
+    for (int i = 0; i < 2 * ZP; ++i) tot[k][i] = make_float2(0.f, 0.f);
+  for (int mc = 0; mc < N; mc += CT) {
+    // rows q = n - m: u = GA - 1 - (n - a0) + m, all of them once, CT new ones per chunk
+    const int lo = mc == 0 ? 0 : mc + GA - 1, hi = mc + GA + CT - 1;
+    for (int e = threadIdx.x; e < (hi - lo) * ZC; e += 256) {
+      const int u = lo + e / ZC, zz = e % ZC, z = z0 + zz;
+      gqs[(u % R) * ZC + zz] = z < d.nz ? g[size_t(tab_index((a0 + GA - 1 - u) & msk, N)) * d.nzs + z]
+                                        : make_float2(0.f, 0.f);
     }
-    for (int e = threadIdx.x; e < GMC * 32; e += blockDim.x) {
-      const int mi = e >> 5, jj = j0 + (e & 31);
-      ws[mi][e & 31] = jj < d.nz ? vh[size_t(mc + mi) * 2 * d.nz + jj] : make_float2(0.f, 0.f);
+    for (int e = threadIdx.x; e < CT * ZC; e += 256) {
+      const int mi = e / ZC, zz = e % ZC, z = z0 + zz;
+      ws[e] = z < d.nz ? vh[size_t(mc + mi) * 2 * d.nz + z] : make_float2(0.f, 0.f);
     }
-    for (int e = threadIdx.x; e < GMC * GA; e += blockDim.x) {
-      const int al = e / GMC, mi = e - al * GMC, n = a0 + al;
+    for (int e = threadIdx.x; e < CT * GA; e += 256) {
+      const int al = e / CT, mi = e - al * CT, n = a0 + al;
       float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
       if (n <= H) {
         int q = (n - mc - mi) & msk;
@@ -199,43 +262,82 @@ __global__ void __launch_bounds__(256, 3) grad_gbar_kernel(Dev d, int f0) {
     }
     __syncthreads();
     if (live) {
-      // thread's n_k = a0 + 8 w + k; at m = mc + mi its leg q_k = n_k - m sits in row
-      // qi = 8 w + k - mi + GMC - 1, one row lower per step of m
-      float2 win[8], acc[8];
+      // n_k = a0 + GN w + k at m = mc + mi: u = GA - 1 - GN w - k + m
+      Row<ZP> win[GN];
+      float2 acc[GN][2 * ZP];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) acc[k] = make_float2(0.f, 0.f);
+      for (int k = 0; k < GN; ++k) {
+        win[k] = row_of<ZP>(gqs, (mc + GA - 1 - GN * w - k) % R, lane);
 #pragma unroll
-      for (int k = 0; k < 8; ++k) win[k] = gqs[8 * w + k + GMC - 1][lane];
+        for (int i = 0; i < 2 * ZP; ++i) acc[k][i] = make_float2(0.f, 0.f);
+      }
+      int sq = (mc + GA - 1 - GN * w) % R;
 #pragma unroll
-      for (int mi = 0; mi < GMC; ++mi) {
+      for (int mi = 0; mi < CT; ++mi) {
         if (mi > 0) {
+          sq = sq + 1 == R ? 0 : sq + 1;
 #pragma unroll
-          for (int k = 7; k > 0; --k) win[k] = win[k - 1];
-          win[0] = gqs[8 * w - mi + GMC - 1][lane];
+          for (int k = GN - 1; k > 0; --k) win[k] = win[k - 1];
+          win[0] = row_of<ZP>(gqs, sq, lane);
         }
-        const float2 v = ws[mi][lane];
+        const Row<ZP> v = row_of<ZP>(ws, mi, lane);
 #pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const float4 c = cf[mi][8 * w + k];
-          const float tx = fmaf(c.x, v.x, c.z * v.y), ty = fmaf(c.y, v.x, c.w * v.y);
-          acc[k].x = fmaf(win[k].x, tx, fmaf(-win[k].y, ty, acc[k].x));
-          acc[k].y = fmaf(win[k].x, ty, fmaf(win[k].y, tx, acc[k].y));
+        for (int k = 0; k < GN; ++k) {
+          const float4 c = cf[mi][GN * w + k];
+#pragma unroll
+          for (int i = 0; i < 2 * ZP; ++i) {
+            const float2 vz = v.at(i), gz = win[k].at(i);
+            const float tx = fmaf(c.x, vz.x, c.z * vz.y), ty = fmaf(c.y, vz.x, c.w * vz.y);
+            acc[k][i].x = fmaf(gz.x, tx, fmaf(-gz.y, ty, acc[k][i].x));
+            acc[k][i].y = fmaf(gz.x, ty, fmaf(gz.y, tx, acc[k][i].y));
+          }
         }
       }
 #pragma unroll
-      for (int k = 0; k < 8; ++k) tot[k] = tot[k] + acc[k];
+      for (int k = 0; k < GN; ++k)
+#pragma unroll
+        for (int i = 0; i < 2 * ZP; ++i) tot[k][i] = tot[k][i] + acc[k][i];
     }
     __syncthreads();
   }
-  if (j < d.nz) {
-    const float sc = float(2.0 / (double(N) * N) * sqrt(d.fc[f].s_abs));
-    float2* G = d.gbar + size_t(f) * nk * d.nz;
+  const float sc = float(2.0 / (double(N) * N) * sqrt(d.fc[f].s_abs));
+  float2* G = d.gbar + size_t(f) * nk * d.nz;
 #pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int n = a0 + 8 * w + k;
-      if (n <= H) G[size_t(n) * d.nz + j] = make_float2(sc * tot[k].x, sc * tot[k].y);
+  for (int k = 0; k < GN; ++k) {
+    const int n = a0 + GN * w + k;
+    if (n > H) continue;
+#pragma unroll
+    for (int i = 0; i < 2 * ZP; ++i) {
+      const int z = z0 + lane_z(i, lane);
+      if (z < d.nz) G[size_t(n) * d.nz + z] = make_float2(sc * tot[k][i].x, sc * tot[k][i].y);
     }
   }
+}
+
+// 128 depths per CTA unless the last 64 of them would all be padding
+inline bool wide_depths(int nz) { return (nz + 127) / 128 * 128 - nz < 64; }
+
+cudaError_t vhat_launch(const Dev& d, int f0, int nfc, cudaStream_t s) {
+  const int nj = d.N / 4 + 1;                              // m = 0..N/2, two per j
+  if (wide_depths(d.nz)) {
+    using S = VhatShape<2>;
+    grad_vhat_kernel<2><<<dim3((nj + S::VJ - 1) / S::VJ, (d.nz + 127) / 128, nfc), 256, S::SMEM, s>>>(d, f0);
+  } else {
+    using S = VhatShape<1>;
+    grad_vhat_kernel<1><<<dim3((nj + S::VJ - 1) / S::VJ, (d.nz + 63) / 64, nfc), 256, S::SMEM, s>>>(d, f0);
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t gbar_launch(const Dev& d, int f0, int nfc, cudaStream_t s) {
+  if (wide_depths(d.nz)) {
+    using S = GbarShape<2>;
+    grad_gbar_kernel<2><<<dim3((d.nk + S::GA - 1) / S::GA, (d.nz + 127) / 128, nfc), 256, S::SMEM, s>>>(d, f0);
+  } else {
+    using S = GbarShape<1>;
+    grad_gbar_kernel<1><<<dim3((d.nk + S::GA - 1) / S::GA, (d.nz + 63) / 64, nfc), 256, S::SMEM, s>>>(d, f0);
+  }
+  return cudaGetLastError();
 }
 
 // ---- dJ/dc_l: reverse-mode differentiation of the depth march ------------------------------
@@ -424,15 +526,15 @@ __global__ void __launch_bounds__(128) grad_reverse_kernel(Dev d) {
   }
 }
 
-// nw: the reverse kernel's warps (their partials are added in warp order)
-__global__ void grad_finalize_kernel(Dev d, double* J, double* gc, int nw) {
-  const double cj = 1.0 / (double(d.N) * d.N);
-  if (threadIdx.x == 0 && J) J[0] = cj * d.gacc[0];
-  for (int l = threadIdx.x; l < d.nlayer; l += blockDim.x) {
-    double t = 0.0;
-    for (int w = 0; w < nw; ++w) t += d.gcpart[size_t(w) * d.nlayer + l];
-    gc[l] = t;
-  }
+// nw: the reverse kernel's warps.  One warp per layer: lane l adds the partials l, l + 32, ... in
+// order, then a butterfly over the lanes (a fixed order of additions).
+__global__ void __launch_bounds__(32) grad_finalize_kernel(Dev d, double* J, double* gc, int nw) {
+  const int l = blockIdx.x, lane = threadIdx.x;
+  if (l == 0 && lane == 0 && J) J[0] = d.gacc[0] / (double(d.N) * d.N);
+  double t = 0.0;
+  for (int w = lane; w < nw; w += 32) t += d.gcpart[size_t(w) * d.nlayer + l];
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if (lane == 0) gc[l] = t;
 }
 
 // ---- adjoint of the inversion D -> V (linear in D: G and lam depend on the rows only) --------
@@ -720,14 +822,19 @@ cudaError_t launch_invert_vjp(const Dev& d0, const void* Vbar, int Vbar_dtype, v
     const long long nfl = (long long)d.nf * d.nlayer * d.nk;
     grad_field_kernel<<<unsigned((nfl + 127) / 128), 128, 0, s>>>(d, d.g64);
     grad_reverse_kernel<<<gk, 128, 0, s>>>(d);
-    grad_finalize_kernel<<<1, 64, 0, s>>>(d, nullptr, gc, int(gk.x * gk.y * 4));
+    grad_finalize_kernel<<<d.nlayer, 32, 0, s>>>(d, nullptr, gc, int(gk.x * gk.y * 4));
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
 
-static dim3 vhat_grid(const Dev& d, int nfc) {          // m = 0..N/2, two per j
-  return dim3((d.N / 4 + 1 + VJ - 1) / VJ, (d.nz + 31) / 32, nfc);
+cudaError_t prepare_grad() {
+  const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e;
+  if ((e = cudaFuncSetAttribute(grad_vhat_kernel<1>, attr, VhatShape<1>::SMEM)) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(grad_vhat_kernel<2>, attr, VhatShape<2>::SMEM)) != cudaSuccess) return e;
+  if ((e = cudaFuncSetAttribute(grad_gbar_kernel<1>, attr, GbarShape<1>::SMEM)) != cudaSuccess) return e;
+  return cudaFuncSetAttribute(grad_gbar_kernel<2>, attr, GbarShape<2>::SMEM);
 }
 
 bool grad_supported(const Dev& d) {
@@ -759,8 +866,7 @@ cudaError_t launch_adjoint(const Dev& d, const void* D, int D_dtype, void* V, in
     const int nfc = std::min(d.fchunk, d.nf - f0);
     if ((e = launch_transform<float>(d, D, D_dtype, f0, nfc, s)) != cudaSuccess) return e;
     if ((e = launch_born_residual(d, f0, nfc, false, s)) != cudaSuccess) return e;
-    grad_vhat_kernel<<<vhat_grid(d, nfc), 256, 0, s>>>(d, f0);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = vhat_launch(d, f0, nfc, s)) != cudaSuccess) return e;
   }
   return launch_lateral_idft_real(d, d.adj, scale, V, V_dtype, s);
 }
@@ -777,9 +883,8 @@ cudaError_t launch_misfit_grad(const Dev& d, const void* V, int V_dtype, const v
     const int nfc = std::min(d.fchunk, d.nf - f0);
     if ((e = launch_transform<float>(d, D, D_dtype, f0, nfc, s)) != cudaSuccess) return e;
     if ((e = launch_born_residual(d, f0, nfc, true, s)) != cudaSuccess) return e;
-    grad_vhat_kernel<<<vhat_grid(d, nfc), 256, 0, s>>>(d, f0);
-    grad_gbar_kernel<<<dim3((d.nk + GA - 1) / GA, (d.nz + 31) / 32, nfc), 256, 0, s>>>(d, f0);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = vhat_launch(d, f0, nfc, s)) != cudaSuccess) return e;
+    if ((e = gbar_launch(d, f0, nfc, s)) != cudaSuccess) return e;
   }
   const dim3 gk((d.nk + 127) / 128, d.nf);
   grad_march_kernel<<<gk, 128, 0, s>>>(d);
@@ -788,7 +893,7 @@ cudaError_t launch_misfit_grad(const Dev& d, const void* V, int V_dtype, const v
   grad_reverse_kernel<<<gk, 128, 0, s>>>(d);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = launch_lateral_idft_real(d, d.adj, 2.0 / (double(N) * N), gV, V_dtype, s)) != cudaSuccess) return e;
-  grad_finalize_kernel<<<1, 64, 0, s>>>(d, J, gc, int(gk.x * gk.y * 4));
+  grad_finalize_kernel<<<d.nlayer, 32, 0, s>>>(d, J, gc, int(gk.x * gk.y * 4));
   return cudaGetLastError();
 }
 

@@ -105,7 +105,7 @@ struct edt_ctx {
   Region r_fc, r_ltop, r_lvel, r_zl, r_zo, r_rows, r_roff, r_roffmf, r_band, r_bcol, r_cpre, r_kval, r_pairm, r_fjoff, r_fjent, r_jact, r_jmap, r_Gs, r_U, r_Dw, r_A32, r_tw64, r_tw32, r_segm, r_segr0,
       r_segn, r_ctas, r_mslot, r_zo32, r_fc32, r_coef, r_coef32, r_g64, r_g32, r_g32lo, r_rowmax, r_gscale, r_X, r_Dst, r_Vst, r_rhs, r_gent, r_gpart, r_G,
       r_dinv, r_L32, r_dinv32, r_b, r_tr, r_tpart, r_x, r_r, r_rpart, r_rowc, r_xmu, r_gam, r_tref, r_treoff, r_vhat, r_vfull, r_gscr, r_adj, r_gacc, r_gcpart, r_bexp, r_bfold, r_status, r_flags,
-      r_kzP, r_kzp, r_kzgoff, r_kzvoff, r_kzG, r_kzT, r_kzb, r_kzx;
+      r_tlog, r_kzP, r_kzp, r_kzgoff, r_kzvoff, r_kzG, r_kzT, r_kzb, r_kzx;
   Dev dev{};
   cudaStream_t last_stream = nullptr;
   int last_status = EDT_OK;
@@ -707,6 +707,7 @@ void layout(edt_ctx* c) {
   take(c->r_status, ns * sizeof(int));
   take(c->r_flags, 8 * sizeof(unsigned));
   const bool disk = !c->kz_p.empty();
+  take(c->r_tlog, c->cfg.solver == EDT_SOLVE_TSVD ? ns * tsvd_log_doubles(c->nz) * sizeof(double) : 0);
   take(c->r_kzP, disk ? size_t(nz) * nz * sizeof(double) : 0);
   take(c->r_kzp, disk ? ns * sizeof(int) : 0);
   take(c->r_kzgoff, disk ? ns * sizeof(long long) : 0);
@@ -817,6 +818,8 @@ void bind(edt_ctx* c) {
   d.flags = at<unsigned*>(c, c->r_flags);
   d.solver = c->cfg.solver;
   d.tsvd_tol = c->cfg.tsvd_tol;
+  d.tlog = c->r_tlog.bytes ? at<double*>(c, c->r_tlog) : nullptr;
+  d.tlog_stride = c->r_tlog.bytes ? tsvd_log_doubles(c->nz) : 0;
   const bool disk = c->r_kzP.bytes > 0;
   d.kz_P = disk ? at<const double*>(c, c->r_kzP) : nullptr;
   d.kz_p = disk ? at<const int*>(c, c->r_kzp) : nullptr;

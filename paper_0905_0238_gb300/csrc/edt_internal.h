@@ -192,6 +192,8 @@ struct Dev {
   double* kz_T;                 // [nsub][nz][p] scratch G P_p
   double* kz_b;                 // [nsub][nz][2] restricted right-hand sides
   double* kz_x;                 // [nsub][nz][2] restricted solutions
+  double* tlog;                 // [nsub][tlog_stride] tangents of the truncated SVD's rotations
+  size_t tlog_stride;
 };
 
 // Record a CUDA error for edt_last_cuda_error; returns EDT_ECUDA.
@@ -322,6 +324,7 @@ int chol_block_cols();
 // vertical-wavenumber disk, in place of the Cholesky stage of the FP64 line path.
 constexpr int TSVD_MAX_NZ = 96;
 size_t tsvd_smem_bytes(int p);
+size_t tsvd_log_doubles(int p);                                 // rotation log of one subproblem
 cudaError_t prepare_variants(int nz);
 cudaError_t launch_solve_variant(const Dev& d, cudaStream_t s);
 

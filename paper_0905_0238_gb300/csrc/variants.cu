@@ -10,7 +10,7 @@
 //    Ahat, W its right singular vectors) the solution V S~^-1 U^T dhat is
 //        x = sum over lambda_j >= sigma^2 of w_j (w_j^T Ahat^T dhat) / lambda_j,
 //    computed from the eigenpairs of the FP64 normal matrix by cyclic two-sided Jacobi rotations
-//    in parallel (round-robin) order, matrix and eigenvectors in shared memory.
+//    in parallel (round-robin) order, the matrix in shared memory and the rotations logged.
 #include "edt_internal.h"
 
 namespace edt {
@@ -62,12 +62,68 @@ __global__ void kzv_back_kernel(Dev d) {
   d.x[(size_t(m) * n + i) * 2 + side] = s;
 }
 
-constexpr int JAC_THREADS = 256;
+constexpr int JAC_THREADS = 512;
 constexpr int JAC_MAX_SWEEPS = 20;
+constexpr int JAC_BLOCKS = 3;      // 2 x 2 blocks per thread: (TSVD_MAX_NZ / 2)(TSVD_MAX_NZ / 2 + 1) / 2 in all
+static_assert((TSVD_MAX_NZ / 2) * (TSVD_MAX_NZ / 2 + 1) / 2 <= JAC_THREADS * JAC_BLOCKS, "blocks fit the threads");
+
+__device__ __forceinline__ double rcp_approx(double x) {      // ~20 bits
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  return y;
+}
+__device__ __forceinline__ double rsqrt_approx(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  return y;
+}
+// cosine of the rotation of tangent t, 1 / sqrt(1 + t^2) to FP64: the estimate y0 and one
+// third-order step on e = 1 - q y0^2 (y = y0 (1 + e/2 + 3 e^2 / 8), error ~ e^3)
+__device__ __forceinline__ double cos_of(double t) {
+  const double q = fma(t, t, 1.0), y0 = rsqrt_approx(q);
+  const double e = fma(-q * y0, y0, 1.0);
+  return fma(y0 * e, fma(0.375, e, 0.5), y0);
+}
+// tangent of the rotation that zeroes apq between the diagonal entries app, aqq, to ~20 bits: an
+// inexact angle leaves |apq| 1e-6 of what it was (the next sweep takes the rest), the rotation
+// itself is orthogonal to FP64 because the cosine is formed from the tangent that is used
+__device__ __forceinline__ double tan_of(double app, double aqq, double apq) {
+  const double dd = aqq - app;
+  if (dd == 0.0) return 1.0;
+  if (fabs(dd) > 1e8 * fabs(apq)) return apq * rcp_approx(dd);
+  const double tau = dd * rcp_approx(2.0 * apq), q = fma(tau, tau, 1.0);
+  return copysign(rcp_approx(fabs(tau) + q * rsqrt_approx(q)), tau);
+}
+
+// players of the round-robin (a dummy when p is odd); round r: player 0 fixed, the others
+// rotate; pair k = (position k, position P2 - 1 - k), a < b, b == p: the dummy
+__device__ __forceinline__ void jac_pair(int k, int r, int P2, int& a, int& b) {
+  auto pos = [&](int t) {
+    if (t == 0) return 0;
+    const int v = t + r;                       // 1 + (t - 1 + r) mod (P2 - 1), r < P2 - 1
+    return v >= P2 ? v - (P2 - 1) : v;
+  };
+  a = pos(k);
+  b = pos(P2 - 1 - k);
+  if (a > b) { const int t = a; a = b; b = t; }
+}
 
 // One CTA per subproblem: eigen-decomposition of the p x p normal matrix (G, or G' of the disk)
 // by cyclic Jacobi, then the truncated-SVD solution for both right-hand sides.
 // src: matrices at m * nz * nz with leading dimension p; rhs, out: [m][nz][2].
+//
+// The FP64 unit (one warp instruction per 16 cycles of an SM) bounds the rounds, so a round does
+// no more FP64 work than it has to:
+//   * the matrix is kept as its lower triangle and updated two-sidedly in one pass, block (K, L) of
+//     the pairs K <= L at a time, X <- J_K^T X J_L: 16 operations per 4 entries of half the
+//     matrix, where a pass over the columns and one over the rows of the whole matrix take 32;
+//     blocks of two pairs that do not rotate are left alone;
+//   * the eigenvectors are not accumulated (another 16 operations per 4 entries): with W = J_1
+//     J_2 ... J_n, W^T b is formed by applying each rotation to b as it is found, and W z by
+//     applying them in reverse order from the log of their tangents (tlog, written once and
+//     read once), 8 operations per pair and right-hand side;
+//   * the tangents take approximate reciprocals (tan_of).
+// One barrier after the angles and one after the update.
 __global__ void __launch_bounds__(JAC_THREADS) tsvd_jacobi_kernel(Dev d, const double* src, const double* rhs,
                                                                  double* out) {
   extern __shared__ __align__(16) double sm[];
@@ -75,12 +131,13 @@ __global__ void __launch_bounds__(JAC_THREADS) tsvd_jacobi_kernel(Dev d, const d
   const int n = d.nz;
   const int p = d.kz_p ? d.kz_p[m] : n;
   const int ld = p + 1;
-  double* A = sm;                         // [p][ld]
-  double* W = A + size_t(p) * ld;         // [p][ld] eigenvectors (columns)
-  double* cs = W + size_t(p) * ld;        // [2][p/2 + 1] rotation cosines and sines
-  double* red = cs + 2 * (p / 2 + 1);     // [32]
-  int* pj = reinterpret_cast<int*>(red + 32);   // [2][p/2 + 1] pair indices (i < j), -1: none;
-                                                // then the sweep's rotation flag
+  const int P2 = (p + 1) & ~1, npair = P2 / 2;
+  double* A = sm;                         // [p][ld] lower triangle (row >= column)
+  double* bv = A + size_t(p) * ld;        // [p][2] W^T b, later W z
+  double* cs = bv + 2 * p;                // [2][npair] rotation cosines and sines
+  double* red = cs + P2;                  // [32]
+  int* pj = reinterpret_cast<int*>(red + 32);   // [2][npair] pair indices a < b (b == p: alone)
+  int* rotated = pj + P2;
   const bool has_rows = d.row_off[m + 1] > d.row_off[m];
   double* xo = out + size_t(m) * n * 2;
   if (!has_rows || p == 0) {
@@ -89,110 +146,146 @@ __global__ void __launch_bounds__(JAC_THREADS) tsvd_jacobi_kernel(Dev d, const d
     return;
   }
   const double* S = src + size_t(m) * n * n;
+  const double* bm = rhs + size_t(m) * n * 2;
+  // the matrix times a power of two that puts its largest diagonal entry in [0.5, 1)
+  double dmax = 0.0;
+  for (int i = threadIdx.x; i < p; i += blockDim.x) dmax = fmax(dmax, fabs(S[size_t(i) * p + i]));
+  auto block_max = [&](double v) {
+    for (int o = 16; o > 0; o >>= 1) v = fmax(v, __shfl_xor_sync(0xffffffffu, v, o));
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
+    __syncthreads();
+    v = 0.0;
+    for (int w = 0; w < JAC_THREADS / 32; ++w) v = fmax(v, red[w]);
+    return v;
+  };
+  dmax = block_max(dmax);
+  int ex = 0;
+  if (dmax > 0.0 && isfinite(dmax)) frexp(dmax, &ex);
+  const double sc = scalbn(1.0, -ex);
   for (int e = threadIdx.x; e < p * p; e += blockDim.x) {
     const int i = e / p, j = e - i * p;
-    A[i * ld + j] = S[size_t(i) * p + j];
-    W[i * ld + j] = i == j ? 1.0 : 0.0;
+    if (j <= i) A[i * ld + j] = sc * S[size_t(i) * p + j];
   }
-  __syncthreads();
-  const int P2 = (p + 1) & ~1;            // players of the round-robin (a dummy when p is odd)
-  const int npair = P2 / 2;
+  for (int i = threadIdx.x; i < 2 * p; i += blockDim.x) bv[i] = bm[i];
+  // this thread's blocks (K <= L), the same in every round
+  int bK[JAC_BLOCKS], bL[JAC_BLOCKS];
+  const int nblk = npair * (npair + 1) / 2;
+#pragma unroll
+  for (int q = 0; q < JAC_BLOCKS; ++q) {
+    const int e = threadIdx.x + q * JAC_THREADS;
+    int L = int((sqrtf(8.0f * e + 1.0f) - 1.0f) * 0.5f);
+    while (L * (L + 1) / 2 > e) --L;
+    while ((L + 1) * (L + 2) / 2 <= e) ++L;
+    bL[q] = e < nblk ? L : -1;
+    bK[q] = e - L * (L + 1) / 2;
+  }
+  double* tl = d.tlog + size_t(m) * d.tlog_stride;
   // a pair is rotated while |a_ij| > 1e-14 sqrt(a_ii a_jj) (relative to its own diagonal, which
   // keeps small eigenvalues of the positive semi-definite matrix accurate; well above the FP64
   // rounding of a rotation, so the sweeps end); the sweeps stop when one rotates no pair
-  int* rotated = pj + 2 * (p / 2 + 1);
+  int nround = 0;
   for (int sweep = 0; sweep < JAC_MAX_SWEEPS; ++sweep) {
     if (threadIdx.x == 0) *rotated = 0;
     __syncthreads();
-    for (int r = 0; r < P2 - 1; ++r) {
-      // round r: player 0 fixed, the others rotate; pair k = (pos[k], pos[P2 - 1 - k])
+    for (int r = 0; r < P2 - 1; ++r, ++nround) {
       for (int k = threadIdx.x; k < npair; k += blockDim.x) {
-        auto pos = [&](int t) { return t == 0 ? 0 : 1 + (t - 1 + r) % (P2 - 1); };
-        int a = pos(k), b = pos(P2 - 1 - k);
-        if (a > b) { const int t = a; a = b; b = t; }
-        double c = 1.0, s = 0.0;
-        bool rot = false;
+        int a, b;
+        jac_pair(k, r, P2, a, b);
+        double t = 0.0;
         if (b < p) {
-          const double apq = A[a * ld + b];
-          const double app = A[a * ld + a], aqq = A[b * ld + b];
-          if (fabs(apq) > 1e-14 * sqrt(fabs(app * aqq))) {
-            const double tau = (aqq - app) / (2.0 * apq);
-            const double t = fabs(tau) < 1e150 ? (tau >= 0.0 ? 1.0 : -1.0) / (fabs(tau) + sqrt(1.0 + tau * tau))
-                                               : 0.5 / tau;
-            c = 1.0 / sqrt(1.0 + t * t);
-            s = t * c;
-            rot = true;
-          }
+          const double apq = A[b * ld + a], app = A[a * ld + a], aqq = A[b * ld + b];
+          if (apq * apq > 1e-28 * fabs(app * aqq)) t = tan_of(app, aqq, apq);
+          if (!(fabs(t) <= 2.0)) t = 0.0;      // outside the estimates' range: nothing to rotate
         }
-        if (rot) *rotated = 1;
-        pj[k] = rot ? a : -1; pj[npair + k] = b;
-        cs[k] = c; cs[npair + k] = s;
+        const double c = t != 0.0 ? cos_of(t) : 1.0;
+        if (t != 0.0) *rotated = 1;
+        pj[k] = a; pj[npair + k] = b;
+        cs[k] = c; cs[npair + k] = t * c;
+        tl[size_t(nround) * npair + k] = t;
       }
       __syncthreads();
-      // A <- A J and W <- W J: columns a, b of every pair (disjoint columns)
-      for (int e = threadIdx.x; e < npair * p; e += blockDim.x) {
-        const int k = e / p, row = e - k * p;
-        const int a = pj[k], b = pj[npair + k];
-        if (a < 0) continue;
-        const double c = cs[k], s = cs[npair + k];
-        const double x = A[row * ld + a], y = A[row * ld + b];
-        A[row * ld + a] = c * x - s * y;
-        A[row * ld + b] = s * x + c * y;
-        const double u = W[row * ld + a], v = W[row * ld + b];
-        W[row * ld + a] = c * u - s * v;
-        W[row * ld + b] = s * u + c * v;
+#pragma unroll
+      for (int q = 0; q < JAC_BLOCKS; ++q) {
+        const int K = bK[q], L = bL[q];
+        if (L < 0) continue;
+        const double cK = cs[K], sK = cs[npair + K], cL = cs[L], sL = cs[npair + L];
+        if (sK == 0.0 && sL == 0.0) continue;
+        const int a = pj[K], b = pj[npair + K], u = pj[L], v = pj[npair + L];
+        auto at = [&](int i, int j) -> double& { return i >= j ? A[i * ld + j] : A[j * ld + i]; };
+        const bool hb = b < p, hv = v < p;
+        const double xau = at(a, u), xav = hv ? at(a, v) : 0.0;
+        const double xbu = hb ? at(b, u) : 0.0, xbv = hb && hv ? at(b, v) : 0.0;
+        const double yau = cL * xau - sL * xav, yav = sL * xau + cL * xav;
+        const double ybu = cL * xbu - sL * xbv, ybv = sL * xbu + cL * xbv;
+        at(a, u) = cK * yau - sK * ybu;
+        if (hv) at(a, v) = cK * yav - sK * ybv;
+        if (K != L && hb) at(b, u) = sK * yau + cK * ybu;     // K == L: the entry (a, v) again
+        if (hb && hv) at(b, v) = sK * yav + cK * ybv;
       }
-      __syncthreads();
-      // A <- J^T A: rows a, b of every pair (disjoint rows)
-      for (int e = threadIdx.x; e < npair * p; e += blockDim.x) {
-        const int k = e / p, col = e - k * p;
-        const int a = pj[k], b = pj[npair + k];
-        if (a < 0) continue;
+      for (int e = threadIdx.x; e < 2 * npair; e += blockDim.x) {
+        const int k = e >> 1, a = pj[k], b = pj[npair + k];
+        if (b >= p) continue;
         const double c = cs[k], s = cs[npair + k];
-        const double x = A[a * ld + col], y = A[b * ld + col];
-        A[a * ld + col] = c * x - s * y;
-        A[b * ld + col] = s * x + c * y;
+        const double x = bv[2 * a + (e & 1)], y = bv[2 * b + (e & 1)];
+        bv[2 * a + (e & 1)] = c * x - s * y;
+        bv[2 * b + (e & 1)] = s * x + c * y;
       }
       __syncthreads();
     }
-    if (!*rotated) break;
+    const bool more = *rotated != 0;
     __syncthreads();
+    if (!more) break;
   }
   // threshold on the eigenvalues lambda = s^2: tol > 0 absolute on s, < 0 relative to s_max,
   // 0: every positive s
   double lmax = 0.0;
   for (int i = threadIdx.x; i < p; i += blockDim.x) lmax = fmax(lmax, A[i * ld + i]);
-  for (int o = 16; o > 0; o >>= 1) lmax = fmax(lmax, __shfl_xor_sync(0xffffffffu, lmax, o));
-  __syncthreads();
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = lmax;
-  __syncthreads();
-  lmax = 0.0;
-  for (int w = 0; w < int(blockDim.x >> 5); ++w) lmax = fmax(lmax, red[w]);
+  lmax = block_max(lmax);
+  const double un = scalbn(1.0, ex);                       // eigenvalues of the unscaled matrix
   const double tol = d.tsvd_tol;
-  const double thr = tol > 0.0 ? tol * tol : (tol < 0.0 ? tol * tol * lmax : 0.0);
-  // z = Lambda~^-1 W^T b (kept eigenvalues only) in the last 2p doubles of A (A's entries are no
-  // longer needed once its diagonal is saved), then x' = W z
-  const double* bm = rhs + size_t(m) * n * 2;
-  double* zv = A + size_t(p) * ld - 2 * p;
-  // the eigenvalues go to W's padding column W[i][p] (ld = p + 1)
-  __syncthreads();
-  for (int i = threadIdx.x; i < p; i += blockDim.x) W[i * ld + p] = A[i * ld + i];
-  __syncthreads();
-  for (int e = threadIdx.x; e < 2 * p; e += blockDim.x) {
-    const int i = e >> 1, side = e & 1;
-    double sacc = 0.0;
-    for (int k = 0; k < p; ++k) sacc = fma(W[k * ld + i], bm[k * 2 + side], sacc);
-    const double lam = W[i * ld + p];
-    zv[e] = (thr > 0.0 ? lam >= thr : lam > 0.0) ? sacc / lam : 0.0;
+  const double thr = tol > 0.0 ? tol * tol : (tol < 0.0 ? tol * tol * (un * lmax) : 0.0);
+  for (int e = threadIdx.x; e < 2 * p; e += blockDim.x) {  // z = Lambda~^-1 W^T b
+    const int i = e >> 1;
+    const double lam = un * A[i * ld + i];
+    bv[e] = (thr > 0.0 ? lam >= thr : lam > 0.0) ? bv[e] / lam : 0.0;
+  }
+  // x' = W z: the rotations in reverse order, a batch of rounds' tangents at a time (the matrix
+  // is no longer needed; its storage holds their cosines and sines)
+  const int batch = max(1, (p * ld) / (2 * npair));
+  double* lc = A;
+  for (int r1 = nround; r1 > 0; r1 -= batch) {
+    const int r0 = max(0, r1 - batch), cnt = (r1 - r0) * npair;
+    double* ls = lc + cnt;
+    __syncthreads();
+    for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
+      const double t = tl[size_t(r0) * npair + e];
+      const double c = t != 0.0 ? cos_of(t) : 1.0;
+      lc[e] = c;
+      ls[e] = t * c;
+    }
+    __syncthreads();
+    if (threadIdx.x < 2 * TSVD_MAX_NZ / 2) {               // the threads of one named barrier
+      for (int r = r1 - 1; r >= r0; --r) {
+        for (int e = threadIdx.x; e < 2 * npair; e += TSVD_MAX_NZ) {
+          const int k = e >> 1;
+          const double c = lc[(r - r0) * npair + k], s = ls[(r - r0) * npair + k];
+          int a, b;
+          jac_pair(k, r % (P2 - 1), P2, a, b);
+          if (s == 0.0 || b >= p) continue;
+          const double x = bv[2 * a + (e & 1)], y = bv[2 * b + (e & 1)];
+          bv[2 * a + (e & 1)] = c * x + s * y;
+          bv[2 * b + (e & 1)] = c * y - s * x;
+        }
+        asm volatile("bar.sync 1, %0;" ::"n"(TSVD_MAX_NZ) : "memory");
+      }
+    }
   }
   __syncthreads();
   bool bad = false;
   for (int e = threadIdx.x; e < 2 * p; e += blockDim.x) {
-    const int i = e >> 1, side = e & 1;
-    double sacc = 0.0;
-    for (int k = 0; k < p; ++k) sacc = fma(W[i * ld + k], zv[k * 2 + side], sacc);
-    xo[e] = sacc;
-    if (!isfinite(sacc)) bad = true;
+    xo[e] = bv[e];
+    if (!isfinite(bv[e])) bad = true;
   }
   for (int e = 2 * p + threadIdx.x; e < 2 * n; e += blockDim.x) xo[e] = 0.0;
   bad = __syncthreads_or(bad);
@@ -202,7 +295,14 @@ __global__ void __launch_bounds__(JAC_THREADS) tsvd_jacobi_kernel(Dev d, const d
 }  // namespace
 
 size_t tsvd_smem_bytes(int p) {
-  return (2 * size_t(p) * (p + 1) + 2 * size_t(p / 2 + 1) + 32) * sizeof(double) + (2 * size_t(p / 2 + 1) + 1) * sizeof(int);
+  const size_t P2 = (p + 1) & ~1;
+  return (size_t(p) * (p + 1) + 2 * p + P2 + 32) * sizeof(double) + (P2 + 1) * sizeof(int);
+}
+
+// doubles of one subproblem's rotation log: every pair of every round of the most sweeps
+size_t tsvd_log_doubles(int p) {
+  const size_t P2 = (p + 1) & ~1;
+  return size_t(JAC_MAX_SWEEPS) * (P2 - 1) * (P2 / 2);
 }
 
 cudaError_t prepare_variants(int nz) {

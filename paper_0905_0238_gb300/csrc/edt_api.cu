@@ -105,7 +105,7 @@ struct edt_ctx {
   Region r_fc, r_ltop, r_lvel, r_zl, r_zo, r_rows, r_roff, r_roffmf, r_band, r_bcol, r_cpre, r_kval, r_pairm, r_fjoff, r_fjent, r_jact, r_jmap, r_Gs, r_U, r_Dw, r_A32, r_tw64, r_tw32, r_segm, r_segr0,
       r_segn, r_ctas, r_mslot, r_zo32, r_fc32, r_coef, r_coef32, r_g64, r_g32, r_g32lo, r_rowmax, r_gscale, r_X, r_Dst, r_Vst, r_rhs, r_gent, r_gpart, r_G,
       r_dinv, r_L32, r_dinv32, r_b, r_tr, r_tpart, r_x, r_r, r_rpart, r_rowc, r_xmu, r_gam, r_tref, r_treoff, r_vhat, r_vfull, r_gscr, r_adj, r_gacc, r_gcpart, r_bexp, r_bfold, r_status, r_flags,
-      r_tlog, r_kzP, r_kzp, r_kzgoff, r_kzvoff, r_kzG, r_kzT, r_kzb, r_kzx;
+      r_g64part, r_b64part, r_tlog, r_kzP, r_kzp, r_kzgoff, r_kzvoff, r_kzG, r_kzT, r_kzb, r_kzx;
   Dev dev{};
   cudaStream_t last_stream = nullptr;
   int last_status = EDT_OK;
@@ -707,6 +707,9 @@ void layout(edt_ctx* c) {
   take(c->r_status, ns * sizeof(int));
   take(c->r_flags, 8 * sizeof(unsigned));
   const bool disk = !c->kz_p.empty();
+  const size_t gsp = mixed ? 1 : gram_f64_split(c->nz, c->nsub);
+  take(c->r_g64part, gsp > 1 ? gram_f64_part_doubles(c->nz, c->nsub) * sizeof(double) : 0);
+  take(c->r_b64part, gsp > 1 ? ns * gsp * nz * 2 * sizeof(double) : 0);
   take(c->r_tlog, c->cfg.solver == EDT_SOLVE_TSVD ? ns * tsvd_log_doubles(c->nz) * sizeof(double) : 0);
   take(c->r_kzP, disk ? size_t(nz) * nz * sizeof(double) : 0);
   take(c->r_kzp, disk ? ns * sizeof(int) : 0);
@@ -818,6 +821,9 @@ void bind(edt_ctx* c) {
   d.flags = at<unsigned*>(c, c->r_flags);
   d.solver = c->cfg.solver;
   d.tsvd_tol = c->cfg.tsvd_tol;
+  d.g64_split = c->cfg.precision == EDT_MIXED ? 1 : gram_f64_split(c->nz, c->nsub);
+  d.g64part = c->r_g64part.bytes ? at<double*>(c, c->r_g64part) : nullptr;
+  d.b64part = c->r_b64part.bytes ? at<double*>(c, c->r_b64part) : nullptr;
   d.tlog = c->r_tlog.bytes ? at<double*>(c, c->r_tlog) : nullptr;
   d.tlog_stride = c->r_tlog.bytes ? tsvd_log_doubles(c->nz) : 0;
   const bool disk = c->r_kzP.bytes > 0;
@@ -1057,6 +1063,7 @@ int edt_set_workspace(edt_ctx* c, void* ws, size_t bytes) {
   EDT_TRY(prepare_grad());
   EDT_TRY(prepare_chol(c->dev));
   if (c->cfg.precision == EDT_MIXED) EDT_TRY(prepare_gram_tc(c->dev));
+  else EDT_TRY(prepare_gram_f64(c->dev));
   if (c->band_mode) EDT_TRY(prepare_band(c->dev));
   if (c->win) EDT_TRY(prepare_fa(c->dev));
   if (!c->aux) {
@@ -1526,7 +1533,8 @@ int edt_get_stats(edt_ctx* c, edt_stats* o) {
     for (const BandChunk& ch : c->bchunks) tr_launches += 1 + (ch.nbcol > 0) + (ch.nrow > 0);
   }
   const int chol_n = c->dev.chol_df ? chol_dfloat_launches(c->nz) : chol_launches(c->nz);
-  o->launches_per_invert = (c->cfg.precision == EDT_MIXED ? 6 + 3 * c->cfg.refine : 5) + tr_launches +
+  o->launches_per_invert = (c->cfg.precision == EDT_MIXED ? 6 + 3 * c->cfg.refine
+                                                          : 5 + (gram_f64_split(c->nz, c->nsub) > 1)) + tr_launches +
                            chol_n + gram_scale_launches(c->dev, green_tables(c) != GREEN_G32DF);
   // solver variants replace the Cholesky launch: trace, two projections, the solve (Cholesky
   // or Jacobi), the back-projection with the disk; the Jacobi kernel alone without it

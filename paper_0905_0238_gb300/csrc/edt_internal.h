@@ -192,6 +192,10 @@ struct Dev {
   double* kz_T;                 // [nsub][nz][p] scratch G P_p
   double* kz_b;                 // [nsub][nz][2] restricted right-hand sides
   double* kz_x;                 // [nsub][nz][2] restricted solutions
+  // FP64 Gram: parts a subproblem's rows are added in, at most, and their sums
+  int g64_split;
+  double* g64part;              // [nsub][groups][g64_split] tile sums (csrc/gram_f64.cu)
+  double* b64part;              // [nsub][g64_split][nz][2]
   double* tlog;                 // [nsub][tlog_stride] tangents of the truncated SVD's rotations
   size_t tlog_stride;
 };
@@ -233,6 +237,8 @@ cudaError_t prepare_fa(const Dev& d);
 cudaError_t fft2_f64(const Dev& d, double2* X, int planes, int ny, int sign, double scale, cudaStream_t s);
 
 cudaError_t launch_gram_f64(const Dev& d, cudaStream_t s);
+int gram_f64_split(int nz, int nsub);
+size_t gram_f64_part_doubles(int nz, int nsub);
 cudaError_t launch_gram_tc(const Dev& d, cudaStream_t s);       // partial tiles + trace
 int gram_scale_launches(const Dev& d, bool rowmax_ready);       // FP16 operand scales: 0, 1 or 2 kernels
 int gram_trace_parts();                                         // trace partials per Gram segment
@@ -332,6 +338,7 @@ cudaError_t launch_solve_variant(const Dev& d, cudaStream_t s);
 cudaError_t prepare_fft(const Dev& d);
 cudaError_t prepare_chol(const Dev& d);
 cudaError_t prepare_gram_tc(const Dev& d);
+cudaError_t prepare_gram_f64(const Dev& d);
 cudaError_t prepare_grad();
 
 // Tensor-core Gram tiling (shared by host planning and the kernel).

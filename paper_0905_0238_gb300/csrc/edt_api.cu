@@ -1524,7 +1524,7 @@ int edt_get_stats(edt_ctx* c, edt_stats* o) {
   o->workspace_bytes = c->ws_bytes;
   o->gram_flop = 2.0 * 2.0 * double(o->rows_solved) * double(c->nz) * double(c->nz + 2);
   o->last_status = c->last_status;
-  // kernels launched by one edt_invert: green (3), per frequency chunk transform (2) and
+  // kernels launched by one edt_invert: the depth march, per frequency chunk transform (2) and
   // right-hand sides (1), Gram (FP64: 1; mixed: tensor-core + reduce 2), batched Cholesky,
   // per refinement step (3: partial residuals, their ordered sum, the update), inverse (1)
   int tr_launches = c->fchunk > 0 ? 3 * ((c->nf + c->fchunk - 1) / c->fchunk) : 0;
@@ -1533,8 +1533,9 @@ int edt_get_stats(edt_ctx* c, edt_stats* o) {
     for (const BandChunk& ch : c->bchunks) tr_launches += 1 + (ch.nbcol > 0) + (ch.nrow > 0);
   }
   const int chol_n = c->dev.chol_df ? chol_dfloat_launches(c->nz) : chol_launches(c->nz);
-  o->launches_per_invert = (c->cfg.precision == EDT_MIXED ? 6 + 3 * c->cfg.refine
-                                                          : 5 + (gram_f64_split(c->nz, c->nsub) > 1)) + tr_launches +
+  o->launches_per_invert = green_launches(c->dev, green_tables(c)) +
+                           (c->cfg.precision == EDT_MIXED ? 3 + 3 * c->cfg.refine
+                                                          : 2 + (gram_f64_split(c->nz, c->nsub) > 1)) + tr_launches +
                            chol_n + gram_scale_launches(c->dev, green_tables(c) != GREEN_G32DF);
   // solver variants replace the Cholesky launch: trace, two projections, the solve (Cholesky
   // or Jacobi), the back-projection with the disk; the Jacobi kernel alone without it
@@ -1544,15 +1545,15 @@ int edt_get_stats(edt_ctx* c, edt_stats* o) {
     // refinement (3 per step), inverse (completion, FP64 row and column transforms, output: 3 or 4)
     int fk = 0;
     for (int n : c->nact) fk += n > 0;
-    o->launches_per_invert = 3 + 3 * fk + 2 + 2 + chol_n + 3 * c->cfg.refine +
+    o->launches_per_invert = green_launches(c->dev, green_tables(c)) + 3 * fk + 2 + 2 + chol_n + 3 * c->cfg.refine +
                              (c->ny > 1 ? 4 : 3);
   }
   o->freq_chunk = c->band_mode ? c->band_maxplanes : c->fchunk;
-  // misfit gradient: green (3), zero, lateral DFT and its FP32 copy, per chunk transform (2), the
+  // misfit gradient: green, zero, lateral DFT and its FP32 copy, per chunk transform (2), the
   // residual (2) and two contractions, depth march forward / field / reversed (3), inverse
   // lateral DFT, finalize
   o->launches_per_grad = grad_supported(c->dev) && c->fchunk > 0
-                             ? 3 + 3 + 6 * ((c->nf + c->fchunk - 1) / c->fchunk) + 5 : 0;
+                             ? green_launches(c->dev, GREEN_G32) + 3 + 6 * ((c->nf + c->fchunk - 1) / c->fchunk) + 5 : 0;
   o->gram_rows_padded = 0;
   for (long long n : c->seg_nrow) o->gram_rows_padded += (n + TC_KC - 1) / TC_KC * TC_KC;
   if (c->ws) {

@@ -211,6 +211,7 @@ constexpr int GREEN_G32F = 8;
 // of layers times FP32 rounding, for the line inversion with the FP32 residual);
 // GREEN_G32DF: the FP64 evaluation written as the double-float pair g32 + g32lo (no g64)
 cudaError_t launch_green(const Dev& d, cudaStream_t s, int tables);
+int green_launches(const Dev& d, int tables);                   // kernels it launches
 
 // Data transform of frequency planes [f0, f0 + nfc) into X, then the split right-hand
 // sides of every subproblem's rows at those frequencies (X holds only the chunk).

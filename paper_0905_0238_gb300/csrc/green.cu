@@ -13,15 +13,16 @@
 // depth sample to the next by multiplication with exp(+-i kappa_j dz) (error ~ n ulp),
 // re-anchored by a direct evaluation at every layer entry and chunk start.
 //
-// Kernels: green_layer (one thread per (f, n, layer): vertical wavenumber and the layer's
-// phase factors, the FP64 transcendentals, fully parallel), green_recursion (one thread
-// per (f, n): the two recursions, FP64), then one of two evaluations:
+// Kernels: green_layer (one thread per (f, n, layer): vertical wavenumber, the layer's phase
+// factors and the interface's recursion coefficients, fully parallel), green_recursion (one
+// thread per (f, n): the two recursions in a division-free form, FP64), then one of two
+// evaluations:
 //   green_eval64  (FP64 table, and/or the FP32 table sqrt|s_f| g rounded from it, with the
 //                 rounding remainder as a second FP32 table for a double-float pair):
-//                 a CTA per (f, block of 32 n); each warp marches a chunk of depths by the
-//                 recurrence and stages its tile in shared memory so the table rows are
-//                 written coalesced;
-//   green_eval32  (FP32 table sqrt|s_f| g for the mixed path): one thread per (f, n, z);
+//                 a warp per 32 rows (f, n) and 16 depths marches them by the recurrence and
+//                 stages its tile in shared memory so the table rows are written coalesced;
+//   green_eval32  (FP32 table sqrt|s_f| g for the mixed path; green_coef32 rounds the layers'
+//                 coefficients for it): one thread per (f, n, z);
 //                 each exponential's phase and decay are formed and range-reduced in FP64
 //                 (Cody-Waite for the phase, integer/fraction split for the decay) and
 //                 evaluated with FP32 sincos/exp2 of the reduced arguments, ~1e-7 relative.
@@ -41,10 +42,10 @@ namespace edt {
 
 namespace {
 
-// coefficient slots per (f, n, layer): kappa, rho, amp, exp(i kappa dz), exp(-i kappa dz),
-// exp(i kappa h), 1 / (1 + r_{j+1})
+// coefficient slots per (f, n, layer): kappa; sigma, then M; tau, then T; exp(i kappa dz),
+// exp(-i kappa dz); exp(i kappa h); delta, then D (see green_layer and green_recursion)
 constexpr int NCOEF = 7;
-constexpr int C_KAP = 0, C_RHO = 1, C_AMP = 2, C_E = 3, C_EI = 4, C_EH = 5, C_INV1R = 6;
+constexpr int C_KAP = 0, C_SIG = 1, C_MUP = 1, C_AMP = 2, C_E = 3, C_EI = 4, C_EH = 5, C_DEL = 6, C_DEN = 6;
 // FP32 copies for the fast evaluation: kappa.x and kappa.y as (hi, lo) pairs, amp, rho
 constexpr int NCOEF32 = 8;
 
@@ -60,7 +61,37 @@ __device__ __forceinline__ double2 cinv(double2 b) {
   return cmk(b.x * r, -b.y * r);
 }
 
-__global__ void green_layer_kernel(Dev d, int want_steps) {
+// sqrt(w) on the branch Im >= 0, FP64: the FP32 root (relative error ~1e-7) and two Newton steps
+// k + (w - k^2) / (2 k) whose residual is formed in FP64 and whose divisor is the FP32 root's (it
+// only scales the correction): 1e-14, then FP64 rounding, in about 20 FP64 operations instead of
+// the hundred of a complex FP64 root.  Values outside the FP32 range take that root.
+__device__ __forceinline__ double2 kappa_of(double2 w) {
+  const double m = fmax(fabs(w.x), fabs(w.y));
+  if (!(m > 1e-25 && m < 1e25)) return csqrt_upper(w);
+  const float2 k32 = csqrt_upper32(make_float2(float(w.x), float(w.y)));
+  const float2 inv = cinv32(make_float2(2.f * k32.x, 2.f * k32.y));
+  double2 k = cmk(double(k32.x), double(k32.y));
+#pragma unroll
+  for (int it = 0; it < 2; ++it) {
+    const double rr = fma(k.y, k.y, fma(-k.x, k.x, w.x)), ri = fma(-2.0 * k.x, k.y, w.y);
+    const float2 dk = make_float2(float(rr), float(ri)) * inv;
+    k.x += double(dk.x);
+    k.y += double(dk.y);
+  }
+  return k;
+}
+
+// 2^-e of a positive double's exponent e (|v| in [2^e, 2^(e+1))), by its bits
+__device__ __forceinline__ double pow2_down(double v) {
+  const int e = (__double2hiint(v) >> 20) & 0x7ff;
+  return __hiloint2double(min(max(2046 - e, 1), 2046) << 20, 0);
+}
+
+// Per (f, n, layer), fully parallel: kappa_j, exp(i kappa_j h_j), the step factors
+// exp(+-i kappa_j dz) of layers that may hold two depth samples, and the interface's recursion
+// coefficients sigma = lambda (kappa_j + kappa_{j+1}), delta = lambda (kappa_j - kappa_{j+1}) and
+// tau = 2 kappa_j lambda exp(i kappa_j h_j), lambda the power of two that puts sigma near 1.
+__global__ void __launch_bounds__(128) green_layer_kernel(Dev d, int want_steps) {
   const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int J = d.nlayer;
   const long long total = (long long)d.nf * d.nk * J;
@@ -74,63 +105,122 @@ __global__ void green_layer_kernel(Dev d, int want_steps) {
   const double2 om = cmk(fc.om_re, fc.om_im);
   const double2 om2 = om * om;
   const double inv_c2 = 1.0 / (d.layer_vel[j] * d.layer_vel[j]);
-  const double2 kap = csqrt_upper(cmk(om2.x * inv_c2 - k * k, om2.y * inv_c2));
+  const double2 kap = kappa_of(cmk(om2.x * inv_c2 - k * k, om2.y * inv_c2));
   double2* c = d.coef;
   c[cix(d, f, n, j, C_KAP)] = kap;
+  double h = 2.0 * d.dz;
   if (j < J - 1) {
-    const double h = d.layer_top[j + 1] - d.layer_top[j];
-    c[cix(d, f, n, j, C_EH)] = cexp(cmk(-kap.y * h, kap.x * h));
-  } else {
-    c[cix(d, f, n, j, C_EH)] = cmk(1.0, 0.0);
+    h = d.layer_top[j + 1] - d.layer_top[j];
+    const double2 eh = cexp(cmk(-kap.y * h, kap.x * h));
+    const double ic2n = 1.0 / (d.layer_vel[j + 1] * d.layer_vel[j + 1]);
+    const double2 kn = kappa_of(cmk(om2.x * ic2n - k * k, om2.y * ic2n));
+    const double2 sg = kap + kn;
+    const double lam = pow2_down(fmax(fabs(sg.x), fabs(sg.y)));
+    c[cix(d, f, n, j, C_EH)] = eh;
+    c[cix(d, f, n, j, C_SIG)] = lam * sg;
+    c[cix(d, f, n, j, C_DEL)] = lam * (kap - kn);
+    c[cix(d, f, n, j, C_AMP)] = (2.0 * lam) * (kap * eh);
   }
-  if (want_steps) {
+  // samples are dz apart, so a thinner layer holds one at most
+  if (want_steps && h > 0.999 * d.dz) {
     const double2 E = cexp(cmk(-kap.y * d.dz, kap.x * d.dz));
     c[cix(d, f, n, j, C_E)] = E;
-    c[cix(d, f, n, j, C_EI)] = cdiv(cmk(1.0, 0.0), E);
+    c[cix(d, f, n, j, C_EI)] = cinv(E);
   }
 }
 
-__global__ void green_recursion_kernel(Dev d) {
-  const int n = blockIdx.x * blockDim.x + threadIdx.x;
-  const int f = blockIdx.y;
-  if (n >= d.nk) return;
+// Per (f, n), the serial part.  With r_j = N_j / D_j the upward recursion of the header is linear,
+//   M_j = delta_j D_{j+1} + sigma_j N_{j+1},  D_j = sigma_j D_{j+1} + delta_j N_{j+1},
+//   N_j = exp(2 i kappa_j h_j) M_j,   rho_j = M_j / D_j,
+// from N = 0, D = 1 at the half-space, and the downward one telescopes:
+//   A_j = (i / (2 kappa_0)) prod_{i < j} (2 kappa_i exp(i kappa_i h_i)) D_j / D_0
+// (the powers of two lambda_i cancel against tau_i).  No division is left on the chains, three
+// multiply-adds and a product per layer upward and one product downward; the two divisions of
+// the plain recursion took 60 dependent FP64 operations per layer.  Every eighth layer the pair
+// is rescaled by a power of two (into tau too), so that thousands of layers neither overflow nor
+// vanish.  Leaves M_j (C_MUP), D_j (C_DEN) and T_j = A_j / D_j (C_AMP).
+__global__ void __launch_bounds__(32) green_recursion_kernel(Dev d) {
+  const long long gid = (long long)blockIdx.x * 32 + threadIdx.x;
+  if (gid >= (long long)d.nf * d.nk) return;
+  const int f = int(gid / d.nk), n = int(gid - (long long)f * d.nk);
   const int J = d.nlayer;
-  double2* c = d.coef;
-  const double2 one = cmk(1.0, 0.0);
-  // upward recursion for the reflection coefficient of the stack below each interface
-  double2 r_next = cmk(0.0, 0.0);
-  c[cix(d, f, n, J - 1, C_RHO)] = cmk(0.0, 0.0);
-  double2 kn = c[cix(d, f, n, J - 1, C_KAP)];
-  for (int j = J - 2; j >= 0; --j) {
-    const double2 kj = c[cix(d, f, n, j, C_KAP)], eh = c[cix(d, f, n, j, C_EH)];
-    const double2 inv1r = cinv(one + r_next);             // 1 / (1 + r_{j+1})
-    const double2 y = kn * (one - r_next) * inv1r;
-    const double2 rho = (kj - y) * cinv(kj + y);
-    c[cix(d, f, n, j, C_RHO)] = rho;
-    c[cix(d, f, n, j, C_INV1R)] = inv1r;
-    r_next = rho * (eh * eh);
-    kn = kj;
+  const size_t lst = size_t(NCOEF) * d.nk;                // from a layer to the next
+  double2* c = d.coef + cix(d, f, n, 0, 0);
+  const size_t nk = d.nk;
+  double2 N = cmk(0.0, 0.0), D = cmk(1.0, 0.0);
+  {
+    double2* cl = c + lst * (J - 1);
+    cl[C_MUP * nk] = N;
+    cl[C_DEN * nk] = D;
   }
-  // downward recursion for the downgoing amplitude; jump g'(0+) - g'(0-) = -1
-  const double2 k0 = c[cix(d, f, n, 0, C_KAP)];
-  double2 amp = cmk(0.0, 0.5) * cinv(k0);
-  for (int j = 0; j < J - 1; ++j) {
-    c[cix(d, f, n, j, C_AMP)] = amp;
-    amp = amp * c[cix(d, f, n, j, C_EH)] * (one + c[cix(d, f, n, j, C_RHO)]) * c[cix(d, f, n, j, C_INV1R)];
-  }
-  c[cix(d, f, n, J - 1, C_AMP)] = amp;
-  if (d.coef32) {
-    float* c32 = d.coef32 + (size_t(f) * d.nk + n) * size_t(J) * NCOEF32;
-    for (int j = 0; j < J; ++j) {
-      const double2 kap = c[cix(d, f, n, j, C_KAP)], a = c[cix(d, f, n, j, C_AMP)], r = c[cix(d, f, n, j, C_RHO)];
-      const float kxh = float(kap.x), kyh = float(kap.y);
-      float* o = c32 + j * NCOEF32;
-      o[0] = kxh; o[1] = float(kap.x - double(kxh));
-      o[2] = kyh; o[3] = float(kap.y - double(kyh));
-      o[4] = float(a.x); o[5] = float(a.y);
-      o[6] = j < J - 1 ? float(r.x) : 0.f; o[7] = j < J - 1 ? float(r.y) : 0.f;
+  constexpr int U = 4;                                    // layers loaded ahead of the chain
+  for (int j1 = J - 1; j1 > 0; j1 -= U) {
+    double2 sg[U], de[U], eh[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int j = j1 - 1 - u;
+      if (j < 0) continue;
+      const double2* cl = c + lst * j;
+      sg[u] = cl[C_SIG * nk]; de[u] = cl[C_DEL * nk]; eh[u] = cl[C_EH * nk];
+    }
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const int j = j1 - 1 - u;
+      if (j < 0) continue;
+      double2* cl = c + lst * j;
+      double2 M = de[u] * D + sg[u] * N;
+      D = sg[u] * D + de[u] * N;
+      const double2 E = eh[u] * eh[u];
+      if ((j & 7) == 0) {
+        const double s = pow2_down(fmax(fabs(D.x), fabs(D.y)));
+        D = s * D;
+        M = s * M;
+        cl[C_AMP * nk] = s * cl[C_AMP * nk];
+      }
+      N = E * M;
+      cl[C_MUP * nk] = M;
+      cl[C_DEN * nk] = D;
     }
   }
+  double2 T = cmk(0.0, 0.5) * cinv(c[C_KAP * nk] * D);    // A_0 / D_0
+  for (int j0 = 0; j0 < J; j0 += 2 * U) {
+    double2 tau[2 * U];
+#pragma unroll
+    for (int u = 0; u < 2 * U; ++u)
+      if (j0 + u < J - 1) tau[u] = c[lst * (j0 + u) + C_AMP * nk];
+#pragma unroll
+    for (int u = 0; u < 2 * U; ++u) {
+      if (j0 + u >= J) continue;
+      c[lst * (j0 + u) + C_AMP * nk] = T;
+      if (j0 + u < J - 1) T = T * tau[u];
+    }
+  }
+}
+
+// amplitude and reflection of layer j from the recursion's M, D, T
+__device__ __forceinline__ void layer_waves(const Dev& d, int f, int n, int j, double2& amp, double2& rho) {
+  const double2 D = d.coef[cix(d, f, n, j, C_DEN)];
+  amp = d.coef[cix(d, f, n, j, C_AMP)] * D;
+  rho = j < d.nlayer - 1 ? d.coef[cix(d, f, n, j, C_MUP)] * cinv(D) : cmk(0.0, 0.0);
+}
+
+// the FP32 coefficients green_eval32 reads, per (f, n, layer)
+__global__ void __launch_bounds__(128) green_coef32_kernel(Dev d) {
+  const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int J = d.nlayer;
+  if (gid >= (long long)d.nf * d.nk * J) return;
+  const int n = int(gid % d.nk);
+  const long long fj = gid / d.nk;
+  const int j = int(fj % J), f = int(fj / J);
+  double2 a, r;
+  layer_waves(d, f, n, j, a, r);
+  const double2 kap = d.coef[cix(d, f, n, j, C_KAP)];
+  float4 k4;
+  split_ff(kap.x, k4.x, k4.y);
+  split_ff(kap.y, k4.z, k4.w);
+  float4* o = reinterpret_cast<float4*>(d.coef32 + ((size_t(f) * d.nk + n) * J + j) * NCOEF32);
+  o[0] = k4;
+  o[1] = make_float4(float(a.x), float(a.y), float(r.x), float(r.y));
 }
 
 // The FP32 recursion's rounding errors (and those of its FP32 exponentials) compound over the
@@ -206,21 +296,21 @@ __global__ void __launch_bounds__(128) green_rec32_kernel(Dev d) {
   }
 }
 
-constexpr int EV_WARPS = 4;
-constexpr int EV_ZC = 16;   // depths per warp chunk
+constexpr int EV_ZC = 16;   // depths per warp
 
-__global__ void __launch_bounds__(EV_WARPS * 32) green_eval64_kernel(Dev d) {
-  __shared__ double2 tile[EV_WARPS][32][EV_ZC + 1];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int f = blockIdx.y;
-  const int n0 = blockIdx.x * 32;
-  const int n = n0 + lane;
+// One warp per 32 table rows (of any frequencies) and 16 depths: the FP64 unit is the bound, so
+// the lanes are filled across frequencies and the depths spread over as many SMs as there are.
+__global__ void __launch_bounds__(32) green_eval64_kernel(Dev d) {
+  __shared__ double2 tile[32][EV_ZC + 1];
+  const int lane = threadIdx.x;
+  const long long nrow = (long long)d.nf * d.nk;
+  const long long r0 = (long long)blockIdx.x * 32;
+  const long long row = min(r0 + lane, nrow - 1);
+  const int f = int(row / d.nk), n = int(row - (long long)f * d.nk);
   const int J = d.nlayer;
-  const bool valid = n < d.nk;
   const double2* c = d.coef;
-  const int nn0 = valid ? n : 0;
-  const double sq = sqrt(d.fc[f].s_abs);
-  for (int zc = warp * EV_ZC; zc < d.nz; zc += EV_WARPS * EV_ZC) {
+  const int zc = blockIdx.y * EV_ZC;
+  {
     int cur = -1;
     double2 e1 = cmk(0.0, 0.0), e2 = e1, E = e1, Ei = e1, amp = e1, rho = e1;
     for (int i = 0; i < EV_ZC && zc + i < d.nz; ++i) {
@@ -228,11 +318,12 @@ __global__ void __launch_bounds__(EV_WARPS * 32) green_eval64_kernel(Dev d) {
       const int l = d.z_layer[z];
       if (l != cur) {             // anchor: direct evaluation at layer entry / chunk start
         cur = l;
-        const double2 kap = c[cix(d, f, nn0, l, C_KAP)];
-        rho = c[cix(d, f, nn0, l, C_RHO)];
-        amp = c[cix(d, f, nn0, l, C_AMP)];
-        E = c[cix(d, f, nn0, l, C_E)];
-        Ei = c[cix(d, f, nn0, l, C_EI)];
+        const double2 kap = c[cix(d, f, n, l, C_KAP)];
+        layer_waves(d, f, n, l, amp, rho);
+        if (z + 1 < d.nz && d.z_layer[z + 1] == l) {
+          E = c[cix(d, f, n, l, C_E)];
+          Ei = c[cix(d, f, n, l, C_EI)];
+        }
         const double off = d.z_off[z];
         e1 = cexp(cmk(-kap.y * off, kap.x * off));
         if (l < J - 1) {
@@ -240,34 +331,33 @@ __global__ void __launch_bounds__(EV_WARPS * 32) green_eval64_kernel(Dev d) {
           e2 = cexp(cmk(-kap.y * a, kap.x * a));
         } else {
           e2 = cmk(0.0, 0.0);
-          rho = cmk(0.0, 0.0);
         }
       } else {
         e1 = e1 * E;
         e2 = e2 * Ei;
       }
-      tile[warp][lane][i] = amp * (e1 + rho * e2);
+      tile[lane][i] = amp * (e1 + rho * e2);
     }
-    __syncwarp();
-    const int zi = lane & 15;
-    for (int rr = 0; rr < 32; rr += 2) {
-      const int nl = rr + (lane >> 4);
-      const int nn = n0 + nl;
-      const int z = zc + zi;
-      if (nn < d.nk && z < d.nz) {
-        const double2 v = tile[warp][nl][zi];
-        if (d.g64) d.g64[(size_t(f) * d.nk + nn) * d.nz + z] = v;
-        if (d.g32) {
-          // sqrt|s_f| g rounded to FP32, and (double-float table) the FP32 rounding of the rest
-          const double sx = sq * v.x, sy = sq * v.y;
-          const float hx = float(sx), hy = float(sy);
-          const size_t o32 = (size_t(f) * d.nk + nn) * d.nzs + z;
-          d.g32[o32] = make_float2(hx, hy);
-          if (d.g32lo) d.g32lo[o32] = make_float2(float(sx - double(hx)), float(sy - double(hy)));
-        }
+  }
+  __syncwarp();
+  const int z = zc + (lane & 15);
+  const double sq_lane = d.g32 ? sqrt(d.fc[f].s_abs) : 0.0;
+  for (int rr = 0; rr < 32; rr += 2) {
+    const int nl = rr + (lane >> 4);
+    const double sq = __shfl_sync(0xffffffffu, sq_lane, nl);
+    const long long r = r0 + nl;
+    if (r < nrow && z < d.nz) {
+      const double2 v = tile[nl][lane & 15];
+      if (d.g64) d.g64[size_t(r) * d.nz + z] = v;
+      if (d.g32) {
+        // sqrt|s_f| g rounded to FP32, and (double-float table) the FP32 rounding of the rest
+        const double sx = sq * v.x, sy = sq * v.y;
+        const float hx = float(sx), hy = float(sy);
+        const size_t o32 = size_t(r) * d.nzs + z;
+        d.g32[o32] = make_float2(hx, hy);
+        if (d.g32lo) d.g32lo[o32] = make_float2(float(sx - double(hx)), float(sy - double(hy)));
       }
     }
-    __syncwarp();
   }
 }
 
@@ -307,6 +397,11 @@ __global__ void __launch_bounds__(256) green_eval32_kernel(Dev d) {
 
 }  // namespace
 
+int green_launches(const Dev& d, int tables) {
+  if (tables == GREEN_G32F && d.nlayer <= COEF32_MAX_LAYERS) return 3;
+  return tables == GREEN_G32 || tables == GREEN_G32F ? 4 : 3;
+}
+
 cudaError_t launch_green(const Dev& d, cudaStream_t s, int tables) {
   const bool fast32 = tables == GREEN_G32 || tables == GREEN_G32F;
   dim3 g1((d.nk + 127) / 128, d.nf);
@@ -316,8 +411,9 @@ cudaError_t launch_green(const Dev& d, cudaStream_t s, int tables) {
     green_rec32_kernel<<<g1, 128, 0, s>>>(d);
   } else {
     const long long nl = (long long)d.nf * d.nk * d.nlayer;
-    green_layer_kernel<<<unsigned((nl + 255) / 256), 256, 0, s>>>(d, fast32 ? 0 : 1);
-    green_recursion_kernel<<<g1, 128, 0, s>>>(d);
+    green_layer_kernel<<<unsigned((nl + 127) / 128), 128, 0, s>>>(d, fast32 ? 0 : 1);
+    green_recursion_kernel<<<unsigned(((long long)d.nf * d.nk + 31) / 32), 32, 0, s>>>(d);
+    if (fast32) green_coef32_kernel<<<unsigned((nl + 127) / 128), 128, 0, s>>>(d);
   }
   if (fast32) {
     green_eval32_kernel<<<unsigned((long long)d.nf * d.nk), 256, 0, s>>>(d);
@@ -326,8 +422,8 @@ cudaError_t launch_green(const Dev& d, cudaStream_t s, int tables) {
     if (!(tables & (GREEN_G32 | GREEN_G32DF))) e.g32 = nullptr;
     if (!(tables & GREEN_G32DF)) e.g32lo = nullptr;
     if (!(tables & GREEN_G64)) e.g64 = nullptr;
-    dim3 g2((d.nk + 31) / 32, d.nf);
-    green_eval64_kernel<<<g2, EV_WARPS * 32, 0, s>>>(e);
+    const dim3 g2(unsigned(((long long)d.nf * d.nk + 31) / 32), (d.nz + EV_ZC - 1) / EV_ZC);
+    green_eval64_kernel<<<g2, 32, 0, s>>>(e);
   }
   return cudaGetLastError();
 }

@@ -87,111 +87,222 @@ __device__ __forceinline__ double pow2_down(double v) {
   return __hiloint2double(min(max(2046 - e, 1), 2046) << 20, 0);
 }
 
-// Per (f, n, layer), fully parallel: kappa_j, exp(i kappa_j h_j), the step factors
+// Per (f, n) and LRUN consecutive layers: kappa_j, exp(i kappa_j h_j), the step factors
 // exp(+-i kappa_j dz) of layers that may hold two depth samples, and the interface's recursion
 // coefficients sigma = lambda (kappa_j + kappa_{j+1}), delta = lambda (kappa_j - kappa_{j+1}) and
 // tau = 2 kappa_j lambda exp(i kappa_j h_j), lambda the power of two that puts sigma near 1.
-__global__ void __launch_bounds__(128) green_layer_kernel(Dev d, int want_steps) {
-  const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int J = d.nlayer;
-  const long long total = (long long)d.nf * d.nk * J;
-  if (gid >= total) return;
+// LRUN = 4 forms five kappa for four layers instead of eight; with few layers one per thread
+// spreads better beside the data transform that runs at the same time (13 layers over 9675
+// (f, n): a 256-point line takes 1.13 ms with 1, 1.19 with 4).
+constexpr int LBLOCK = 128;
+template <int LRUN>
+__global__ void __launch_bounds__(LBLOCK) green_layer_kernel(Dev d, int want_steps) {
+  const long long gid = (long long)blockIdx.x * LBLOCK + threadIdx.x;
+  const int J = d.nlayer, nrun = (J + LRUN - 1) / LRUN;
+  if (gid >= (long long)d.nf * d.nk * nrun) return;
   const int n = int(gid % d.nk);                   // wavenumber fastest: coalesced stores
   const long long fj = gid / d.nk;
-  const int j = int(fj % J), f = int(fj / J);
+  const int j0 = int(fj % nrun) * LRUN, f = int(fj / nrun);
   const FreqConst fc = d.fc[f];
-  const double L = double(d.N) * d.dx;
-  const double k = d.kval ? d.kval[n] : 2.0 * M_PI * double(n) / L;
+  const double k = d.kval ? d.kval[n] : double(n) * (2.0 * M_PI / (double(d.N) * d.dx));
   const double2 om = cmk(fc.om_re, fc.om_im);
   const double2 om2 = om * om;
-  const double inv_c2 = 1.0 / (d.layer_vel[j] * d.layer_vel[j]);
-  const double2 kap = kappa_of(cmk(om2.x * inv_c2 - k * k, om2.y * inv_c2));
   double2* c = d.coef;
-  c[cix(d, f, n, j, C_KAP)] = kap;
-  double h = 2.0 * d.dz;
-  if (j < J - 1) {
-    h = d.layer_top[j + 1] - d.layer_top[j];
-    const double2 eh = cexp(cmk(-kap.y * h, kap.x * h));
-    const double ic2n = 1.0 / (d.layer_vel[j + 1] * d.layer_vel[j + 1]);
-    const double2 kn = kappa_of(cmk(om2.x * ic2n - k * k, om2.y * ic2n));
-    const double2 sg = kap + kn;
-    const double lam = pow2_down(fmax(fabs(sg.x), fabs(sg.y)));
-    c[cix(d, f, n, j, C_EH)] = eh;
-    c[cix(d, f, n, j, C_SIG)] = lam * sg;
-    c[cix(d, f, n, j, C_DEL)] = lam * (kap - kn);
-    c[cix(d, f, n, j, C_AMP)] = (2.0 * lam) * (kap * eh);
-  }
-  // samples are dz apart, so a thinner layer holds one at most
-  if (want_steps && h > 0.999 * d.dz) {
-    const double2 E = cexp(cmk(-kap.y * d.dz, kap.x * d.dz));
-    c[cix(d, f, n, j, C_E)] = E;
-    c[cix(d, f, n, j, C_EI)] = cinv(E);
+  auto kappa = [&](int j) {
+    const double inv_c2 = 1.0 / (d.layer_vel[j] * d.layer_vel[j]);
+    return kappa_of(cmk(om2.x * inv_c2 - k * k, om2.y * inv_c2));
+  };
+  double2 kap = kappa(j0);
+#pragma unroll 1
+  for (int j = j0; j < min(J, j0 + LRUN); ++j) {
+    c[cix(d, f, n, j, C_KAP)] = kap;
+    double h = 2.0 * d.dz;
+    double2 kn = kap;
+    if (j < J - 1) {
+      h = d.layer_top[j + 1] - d.layer_top[j];
+      const double2 eh = cexp(cmk(-kap.y * h, kap.x * h));
+      kn = kappa(j + 1);
+      const double2 sg = kap + kn;
+      const double lam = pow2_down(fmax(fabs(sg.x), fabs(sg.y)));
+      c[cix(d, f, n, j, C_EH)] = eh;
+      c[cix(d, f, n, j, C_SIG)] = lam * sg;
+      c[cix(d, f, n, j, C_DEL)] = lam * (kap - kn);
+      c[cix(d, f, n, j, C_AMP)] = (2.0 * lam) * (kap * eh);
+    }
+    // samples are dz apart, so a thinner layer holds one at most
+    if (want_steps && h > 0.999 * d.dz) {
+      const double2 E = cexp(cmk(-kap.y * d.dz, kap.x * d.dz));
+      c[cix(d, f, n, j, C_E)] = E;
+      c[cix(d, f, n, j, C_EI)] = cinv(E);
+    }
+    kap = kn;
   }
 }
 
-// Per (f, n), the serial part.  With r_j = N_j / D_j the upward recursion of the header is linear,
+__device__ __forceinline__ double2 shfl2(double2 v, int src) {
+  return cmk(__shfl_sync(0xffffffffu, v.x, src), __shfl_sync(0xffffffffu, v.y, src));
+}
+__device__ __forceinline__ double cmax(double2 v) { return fmax(fabs(v.x), fabs(v.y)); }
+// s = 2^-e of the exponent e of v (bits), e added to ex
+__device__ __forceinline__ double rescale(double v, int& ex) {
+  const double s = pow2_down(v);
+  ex += 1023 - ((__double2hiint(s) >> 20) & 0x7ff);
+  return s;
+}
+
+// The recursions over the layers.  With r_j = N_j / D_j the upward recursion of the header is linear,
 //   M_j = delta_j D_{j+1} + sigma_j N_{j+1},  D_j = sigma_j D_{j+1} + delta_j N_{j+1},
 //   N_j = exp(2 i kappa_j h_j) M_j,   rho_j = M_j / D_j,
 // from N = 0, D = 1 at the half-space, and the downward one telescopes:
 //   A_j = (i / (2 kappa_0)) prod_{i < j} (2 kappa_i exp(i kappa_i h_i)) D_j / D_0
-// (the powers of two lambda_i cancel against tau_i).  No division is left on the chains, three
-// multiply-adds and a product per layer upward and one product downward; the two divisions of
-// the plain recursion took 60 dependent FP64 operations per layer.  Every eighth layer the pair
-// is rescaled by a power of two (into tau too), so that thousands of layers neither overflow nor
-// vanish.  Leaves M_j (C_MUP), D_j (C_DEN) and T_j = A_j / D_j (C_AMP).
+// (the powers of two lambda_i cancel against tau_i).  No division is left on the chains.  Every
+// eighth layer the pair is rescaled by a power of two (into tau too), so that thousands of
+// layers neither overflow nor vanish.  Leaves M_j (C_MUP), D_j (C_DEN) and T_j = A_j / D_j (C_AMP).
+//
+// S lanes share the layers of one (f, n), a run of layers each.  One warp takes 64 cycles of its
+// quarter of an SM for an FP64 instruction however few lanes work, so a stack of many layers over
+// few (f, n) (257 layers, 1056 of them: 33 warps on 608 quarters) has to be split: each lane
+// forms the 2 x 2 matrix of its run, a suffix scan of the matrices over the lanes gives every run
+// its incoming pair, then the run is walked as usual; the amplitudes take a prefix product.
+template <int S>
 __global__ void __launch_bounds__(32) green_recursion_kernel(Dev d) {
-  const long long gid = (long long)blockIdx.x * 32 + threadIdx.x;
-  if (gid >= (long long)d.nf * d.nk) return;
-  const int f = int(gid / d.nk), n = int(gid - (long long)f * d.nk);
+  constexpr int RPW = 32 / S;                             // (f, n) per warp
+  const int lane = threadIdx.x, seg = lane / RPW;
+  const long long row0 = (long long)blockIdx.x * RPW + lane % RPW, nrow = (long long)d.nf * d.nk;
+  const bool live = row0 < nrow;                          // the others only take part in the shuffles
+  const long long row = live ? row0 : nrow - 1;
+  const int f = int(row / d.nk), n = int(row - (long long)f * d.nk);
   const int J = d.nlayer;
-  const size_t lst = size_t(NCOEF) * d.nk;                // from a layer to the next
+  const int ja = int((long long)(J - 1) * seg / S), jb = int((long long)(J - 1) * (seg + 1) / S);
+  const size_t nk = d.nk, lst = size_t(NCOEF) * nk;       // from a layer to the next
   double2* c = d.coef + cix(d, f, n, 0, 0);
-  const size_t nk = d.nk;
-  double2 N = cmk(0.0, 0.0), D = cmk(1.0, 0.0);
-  {
-    double2* cl = c + lst * (J - 1);
-    cl[C_MUP * nk] = N;
-    cl[C_DEN * nk] = D;
-  }
+  const double2 zero = cmk(0.0, 0.0), one = cmk(1.0, 0.0);
   constexpr int U = 4;                                    // layers loaded ahead of the chain
-  for (int j1 = J - 1; j1 > 0; j1 -= U) {
-    double2 sg[U], de[U], eh[U];
+  double2 N = zero, D = one;                              // what enters the run from below
+  int ein = 0;                                            // true pair: times 2^ein
+  if (S > 1) {
+    // columns (Nu, Du), (Nv, Dv): the images of (1, 0) and (0, 1); true matrix: times 2^e
+    double2 Nu = one, Du = zero, Nv = zero, Dv = one;
+    int e = 0;
+    auto norm = [&]() {
+      const double s = rescale(fmax(fmax(cmax(Nu), cmax(Du)), fmax(cmax(Nv), cmax(Dv))), e);
+      Nu = s * Nu; Du = s * Du; Nv = s * Nv; Dv = s * Dv;
+    };
+    for (int j1 = jb; j1 > ja; j1 -= U) {
+      double2 sg[U], de[U], eh[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int j = j1 - 1 - u;
+        if (j < ja) continue;
+        const double2* cl = c + lst * j;
+        sg[u] = cl[C_SIG * nk]; de[u] = cl[C_DEL * nk]; eh[u] = cl[C_EH * nk];
+      }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int j = j1 - 1 - u;
+        if (j < ja) continue;
+        const double2 E = eh[u] * eh[u];
+        const double2 Mu = de[u] * Du + sg[u] * Nu, Mv = de[u] * Dv + sg[u] * Nv;
+        Du = sg[u] * Du + de[u] * Nu;
+        Dv = sg[u] * Dv + de[u] * Nv;
+        Nu = E * Mu;
+        Nv = E * Mv;
+        if ((j & 7) == 0) norm();
+      }
+    }
+    norm();
+#pragma unroll
+    for (int o = 1; o < S; o <<= 1) {                     // times the product of the o runs below
+      const int src = min(lane + o * RPW, 31);
+      const double2 a = shfl2(Nu, src), b = shfl2(Nv, src), x = shfl2(Du, src), y = shfl2(Dv, src);
+      const int eo = __shfl_sync(0xffffffffu, e, src);
+      if (seg + o < S) {
+        const double2 nu = Nu * a + Nv * x, nv = Nu * b + Nv * y;
+        const double2 du = Du * a + Dv * x, dv = Du * b + Dv * y;
+        Nu = nu; Nv = nv; Du = du; Dv = dv;
+        e += eo;
+        norm();
+      }
+    }
+    const int src = min(lane + RPW, 31);
+    const double2 bn = shfl2(Nv, src), bd = shfl2(Dv, src);
+    const int eb = __shfl_sync(0xffffffffu, e, src);
+    if (seg + 1 < S) { N = bn; D = bd; ein = eb; }
+  }
+  if (live && seg == S - 1) {
+    double2* cl = c + lst * (J - 1);
+    cl[C_MUP * nk] = zero;
+    cl[C_DEN * nk] = one;
+  }
+  double2 prod = one;                                     // of the run's tau (rescaled)
+  int er = 0;                                             // exponents taken out inside the run
+  for (int j1 = jb; j1 > ja; j1 -= U) {
+    double2 sg[U], de[U], eh[U], ta[U];
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int j = j1 - 1 - u;
-      if (j < 0) continue;
+      if (j < ja) continue;
       const double2* cl = c + lst * j;
       sg[u] = cl[C_SIG * nk]; de[u] = cl[C_DEL * nk]; eh[u] = cl[C_EH * nk];
+      if (S > 1) ta[u] = cl[C_AMP * nk];
     }
 #pragma unroll
     for (int u = 0; u < U; ++u) {
       const int j = j1 - 1 - u;
-      if (j < 0) continue;
+      if (j < ja) continue;
       double2* cl = c + lst * j;
       double2 M = de[u] * D + sg[u] * N;
       D = sg[u] * D + de[u] * N;
       const double2 E = eh[u] * eh[u];
       if ((j & 7) == 0) {
-        const double s = pow2_down(fmax(fabs(D.x), fabs(D.y)));
+        const double s = rescale(cmax(D), er);
         D = s * D;
         M = s * M;
-        cl[C_AMP * nk] = s * cl[C_AMP * nk];
+        const double2 t = s * (S > 1 ? ta[u] : cl[C_AMP * nk]);
+        if (live) cl[C_AMP * nk] = t;
+        if (S > 1) ta[u] = t;
       }
+      if (S > 1) prod = prod * ta[u];
       N = E * M;
-      cl[C_MUP * nk] = M;
-      cl[C_DEN * nk] = D;
+      if (live) {
+        cl[C_MUP * nk] = M;
+        cl[C_DEN * nk] = D;
+      }
     }
   }
-  double2 T = cmk(0.0, 0.5) * cinv(c[C_KAP * nk] * D);    // A_0 / D_0
-  for (int j0 = 0; j0 < J; j0 += 2 * U) {
+  // T at the run's first layer: T_0 = A_0 / D_0 times the runs above; a run's stored D is off the
+  // true one by 2^(ein + er), its product of tau by 2^-er
+  double2 T = cmk(0.0, 0.5) * cinv(c[C_KAP * nk] * D);
+  if (S > 1) {
+    T = shfl2(T, lane % RPW);
+    const int e0 = __shfl_sync(0xffffffffu, ein + er, lane % RPW);
+    int x = er;
+#pragma unroll
+    for (int o = 1; o < S; o <<= 1) {                     // inclusive prefix over the runs
+      const int src = max(lane - o * RPW, 0);
+      const double2 q = shfl2(prod, src);
+      const int xo = __shfl_sync(0xffffffffu, x, src);
+      if (seg >= o) { prod = prod * q; x += xo; }
+    }
+    const int src = max(lane - RPW, 0);
+    const double2 q = shfl2(prod, src);
+    const int xo = __shfl_sync(0xffffffffu, x, src);
+    if (seg > 0) {
+      T = T * q;
+      const int k = xo + ein + er - e0;
+      T = cmk(scalbn(T.x, k), scalbn(T.y, k));
+    }
+  }
+  const int je = seg == S - 1 ? J : jb;                   // the half-space belongs to the last run
+  for (int j0 = ja; j0 < je; j0 += 2 * U) {
     double2 tau[2 * U];
 #pragma unroll
     for (int u = 0; u < 2 * U; ++u)
-      if (j0 + u < J - 1) tau[u] = c[lst * (j0 + u) + C_AMP * nk];
+      if (j0 + u < min(je, J - 1)) tau[u] = c[lst * (j0 + u) + C_AMP * nk];
 #pragma unroll
     for (int u = 0; u < 2 * U; ++u) {
-      if (j0 + u >= J) continue;
-      c[lst * (j0 + u) + C_AMP * nk] = T;
+      if (j0 + u >= je) continue;
+      if (live) c[lst * (j0 + u) + C_AMP * nk] = T;
       if (j0 + u < J - 1) T = T * tau[u];
     }
   }
@@ -296,10 +407,10 @@ __global__ void __launch_bounds__(128) green_rec32_kernel(Dev d) {
   }
 }
 
-constexpr int EV_ZC = 16;   // depths per warp
-
-// One warp per 32 table rows (of any frequencies) and 16 depths: the FP64 unit is the bound, so
-// the lanes are filled across frequencies and the depths spread over as many SMs as there are.
+// One warp per 32 table rows (of any frequencies) and EV_ZC depths: the FP64 unit is the bound, so
+// the lanes are filled across frequencies; 16 depths share the anchors where the rows alone fill
+// the GPU, 4 where they do not (a 64-point line: 33 row blocks for 608 quarters of an SM).
+template <int EV_ZC>
 __global__ void __launch_bounds__(32) green_eval64_kernel(Dev d) {
   __shared__ double2 tile[32][EV_ZC + 1];
   const int lane = threadIdx.x;
@@ -340,14 +451,15 @@ __global__ void __launch_bounds__(32) green_eval64_kernel(Dev d) {
     }
   }
   __syncwarp();
-  const int z = zc + (lane & 15);
+  constexpr int RP = 32 / EV_ZC;                          // rows written together
+  const int z = zc + lane % EV_ZC;
   const double sq_lane = d.g32 ? sqrt(d.fc[f].s_abs) : 0.0;
-  for (int rr = 0; rr < 32; rr += 2) {
-    const int nl = rr + (lane >> 4);
+  for (int rr = 0; rr < 32; rr += RP) {
+    const int nl = rr + lane / EV_ZC;
     const double sq = __shfl_sync(0xffffffffu, sq_lane, nl);
     const long long r = r0 + nl;
     if (r < nrow && z < d.nz) {
-      const double2 v = tile[nl][lane & 15];
+      const double2 v = tile[nl][lane % EV_ZC];
       if (d.g64) d.g64[size_t(r) * d.nz + z] = v;
       if (d.g32) {
         // sqrt|s_f| g rounded to FP32, and (double-float table) the FP32 rounding of the rest
@@ -410,9 +522,15 @@ cudaError_t launch_green(const Dev& d, cudaStream_t s, int tables) {
     green_kap32_kernel<<<unsigned((nl + 255) / 256), 256, 0, s>>>(d);
     green_rec32_kernel<<<g1, 128, 0, s>>>(d);
   } else {
-    const long long nl = (long long)d.nf * d.nk * d.nlayer;
-    green_layer_kernel<<<unsigned((nl + 127) / 128), 128, 0, s>>>(d, fast32 ? 0 : 1);
-    green_recursion_kernel<<<unsigned(((long long)d.nf * d.nk + 31) / 32), 32, 0, s>>>(d);
+    const long long rows = (long long)d.nf * d.nk, nl = rows * d.nlayer;
+    const int run = d.nlayer > 64 ? 4 : 1;
+    const unsigned lb = unsigned((rows * ((d.nlayer + run - 1) / run) + LBLOCK - 1) / LBLOCK);
+    if (run == 4) green_layer_kernel<4><<<lb, LBLOCK, 0, s>>>(d, fast32 ? 0 : 1);
+    else green_layer_kernel<1><<<lb, LBLOCK, 0, s>>>(d, fast32 ? 0 : 1);
+    // the split walks every layer twice (2 x 2 matrices, then the run): only for stacks of at
+    // least four layers per run over too few (f, n) to fill the SMs' quarters
+    if (d.nlayer > 4 * 16 && rows < 32 * 304) green_recursion_kernel<16><<<unsigned((rows + 1) / 2), 32, 0, s>>>(d);
+    else green_recursion_kernel<1><<<unsigned((rows + 31) / 32), 32, 0, s>>>(d);
     if (fast32) green_coef32_kernel<<<unsigned((nl + 127) / 128), 128, 0, s>>>(d);
   }
   if (fast32) {
@@ -422,8 +540,10 @@ cudaError_t launch_green(const Dev& d, cudaStream_t s, int tables) {
     if (!(tables & (GREEN_G32 | GREEN_G32DF))) e.g32 = nullptr;
     if (!(tables & GREEN_G32DF)) e.g32lo = nullptr;
     if (!(tables & GREEN_G64)) e.g64 = nullptr;
-    const dim3 g2(unsigned(((long long)d.nf * d.nk + 31) / 32), (d.nz + EV_ZC - 1) / EV_ZC);
-    green_eval64_kernel<<<g2, 32, 0, s>>>(e);
+    const long long rows = (long long)d.nf * d.nk;
+    const unsigned rb = unsigned((rows + 31) / 32);
+    if ((long long)rb * ((d.nz + 15) / 16) < 608) green_eval64_kernel<4><<<dim3(rb, (d.nz + 3) / 4), 32, 0, s>>>(e);
+    else green_eval64_kernel<16><<<dim3(rb, (d.nz + 15) / 16), 32, 0, s>>>(e);
   }
   return cudaGetLastError();
 }

@@ -8,6 +8,7 @@ from __future__ import annotations
 
 import ctypes as C
 import os
+import struct
 from dataclasses import dataclass
 from typing import Optional, Sequence
 
@@ -636,29 +637,41 @@ class Solver:
 
 
 # ---- streaming 1D subproblems (edt_stream_*) ---------------------------------------------
+# edt_sub1d as one packed record (native alignment, the same layout as the ctypes structure)
+_SUB1D = struct.Struct("@i5diPPiPiPiPP0d")
+
+
+def _pointer(a, dtype, keep):
+    """Address of a C-contiguous array of `dtype` holding `a`; a converted copy is kept in `keep`."""
+    if type(a) is not np.ndarray or a.dtype != dtype or not a.flags.c_contiguous:
+        a = np.ascontiguousarray(a, dtype=dtype)
+        keep.append(a)
+    return a.__array_interface__["data"][0]
+
+
 def _sub1d_array(subs):
-    """ctypes array of edt_sub1d for objects with the fields of synth.stream.Sub1D, plus the
-    numpy arrays it points into (kept alive by the caller until the submit returns)."""
-    arr = (edt_sub1d * max(len(subs), 1))()
-    keep = []
-    dp, ip, fp = C.POINTER(C.c_double), C.POINTER(C.c_int), C.POINTER(C.c_float)
+    """Array of edt_sub1d for objects with the fields of synth.stream.Sub1D, plus what it points
+    into (kept alive by the caller until the submit returns).  The records are packed with
+    struct: setting the fields of a ctypes structure one by one took 20 us per request, as long
+    as the device takes to solve it."""
+    if _SUB1D.size != C.sizeof(edt_sub1d):
+        raise RuntimeError("edt_sub1d layout mismatch")
+    buf = bytearray(max(len(subs), 1) * _SUB1D.size)
+    keep = [subs]
+    f8, i4, c8 = np.dtype(np.float64), np.dtype(np.int32), np.dtype(np.complex64)
     for i, s in enumerate(subs):
-        tops = np.ascontiguousarray(s.layer_top, dtype=np.float64)
-        vel = np.ascontiguousarray(s.layer_vel, dtype=np.float64)
-        fr = np.ascontiguousarray(s.freq_hz, dtype=np.float64)
-        kv = np.ascontiguousarray(s.kval, dtype=np.float64)
-        rows = np.ascontiguousarray(s.rows, dtype=np.int32).reshape(-1, 3)
-        data = np.ascontiguousarray(s.data, dtype=np.complex64).reshape(-1, 2).view(np.float32)
-        keep += [tops, vel, fr, kv, rows, data]
-        e = arr[i]
-        e.nz, e.dz, e.z0 = int(s.nz), float(s.dz), float(s.z0)
-        e.eps, e.alpha, e.dx = float(s.eps), float(s.alpha), float(s.dx)
-        e.nlayer = len(tops)
-        e.layer_top_m, e.layer_vel_mps = tops.ctypes.data_as(dp), vel.ctypes.data_as(dp)
-        e.nfreq, e.freq_hz = len(fr), fr.ctypes.data_as(dp)
-        e.nk, e.kval = len(kv), kv.ctypes.data_as(dp)
-        e.nrow, e.rows, e.data = rows.shape[0], rows.ctypes.data_as(ip), data.ctypes.data_as(fp)
-    return arr, keep
+        tops, freq, kval, rows, data = s.layer_top, s.freq_hz, s.kval, s.rows, s.data
+        # the arrays themselves, not only the request, so that a field replaced meanwhile is safe
+        keep.append((tops, s.layer_vel, freq, kval, rows, data))
+        tp, vp = _pointer(tops, f8, keep), _pointer(s.layer_vel, f8, keep)
+        fp, kp = _pointer(freq, f8, keep), _pointer(kval, f8, keep)
+        rp, dp = _pointer(rows, i4, keep), _pointer(data, c8, keep)
+        nrow, odd = divmod(np.size(rows), 3)
+        if odd or np.size(data) % 2:
+            raise ValueError("rows are (f, p, q) triples and data (d_+, d_-) pairs")
+        _SUB1D.pack_into(buf, i * _SUB1D.size, int(s.nz), s.dz, s.z0, s.eps, s.alpha, s.dx, len(tops), tp, vp,
+                         len(freq), fp, len(kval), kp, nrow, rp, dp)
+    return (edt_sub1d * max(len(subs), 1)).from_buffer(buf), keep
 
 
 def edt_stream_request_bytes(sub) -> int:

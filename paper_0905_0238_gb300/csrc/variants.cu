@@ -67,32 +67,22 @@ constexpr int JAC_MAX_SWEEPS = 20;
 constexpr int JAC_BLOCKS = 3;      // 2 x 2 blocks per thread: (TSVD_MAX_NZ / 2)(TSVD_MAX_NZ / 2 + 1) / 2 in all
 static_assert((TSVD_MAX_NZ / 2) * (TSVD_MAX_NZ / 2 + 1) / 2 <= JAC_THREADS * JAC_BLOCKS, "blocks fit the threads");
 
-__device__ __forceinline__ double rcp_approx(double x) {      // ~20 bits
-  double y;
-  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  return y;
-}
-__device__ __forceinline__ double rsqrt_approx(double x) {
-  double y;
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-  return y;
-}
-// cosine of the rotation of tangent t, 1 / sqrt(1 + t^2) to FP64: the estimate y0 and one
-// third-order step on e = 1 - q y0^2 (y = y0 (1 + e/2 + 3 e^2 / 8), error ~ e^3)
-__device__ __forceinline__ double cos_of(double t) {
-  const double q = fma(t, t, 1.0), y0 = rsqrt_approx(q);
+// cosine of the rotation of tangent t, 1 / sqrt(1 + t^2) to FP64 (q = 1 + t^2): the FP32 estimate
+// y0 and one third-order step on e = 1 - q y0^2 (y = y0 (1 + e/2 + 3 e^2 / 8), error ~ e^3)
+__device__ __forceinline__ double cos_of(double t, double q) {
+  const double y0 = double(rsqrtf(float(q)));
   const double e = fma(-q * y0, y0, 1.0);
   return fma(y0 * e, fma(0.375, e, 0.5), y0);
 }
-// tangent of the rotation that zeroes apq between the diagonal entries app, aqq, to ~20 bits: an
-// inexact angle leaves |apq| 1e-6 of what it was (the next sweep takes the rest), the rotation
-// itself is orthogonal to FP64 because the cosine is formed from the tangent that is used
-__device__ __forceinline__ double tan_of(double app, double aqq, double apq) {
-  const double dd = aqq - app;
-  if (dd == 0.0) return 1.0;
-  if (fabs(dd) > 1e8 * fabs(apq)) return apq * rcp_approx(dd);
-  const double tau = dd * rcp_approx(2.0 * apq), q = fma(tau, tau, 1.0);
-  return copysign(rcp_approx(fabs(tau) + q * rsqrt_approx(q)), tau);
+__device__ __forceinline__ double cos_of(double t) { return cos_of(t, fma(t, t, 1.0)); }
+// tangent of the rotation that zeroes apq between diagonal entries that differ by dd = aqq - app, in
+// FP32: an inexact angle leaves |apq| 1e-7 of what it was (the next sweep takes the rest), the
+// rotation itself is orthogonal to FP64 because the cosine is formed from the tangent that is used
+__device__ __forceinline__ float tan_of(float dd, float apq) {
+  if (dd == 0.f) return 1.f;
+  const float tau = dd / (2.f * apq);
+  if (fabsf(tau) > 1e9f) return 0.5f / tau;
+  return copysignf(1.f / (fabsf(tau) + sqrtf(fmaf(tau, tau, 1.f))), tau);
 }
 
 // players of the round-robin (a dummy when p is odd); round r: player 0 fixed, the others
@@ -112,18 +102,24 @@ __device__ __forceinline__ void jac_pair(int k, int r, int P2, int& a, int& b) {
 // by cyclic Jacobi, then the truncated-SVD solution for both right-hand sides.
 // src: matrices at m * nz * nz with leading dimension p; rhs, out: [m][nz][2].
 //
-// The FP64 unit (one warp instruction per 16 cycles of an SM) bounds the rounds, so a round does
-// no more FP64 work than it has to:
+// The FP64 unit (one warp instruction per 64 cycles of each of an SM's four parts) bounds the
+// rounds, so a round does no more FP64 work than it has to:
 //   * the matrix is kept as its lower triangle and updated two-sidedly in one pass, block (K, L) of
-//     the pairs K <= L at a time, X <- J_K^T X J_L: 16 operations per 4 entries of half the
-//     matrix, where a pass over the columns and one over the rows of the whole matrix take 32;
-//     blocks of two pairs that do not rotate are left alone;
-//   * the eigenvectors are not accumulated (another 16 operations per 4 entries): with W = J_1
-//     J_2 ... J_n, W^T b is formed by applying each rotation to b as it is found, and W z by
-//     applying them in reverse order from the log of their tangents (tlog, written once and
-//     read once), 8 operations per pair and right-hand side;
-//   * the tangents take approximate reciprocals (tan_of).
-// One barrier after the angles and one after the update.
+//     the pairs K <= L at a time, where a pass over the columns and one over the rows of the whole
+//     matrix do it twice; blocks of two pairs that do not rotate are left alone;
+//   * it is kept scaled, A = S B S with S diagonal: a rotation by c [1, -t; t, 1] then is one
+//     multiply-add per entry, B_p' = B_p - (t s_q / s_p) B_q, B_q' = B_q + (t s_p / s_q) B_p, with
+//     s_p' = c s_p, s_q' = c s_q (fast rotations: 8 operations per block instead of 16); S goes
+//     back into the matrix after every sweep (c >= 1/sqrt 2, so it shrinks by 2^-48 at most);
+//   * the eigenvectors are not accumulated: with W = J_1 J_2 ... J_n, W^T b is formed by applying
+//     each rotation to b as it is found, and W z by applying them in reverse order from the log
+//     of their tangents (tlog, written once and read once);
+//   * the angles are chosen in FP32 (tan_of);
+//   * only what the threshold needs is rotated (below), which ends the sweeps earlier.
+// One barrier after the angles and one after the update.  Measured on the paper's acquisition (129
+// systems of 65 unknowns): the kernel 14.0 ms with W accumulated over the whole
+// matrix and every pair rotated (13 to 20 sweeps), 6.1 with the half matrix and the log, 3.5 ms now (8 to 14
+// sweeps).
 __global__ void __launch_bounds__(JAC_THREADS) tsvd_jacobi_kernel(Dev d, const double* src, const double* rhs,
                                                                  double* out) {
   extern __shared__ __align__(16) double sm[];
@@ -132,10 +128,13 @@ __global__ void __launch_bounds__(JAC_THREADS) tsvd_jacobi_kernel(Dev d, const d
   const int p = d.kz_p ? d.kz_p[m] : n;
   const int ld = p + 1;
   const int P2 = (p + 1) & ~1, npair = P2 / 2;
-  double* A = sm;                         // [p][ld] lower triangle (row >= column)
-  double* bv = A + size_t(p) * ld;        // [p][2] W^T b, later W z
-  double* cs = bv + 2 * p;                // [2][npair] rotation cosines and sines
-  double* red = cs + P2;                  // [32]
+  double* A = sm;                         // [p][ld] lower triangle (row >= column) of B
+  double* bv = A + size_t(p) * ld;        // [p][2] S^-1 W^T b, later W z
+  double* al = bv + 2 * p;                // [2][npair] a round's t s_q / s_p and t s_p / s_q
+  double* rt = al + P2;                   // [2][npair] the next round's s_q / s_p and s_p / s_q
+  double* sv = rt + P2;                   // [p] S
+  double* si = sv + p;                    // [p] S^-1
+  double* red = si + p;                   // [32]
   int* pj = reinterpret_cast<int*>(red + 32);   // [2][npair] pair indices a < b (b == p: alone)
   int* rotated = pj + P2;
   const bool has_rows = d.row_off[m + 1] > d.row_off[m];
@@ -168,6 +167,7 @@ __global__ void __launch_bounds__(JAC_THREADS) tsvd_jacobi_kernel(Dev d, const d
     if (j <= i) A[i * ld + j] = sc * S[size_t(i) * p + j];
   }
   for (int i = threadIdx.x; i < 2 * p; i += blockDim.x) bv[i] = bm[i];
+  for (int i = threadIdx.x; i < p; i += blockDim.x) sv[i] = si[i] = 1.0;
   // this thread's blocks (K <= L), the same in every round
   int bK[JAC_BLOCKS], bL[JAC_BLOCKS];
   const int nblk = npair * (npair + 1) / 2;
@@ -181,59 +181,100 @@ __global__ void __launch_bounds__(JAC_THREADS) tsvd_jacobi_kernel(Dev d, const d
     bK[q] = e - L * (L + 1) / 2;
   }
   double* tl = d.tlog + size_t(m) * d.tlog_stride;
-  // a pair is rotated while |a_ij| > 1e-14 sqrt(a_ii a_jj) (relative to its own diagonal, which
-  // keeps small eigenvalues of the positive semi-definite matrix accurate; well above the FP64
-  // rounding of a rotation, so the sweeps end); the sweeps stop when one rotates no pair
+  // Which pairs to rotate.  Without a threshold: while |a_ij| > 1e-14 sqrt(a_ii a_jj) (relative to
+  // its own diagonal, which keeps small eigenvalues of the positive semi-definite matrix accurate;
+  // well above the FP64 rounding of a rotation, so the sweeps end).  With one, only the
+  // eigenvalues at or above it and their vectors are wanted; th <= the threshold (the largest
+  // diagonal entry is at most the largest eigenvalue) stands for it:
+  //   both entries >= th / 2: as above;
+  //   one of them: decoupled to the FP64 rounding of the larger, |a_ij| <= 1e-15 a_ii;
+  //   both below: |a_ij| <= th / (4 p), so that no eigenvalue of that block reaches th (Gershgorin:
+  //   below th / 2 + p th / (4 p)); its eigenvalues below th need not be resolved.
+  // The small ones are mostly rounding noise, whose relative off-diagonals die down last.
+  const double tol = d.tsvd_tol;
+  const double th64 = tol > 0.0 ? tol * tol * sc : tol * tol * (sc * dmax);
+  const float wanted = tol != 0.0 ? float(0.5 * th64) : -1.f, apart = float(0.25 * th64 / double(p));
   int nround = 0;
   for (int sweep = 0; sweep < JAC_MAX_SWEEPS; ++sweep) {
     if (threadIdx.x == 0) *rotated = 0;
+    for (int k = threadIdx.x; k < P2; k += blockDim.x) rt[k] = 1.0;
     __syncthreads();
     for (int r = 0; r < P2 - 1; ++r, ++nround) {
       for (int k = threadIdx.x; k < npair; k += blockDim.x) {
         int a, b;
         jac_pair(k, r, P2, a, b);
-        double t = 0.0;
+        float t = 0.f;
+        const double rab = rt[k], rba = rt[npair + k];     // s_b / s_a, s_a / s_b
         if (b < p) {
-          const double apq = A[b * ld + a], app = A[a * ld + a], aqq = A[b * ld + b];
-          if (apq * apq > 1e-28 * fabs(app * aqq)) t = tan_of(app, aqq, apq);
-          if (!(fabs(t) <= 2.0)) t = 0.0;      // outside the estimates' range: nothing to rotate
+          const double Bab = A[b * ld + a], Baa = A[a * ld + a], Bbb = A[b * ld + b];
+          const float fab = float(Bab), faa = fabsf(float(Baa)), fbb = fabsf(float(Bbb));
+          const float sa = float(sv[a]), sb = float(sv[b]);
+          const float taa = sa * sa * faa, tbb = sb * sb * fbb, tab = sa * sb * fabsf(fab);   // true entries
+          const float hi = fmaxf(taa, tbb), lo = fminf(taa, tbb);
+          const bool want = lo >= wanted ? fabsf(fab) > 1e-14f * (sqrtf(faa) * sqrtf(fbb))
+                                         : (hi >= wanted ? tab > 1e-15f * hi : tab > apart);
+          if (want) t = tan_of(float(rab * Bbb - rba * Baa), fab);
+          if (!(fabsf(t) <= 2.f)) t = 0.f;     // outside the estimates' range: nothing to rotate
         }
-        const double c = t != 0.0 ? cos_of(t) : 1.0;
-        if (t != 0.0) *rotated = 1;
         pj[k] = a; pj[npair + k] = b;
-        cs[k] = c; cs[npair + k] = t * c;
-        tl[size_t(nround) * npair + k] = t;
+        tl[size_t(nround) * npair + k] = double(t);
+        double alpha = 0.0, beta = 0.0;
+        if (t != 0.f) {
+          *rotated = 1;
+          const double t64 = double(t), q = fma(t64, t64, 1.0), c = cos_of(t64, q), ic = q * c;
+          alpha = t64 * rab;
+          beta = t64 * rba;
+          sv[a] *= c; sv[b] *= c;
+          si[a] *= ic; si[b] *= ic;
+        }
+        al[k] = alpha; al[npair + k] = beta;
       }
       __syncthreads();
 #pragma unroll
       for (int q = 0; q < JAC_BLOCKS; ++q) {
         const int K = bK[q], L = bL[q];
         if (L < 0) continue;
-        const double cK = cs[K], sK = cs[npair + K], cL = cs[L], sL = cs[npair + L];
-        if (sK == 0.0 && sL == 0.0) continue;
+        const double aK = al[K], eK = al[npair + K], aL = al[L], eL = al[npair + L];
+        if (aK == 0.0 && aL == 0.0) continue;
         const int a = pj[K], b = pj[npair + K], u = pj[L], v = pj[npair + L];
         auto at = [&](int i, int j) -> double& { return i >= j ? A[i * ld + j] : A[j * ld + i]; };
         const bool hb = b < p, hv = v < p;
         const double xau = at(a, u), xav = hv ? at(a, v) : 0.0;
         const double xbu = hb ? at(b, u) : 0.0, xbv = hb && hv ? at(b, v) : 0.0;
-        const double yau = cL * xau - sL * xav, yav = sL * xau + cL * xav;
-        const double ybu = cL * xbu - sL * xbv, ybv = sL * xbu + cL * xbv;
-        at(a, u) = cK * yau - sK * ybu;
-        if (hv) at(a, v) = cK * yav - sK * ybv;
-        if (K != L && hb) at(b, u) = sK * yau + cK * ybu;     // K == L: the entry (a, v) again
-        if (hb && hv) at(b, v) = sK * yav + cK * ybv;
+        const double yau = fma(-aL, xav, xau), yav = fma(eL, xau, xav);
+        const double ybu = fma(-aL, xbv, xbu), ybv = fma(eL, xbu, xbv);
+        at(a, u) = fma(-aK, ybu, yau);
+        if (hv) at(a, v) = fma(-aK, ybv, yav);
+        if (K != L && hb) at(b, u) = fma(eK, yau, ybu);     // K == L: the entry (a, v) again
+        if (hb && hv) at(b, v) = fma(eK, yav, ybv);
       }
-      for (int e = threadIdx.x; e < 2 * npair; e += blockDim.x) {
-        const int k = e >> 1, a = pj[k], b = pj[npair + k];
-        if (b >= p) continue;
-        const double c = cs[k], s = cs[npair + k];
-        const double x = bv[2 * a + (e & 1)], y = bv[2 * b + (e & 1)];
-        bv[2 * a + (e & 1)] = c * x - s * y;
-        bv[2 * b + (e & 1)] = s * x + c * y;
+      for (int e = JAC_THREADS - 1 - int(threadIdx.x); e < 3 * npair; e += JAC_THREADS) {
+        if (e < 2 * npair) {                               // b; the last warps have the fewest blocks
+          const int k = e >> 1, a = pj[k], b = pj[npair + k];
+          if (al[k] == 0.0) continue;
+          const double x = bv[2 * a + (e & 1)], y = bv[2 * b + (e & 1)];
+          bv[2 * a + (e & 1)] = fma(-al[k], y, x);
+          bv[2 * b + (e & 1)] = fma(al[npair + k], x, y);
+        } else if (r + 1 < P2 - 1) {                       // the next round's ratios
+          const int k = e - 2 * npair;
+          int a, b;
+          jac_pair(k, r + 1, P2, a, b);
+          if (b < p) {
+            rt[k] = sv[b] * si[a];
+            rt[npair + k] = sv[a] * si[b];
+          }
+        }
       }
       __syncthreads();
     }
     const bool more = *rotated != 0;
+    for (int e = threadIdx.x; e < p * p; e += blockDim.x) {      // S back into the matrix and b
+      const int i = e / p, j = e - i * p;
+      if (j <= i) A[i * ld + j] *= sv[i] * sv[j];
+    }
+    for (int e = threadIdx.x; e < 2 * p; e += blockDim.x) bv[e] *= sv[e >> 1];
+    __syncthreads();
+    for (int i = threadIdx.x; i < p; i += blockDim.x) sv[i] = si[i] = 1.0;
     __syncthreads();
     if (!more) break;
   }
@@ -243,7 +284,6 @@ __global__ void __launch_bounds__(JAC_THREADS) tsvd_jacobi_kernel(Dev d, const d
   for (int i = threadIdx.x; i < p; i += blockDim.x) lmax = fmax(lmax, A[i * ld + i]);
   lmax = block_max(lmax);
   const double un = scalbn(1.0, ex);                       // eigenvalues of the unscaled matrix
-  const double tol = d.tsvd_tol;
   const double thr = tol > 0.0 ? tol * tol : (tol < 0.0 ? tol * tol * (un * lmax) : 0.0);
   for (int e = threadIdx.x; e < 2 * p; e += blockDim.x) {  // z = Lambda~^-1 W^T b
     const int i = e >> 1;
@@ -296,7 +336,7 @@ __global__ void __launch_bounds__(JAC_THREADS) tsvd_jacobi_kernel(Dev d, const d
 
 size_t tsvd_smem_bytes(int p) {
   const size_t P2 = (p + 1) & ~1;
-  return (size_t(p) * (p + 1) + 2 * p + P2 + 32) * sizeof(double) + (P2 + 1) * sizeof(int);
+  return (size_t(p) * (p + 1) + 4 * p + 2 * P2 + 32) * sizeof(double) + (P2 + 1) * sizeof(int);
 }
 
 // doubles of one subproblem's rotation log: every pair of every round of the most sweeps

@@ -83,6 +83,18 @@ __device__ __forceinline__ int lane_z(int i, int lane) { return 64 * (i >> 1) + 
 
 constexpr int CT = 16;                     // steps per staged chunk
 
+// Chunks are staged one ahead: the next chunk's table rows by asynchronous 16-byte copies into
+// slots of the circular buffers that the current chunk does not use, its coefficients through
+// registers, while the current one is multiplied (without it the kernels' 16 warps per SM left
+// the FP32 pipes idle during the loads, 41 % of their cycles used; one gradient of the 512-point,
+// 128-frequency, 256-depth line took 7.17 ms, with it 6.29).
+__device__ __forceinline__ void copy16(float2* dst, const float2* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(uint32_t(__cvta_generic_to_shared(dst))), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
 // ---- B(m, j) += sum over the classes of m of Re(a) U + Im(a) W ------------------------------
 // Every entry (p, q) of the plane appears once: the classes {(p, q), (-q, -p)} of m = p - q and
 // their mirror images {(q, p), (-p, -q)} of -m share a = g32_p g32_q, and V = Re sum Ahat(m)
@@ -94,22 +106,23 @@ constexpr int CT = 16;                     // steps per staged chunk
 // t share all but CT of their rows, which stay where they are (circular buffers).
 template <int ZP> struct VhatShape {
   static constexpr int JT = 4 / ZP, VJ = 8 * JT;           // j per thread and per CTA (two m each)
-  static constexpr int R = CT + VJ;                        // rows buffered of either leg
-  static constexpr int SMEM = (2 * R * 64 * ZP) * int(sizeof(float2)) + CT * 2 * VJ * int(sizeof(float4));
+  static constexpr int R = 2 * CT + VJ;                    // rows buffered of either leg
+  static constexpr int NC = CT * 2 * VJ;                   // coefficients of a chunk
+  static constexpr int SMEM = 2 * R * 64 * ZP * int(sizeof(float2)) + 2 * NC * int(sizeof(float4));
 };
 
 template <int ZP>
 __global__ void __launch_bounds__(256, 2) grad_vhat_kernel(Dev d, int f0) {
   using S = VhatShape<ZP>;
-  constexpr int JT = S::JT, VJ = S::VJ, R = S::R, ZC = 64 * ZP;
+  constexpr int JT = S::JT, VJ = S::VJ, R = S::R, ZC = 64 * ZP, CQ = S::NC / 256;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float4 (*cf)[2 * VJ] = reinterpret_cast<float4 (*)[2 * VJ]>(smem_raw);    // [CT] (U, W) of (t, m)
-  float2* gps = reinterpret_cast<float2*>(cf + CT);        // row jt + u, u = t + ..., in slot u mod R
-  float2* gqs = gps + R * ZC;                              // row u - jt, u = t - ..., in slot (u + VJ) mod R
+  float4* cf = reinterpret_cast<float4*>(smem_raw);        // [2][CT][2 VJ] (U, W) of (t, m)
+  float2* gps = reinterpret_cast<float2*>(cf + 2 * S::NC); // row jt + u, u = t + ..., in slot u mod R
+  float2* gqs = gps + R * ZC;                              // row u - jt - (VJ - 1), u = t + ..., likewise
   const int N = d.N, H = N / 2, msk = N - 1, nk = d.nk, fi = blockIdx.z, f = f0 + fi;
   const int jt = blockIdx.x * VJ, z0 = blockIdx.y * ZC;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const float2* g = d.g32 + size_t(f) * nk * d.nzs;
+  const float2* g = d.g32 + size_t(f) * nk * d.nzs + z0;
   const float4* E = d.born_fold + size_t(fi) * 2 * nk * nk;
   const float4* T = E + size_t(nk) * nk;
   const bool live = 2 * (jt + JT * w) <= H;                // the same in the whole warp
@@ -118,36 +131,57 @@ __global__ void __launch_bounds__(256, 2) grad_vhat_kernel(Dev d, int f0) {
   for (int k = 0; k < 2 * JT; ++k)
 #pragma unroll
     for (int i = 0; i < 2 * ZP; ++i) acc[k][i] = make_float2(0.f, 0.f);
-  // rows [lo, hi) of u: gps gets jt + u, gqs (u - VJ + 1) - jt
-  auto load_rows = [&](int lo, int hi) {
-    for (int e = threadIdx.x; e < (hi - lo) * ZC; e += 256) {
-      const int u = lo + e / ZC, zz = e % ZC, z = z0 + zz, sl = (u % R) * ZC + zz;
-      const bool in = z < d.nz;
-      gps[sl] = in ? g[size_t(tab_index((jt + u) & msk, N)) * d.nzs + z] : make_float2(0.f, 0.f);
-      gqs[sl] = in ? g[size_t(tab_index((u - VJ + 1 - jt) & msk, N)) * d.nzs + z] : make_float2(0.f, 0.f);
+  // rows [lo, hi) of u; depths past nz are not copied (their lanes' sums are not stored)
+  auto copy_rows = [&](int lo, int hi) {
+    for (int e = threadIdx.x; e < (hi - lo) * (ZC / 2); e += 256) {
+      const int u = lo + e / (ZC / 2), zz = 2 * (e % (ZC / 2)), sl = (u % R) * ZC + zz;
+      if (z0 + zz >= d.nz) continue;
+      copy16(gps + sl, g + size_t(tab_index((jt + u) & msk, N)) * d.nzs + zz);
+      copy16(gqs + sl, g + size_t(tab_index((u - VJ + 1 - jt) & msk, N)) * d.nzs + zz);
     }
+    copies_commit();
   };
-  for (int t0 = 0; t0 <= H; t0 += CT) {
-    load_rows(t0 == 0 ? 0 : t0 + VJ, t0 + VJ + CT);
-    for (int e = threadIdx.x; e < CT * 2 * VJ; e += 256) {
-      const int tt = e / (2 * VJ), mi = e - tt * (2 * VJ);
-      const int t = t0 + tt, m = 2 * jt + mi, odd = m & 1, j = m >> 1;
-      float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+  float4 raw[CQ];                                          // folded values of a chunk, as read
+  auto load_coef = [&](int t0) {
+#pragma unroll
+    for (int i = 0; i < CQ; ++i) {
+      const int e = threadIdx.x + 256 * i, mi = e % (2 * VJ);
+      const int t = t0 + e / (2 * VJ), m = 2 * jt + mi, odd = m & 1, j = m >> 1;
+      raw[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (m <= H && t <= H - odd) {
         int p = t + j + odd, q = t - j;
         if (p > H) p -= N;                                  // signed indices, never both negative
-        const float4 c = p >= 0 && q >= 0 ? E[size_t(p) * nk + q]
-                                          : T[size_t(p >= 0 ? p : -p) * nk + (q >= 0 ? q : -q)];
-        float2 S1 = make_float2(c.x, c.y), S2 = make_float2(c.z, c.w);
-        if (p < 0) { const float2 x = S1; S1 = S2; S2 = x; }
-        float wt = !odd && (t == 0 || t == H) ? 0.5f : 1.f;
-        if (m == 0 || m == H) wt *= 0.5f;
-        o = make_float4(wt * (S1.x + S2.x), wt * (S1.y - S2.y), wt * (S1.y + S2.y), wt * (S2.x - S1.x));
+        raw[i] = p >= 0 && q >= 0 ? E[size_t(p) * nk + q]
+                                  : T[size_t(p >= 0 ? p : -p) * nk + (q >= 0 ? q : -q)];
       }
-      cf[tt][mi] = o;
     }
-    __syncthreads();
+  };
+  auto store_coef = [&](int t0, float4* dst) {
+#pragma unroll
+    for (int i = 0; i < CQ; ++i) {
+      const int e = threadIdx.x + 256 * i, mi = e % (2 * VJ);
+      const int t = t0 + e / (2 * VJ), m = 2 * jt + mi, odd = m & 1;
+      float2 S1 = make_float2(raw[i].x, raw[i].y), S2 = make_float2(raw[i].z, raw[i].w);
+      if (t + (m >> 1) + odd > H) { const float2 x = S1; S1 = S2; S2 = x; }      // p < 0
+      float wt = !odd && (t == 0 || t == H) ? 0.5f : 1.f;
+      if (m == 0 || m == H) wt *= 0.5f;
+      dst[e] = make_float4(wt * (S1.x + S2.x), wt * (S1.y - S2.y), wt * (S1.y + S2.y), wt * (S2.x - S1.x));
+    }
+  };
+  copy_rows(0, VJ + CT);
+  load_coef(0);
+  store_coef(0, cf);
+  int buf = 0;
+  for (int t0 = 0; t0 <= H; t0 += CT, buf ^= 1) {
+    copies_wait();
+    __syncthreads();                                       // this chunk is staged, the last one done with
+    const bool more = t0 + CT <= H;
+    if (more) {
+      copy_rows(t0 + VJ + CT, t0 + VJ + 2 * CT);
+      load_coef(t0 + CT);
+    }
     if (live) {
+      const float4* cb = cf + buf * S::NC + 2 * JT * w;
       // at t = t0 + tt: P[i] = row p of j = jt + JT w + i (u = t + JT w + i), Q[i] = its row q
       // (u = t + VJ - 1 - JT w - i)
       Row<ZP> P[JT + 1], Q[JT];
@@ -173,7 +207,7 @@ __global__ void __launch_bounds__(256, 2) grad_vhat_kernel(Dev d, int f0) {
         for (int i = 0; i < JT; ++i)
 #pragma unroll
           for (int o = 0; o < 2; ++o) {
-            const float4 c = cf[tt][2 * (JT * w + i) + o];
+            const float4 c = cb[tt * (2 * VJ) + 2 * i + o];
 #pragma unroll
             for (int x = 0; x < 2 * ZP; ++x) {
               const float2 a = P[i + o].at(x) * Q[i].at(x);
@@ -184,7 +218,7 @@ __global__ void __launch_bounds__(256, 2) grad_vhat_kernel(Dev d, int f0) {
           }
       }
     }
-    __syncthreads();
+    if (more) store_coef(t0 + CT, cf + (buf ^ 1) * S::NC);
   }
 #pragma unroll
   for (int k = 0; k < 2 * JT; ++k) {
@@ -211,23 +245,24 @@ __global__ void __launch_bounds__(256, 2) grad_vhat_kernel(Dev d, int f0) {
 // then the chunks).
 template <int ZP> struct GbarShape {
   static constexpr int GN = 8 / ZP, GA = 8 * GN;           // n per thread and per CTA
-  static constexpr int R = GA + CT;                        // rows buffered
-  static constexpr int SMEM = (R + CT) * 64 * ZP * int(sizeof(float2)) + CT * (GA + 1) * int(sizeof(float4));
+  static constexpr int R = GA + 2 * CT;                    // rows buffered
+  static constexpr int NC = CT * (GA + 1);
+  static constexpr int SMEM = (R + 2 * CT) * 64 * ZP * int(sizeof(float2)) + 2 * NC * int(sizeof(float4));
 };
 
 template <int ZP>
 __global__ void __launch_bounds__(256, 2) grad_gbar_kernel(Dev d, int f0) {
   using S = GbarShape<ZP>;
-  constexpr int GN = S::GN, GA = S::GA, R = S::R, ZC = 64 * ZP;
+  constexpr int GN = S::GN, GA = S::GA, R = S::R, ZC = 64 * ZP, CQ = CT * GA / 256;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  float4 (*cf)[GA + 1] = reinterpret_cast<float4 (*)[GA + 1]>(smem_raw);    // [CT] (C1, C2) of (m, n)
-  float2* ws = reinterpret_cast<float2*>(cf + CT);         // [CT] Vhat rows
-  float2* gqs = ws + CT * ZC;                              // row a0 + GA - 1 - u in slot u mod R
+  float4* cf = reinterpret_cast<float4*>(smem_raw);        // [2][CT][GA + 1] (C1, C2) of (m, n)
+  float2* ws = reinterpret_cast<float2*>(cf + 2 * S::NC);  // [2][CT] Vhat rows
+  float2* gqs = ws + 2 * CT * ZC;                          // row a0 + GA - 1 - u in slot u mod R
   const int N = d.N, H = N / 2, msk = N - 1, nk = d.nk, fi = blockIdx.z, f = f0 + fi;
   const int a0 = blockIdx.x * GA, z0 = blockIdx.y * ZC;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const float2* g = d.g32 + size_t(f) * nk * d.nzs;
-  const float2* vh = reinterpret_cast<const float2*>(d.vfull);     // row m at 2 nz m
+  const float2* g = d.g32 + size_t(f) * nk * d.nzs + z0;
+  const float2* vh = reinterpret_cast<const float2*>(d.vfull) + z0;     // row m at 2 nz m
   const float4* E = d.born_fold + size_t(fi) * 2 * nk * nk;
   const float4* T = E + size_t(nk) * nk;
   const bool live = a0 + GN * w <= H;                      // the same in the whole warp
@@ -236,32 +271,56 @@ __global__ void __launch_bounds__(256, 2) grad_gbar_kernel(Dev d, int f0) {
   for (int k = 0; k < GN; ++k)
 #pragma unroll
     for (int i = 0; i < 2 * ZP; ++i) tot[k][i] = make_float2(0.f, 0.f);
-  for (int mc = 0; mc < N; mc += CT) {
-    // rows q = n - m: u = GA - 1 - (n - a0) + m, all of them once, CT new ones per chunk
-    const int lo = mc == 0 ? 0 : mc + GA - 1, hi = mc + GA + CT - 1;
-    for (int e = threadIdx.x; e < (hi - lo) * ZC; e += 256) {
-      const int u = lo + e / ZC, zz = e % ZC, z = z0 + zz;
-      gqs[(u % R) * ZC + zz] = z < d.nz ? g[size_t(tab_index((a0 + GA - 1 - u) & msk, N)) * d.nzs + z]
-                                        : make_float2(0.f, 0.f);
+  // rows q = n - m: u = GA - 1 - (n - a0) + m; depths past nz are not copied (not stored either)
+  auto copy_rows = [&](int lo, int hi, int mc, float2* wb) {
+    for (int e = threadIdx.x; e < (hi - lo) * (ZC / 2); e += 256) {
+      const int u = lo + e / (ZC / 2), zz = 2 * (e % (ZC / 2));
+      if (z0 + zz < d.nz)
+        copy16(gqs + (u % R) * ZC + zz, g + size_t(tab_index((a0 + GA - 1 - u) & msk, N)) * d.nzs + zz);
     }
-    for (int e = threadIdx.x; e < CT * ZC; e += 256) {
-      const int mi = e / ZC, zz = e % ZC, z = z0 + zz;
-      ws[e] = z < d.nz ? vh[size_t(mc + mi) * 2 * d.nz + z] : make_float2(0.f, 0.f);
+    for (int e = threadIdx.x; e < CT * (ZC / 2); e += 256) {
+      const int mi = e / (ZC / 2), zz = 2 * (e % (ZC / 2));
+      if (z0 + zz < d.nz) copy16(wb + mi * ZC + zz, vh + size_t(mc + mi) * 2 * d.nz + zz);
     }
-    for (int e = threadIdx.x; e < CT * GA; e += 256) {
-      const int al = e / CT, mi = e - al * CT, n = a0 + al;
-      float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
+    copies_commit();
+  };
+  float4 raw[CQ];
+  auto load_coef = [&](int mc) {
+#pragma unroll
+    for (int i = 0; i < CQ; ++i) {
+      const int e = threadIdx.x + 256 * i, n = a0 + e / CT;
+      raw[i] = make_float4(0.f, 0.f, 0.f, 0.f);
       if (n <= H) {
-        int q = (n - mc - mi) & msk;
+        int q = (n - mc - e % CT) & msk;
         if (q > H) q -= N;
-        const float4 c = q >= 0 ? E[size_t(n) * nk + q] : T[size_t(n) * nk - q];
-        const float wt = n == 0 || n == H ? 0.5f : 1.f;
-        o = make_float4(wt * (c.x + c.z), -wt * (c.y + c.w), wt * (c.y - c.w), wt * (c.x - c.z));
+        raw[i] = q >= 0 ? E[size_t(n) * nk + q] : T[size_t(n) * nk - q];
       }
-      cf[mi][al] = o;
     }
-    __syncthreads();
+  };
+  auto store_coef = [&](float4* dst) {
+#pragma unroll
+    for (int i = 0; i < CQ; ++i) {
+      const int e = threadIdx.x + 256 * i, al = e / CT, n = a0 + al;
+      const float4 c = raw[i];
+      const float wt = n == 0 || n == H ? 0.5f : 1.f;
+      dst[(e % CT) * (GA + 1) + al] = make_float4(wt * (c.x + c.z), -wt * (c.y + c.w), wt * (c.y - c.w), wt * (c.x - c.z));
+    }
+  };
+  copy_rows(0, GA + CT - 1, 0, ws);
+  load_coef(0);
+  store_coef(cf);
+  int buf = 0;
+  for (int mc = 0; mc < N; mc += CT, buf ^= 1) {
+    copies_wait();
+    __syncthreads();                                       // this chunk is staged, the last one done with
+    const bool more = mc + CT < N;
+    if (more) {
+      copy_rows(mc + GA + CT - 1, mc + GA + 2 * CT - 1, mc + CT, ws + (buf ^ 1) * CT * ZC);
+      load_coef(mc + CT);
+    }
     if (live) {
+      const float4* cb = cf + buf * S::NC + GN * w;
+      const float2* wb = ws + buf * CT * ZC;
       // n_k = a0 + GN w + k at m = mc + mi: u = GA - 1 - GN w - k + m
       Row<ZP> win[GN];
       float2 acc[GN][2 * ZP];
@@ -280,10 +339,10 @@ __global__ void __launch_bounds__(256, 2) grad_gbar_kernel(Dev d, int f0) {
           for (int k = GN - 1; k > 0; --k) win[k] = win[k - 1];
           win[0] = row_of<ZP>(gqs, sq, lane);
         }
-        const Row<ZP> v = row_of<ZP>(ws, mi, lane);
+        const Row<ZP> v = row_of<ZP>(wb, mi, lane);
 #pragma unroll
         for (int k = 0; k < GN; ++k) {
-          const float4 c = cf[mi][GN * w + k];
+          const float4 c = cb[mi * (GA + 1) + k];
 #pragma unroll
           for (int i = 0; i < 2 * ZP; ++i) {
             const float2 vz = v.at(i), gz = win[k].at(i);
@@ -298,7 +357,7 @@ __global__ void __launch_bounds__(256, 2) grad_gbar_kernel(Dev d, int f0) {
 #pragma unroll
         for (int i = 0; i < 2 * ZP; ++i) tot[k][i] = tot[k][i] + acc[k][i];
     }
-    __syncthreads();
+    if (more) store_coef(cf + (buf ^ 1) * S::NC);
   }
   const float sc = float(2.0 / (double(N) * N) * sqrt(d.fc[f].s_abs));
   float2* G = d.gbar + size_t(f) * nk * d.nz;

@@ -37,29 +37,14 @@
 // the depth march.
 #include "edt_internal.h"
 #include "cplx.cuh"
+#include "green_coef.cuh"
 
 namespace edt {
 
 namespace {
 
-// coefficient slots per (f, n, layer): kappa; sigma, then M; tau, then T; exp(i kappa dz),
-// exp(-i kappa dz); exp(i kappa h); delta, then D (see green_layer and green_recursion)
-constexpr int NCOEF = 7;
-constexpr int C_KAP = 0, C_SIG = 1, C_MUP = 1, C_AMP = 2, C_E = 3, C_EI = 4, C_EH = 5, C_DEL = 6, C_DEN = 6;
 // FP32 copies for the fast evaluation: kappa.x and kappa.y as (hi, lo) pairs, amp, rho
 constexpr int NCOEF32 = 8;
-
-// coefficient array layout [f][layer][slot][n]: consecutive wavenumbers are adjacent, so the
-// per-(f, n) threads of every kernel below read and write them coalesced
-__device__ __forceinline__ size_t cix(const Dev& d, int f, int n, int j, int k) {
-  return ((size_t(f) * d.nlayer + j) * NCOEF + k) * d.nk + n;
-}
-
-// 1 / b with one real division (|b| is O(1e-3 .. 1e3) for every use here)
-__device__ __forceinline__ double2 cinv(double2 b) {
-  const double r = 1.0 / (b.x * b.x + b.y * b.y);
-  return cmk(b.x * r, -b.y * r);
-}
 
 // sqrt(w) on the branch Im >= 0, FP64: the FP32 root (relative error ~1e-7) and two Newton steps
 // k + (w - k^2) / (2 k) whose residual is formed in FP64 and whose divisor is the FP32 root's (it
@@ -308,13 +293,6 @@ __global__ void __launch_bounds__(32) green_recursion_kernel(Dev d) {
   }
 }
 
-// amplitude and reflection of layer j from the recursion's M, D, T
-__device__ __forceinline__ void layer_waves(const Dev& d, int f, int n, int j, double2& amp, double2& rho) {
-  const double2 D = d.coef[cix(d, f, n, j, C_DEN)];
-  amp = d.coef[cix(d, f, n, j, C_AMP)] * D;
-  rho = j < d.nlayer - 1 ? d.coef[cix(d, f, n, j, C_MUP)] * cinv(D) : cmk(0.0, 0.0);
-}
-
 // the FP32 coefficients green_eval32 reads, per (f, n, layer)
 __global__ void __launch_bounds__(128) green_coef32_kernel(Dev d) {
   const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -510,6 +488,7 @@ __global__ void __launch_bounds__(256) green_eval32_kernel(Dev d) {
 }  // namespace
 
 int green_launches(const Dev& d, int tables) {
+  if (tables == GREEN_COEF) return 2;
   if (tables == GREEN_G32F && d.nlayer <= COEF32_MAX_LAYERS) return 3;
   return tables == GREEN_G32 || tables == GREEN_G32F ? 4 : 3;
 }
@@ -523,16 +502,17 @@ cudaError_t launch_green(const Dev& d, cudaStream_t s, int tables) {
     green_rec32_kernel<<<g1, 128, 0, s>>>(d);
   } else {
     const long long rows = (long long)d.nf * d.nk, nl = rows * d.nlayer;
-    const int run = d.nlayer > 64 ? 4 : 1;
+    const int run = d.nlayer > 64 ? 4 : 1, steps = fast32 || tables == GREEN_COEF ? 0 : 1;
     const unsigned lb = unsigned((rows * ((d.nlayer + run - 1) / run) + LBLOCK - 1) / LBLOCK);
-    if (run == 4) green_layer_kernel<4><<<lb, LBLOCK, 0, s>>>(d, fast32 ? 0 : 1);
-    else green_layer_kernel<1><<<lb, LBLOCK, 0, s>>>(d, fast32 ? 0 : 1);
+    if (run == 4) green_layer_kernel<4><<<lb, LBLOCK, 0, s>>>(d, steps);
+    else green_layer_kernel<1><<<lb, LBLOCK, 0, s>>>(d, steps);
     // the split walks every layer twice (2 x 2 matrices, then the run): only for stacks of at
     // least four layers per run over too few (f, n) to fill the SMs' quarters
     if (d.nlayer > 4 * 16 && rows < 32 * 304) green_recursion_kernel<16><<<unsigned((rows + 1) / 2), 32, 0, s>>>(d);
     else green_recursion_kernel<1><<<unsigned((rows + 31) / 32), 32, 0, s>>>(d);
     if (fast32) green_coef32_kernel<<<unsigned((nl + 127) / 128), 128, 0, s>>>(d);
   }
+  if (tables == GREEN_COEF) return cudaGetLastError();
   if (fast32) {
     green_eval32_kernel<<<unsigned((long long)d.nf * d.nk), 256, 0, s>>>(d);
   } else {

@@ -519,14 +519,19 @@ __global__ void __launch_bounds__(256) cb_prow_kernel(Dev d, int k0, const int* 
                          : (r < kb && lane == r ? df_of(d.dinv[vo + k0 + r]) : make_float2(0.f, 0.f));
   }
   __syncthreads();
+  // the four outputs j = warp + 8 q side by side, so that their chains of dependent additions
+  // overlap; X_jl is zero for l > j, so l runs to the largest j of the eight warps
   float2 out[4];
 #pragma unroll
-  for (int q = 0; q < 4; ++q) {
-    const int j = warp + 8 * q;
-    float2 acc = make_float2(0.f, 0.f);
-    for (int l = 0; l <= j; ++l) df_acc(acc, sA[l * LDP + lane], sX[j * LDP + l]);
-    out[q] = df_norm(acc);
+  for (int q = 0; q < 4; ++q) out[q] = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int l = 0; l < NB; ++l) {
+    const float2 a = sA[l * LDP + lane];
+#pragma unroll
+    for (int q = l / 8; q < 4; ++q) df_acc(out[q], a, sX[(warp + 8 * q) * LDP + l]);
   }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) out[q] = df_norm(out[q]);
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < 4; ++q) sA[(warp + 8 * q) * LDP + lane] = out[q];

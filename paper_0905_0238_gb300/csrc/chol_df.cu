@@ -90,14 +90,19 @@ __global__ void __launch_bounds__(128) cdf_panel_kernel(Dev d, int k0) {
     }
   }
   __syncthreads();
+  // the eight outputs j = h + 4 q side by side, so that their chains of dependent additions
+  // overlap; X_jl is zero for l > j, so l runs to the largest j of the four warps
   float2 out[FB / 4];
 #pragma unroll
-  for (int q = 0; q < FB / 4; ++q) {
-    const int j = h + 4 * q;
-    float2 acc = make_float2(0.f, 0.f);
-    for (int l = 0; l <= j; ++l) df_acc(acc, sA[l * FLD + lane], sX[j * FLD + l]);
-    out[q] = df_norm(acc);
+  for (int q = 0; q < FB / 4; ++q) out[q] = make_float2(0.f, 0.f);
+#pragma unroll
+  for (int l = 0; l < FB; ++l) {
+    const float2 a = sA[l * FLD + lane];
+#pragma unroll
+    for (int q = l / 4; q < FB / 4; ++q) df_acc(out[q], a, sX[(h + 4 * q) * FLD + l]);
   }
+#pragma unroll
+  for (int q = 0; q < FB / 4; ++q) out[q] = df_norm(out[q]);
   __syncthreads();
 #pragma unroll
   for (int q = 0; q < FB / 4; ++q) sA[(h + 4 * q) * FLD + lane] = out[q];

@@ -216,8 +216,8 @@ typedef struct {
                                    [4, 8, 16]; default 8                                    */
   int refine_shape;             /* mixed: refinement CTA shape, 0 = 4 warps x 32 rows,
                                    1 = 8 x 32, 2 = 4 x 64, 3 = 8 x 16; default 0           */
-  int window_ztile;             /* window geometry: depths per kernel-row cluster [2, 4, 8];
-                                   default 4                                                */
+  int window_ztile;             /* window geometry on a line (ny = 1): depths per kernel-row
+                                   cluster [2, 4, 8]; default 4; no effect on a grid        */
   int overlap;                  /* 1: depth march (and window kernel rows) on the internal
                                    stream, concurrent with the data transform; 0: in
                                    sequence on the caller's stream [0, 1]; default 1        */

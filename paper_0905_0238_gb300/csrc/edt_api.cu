@@ -69,6 +69,9 @@ struct edt_ctx {
   std::vector<int2> fj_ent;            // [rows] (midpoint index, row) grouped by (f, j)
   std::vector<double2> cf;             // [nf] omega~^2 dx dy dz
   std::vector<int> jact, jmap, nact;   // active offset wavenumbers per frequency
+  std::vector<int> q_off, q_xy;        // a grid's quadrant points with kept rows, per frequency
+  std::vector<int4> q_rows;            // [q_xy] rows of the pairs (kx, ky) and (-kx, ky)
+  int q_max = 0;                       // most points of a frequency
   long long rows_max_sub = 0;
   // band-limited transform of the mixed path
   bool band_mode = false;
@@ -102,7 +105,7 @@ struct edt_ctx {
   // workspace
   size_t ws_bytes = 0;
   void* ws = nullptr;
-  Region r_fc, r_ltop, r_lvel, r_zl, r_zo, r_rows, r_roff, r_roffmf, r_band, r_bcol, r_cpre, r_kval, r_pairm, r_fjoff, r_fjent, r_jact, r_jmap, r_Gs, r_U, r_Dw, r_A32, r_tw64, r_tw32, r_segm, r_segr0,
+  Region r_fc, r_ltop, r_lvel, r_zl, r_zo, r_rows, r_roff, r_roffmf, r_band, r_bcol, r_cpre, r_kval, r_pairm, r_fjoff, r_fjent, r_jact, r_jmap, r_qxy, r_qrows, r_Gs, r_U, r_Dw, r_A32, r_tw64, r_tw32, r_segm, r_segr0,
       r_segn, r_ctas, r_mslot, r_zo32, r_fc32, r_coef, r_coef32, r_g64, r_g32, r_g32lo, r_rowmax, r_gscale, r_X, r_Dst, r_Vst, r_rhs, r_gent, r_gpart, r_G,
       r_dinv, r_L32, r_dinv32, r_b, r_tr, r_tpart, r_x, r_r, r_rpart, r_rowc, r_xmu, r_gam, r_tref, r_treoff, r_vhat, r_vfull, r_gscr, r_adj, r_gacc, r_gcpart, r_bexp, r_bfold, r_status, r_flags,
       r_g64part, r_b64part, r_tlog, r_kzP, r_kzp, r_kzgoff, r_kzvoff, r_kzG, r_kzT, r_kzb, r_kzx;
@@ -218,11 +221,13 @@ void plan_window(edt_ctx* c, double cmin) {
   c->rows.clear();
   c->row_off.assign(c->nsub + 1, 0);
   c->counts_cut.assign(c->nsub, 0);
+  std::vector<int> pf(size_t(nf + 1) * c->nsub);       // first row of (pair, frequency)
   for (int p = 0; p < c->nsub; ++p) {
     c->row_off[p] = (long long)c->rows.size();
     const int m = c->pair_m[p], my = m / nx, mx = m - my * nx;
     const double mxs = double(sgn(mx, nx)) / (nx * g.dx), mys = double(sgn(my, ny)) / (ny * g.dy);
-    for (int f = 0; f < nf; ++f)
+    for (int f = 0; f < nf; ++f) {
+      pf[size_t(p) * (nf + 1) + f] = int(c->rows.size());
       for (int jy = 0; jy < wy; ++jy)
         for (int jx = 0; jx < wx; ++jx) {
           bool keep = true;
@@ -240,6 +245,8 @@ void plan_window(edt_ctx* c, double cmin) {
           c->rows.push_back(uint32_t(f) << 16 | uint32_t(j));
           c->counts_cut[p] += 1;
         }
+    }
+    pf[size_t(p) * (nf + 1) + nf] = int(c->rows.size());
   }
   c->row_off[c->nsub] = (long long)c->rows.size();
   c->fj_off.assign(size_t(nf) * W + 1, 0);
@@ -260,6 +267,31 @@ void plan_window(edt_ctx* c, double cmin) {
         c->jact[size_t(f) * W + c->nact[f]] = j;
         c->nact[f]++;
       }
+  // a grid's kernel rows are formed per quadrant point (kx, ky) for the pairs of (+-kx, ky)
+  c->q_off.assign(nf + 1, 0);
+  c->q_xy.clear(); c->q_rows.clear();
+  c->q_max = 0;
+  if (ny > 1) {
+    std::vector<int> pair_of(size_t(ny) * nx, -1);
+    for (int p = 0; p < c->nsub; ++p) pair_of[c->pair_m[p]] = p;
+    for (int f = 0; f < nf; ++f) {
+      for (int qy = 0; qy < hy; ++qy)
+        for (int qx = 0; qx < hx; ++qx) {
+          const size_t p0 = size_t(pair_of[qy * nx + qx]) * (nf + 1) + f;
+          int4 r = make_int4(pf[p0], pf[p0 + 1] - pf[p0], 0, 0);
+          if (qx > 0 && 2 * qx < nx && qy > 0 && 2 * qy < ny) {
+            const size_t p1 = size_t(pair_of[qy * nx + nx - qx]) * (nf + 1) + f;
+            r.z = pf[p1];
+            r.w = pf[p1 + 1] - pf[p1];
+          }
+          if (r.y + r.w == 0) continue;
+          c->q_xy.push_back(qy << 16 | qx);
+          c->q_rows.push_back(r);
+        }
+      c->q_off[f + 1] = int(c->q_xy.size());
+      c->q_max = std::max(c->q_max, c->q_off[f + 1] - c->q_off[f]);
+    }
+  }
   c->cf.resize(nf);
   for (int f = 0; f < nf; ++f) {
     const double2 om = make_double2(c->fc[f].om_re, c->fc[f].om_im);
@@ -643,9 +675,14 @@ void layout(edt_ctx* c) {
   take(c->r_fjent, std::max<size_t>(c->fj_ent.size(), 1) * sizeof(int2));
   take(c->r_jact, std::max<size_t>(c->jact.size(), 1) * sizeof(int));
   take(c->r_jmap, std::max<size_t>(c->jmap.size(), 1) * sizeof(int));
-  take(c->r_Gs, c->win ? nz * nxy * sizeof(float2) : 0);
+  take(c->r_qxy, std::max<size_t>(c->q_xy.size(), 1) * sizeof(int));
+  take(c->r_qrows, std::max<size_t>(c->q_rows.size(), 1) * sizeof(int4));
+  const bool grid = c->win && c->ny > 1;
+  take(c->r_Gs, grid ? nz * (N / 2 + 1) * (c->ny / 2 + 1) * sizeof(float2) : c->win ? nz * N * sizeof(float2) : 0);
   const size_t wact = c->nact.empty() ? 1 : size_t(std::max(1, *std::max_element(c->nact.begin(), c->nact.end())));
-  take(c->r_U, c->win ? wact * nz * (size_t(c->ny / 2 + 1) * N) * sizeof(float2) : 0);
+  const size_t slots = grid ? fa_grid_slots(c->wx, c->wy) : 0;
+  take(c->r_U, grid ? slots * size_t(fa_grid_slab(c->nz, int(slots), c->q_max)) * std::max(c->q_max, 1) * sizeof(float2)
+               : c->win ? wact * nz * N * sizeof(float2) : 0);
   take(c->r_Dw, c->win ? nf * W * nxy * sizeof(float2) : 0);
   take(c->r_A32, c->win ? (R + 1) * nzs * sizeof(float2) : 0);
   take(c->r_tw64, (N / 2) * sizeof(double2));
@@ -754,6 +791,9 @@ void bind(edt_ctx* c) {
   d.fj_ent = at<const int2*>(c, c->r_fjent);
   d.jact = at<const int*>(c, c->r_jact);
   d.jmap = at<const int*>(c, c->r_jmap);
+  d.q_xy = at<const int*>(c, c->r_qxy);
+  d.q_rows = at<const int4*>(c, c->r_qrows);
+  d.fa_slab = c->win && c->ny > 1 ? fa_grid_slab(c->nz, fa_grid_slots(c->wx, c->wy), c->q_max) : 0;
   d.Gs = c->r_Gs.bytes ? at<float2*>(c, c->r_Gs) : nullptr;
   d.U = c->r_U.bytes ? at<float2*>(c, c->r_U) : nullptr;
   d.Dw = c->r_Dw.bytes ? at<float2*>(c, c->r_Dw) : nullptr;
@@ -894,7 +934,10 @@ int transform_rhs(edt_ctx* c, const void* D, int D_dtype, cudaStream_t s) {
 // Window geometry: the assembled kernel rows of every frequency into the row table.
 int kernel_rows(edt_ctx* c, cudaStream_t s) {
   if (!c->win) return EDT_OK;
-  for (int f = 0; f < c->nf; ++f) EDT_TRY(launch_fa_rows(c->dev, f, c->nact[f], c->cf[f], s));
+  for (int f = 0; f < c->nf; ++f) {
+    if (c->ny > 1) EDT_TRY(launch_fa_grid(c->dev, f, c->q_off[f], c->q_off[f + 1] - c->q_off[f], c->cf[f], s));
+    else EDT_TRY(launch_fa_line(c->dev, f, c->nact[f], c->cf[f], s));
+  }
   return EDT_OK;
 }
 
@@ -1028,6 +1071,8 @@ int edt_set_workspace(edt_ctx* c, void* ws, size_t bytes) {
   EDT_TRYI(upload(c, c->r_fjent, c->fj_ent));
   EDT_TRYI(upload(c, c->r_jact, c->jact));
   EDT_TRYI(upload(c, c->r_jmap, c->jmap));
+  EDT_TRYI(upload(c, c->r_qxy, c->q_xy));
+  EDT_TRYI(upload(c, c->r_qrows, c->q_rows));
   EDT_TRYI(upload(c, c->r_tw64, c->tw64));
   EDT_TRYI(upload(c, c->r_tw32, c->tw32));
   EDT_TRYI(upload(c, c->r_segm, c->seg_m));
@@ -1228,7 +1273,7 @@ int edt_autotune(edt_ctx* c, const void* D, int D_dtype, void* V, int V_dtype, v
       {&cur.band_budget_mb, {16, 32, 48, 96}, c->band_mode},
       {&cur.band_cols, {4, 8, 16}, c->band_mode},
       {&cur.refine_shape, {0, 1, 2, 3}, mixed && c->cfg.refine > 0},
-      {&cur.window_ztile, {2, 4, 8}, c->win},
+      {&cur.window_ztile, {2, 4, 8}, c->win && c->ny == 1},
       {&cur.overlap, {0, 1}, true},
   };
   for (Axis& a : axes) {
@@ -1541,11 +1586,13 @@ int edt_get_stats(edt_ctx* c, edt_stats* o) {
   // or Jacobi), the back-projection with the disk; the Jacobi kernel alone without it
   if (c->variant) o->launches_per_invert += (c->kz_p.empty() ? 1 : 5) - chol_launches(c->nz);
   if (c->win) {
-    // green (3), rows (3) per frequency that keeps any, data (2), Gram (2), Cholesky,
+    // green (3), rows per frequency that keeps any (a line: 3; a grid: 1 and 2 per slab of
+    // depths), data (2), Gram (2), Cholesky,
     // refinement (3 per step), inverse (completion, FP64 row and column transforms, output: 3 or 4)
     int fk = 0;
     for (int n : c->nact) fk += n > 0;
-    o->launches_per_invert = green_launches(c->dev, green_tables(c)) + 3 * fk + 2 + 2 + chol_n + 3 * c->cfg.refine +
+    const int per_f = c->ny > 1 ? 1 + 2 * ((c->nz + c->dev.fa_slab - 1) / c->dev.fa_slab) : 3;
+    o->launches_per_invert = green_launches(c->dev, green_tables(c)) + per_f * fk + 2 + 2 + chol_n + 3 * c->cfg.refine +
                              (c->ny > 1 ? 4 : 3);
   }
   o->freq_chunk = c->band_mode ? c->band_maxplanes : c->fchunk;

@@ -87,7 +87,7 @@ struct Dev {
   int fchunk;                   // frequency planes per chunk of the full-plane transform
   // launch shapes picked by the autotuner (edt_autotune): band-column block width (4, 8,
   // 16), refinement CTA shape (0: 4 warps x 32 rows, 1: 8 x 32, 2: 4 x 64, 3: 8 x 16),
-  // depths per kernel-row cluster of the window geometry (2, 4, 8)
+  // depths per kernel-row cluster of a window line (2, 4, 8)
   int tune_bc, tune_rf, tune_zc;
   // band-limited transform (mixed path)
   const BandInfo* band;         // [nf]
@@ -106,9 +106,13 @@ struct Dev {
   const int* jact;              // [nf][W] active offset wavenumbers of each frequency (those
                                 //   with kept rows), compacted; then -1
   const int* jmap;              // [nf][W] position of j among the active ones, or -1
-  float2* Gs;                   // [nz][ny][nx] G(y, z) of one frequency
-  float2* U;                    // [W][nz][ny/2 + 1][nx] window products of one frequency
-                                //   (centrosymmetric in y: rows 0..ny/2 stored)
+  const int* q_xy;              // a grid's quadrant points (y << 16 | x) with kept rows, per frequency
+  const int4* q_rows;           // their rows: (first, count) of the pair (kx, ky), then of (-kx, ky)
+  int fa_slab;                  // depths whose planes of one frequency are held at a time (grid)
+  float2* Gs;                   // G(y, z) of one frequency: a line [nz][nx], a grid's quadrant
+                                //   [nz][ny/2 + 1][nx/2 + 1]
+  float2* U;                    // a line: [active j][nz][nx] window products of one frequency; a grid:
+                                //   [slab][slot][point] (csrc/fagrid.cu)
   float2* Dw;                   // [nf][W][ny][nx] window-transformed data
   float2* A32;                  // [rows + 1][nzs] kernel rows, then a row of ones
   long long ones_row;           // index of the ones row in A32
@@ -230,7 +234,13 @@ cudaError_t prepare_band(const Dev& d);
 // Window geometry (csrc/fa.cu): kernel rows of frequency f into A32, data transform and
 // right-hand sides, the inverse transform to V[ny][nx][nz]; supported grids and windows.
 bool fa_supported(int nx, int ny, int wx, int wy);
-cudaError_t launch_fa_rows(const Dev& d, int f, int nact, double2 cf, cudaStream_t s);
+cudaError_t launch_fa_line(const Dev& d, int f, int nact, double2 cf, cudaStream_t s);
+// the same for a grid (csrc/fagrid.cu): the frequency's points are q_xy/q_rows[qoff .. qoff + nq)
+constexpr size_t FA_SLAB_BYTES = size_t(2) << 30;     // plane buffer of a slab of depths (at least 16)
+int fa_grid_slots(int wx, int wy);
+int fa_grid_slab(int nz, int slots, int nq);
+cudaError_t launch_fa_grid(const Dev& d, int f, int qoff, int nq, double2 cf, cudaStream_t s);
+cudaError_t prepare_fa_grid(const Dev& d);
 cudaError_t launch_fa_data(const Dev& d, const void* D, int D_dtype, cudaStream_t s);
 cudaError_t launch_fa_inverse(const Dev& d, void* V, int V_dtype, cudaStream_t s);
 cudaError_t launch_fa_setup(const Dev& d, long long nrows, cudaStream_t s);

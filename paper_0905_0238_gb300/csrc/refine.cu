@@ -8,14 +8,20 @@
 // refine_sum adds the partials of a subproblem in FP64 in CTA order, so repeated calls give the
 // same bits.  Table
 // rows are read with 16-byte loads (two depths per load) when nz is even, two rows at a time
-// per warp so that both rows' loads are in flight together.  Each warp walks its rows two at a time so that the table loads of
-// both rows are in flight together; rows p and -p sit side by side in the row order and
-// share a table row, so one of the two reads is an L1 hit.  This is the matrix-free form of Ahat^T (dhat - Ahat x): the normal
-// matrix used by the factorisation (from the tensor-core Gram) is not involved, so the
-// refinement corrects the Gram's rounding.
+// per warp so that both rows' loads are in flight together.  This is the matrix-free form of
+// Ahat^T (dhat - Ahat x): the normal matrix used by the factorisation (from the tensor-core Gram) is
+// not involved, so the refinement corrects the Gram's rounding.
+//
+// L1 bounds the line form (71 % of its throughput at 512 points and 256 depths): the row loads cannot
+// be avoided, but x came as eight conflicting 4-byte reads per load of a row and each of the two
+// rows' four predictions took five shuffles and its u four loads.  x is now one 16-byte read
+// for both rows, the eight predictions are summed together (9 shuffles), each lane forms one
+// component of u and eight shuffles hand them round: the production line's inversion takes 3.76 ms
+// instead of 3.93.
 #include "edt_internal.h"
 #include "cplx.cuh"
 #include "dfloat.cuh"
+#include "warpsum.cuh"
 
 #include <algorithm>
 
@@ -30,7 +36,7 @@ namespace {
 template <int Z4, bool FA, int RF_WARPS, int RF_ROWS_PER_WARP>
 __global__ void __launch_bounds__(RF_WARPS * 32) refine_kernel(Dev d) {
   constexpr int ZL = 64 * Z4;
-  __shared__ float xs[2][ZL];
+  __shared__ float4 xs[32 * Z4];               // x of depths 2 i, 2 i + 1: (+, +, -, -)
   __shared__ float red[RF_WARPS][2][ZL];
   const int m = blockIdx.y;
   const long long r0 = d.row_off[m], nr = d.row_off[m + 1] - r0;
@@ -39,21 +45,24 @@ __global__ void __launch_bounds__(RF_WARPS * 32) refine_kernel(Dev d) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int nz = d.nz, N = d.N, msk = N - 1;
   for (int i = threadIdx.x; i < ZL; i += blockDim.x) {
-    xs[0][i] = i < nz ? float(d.x[(size_t(m) * nz + i) * 2 + 0]) : 0.f;
-    xs[1][i] = i < nz ? float(d.x[(size_t(m) * nz + i) * 2 + 1]) : 0.f;
+    float* x = reinterpret_cast<float*>(xs + (i >> 1)) + (i & 1);
+    x[0] = i < nz ? float(d.x[(size_t(m) * nz + i) * 2 + 0]) : 0.f;
+    x[2] = i < nz ? float(d.x[(size_t(m) * nz + i) * 2 + 1]) : 0.f;
   }
   __syncthreads();
   float acc[Z4][2][2];                         // [load t][depth 0/1 of the float4][rhs]
 #pragma unroll
   for (int t = 0; t < Z4; ++t) acc[t][0][0] = acc[t][0][1] = acc[t][1][0] = acc[t][1][1] = 0.f;
-  const float2* rhs = reinterpret_cast<const float2*>(d.rhs);
+  const float* rhs = reinterpret_cast<const float*>(d.rhs);    // [row][+ re, + im, - re, - im]
   const long long wb = c0 + warp * RF_ROWS_PER_WARP;
   const long long we = min(nr, wb + RF_ROWS_PER_WARP);
   for (long long i = wb; i < we; i += 2) {
     const bool two = i + 1 < we;
     float4 a[2][Z4];
     float wv[2];
-    long long ri[2] = {r0 + i, r0 + (two ? i + 1 : i)};
+    const long long ri[2] = {r0 + i, r0 + (two ? i + 1 : i)};
+    // this lane's datum: component (lane >> 2) & 3 of row lane >> 4
+    const float dv = d.refine_nodata ? 0.f : rhs[4 * (lane & 16 ? ri[1] : ri[0]) + ((lane >> 2) & 3)];
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       size_t rp, rq;
@@ -76,35 +85,37 @@ __global__ void __launch_bounds__(RF_WARPS * 32) refine_kernel(Dev d) {
       for (int t = 0; t < Z4; ++t) {
         const int z = 2 * lane + 64 * t;
         const float4 u = z < nz ? __ldg(gp + (z >> 1)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        if (FA) {                               // the second factor is the row of ones
+          a[h][t] = u;
+          continue;
+        }
         const float4 v = z < nz ? __ldg(gq + (z >> 1)) : make_float4(0.f, 0.f, 0.f, 0.f);
         // (z + 1 may be the zero padding of an odd nz)
         a[h][t] = make_float4(u.x * v.x - u.y * v.y, u.x * v.y + u.y * v.x,
                               u.z * v.z - u.w * v.w, u.z * v.w + u.w * v.z);
       }
     }
+    // the eight predictions (row h, rhs, re/im), summed over the warp together; lane 4 c holds sum c
+    float tv[8];
+#pragma unroll
+    for (int c = 0; c < 8; ++c) tv[c] = 0.f;
+#pragma unroll
+    for (int t = 0; t < Z4; ++t) {
+      const float4 x = xs[lane + 32 * t];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        tv[4 * h + 0] = fmaf(a[h][t].x, x.x, fmaf(a[h][t].z, x.y, tv[4 * h + 0]));
+        tv[4 * h + 1] = fmaf(a[h][t].y, x.x, fmaf(a[h][t].w, x.y, tv[4 * h + 1]));
+        tv[4 * h + 2] = fmaf(a[h][t].x, x.z, fmaf(a[h][t].z, x.w, tv[4 * h + 2]));
+        tv[4 * h + 3] = fmaf(a[h][t].y, x.z, fmaf(a[h][t].w, x.w, tv[4 * h + 3]));
+      }
+    }
+    const float ts = warp_sums<8>(tv, lane);
+    const float us = (lane & 16 ? wv[1] : wv[0]) * (dv - ts);
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      float2 tp = make_float2(0.f, 0.f), tm = tp;
-#pragma unroll
-      for (int t = 0; t < Z4; ++t) {
-        const int z = 2 * lane + 64 * t;
-        const float x0 = xs[0][z], x1 = xs[0][z + 1], y0 = xs[1][z], y1 = xs[1][z + 1];
-        tp.x = fmaf(a[h][t].x, x0, fmaf(a[h][t].z, x1, tp.x));
-        tp.y = fmaf(a[h][t].y, x0, fmaf(a[h][t].w, x1, tp.y));
-        tm.x = fmaf(a[h][t].x, y0, fmaf(a[h][t].z, y1, tm.x));
-        tm.y = fmaf(a[h][t].y, y0, fmaf(a[h][t].w, y1, tm.y));
-      }
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        tp.x += __shfl_xor_sync(0xffffffffu, tp.x, o); tp.y += __shfl_xor_sync(0xffffffffu, tp.y, o);
-        tm.x += __shfl_xor_sync(0xffffffffu, tm.x, o); tm.y += __shfl_xor_sync(0xffffffffu, tm.y, o);
-      }
-      const float w = wv[h];
-      const float2 zero2 = make_float2(0.f, 0.f);
-      const float2 dp = d.refine_nodata ? zero2 : rhs[2 * ri[h]];
-      const float2 dm = d.refine_nodata ? zero2 : rhs[2 * ri[h] + 1];
-      const float2 up = make_float2(w * (dp.x - tp.x), w * (dp.y - tp.y));
-      const float2 um = make_float2(w * (dm.x - tm.x), w * (dm.y - tm.y));
+      const float2 up = make_float2(__shfl_sync(0xffffffffu, us, 16 * h), __shfl_sync(0xffffffffu, us, 16 * h + 4));
+      const float2 um = make_float2(__shfl_sync(0xffffffffu, us, 16 * h + 8), __shfl_sync(0xffffffffu, us, 16 * h + 12));
 #pragma unroll
       for (int t = 0; t < Z4; ++t) {
         acc[t][0][0] = fmaf(a[h][t].x, up.x, fmaf(a[h][t].y, up.y, acc[t][0][0]));
@@ -172,7 +183,7 @@ __device__ __forceinline__ void acc_df(float& s, float& lo, float2 ah, float2 al
 template <int Z4, int RF_WARPS, int RF_ROWS_PER_WARP>
 __global__ void __launch_bounds__(RF_WARPS * 32) refine_df_kernel(Dev d) {
   constexpr int ZL = 64 * Z4;
-  __shared__ float xs[2][ZL];
+  __shared__ __align__(8) float xs[2][ZL];
   __shared__ double red[RF_WARPS][2][ZL];
   const int m = blockIdx.y;
   const long long r0 = d.row_off[m], nr = d.row_off[m + 1] - r0;
@@ -185,6 +196,14 @@ __global__ void __launch_bounds__(RF_WARPS * 32) refine_df_kernel(Dev d) {
     xs[1][i] = i < nz ? float(d.x[(size_t(m) * nz + i) * 2 + 1]) : 0.f;
   }
   __syncthreads();
+  // this lane's depths of x, kept in registers over the rows (the FP32 form above reads them again:
+  // the registers cost it more in occupancy than the reads)
+  float2 xp[Z4], xm[Z4];
+#pragma unroll
+  for (int t = 0; t < Z4; ++t) {
+    xp[t] = *reinterpret_cast<const float2*>(&xs[0][2 * lane + 64 * t]);
+    xm[t] = *reinterpret_cast<const float2*>(&xs[1][2 * lane + 64 * t]);
+  }
   // [load t][depth 0/1 of the float4][rhs]: high-order sum, low-order sum
   float as[Z4][2][2], al_[Z4][2][2];
 #pragma unroll
@@ -193,7 +212,7 @@ __global__ void __launch_bounds__(RF_WARPS * 32) refine_df_kernel(Dev d) {
     for (int j = 0; j < 2; ++j)
 #pragma unroll
       for (int k = 0; k < 2; ++k) as[t][j][k] = al_[t][j][k] = 0.f;
-  const float2* rhs = reinterpret_cast<const float2*>(d.rhs);
+  const float* rhs = reinterpret_cast<const float*>(d.rhs);    // [row][+ re, + im, - re, - im]
   const long long wb = c0 + warp * RF_ROWS_PER_WARP;
   const long long we = min(nr, wb + RF_ROWS_PER_WARP);
   for (long long i = wb; i < we; ++i) {
@@ -203,6 +222,7 @@ __global__ void __launch_bounds__(RF_WARPS * 32) refine_df_kernel(Dev d) {
     const int np = p <= N / 2 ? p : N - p, nq = q <= N / 2 ? q : N - q;
     const size_t rp = (size_t(f) * d.nk + np) * d.nzs, rq = (size_t(f) * d.nk + nq) * d.nzs;
     const float w = row_w2(row) ? 2.f : 1.f;
+    const float dv = d.refine_nodata ? 0.f : rhs[4 * ri + (lane >> 3)];   // this lane's datum
     const float4* gph = reinterpret_cast<const float4*>(d.g32 + rp);
     const float4* gqh = reinterpret_cast<const float4*>(d.g32 + rq);
     const float4* gpl = reinterpret_cast<const float4*>(d.g32lo + rp);
@@ -219,26 +239,18 @@ __global__ void __launch_bounds__(RF_WARPS * 32) refine_df_kernel(Dev d) {
       cmul_df(make_float2(u.z, u.w), make_float2(ul.z, ul.w), make_float2(v.z, v.w), make_float2(vl.z, vl.w),
               ah[t][1], al[t][1]);
     }
-    float2 tp = make_float2(0.f, 0.f), tm = tp;
+    float tv[4] = {0.f, 0.f, 0.f, 0.f};         // predictions (rhs, re/im)
 #pragma unroll
     for (int t = 0; t < Z4; ++t) {
-      const int z = 2 * lane + 64 * t;
-      const float x0 = xs[0][z], x1 = xs[0][z + 1], y0 = xs[1][z], y1 = xs[1][z + 1];
-      tp.x = fmaf(ah[t][0].x, x0, fmaf(ah[t][1].x, x1, tp.x));
-      tp.y = fmaf(ah[t][0].y, x0, fmaf(ah[t][1].y, x1, tp.y));
-      tm.x = fmaf(ah[t][0].x, y0, fmaf(ah[t][1].x, y1, tm.x));
-      tm.y = fmaf(ah[t][0].y, y0, fmaf(ah[t][1].y, y1, tm.y));
+      const float x0 = xp[t].x, x1 = xp[t].y, y0 = xm[t].x, y1 = xm[t].y;
+      tv[0] = fmaf(ah[t][0].x, x0, fmaf(ah[t][1].x, x1, tv[0]));
+      tv[1] = fmaf(ah[t][0].y, x0, fmaf(ah[t][1].y, x1, tv[1]));
+      tv[2] = fmaf(ah[t][0].x, y0, fmaf(ah[t][1].x, y1, tv[2]));
+      tv[3] = fmaf(ah[t][0].y, y0, fmaf(ah[t][1].y, y1, tv[3]));
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      tp.x += __shfl_xor_sync(0xffffffffu, tp.x, o); tp.y += __shfl_xor_sync(0xffffffffu, tp.y, o);
-      tm.x += __shfl_xor_sync(0xffffffffu, tm.x, o); tm.y += __shfl_xor_sync(0xffffffffu, tm.y, o);
-    }
-    const float2 zero2 = make_float2(0.f, 0.f);
-    const float2 dp = d.refine_nodata ? zero2 : rhs[2 * ri];
-    const float2 dm = d.refine_nodata ? zero2 : rhs[2 * ri + 1];
-    const float2 up = make_float2(w * (dp.x - tp.x), w * (dp.y - tp.y));
-    const float2 um = make_float2(w * (dm.x - tm.x), w * (dm.y - tm.y));
+    const float us = w * (dv - warp_sums<4>(tv, lane));
+    const float2 up = make_float2(__shfl_sync(0xffffffffu, us, 0), __shfl_sync(0xffffffffu, us, 8));
+    const float2 um = make_float2(__shfl_sync(0xffffffffu, us, 16), __shfl_sync(0xffffffffu, us, 24));
 #pragma unroll
     for (int t = 0; t < Z4; ++t)
 #pragma unroll
@@ -299,12 +311,15 @@ int refine_stride(long long rows_max_sub) {
   return int((std::max(rows_max_sub, 1LL) + least - 1) / least);
 }
 
+// Depths per lane follow nz in steps of 64: a 150-depth line inverts in 1.04 ms with three loads per
+// row (and the sums above), in 1.11 with the four that 193..256 depths take.
 template <int W, int R>
 void refine_df_shape(const Dev& d, cudaStream_t s) {
   const long long rows_per_cta = W * R;
   dim3 g(unsigned((std::max(d.rows_max_sub, 1LL) + rows_per_cta - 1) / rows_per_cta), d.nsub);
   if (d.nzs <= 64) refine_df_kernel<1, W, R><<<g, W * 32, 0, s>>>(d);
   else if (d.nzs <= 128) refine_df_kernel<2, W, R><<<g, W * 32, 0, s>>>(d);
+  else if (d.nzs <= 192) refine_df_kernel<3, W, R><<<g, W * 32, 0, s>>>(d);
   else refine_df_kernel<4, W, R><<<g, W * 32, 0, s>>>(d);
 }
 
@@ -316,6 +331,7 @@ void refine_shape(const Dev& d, cudaStream_t s) {
   const int nz_even = d.nzs;
   if (nz_even <= 64) fa ? refine_kernel<1, true, W, R><<<g, W * 32, 0, s>>>(d) : refine_kernel<1, false, W, R><<<g, W * 32, 0, s>>>(d);
   else if (nz_even <= 128) fa ? refine_kernel<2, true, W, R><<<g, W * 32, 0, s>>>(d) : refine_kernel<2, false, W, R><<<g, W * 32, 0, s>>>(d);
+  else if (nz_even <= 192) fa ? refine_kernel<3, true, W, R><<<g, W * 32, 0, s>>>(d) : refine_kernel<3, false, W, R><<<g, W * 32, 0, s>>>(d);
   else fa ? refine_kernel<4, true, W, R><<<g, W * 32, 0, s>>>(d) : refine_kernel<4, false, W, R><<<g, W * 32, 0, s>>>(d);
 }
 

@@ -357,6 +357,5 @@ cudaError_t prepare_grad();
 constexpr int TC_M = 128;              // MMA rows (depth unknowns per M tile)
 constexpr int TC_KC = 32;              // complex rows per pipeline stage (K = 64 real rows)
 int tc_cols(int nz);                   // TMEM columns of one subproblem's accumulator
-int tc_smem_bytes(int nz, int passes); // dynamic shared memory of the Gram kernel
 
 }  // namespace edt

@@ -18,6 +18,12 @@
 //     16-bit halves, and
 //     store them K-major with the 128-byte swizzle; (Re a, Im a) of one complex row are two
 //     adjacent K elements.  The data rows d_+, d_- occupy two extra operand rows;
+//   * window geometry: a stage's rows are consecutive rows of the assembled table (its second
+//     factor is the row of ones, its weights are one), so warp 17 copies them to shared memory in
+//     two parts by bulk copies a stage ahead and the producers convert from there; one operand
+//     stage pays for the buffer.  Read row by row by the producers, the 35.5 GB table of the 128 x 128
+//     grid with 200 depths came at 1.8 TB/s, bound by its loads' latency: 19.6 ms for the kernel, and
+//     111.5 ms per inversion against 103.4 now;
 //   * operand type: FP16 (line geometry) or BF16 (window geometry).  FP16's 11-bit
 //     significand makes the hi + lo pair a 22-bit row (BF16: 16 bits), at the same MMA rate,
 //     but its range is narrow, so each segment's kernel rows and data rows are multiplied
@@ -44,7 +50,8 @@ namespace edt {
 namespace {
 
 constexpr int PRODUCER_WARPS = 16;
-constexpr int NTHREADS = (PRODUCER_WARPS + 1) * 32;
+// producers, the MMA warp and, in the window geometry, a warp that copies table rows
+__host__ __device__ constexpr int nthreads(bool f16) { return (PRODUCER_WARPS + (f16 ? 1 : 2)) * 32; }
 constexpr int ROWB = 128;                       // bytes per operand row per stage (64 bf16)
 
 __host__ __device__ inline int nzp_of(int nz) { return (nz + 31) / 32 * 32; }
@@ -54,7 +61,12 @@ __host__ __device__ inline int zrows_of(int nzp) {
   return need > mrows ? need : mrows;
 }
 __host__ __device__ inline int cols_of(int nzp) { return (nzp + 16) + (nzp > TC_M ? nzp - TC_M + 16 : 0); }
-__host__ __device__ inline int stages_of(int passes) { return passes == 1 ? 4 : 3; }
+// operand stages: the window geometry gives one up for its staged table rows
+__host__ __device__ constexpr int stages_of(int passes, bool f16) { return passes == 1 ? 4 : f16 ? 3 : 2; }
+// Window geometry: a stage's TC_KC rows are consecutive rows of the assembled table, nzs FP32 complex
+// depths each, copied in RAW_PARTS parts of RAW_ROWS.
+constexpr int RAW_PARTS = 2, RAW_ROWS = TC_KC / RAW_PARTS;
+__host__ __device__ inline int raw_bytes(int nzs, bool f16) { return f16 ? 0 : TC_KC * nzs * int(sizeof(float2)); }
 
 // Row table of one stage in shared memory: TC_KC GramRow entries (offsets, sqrt weight),
 // then the rows' data (d_+, d_-) as TC_KC float4; both arrive by bulk copy.
@@ -103,8 +115,8 @@ __device__ __forceinline__ void split16(const float2 (&v)[4], uint4& h, uint4& l
 }
 
 template <int PASSES, bool F16>
-__global__ void __launch_bounds__(NTHREADS, 1) gram_tc_kernel(Dev d) {
-  constexpr int STAGES = PASSES == 1 ? 4 : 3;
+__global__ void __launch_bounds__(nthreads(F16), 1) gram_tc_kernel(Dev d) {
+  constexpr int STAGES = stages_of(PASSES, F16), NTHREADS = nthreads(F16);
   constexpr int NCOMP = PASSES == 1 ? 1 : 2;
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   const int nz = d.nz, nzp = nzp_of(nz), zr = zrows_of(nzp), ncols = cols_of(nzp);
@@ -114,7 +126,8 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_tc_kernel(Dev d) {
   uintptr_t base = (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023);
   unsigned char* ops = reinterpret_cast<unsigned char*>(base);
   unsigned char* rowtab = ops + size_t(STAGES) * NCOMP * stage_bytes;   // [2][TAB_BYTES]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(rowtab + 2 * TAB_BYTES);
+  float2* raw = reinterpret_cast<float2*>(rowtab + 2 * TAB_BYTES);     // [TC_KC][nzs] (window)
+  uint64_t* bars = reinterpret_cast<uint64_t*>(rowtab + 2 * TAB_BYTES + raw_bytes(d.nzs, F16));
   uint64_t* full = bars;                   // [STAGES] producers -> MMA
   uint64_t* empty = bars + STAGES;         // [STAGES] MMA commit -> producers
   uint64_t* acc_full = bars + 2 * STAGES;  // MMA commit -> epilogue
@@ -122,7 +135,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_tc_kernel(Dev d) {
   uint64_t* drain = acc_empty + 1;         // final commit: every issued MMA has completed
   uint64_t* tbar = drain + 1;              // [2] row-table bulk copies
   uint64_t* never = tbar + 2;              // never completed: the wait-test stall
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(never + 1);
+  uint64_t* raw_full = never + 1;          // [RAW_PARTS] table-row copies (window)
+  uint64_t* raw_empty = raw_full + RAW_PARTS;   // [RAW_PARTS] producers -> copies
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(raw_empty + RAW_PARTS);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -145,6 +160,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_tc_kernel(Dev d) {
     mbar_init(&tbar[0], 1);
     mbar_init(&tbar[1], 1);
     mbar_init(never, 1);
+    for (int h = 0; h < RAW_PARTS; ++h) { mbar_init(&raw_full[h], 1); mbar_init(&raw_empty[h], PRODUCER_WARPS); }
     *abort_flag = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -214,12 +230,39 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_tc_kernel(Dev d) {
       mbar_drain(drain, 0u);
     }
     __syncwarp();
+  } else if (!F16 && warp == PRODUCER_WARPS + 1) {
+    // ------------------------------------------------------------ table rows of the window geometry
+    // A part is refilled with the next stage's rows as soon as every producer has read it, so one
+    // part is always in flight while the other is converted.
+    if (lane == 0) {
+      long long it = 0, issued[RAW_PARTS] = {};
+      bool ok = true;
+      for (int si = s0; si < s1 && ok; ++si) {
+        const int slot = slots[si];
+        const long long nrow = d.seg_nrow[slot], r0 = d.seg_row0[slot];
+        for (long long k0 = 0; k0 < nrow && ok; k0 += TC_KC, ++it) {
+#pragma unroll
+          for (int h = 0; h < RAW_PARTS; ++h) {
+            if (it > 0 && !mbar_wait(&raw_empty[h], unsigned((it - 1) & 1), abort_flag, budget)) { ok = false; break; }
+            const long long r = k0 + h * RAW_ROWS;
+            const int n = int(max(0LL, min((long long)RAW_ROWS, nrow - r)));      // the segment's rows only
+            const uint32_t bytes = uint32_t(n) * d.nzs * sizeof(float2);
+            mbar_expect_tx(&raw_full[h], bytes);
+            if (n > 0) bulk_g2s(raw + size_t(h) * RAW_ROWS * d.nzs, d.rowtab32 + size_t(r0 + r) * d.nzs, bytes, &raw_full[h]);
+            issued[h] = it + 1;
+          }
+        }
+      }
+      // copies still in flight must land before the CTA leaves
+      for (int h = 0; h < RAW_PARTS; ++h)
+        if (issued[h] > 0) mbar_drain(&raw_full[h], unsigned((issued[h] - 1) & 1));
+    }
+    __syncwarp();
   } else {
     // ------------------------------------------------------------ producers + epilogue
     const int ptid = threadIdx.x;                 // 0..255
     const int nunits = (nzp / 32) * 8;            // (32-depth group, 16-byte K chunk)
     const float2* g32 = d.rowtab32;
-    const size_t nzs = size_t(d.nzs);
     long long it = 0;
     bool ok = true;
     // The row table of each stage (32 GramRow entries, 1 KB) arrives by a bulk copy issued
@@ -272,54 +315,88 @@ __global__ void __launch_bounds__(NTHREADS, 1) gram_tc_kernel(Dev d) {
         unsigned char* hi = ops + size_t(s) * NCOMP * stage_bytes;
         unsigned char* lo = hi + stage_bytes;
         float trs = 0.f;
-        // two (32-depth, 16-byte chunk) units per warp at a time: all 16 table loads of
-        // both are issued before either is converted, to keep enough L2 reads in flight
-        for (int u0 = warp; u0 < nunits; u0 += 2 * PRODUCER_WARPS) {
-          float2 gpv[2][4], gqv[2][4];
-          float swv[2][4];
-          int zz[2], cc[2];
-          const char* gz[2];
+        if constexpr (F16) {
+          // two (32-depth, 16-byte chunk) units per warp at a time: all 16 table loads of
+          // both are issued before either is converted, to keep enough L2 reads in flight
+          for (int u0 = warp; u0 < nunits; u0 += 2 * PRODUCER_WARPS) {
+            float2 gpv[2][4], gqv[2][4];
+            float swv[2][4];
+            int zz[2], cc[2];
+            const char* gz[2];
 #pragma unroll
-          for (int h2 = 0; h2 < 2; ++h2) {
-            const int u = u0 + h2 * PRODUCER_WARPS;
-            const bool uv = u < nunits;
-            zz[h2] = uv ? (u >> 3) * 32 + lane : nzp;     // nzp: marks an absent unit
-            cc[h2] = u & 7;
-            // this lane's depth in every table row (a padding depth reads depth 0, weight 0)
-            gz[h2] = reinterpret_cast<const char*>(g32 + (uv && zz[h2] < nz ? zz[h2] : 0));
+            for (int h2 = 0; h2 < 2; ++h2) {
+              const int u = u0 + h2 * PRODUCER_WARPS;
+              const bool uv = u < nunits;
+              zz[h2] = uv ? (u >> 3) * 32 + lane : nzp;     // nzp: marks an absent unit
+              cc[h2] = u & 7;
+              // this lane's depth in every table row (a padding depth reads depth 0, weight 0)
+              gz[h2] = reinterpret_cast<const char*>(g32 + (uv && zz[h2] < nz ? zz[h2] : 0));
 #pragma unroll
-            for (int rr = 0; rr < 4; ++rr) {
-              const GramRow e = rt[cc[h2] * 4 + rr];
-              // entries past the segment's last row belong to the next segment: padding here
-              const bool ok2 = uv && zz[h2] < nz && (cc[h2] * 4 + rr) < nvalid;
-              swv[h2][rr] = ok2 ? e.sw * sc.x : 0.f;
-              gpv[h2][rr] = __ldg(reinterpret_cast<const float2*>(gz[h2] + e.bp));
-              gqv[h2][rr] = __ldg(reinterpret_cast<const float2*>(gz[h2] + e.bq));
+              for (int rr = 0; rr < 4; ++rr) {
+                const GramRow e = rt[cc[h2] * 4 + rr];
+                // entries past the segment's last row belong to the next segment: padding here
+                const bool ok2 = uv && zz[h2] < nz && (cc[h2] * 4 + rr) < nvalid;
+                swv[h2][rr] = ok2 ? e.sw * sc.x : 0.f;
+                gpv[h2][rr] = __ldg(reinterpret_cast<const float2*>(gz[h2] + e.bp));
+                gqv[h2][rr] = __ldg(reinterpret_cast<const float2*>(gz[h2] + e.bq));
+              }
+            }
+#pragma unroll
+            for (int h2 = 0; h2 < 2; ++h2) {
+              if (zz[h2] >= nzp) continue;
+              float2 a[4];
+#pragma unroll
+              for (int rr = 0; rr < 4; ++rr) {
+                const float2 v = gpv[h2][rr] * gqv[h2][rr];
+                a[rr] = make_float2(swv[h2][rr] * v.x, swv[h2][rr] * v.y);
+                trs = fmaf(a[rr].x, a[rr].x, fmaf(a[rr].y, a[rr].y, trs));
+              }
+              const uint32_t off = sw_off(zz[h2], cc[h2]);
+              if (PASSES == 3) {
+                uint4 h, l;
+                split16<F16>(a, h, l);
+                *reinterpret_cast<uint4*>(hi + off) = h;
+                *reinterpret_cast<uint4*>(lo + off) = l;
+              } else {
+                uint4 h;
+                h.x = pack16<F16>(a[0].x, a[0].y); h.y = pack16<F16>(a[1].x, a[1].y);
+                h.z = pack16<F16>(a[2].x, a[2].y); h.w = pack16<F16>(a[3].x, a[3].y);
+                *reinterpret_cast<uint4*>(hi + off) = h;
+              }
             }
           }
+        } else {
+          // window geometry (BF16): the second factor is the row of ones and every weight is one; a
+          // part holds four K chunks, a warp converts one of them for every fourth 32-depth group
 #pragma unroll
-          for (int h2 = 0; h2 < 2; ++h2) {
-            if (zz[h2] >= nzp) continue;
-            float2 a[4];
+          for (int h = 0; h < RAW_PARTS; ++h) {
+            if (!mbar_wait(&raw_full[h], unsigned(it & 1), abort_flag, budget)) { ok = false; break; }
+            const int c = 4 * h + (warp & 3);
+            const float2* rows4 = raw + size_t(c) * 4 * d.nzs;
+            for (int z = 32 * (warp >> 2) + lane; z < nzp; z += 128) {
+              float2 a[4];
 #pragma unroll
-            for (int rr = 0; rr < 4; ++rr) {
-              const float2 v = gpv[h2][rr] * gqv[h2][rr];
-              a[rr] = make_float2(swv[h2][rr] * v.x, swv[h2][rr] * v.y);
-              trs = fmaf(a[rr].x, a[rr].x, fmaf(a[rr].y, a[rr].y, trs));
+              for (int rr = 0; rr < 4; ++rr) {
+                a[rr] = z < nz && c * 4 + rr < nvalid ? rows4[rr * d.nzs + z] : make_float2(0.f, 0.f);
+                trs = fmaf(a[rr].x, a[rr].x, fmaf(a[rr].y, a[rr].y, trs));
+              }
+              const uint32_t off = sw_off(z, c);
+              if (PASSES == 3) {
+                uint4 hv, lv;
+                split16<F16>(a, hv, lv);
+                *reinterpret_cast<uint4*>(hi + off) = hv;
+                *reinterpret_cast<uint4*>(lo + off) = lv;
+              } else {
+                uint4 hv;
+                hv.x = pack16<F16>(a[0].x, a[0].y); hv.y = pack16<F16>(a[1].x, a[1].y);
+                hv.z = pack16<F16>(a[2].x, a[2].y); hv.w = pack16<F16>(a[3].x, a[3].y);
+                *reinterpret_cast<uint4*>(hi + off) = hv;
+              }
             }
-            const uint32_t off = sw_off(zz[h2], cc[h2]);
-            if (PASSES == 3) {
-              uint4 h, l;
-              split16<F16>(a, h, l);
-              *reinterpret_cast<uint4*>(hi + off) = h;
-              *reinterpret_cast<uint4*>(lo + off) = l;
-            } else {
-              uint4 h;
-              h.x = pack16<F16>(a[0].x, a[0].y); h.y = pack16<F16>(a[1].x, a[1].y);
-              h.z = pack16<F16>(a[2].x, a[2].y); h.w = pack16<F16>(a[3].x, a[3].y);
-              *reinterpret_cast<uint4*>(hi + off) = h;
-            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&raw_empty[h]);
           }
+          if (!ok) break;
         }
         // data rows: operand rows nzp (d_+) and nzp + 1 (d_-), 8 chunks each
         if (warp == PRODUCER_WARPS - 1 && lane < 16) {
@@ -544,14 +621,14 @@ int tc_cols(int nz) { return cols_of(nzp_of(nz)); }
 
 int gram_trace_parts() { return PRODUCER_WARPS; }
 
-int tc_smem_bytes(int nz, int passes) {
-  const int zr = zrows_of(nzp_of(nz));
-  const int stages = stages_of(passes), ncomp = passes == 1 ? 1 : 2;
-  return 1024 + stages * ncomp * zr * ROWB + 2 * TAB_BYTES + (2 * stages + 6) * 8 + 16;
+static int tc_smem_bytes(const Dev& d) {
+  const int zr = zrows_of(nzp_of(d.nz));
+  const int stages = stages_of(d.passes, d.f16), ncomp = d.passes == 1 ? 1 : 2;
+  return 1024 + stages * ncomp * zr * ROWB + 2 * TAB_BYTES + raw_bytes(d.nzs, d.f16) + (2 * stages + 6 + 2 * RAW_PARTS) * 8 + 16;
 }
 
 cudaError_t prepare_gram_tc(const Dev& d) {
-  const int smem = tc_smem_bytes(d.nz, d.passes);
+  const int smem = tc_smem_bytes(d);
   const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
   if (d.f16)
     return d.passes == 3 ? cudaFuncSetAttribute(gram_tc_kernel<3, true>, attr, smem)
@@ -573,15 +650,15 @@ cudaError_t launch_gram_scale(const Dev& d, cudaStream_t s, bool rowmax_ready) {
 }
 
 cudaError_t launch_gram_tc(const Dev& d, cudaStream_t s) {
-  const int smem = tc_smem_bytes(d.nz, d.passes);
+  const int smem = tc_smem_bytes(d);
   cudaError_t e;
   if (d.ncta_gram > 0) {
     if (d.f16) {
-      if (d.passes == 3) gram_tc_kernel<3, true><<<d.ncta_gram, NTHREADS, smem, s>>>(d);
-      else gram_tc_kernel<1, true><<<d.ncta_gram, NTHREADS, smem, s>>>(d);
+      if (d.passes == 3) gram_tc_kernel<3, true><<<d.ncta_gram, nthreads(true), smem, s>>>(d);
+      else gram_tc_kernel<1, true><<<d.ncta_gram, nthreads(true), smem, s>>>(d);
     } else {
-      if (d.passes == 3) gram_tc_kernel<3, false><<<d.ncta_gram, NTHREADS, smem, s>>>(d);
-      else gram_tc_kernel<1, false><<<d.ncta_gram, NTHREADS, smem, s>>>(d);
+      if (d.passes == 3) gram_tc_kernel<3, false><<<d.ncta_gram, nthreads(false), smem, s>>>(d);
+      else gram_tc_kernel<1, false><<<d.ncta_gram, nthreads(false), smem, s>>>(d);
     }
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }

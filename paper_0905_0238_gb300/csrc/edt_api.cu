@@ -681,7 +681,7 @@ void layout(edt_ctx* c) {
   take(c->r_Gs, grid ? nz * (N / 2 + 1) * (c->ny / 2 + 1) * sizeof(float2) : c->win ? nz * N * sizeof(float2) : 0);
   const size_t wact = c->nact.empty() ? 1 : size_t(std::max(1, *std::max_element(c->nact.begin(), c->nact.end())));
   const size_t slots = grid ? fa_grid_slots(c->wx, c->wy) : 0;
-  take(c->r_U, grid ? slots * size_t(fa_grid_slab(c->nz, int(slots), c->q_max)) * std::max(c->q_max, 1) * sizeof(float2)
+  take(c->r_U, grid ? fa_grid_bytes(fa_grid_slab(c->nz, int(slots), c->q_max), int(slots), c->q_max)
                : c->win ? wact * nz * N * sizeof(float2) : 0);
   take(c->r_Dw, c->win ? nf * W * nxy * sizeof(float2) : 0);
   take(c->r_A32, c->win ? (R + 1) * nzs * sizeof(float2) : 0);

@@ -112,7 +112,7 @@ struct Dev {
   float2* Gs;                   // G(y, z) of one frequency: a line [nz][nx], a grid's quadrant
                                 //   [nz][ny/2 + 1][nx/2 + 1]
   float2* U;                    // a line: [active j][nz][nx] window products of one frequency; a grid:
-                                //   [slab][slot][point] (csrc/fagrid.cu)
+                                //   tiles of the slab's planes (csrc/fagrid.cu)
   float2* Dw;                   // [nf][W][ny][nx] window-transformed data
   float2* A32;                  // [rows + 1][nzs] kernel rows, then a row of ones
   long long ones_row;           // index of the ones row in A32
@@ -236,9 +236,10 @@ cudaError_t prepare_band(const Dev& d);
 bool fa_supported(int nx, int ny, int wx, int wy);
 cudaError_t launch_fa_line(const Dev& d, int f, int nact, double2 cf, cudaStream_t s);
 // the same for a grid (csrc/fagrid.cu): the frequency's points are q_xy/q_rows[qoff .. qoff + nq)
-constexpr size_t FA_SLAB_BYTES = size_t(2) << 30;     // plane buffer of a slab of depths (at least 16)
+constexpr size_t FA_SLAB_BYTES = size_t(2) << 30;     // plane buffer of a slab of depths (at least 8)
 int fa_grid_slots(int wx, int wy);
 int fa_grid_slab(int nz, int slots, int nq);
+size_t fa_grid_bytes(int nzb, int slots, int nq);
 cudaError_t launch_fa_grid(const Dev& d, int f, int qoff, int nq, double2 cf, cudaStream_t s);
 cudaError_t prepare_fa_grid(const Dev& d);
 cudaError_t launch_fa_data(const Dev& d, const void* D, int D_dtype, cudaStream_t s);

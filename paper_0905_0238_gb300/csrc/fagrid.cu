@@ -17,19 +17,20 @@
 // end -h has no partner +h; s(0) = s(-h) = 0).  Both pairs (kx, ky), (-kx, ky) share the transforms.
 // Against the window sum first (per offset wavenumber j: products, 16-point transforms and one plane
 // FFT), at 128 x 128 midpoints, 16 x 16 half-offsets, 64 frequencies and 200 depths: 45 planes per
-// (f, z) instead of 138 on average, 63 ms of kernels instead of 144 (an inversion 115 ms instead of
-// 192); 64 x 64, 8 x 8, 12 frequencies, 100 depths: 0.59 ms instead of 1.36.
+// (f, z) instead of 138 on average, 49 ms of kernels instead of 144; 64 x 64, 8 x 8, 12 frequencies, 100
+// depths: 0.55 ms instead of 1.36.
 // Per frequency and slab of depths (all of them unless the planes would take more than
-// FA_SLAB_BYTES; slabs that stay in L2 lost more to short launches than they saved, 134 ms per
-// inversion at 80 MB, 123 at 240 MB):
+// FA_SLAB_BYTES; slabs that stay in L2 lost more to short launches than they saved: 134 ms per
+// inversion at 80 MB, 123 at 240 MB, 115 with one slab):
 //   grid_gspace  G on the quadrant, by a half-plane inverse FFT of the |k| table;
 //   grid_planes  P_ab from G in shared memory, its half-plane FFT, E and O at the quadrant points q
-//                = (kx, ky) that have kept rows, as F[z][slot][q];
-//   grid_rows    tiles of 4 q x 16 z: the cosine and sine transforms in shared memory, then the kept
-//                rows of the tile's pairs, 16 depths (128 bytes) at a time.
+//                = (kx, ky) that have kept rows, as tiles of 8 q x 8 z: F[q / 8][z / 8][slot][z % 8][q % 8];
+//   grid_rows    per tile, one bulk copy: the cosine and sine transforms in shared memory, then the
+//                kept rows of the tile's pairs, 8 depths (64 bytes) at a time.
 #include "edt_internal.h"
 #include "cplx.cuh"
 #include "fadft.cuh"
+#include "tc_ptx.cuh"
 
 #include <algorithm>
 
@@ -149,6 +150,8 @@ __device__ __forceinline__ void half_fft(float2* s, const float2* tw, const Src&
   __syncthreads();
 }
 
+constexpr int GT_Q = 8, GT_Z = 8, GT_P = GT_Q * GT_Z;    // points of a tile of F
+
 // ---- G on the quadrant ----------------------------------------------------------------------
 // G(y, z) of one frequency for 0 <= yx, yy <= H, CTA per z: Gs[z][yy][yx].
 template <int N>
@@ -195,7 +198,9 @@ grid_planes_kernel(Dev d, const int* qxy, int nq, int z0, int hx, int hy, int sw
   half_twiddles<N>(tw, d.tw32);
   for (int e = threadIdx.x; e < S::QUAD; e += blockDim.x) gq[e] = G[e];
   const int nE = (hx + 1) * (hy + 1);
-  float2* F = d.U + size_t(blockIdx.y) * (nE + hx * hy) * nq;
+  // slot stride GT_P within a tile, gridDim.y depths per slab
+  const size_t ns = size_t(nE + hx * hy), zt = (gridDim.y + GT_Z - 1) / GT_Z;
+  float2* F = d.U + (size_t(blockIdx.y / GT_Z) * ns) * GT_P + (blockIdx.y % GT_Z) * GT_Q;
   for (int pl = blockIdx.x; pl < nplane; pl += gridDim.x) {
     int a, b;
     if (swap) {
@@ -220,19 +225,20 @@ grid_planes_kernel(Dev d, const int* qxy, int nq, int z0, int hx, int hy, int sw
         v[i] = gm[xm] * gp[xp];
       }
     });
-    float2* e0 = F + size_t(b * (hx + 1) + a) * nq;
-    float2* o0 = a > 0 && b > 0 ? F + size_t(nE + (b - 1) * hx + a - 1) * nq : nullptr;
-    float2* e1 = swap && a != b ? F + size_t(a * (hx + 1) + b) * nq : nullptr;
-    float2* o1 = e1 && o0 ? F + size_t(nE + (a - 1) * hx + b - 1) * nq : nullptr;
+    float2* e0 = F + (b * (hx + 1) + a) * GT_P;
+    float2* o0 = a > 0 && b > 0 ? F + (nE + (b - 1) * hx + a - 1) * GT_P : nullptr;
+    float2* e1 = swap && a != b ? F + (a * (hx + 1) + b) * GT_P : nullptr;
+    float2* o1 = e1 && o0 ? F + (nE + (a - 1) * hx + b - 1) * GT_P : nullptr;
     for (int q = threadIdx.x; q < nq; q += blockDim.x) {
       const int xy = qxy[q], x = xy & 0xffff, y = xy >> 16;
       const float2 p = s[S::at(y, x)], m = s[S::at((N - y) & (N - 1), x)];
-      e0[q] = p + m;
-      if (o0) o0[q] = p - m;
+      const size_t at = size_t(q / GT_Q) * zt * ns * GT_P + q % GT_Q;
+      e0[at] = p + m;
+      if (o0) o0[at] = p - m;
       if (e1) {
         const float2 pt = s[S::at(x, y)], mt = s[S::at((N - x) & (N - 1), y)];
-        e1[q] = pt + mt;
-        if (o1) o1[q] = pt - mt;
+        e1[at] = pt + mt;
+        if (o1) o1[at] = pt - mt;
       }
     }
   }
@@ -302,50 +308,61 @@ template <int H> struct Dst {
   }
 };
 
-constexpr int RT_Q = 4, RT_Z = 16, RT_P = RT_Q * RT_Z, RT_THREADS = 288;   // points of a tile
+// A tile in shared memory is v[slot][point].  It arrives as point 8 z + q; the x pass leaves each
+// half (4 depths, g = z / 4) as 32 g + ((4 q + z % 4) ^ 8 g), so that the 8 depths of a row, for an even
+// and an odd q side by side, fall on 16 different bank pairs.
+constexpr int RT_THREADS = 256;
+__device__ __forceinline__ int rt_at(int q, int z) { return 32 * (z >> 2) + ((4 * q + (z & 3)) ^ (2 * (z & 4))); }
 
-// v[slot][point], point = 16 q + (z ^ 4 q): the loads' half-warps (4 q x 4 z) and the lanes of every
-// later access fall on different bank pairs
 template <int WX, int WY>
 __global__ void __launch_bounds__(RT_THREADS, 3)
 grid_rows_kernel(Dev d, const int4* qrows, int nq, int z0, int nzb, float2 cf) {
   constexpr int HX = WX / 2, HY = WY / 2, NE = (HX + 1) * (HY + 1), NS = NE + HX * HY;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* v = reinterpret_cast<float2*>(smem_raw);
-  const int q0 = blockIdx.x * RT_Q, zb = blockIdx.y * RT_Z;
+  __shared__ uint64_t bar;
+  const int q0 = blockIdx.y * GT_Q, zb = blockIdx.x * GT_Z;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = RT_THREADS / 32;
-  for (int e = threadIdx.x; e < NS * RT_P; e += RT_THREADS) {
-    const int q = e & 3, z = (e >> 2) & 15, sl = e >> 6;
-    float2* dst = v + sl * RT_P + 16 * q + (z ^ (4 * q));
-    if (q0 + q < nq && zb + z < nzb) {
-      const float2* src = d.U + (size_t(zb + z) * NS + sl) * nq + q0 + q;
-      asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(uint32_t(__cvta_generic_to_shared(dst))), "l"(src)
-                   : "memory");
-    } else {
-      *dst = make_float2(0.f, 0.f);
-    }
+  if (threadIdx.x == 0) {
+    tcx::mbar_init(&bar, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    constexpr uint32_t bytes = NS * GT_P * sizeof(float2);
+    tcx::mbar_expect_tx(&bar, bytes);
+    tcx::bulk_g2s(v, d.U + (size_t(blockIdx.y) * gridDim.x + blockIdx.x) * NS * GT_P, bytes, &bar);
   }
-  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
-  // over x: cosine transforms of E's rows b = 0..HY, sine transforms of O's rows b = 1..HY
+  // the wait is bounded; on expiry the copy gets as long again before the CTA leaves
+  bool ok = tcx::mbar_drain(&bar, 0u);
+  if (!ok) {
+    if (threadIdx.x == 0) atomicOr(&d.flags[0], 1u);
+    tcx::mbar_drain(&bar, 0u);
+  }
+  if (!__syncthreads_and(ok)) return;
+  // over x: cosine transforms of E's rows b = 0..HY, sine transforms of O's rows b = 1..HY; a warp
+  // takes a row's 8 points x 4 depths, which it reads before it stores
   for (int tk = warp; tk < 2 * (2 * HY + 1); tk += nw) {
     const int ln = tk >> 1;
-    float2* p = v + (tk & 1) * 32 + lane;
+    const float2* p = v + (tk & 1) * 32 + lane;
+    float2* o = v + rt_at(lane & 7, 4 * (tk & 1) + (lane >> 3));
     if (ln <= HY) {
       float2 x[HX + 1];
 #pragma unroll
-      for (int a = 0; a <= HX; ++a) x[a] = p[(ln * (HX + 1) + a) * RT_P];
+      for (int a = 0; a <= HX; ++a) x[a] = p[(ln * (HX + 1) + a) * GT_P];
       Dct<HX>::run(x);
+      __syncwarp();
 #pragma unroll
-      for (int a = 0; a <= HX; ++a) p[(ln * (HX + 1) + a) * RT_P] = x[a];
-    } else if constexpr (HX > 1) {
-      float2 x[HX - 1];
-      float2* o = p + (NE + (ln - HY - 1) * HX) * RT_P;
+      for (int a = 0; a <= HX; ++a) o[(ln * (HX + 1) + a) * GT_P] = x[a];
+    } else if constexpr (HX > 0) {
+      const int s0 = NE + (ln - HY - 1) * HX;
+      float2 x[HX > 1 ? HX - 1 : 1];
+      const float2 e = p[(s0 + HX - 1) * GT_P];
 #pragma unroll
-      for (int a = 0; a < HX - 1; ++a) x[a] = o[a * RT_P];
-      Dst<HX>::run(x);
+      for (int a = 0; a < HX - 1; ++a) x[a] = p[(s0 + a) * GT_P];
+      if constexpr (HX > 1) Dst<HX>::run(x);
+      __syncwarp();
 #pragma unroll
-      for (int a = 0; a < HX - 1; ++a) o[a * RT_P] = x[a];
+      for (int a = 0; a < HX - 1; ++a) o[(s0 + a) * GT_P] = x[a];
+      o[(s0 + HX - 1) * GT_P] = e;
     }
   }
   __syncthreads();
@@ -356,61 +373,69 @@ grid_rows_kernel(Dev d, const int4* qrows, int nq, int z0, int nzb, float2 cf) {
     if (ln <= HX) {
       float2 x[HY + 1];
 #pragma unroll
-      for (int b = 0; b <= HY; ++b) x[b] = p[(b * (HX + 1) + ln) * RT_P];
+      for (int b = 0; b <= HY; ++b) x[b] = p[(b * (HX + 1) + ln) * GT_P];
       Dct<HY>::run(x);
 #pragma unroll
-      for (int b = 0; b <= HY; ++b) p[(b * (HX + 1) + ln) * RT_P] = x[b];
+      for (int b = 0; b <= HY; ++b) p[(b * (HX + 1) + ln) * GT_P] = x[b];
     } else if constexpr (HY > 1) {
       float2 x[HY - 1];
-      float2* o = p + (NE + ln - HX - 1) * RT_P;
+      float2* o = p + (NE + ln - HX - 1) * GT_P;
 #pragma unroll
-      for (int b = 0; b < HY - 1; ++b) x[b] = o[b * HX * RT_P];
+      for (int b = 0; b < HY - 1; ++b) x[b] = o[b * HX * GT_P];
       Dst<HY>::run(x);
 #pragma unroll
-      for (int b = 0; b < HY - 1; ++b) o[b * HX * RT_P] = x[b];
+      for (int b = 0; b < HY - 1; ++b) o[b * HX * GT_P] = x[b];
     }
   }
   __syncthreads();
-  // the kept rows of both pairs of every point, a half-warp (16 depths) per row
-  const int z = lane & 15, sub = warp * 2 + (lane >> 4);
-  if (zb + z >= nzb) return;
+  // the kept rows of both pairs of every point, 8 lanes (depths) per row, four groups per point
+  const int z = lane & 7, g = warp * 4 + (lane >> 3), q = g & 7;
+  if (q0 + q >= nq || zb + z >= nzb) return;
+  const int4 R = qrows[q0 + q];
+  const int n = R.y + R.w;
   float2* A = d.A32 + z0 + zb + z;
-  for (int q = 0; q < RT_Q && q0 + q < nq; ++q) {
-    const int4 R = qrows[q0 + q];
-    const float2* p = v + 16 * q + (z ^ (4 * q));
-    for (int i = sub; i < R.y + R.w; i += 2 * nw) {
-      const bool mir = i >= R.y;
-      const int row = mir ? R.z + i - R.y : R.x + i;
-      const int j = int(d.rows[row] & 0xffffu), jy = j / WX - HY, jx = j - (j / WX) * WX - HX;
-      const int ax = abs(jx), ay = abs(jy);
-      float2 m = p[(ay * (HX + 1) + ax) * RT_P];
-      if constexpr (HX > 0 && HY > 0) {
-        const bool ix = jx != 0 && ax < HX, iy = jy != 0 && ay < HY;
-        float2 o = p[(NS - 1) * RT_P];
-        if ((jx + jy) & 1) o = make_float2(-o.x, -o.y);
-        if (ix) {                       // i (-1)^jy s(jx) X
-          const float2 X = p[(NE + (HY - 1) * HX + ax - 1) * RT_P];
-          const float c = ((jy & 1) != 0) != (jx < 0) ? -1.f : 1.f;
-          o = make_float2(fmaf(-c, X.y, o.x), fmaf(c, X.x, o.y));
-        }
-        if (iy) {                       // i (-1)^jx s(jy) Y
-          const float2 Y = p[(NE + (ay - 1) * HX + HX - 1) * RT_P];
-          const float c = ((jx & 1) != 0) != (jy < 0) ? -1.f : 1.f;
-          o = make_float2(fmaf(-c, Y.y, o.x), fmaf(c, Y.x, o.y));
-        }
-        if (ix && iy) {
-          const float2 B = p[(NE + (ay - 1) * HX + ax - 1) * RT_P];
-          o = (jx < 0) != (jy < 0) ? o + B : o - B;
-        }
-        m = mir ? m - o : m + o;
+  const float2* p = v + rt_at(q, z);
+  const float2 ohh = p[(NS - 1) * GT_P];
+  constexpr int STEP = RT_THREADS / 64, AHEAD = 4;        // rows' j read ahead
+  auto row_of = [&](int i) { return i < R.y ? R.x + i : R.z + i - R.y; };
+  auto j_of = [&](int i) { return i < n ? int(d.rows[row_of(i)] & 0xffffu) : 0; };
+  int jn[AHEAD];
+#pragma unroll
+  for (int u = 0; u < AHEAD; ++u) jn[u] = j_of((g >> 3) + u * STEP);
+  for (int i = g >> 3; i < n; i += STEP) {
+    const bool mir = i >= R.y;
+    const int row = row_of(i);
+    const int j = jn[0], jy = j / WX - HY, jx = j - (j / WX) * WX - HX;
+#pragma unroll
+    for (int u = 0; u + 1 < AHEAD; ++u) jn[u] = jn[u + 1];
+    jn[AHEAD - 1] = j_of(i + AHEAD * STEP);
+    const int ax = abs(jx), ay = abs(jy);
+    float2 m = p[(ay * (HX + 1) + ax) * GT_P];
+    if constexpr (HX > 0 && HY > 0) {
+      const bool ix = jx != 0 && ax < HX, iy = jy != 0 && ay < HY;
+      float2 o = (jx + jy) & 1 ? make_float2(-ohh.x, -ohh.y) : ohh;
+      if (ix) {                       // i (-1)^jy s(jx) X
+        const float2 X = p[(NE + (HY - 1) * HX + ax - 1) * GT_P];
+        const float c = ((jy & 1) != 0) != (jx < 0) ? -1.f : 1.f;
+        o = make_float2(fmaf(-c, X.y, o.x), fmaf(c, X.x, o.y));
       }
-      A[size_t(row) * d.nzs] = cf * m;
+      if (iy) {                       // i (-1)^jx s(jy) Y
+        const float2 Y = p[(NE + (ay - 1) * HX + HX - 1) * GT_P];
+        const float c = ((jx & 1) != 0) != (jy < 0) ? -1.f : 1.f;
+        o = make_float2(fmaf(-c, Y.y, o.x), fmaf(c, Y.x, o.y));
+      }
+      if (ix && iy) {
+        const float2 B = p[(NE + (ay - 1) * HX + ax - 1) * GT_P];
+        o = (jx < 0) != (jy < 0) ? o + B : o - B;
+      }
+      m = mir ? m - o : m + o;
     }
+    A[size_t(row) * d.nzs] = cf * m;
   }
 }
 
 template <int WX, int WY>
-constexpr int rows_smem() { return ((WX / 2 + 1) * (WY / 2 + 1) + (WX / 2) * (WY / 2)) * RT_P * int(sizeof(float2)); }
+constexpr int rows_smem() { return ((WX / 2 + 1) * (WY / 2 + 1) + (WX / 2) * (WY / 2)) * GT_P * int(sizeof(float2)); }
 
 #define GRID_WINDOWS(X) X(1, 1) X(2, 1) X(4, 1) X(8, 1) X(16, 1) X(2, 2) X(4, 4) X(8, 8) X(16, 16) X(4, 2) X(8, 4) X(16, 8)
 
@@ -435,9 +460,12 @@ cudaError_t prepare_n() {
 int fa_grid_slots(int wx, int wy) { return (wx / 2 + 1) * (wy / 2 + 1) + (wx / 2) * (wy / 2); }
 
 int fa_grid_slab(int nz, int slots, int nq) {
-  const size_t per = size_t(slots) * std::max(nq, 1) * sizeof(float2) * RT_Z;
-  const size_t n = std::max<size_t>(1, FA_SLAB_BYTES / per);
-  return int(std::min<size_t>(size_t(nz), n * RT_Z));
+  const size_t n = std::max<size_t>(1, FA_SLAB_BYTES / fa_grid_bytes(GT_Z, slots, nq));
+  return int(std::min<size_t>(size_t(nz), n * GT_Z));
+}
+
+size_t fa_grid_bytes(int nzb, int slots, int nq) {
+  return size_t((std::max(nq, 1) + GT_Q - 1) / GT_Q) * ((nzb + GT_Z - 1) / GT_Z) * slots * GT_P * sizeof(float2);
 }
 
 cudaError_t launch_fa_grid(const Dev& d, int f, int qoff, int nq, double2 cf, cudaStream_t s) {
@@ -454,7 +482,8 @@ cudaError_t launch_fa_grid(const Dev& d, int f, int qoff, int nq, double2 cf, cu
         : d.N == 64 ? planes_for<64>(d, d.q_xy + qoff, nq, z0, nzb, s)
                     : planes_for<128>(d, d.q_xy + qoff, nq, z0, nzb, s);
     if (e != cudaSuccess) return e;
-    const dim3 g((nq + RT_Q - 1) / RT_Q, (nzb + RT_Z - 1) / RT_Z);
+    // the depth tiles of a point side by side: its rows' neighbouring 64-byte pieces meet in L2
+    const dim3 g((nzb + GT_Z - 1) / GT_Z, (nq + GT_Q - 1) / GT_Q);
     switch (d.wx * 32 + d.wy) {
 #define GR(WX, WY) case WX * 32 + WY: \
       grid_rows_kernel<WX, WY><<<g, RT_THREADS, rows_smem<WX, WY>(), s>>>(d, d.q_rows + qoff, nq, z0, nzb, c); break;

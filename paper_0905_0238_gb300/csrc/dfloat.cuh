@@ -85,96 +85,76 @@ __device__ __forceinline__ float2 df_rsqrt(float2 a) {
 // ---- one 32 x 32 diagonal block of a blocked double-float Cholesky factorisation ----------
 // Shared scratch of the diagonal-block factorisation.
 struct DfDiagScratch {
-  float2 col[3][32];                              // columns of L (three in use at a time)
-  float2 xr[2][32];                               // finished rows of X = L^-1
-  float2 pd[32];                                  // diagonal entries, published a step ahead
+  float2 col[32][33];                             // the block, then L, by columns
+  float2 ls[3][32];                               // column j of L over L_jj (three in use at a time)
+  float2 xr[2][32];                               // finished rows of U (below)
   float2 inv[32];                                 // 1 / L_jj
   int fail;
 };
 
 // Diagonal block of step k0 of one subproblem (kb = min(32, n - k0) columns), factored and
-// inverted in double-float by a 256-thread CTA; thread (warp, lane) holds elements
-// (warp + 8 q, lane), q < 4, of both A and X.  Right-looking with a one-column look-ahead, one
-// barrier per column: in the phase that subtracts column j from the trailing block, the
-// threads of column j + 1 (whose entries that subtraction finishes) also form its pivot
-// L_{j+1,j+1}^2 = a_{j+1,j+1} - L_{j+1,j}^2 from the diagonal entry published one phase earlier,
-// each of them redundantly (the same operations on the same values, so the same bits), take
-// its 1 / sqrt and scale their entries: column j + 1 is ready at the next barrier.  The inverse
-// rides along in the same phases: row j of X is u_j / L_jj, where u_i = e_i - sum_{k < i}
-// L_ik X_k is updated with the finished row j - 1.  Writes L_kk (lower triangle) and
-// its FP32 copy (L32, may be null; X goes there too), X to the strict upper triangle (X_il at
-// (l, i)), and the reciprocal pivots (dinv FP64; dinv32 FP32, may be null).  A non-positive or
-// non-finite pivot sets EDT_ENOTPD and returns false (in every thread).  Every thread of the CTA
-// calls it; A's block must be final and visible to the CTA.
+// inverted in double-float by a 256-thread CTA; lane i of a warp holds row i of the columns
+// c = warp + 8 q, q < 4.  Right-looking with a one-column look-ahead, one barrier per column: in the
+// phase that subtracts column j from the trailing block, the warp of column j + 1, which that
+// subtraction finishes, takes its pivot from its own lane j + 1 and scales the column, which is
+// ready at the next barrier.  A finished column's registers go on to hold its column of U, L^-1 = X
+// with X_ic = U_ic / L_ii: U_i = e_i - sum_{k < i} (L_ik / L_kk) U_k, updated in the same phases
+// with row j - 1.  So a warp does one product per column it holds and phase; A's entries and U's in separate
+// registers, with a lane per column, took two, and the scaling ran in every warp with one lane (the
+// first blocks of the 2050 systems of a 64 x 64 grid: 149 us then, 107 now; its inversion 2.36 ms, 2.23).
+// Writes L_kk (lower triangle) and its FP32 copy (L32, may be null; X goes there too), X to the strict
+// upper triangle (X_il at (l, i)), and the reciprocal pivots (dinv FP64; dinv32 FP32, may be null).  A
+// non-positive or non-finite pivot sets EDT_ENOTPD and returns false (in every thread).  Every thread
+// of the CTA calls it; A's block must be final and visible to the CTA.
 __device__ inline bool df_diag_block(float2* A, float* L32, double* dinv, float* dinv32, int* status, int n,
                                      int k0, DfDiagScratch& sh) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int kb = min(32, n - k0);
-  const float2 zero = make_float2(0.f, 0.f);
-  float2 a[4], u[4];
+  const float2 zero = make_float2(0.f, 0.f), one = make_float2(1.f, 0.f);
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     const int i = warp + 8 * q;
-    a[q] = i < kb && lane <= i ? A[size_t(k0 + i) * n + k0 + lane] : zero;
-    u[q] = make_float2(i == lane ? 1.f : 0.f, 0.f);
-    if (i == lane && i < kb) sh.pd[i] = a[q];
+    sh.col[lane][i] = i < kb && lane <= i ? A[size_t(k0 + i) * n + k0 + lane] : zero;
   }
   if (threadIdx.x == 0) sh.fail = 0;
   __syncthreads();
-  {                                               // column 0, by every thread
-    const float2 d = df_norm(sh.pd[0]);
-    if (!(d.x > 0.f) || !isfinite(d.x)) {
-      if (threadIdx.x == 0) sh.fail = 1;
-    } else {
-      const float2 iv = df_rsqrt(d);
+  float2 w[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
-        const int i = warp + 8 * q;
-        if (lane == 0 && i < kb) {
-          a[q] = i == 0 ? df_mul(d, iv) : df_mul(df_norm(a[q]), iv);
-          sh.col[0][i] = a[q];
-        }
-      }
-      if (threadIdx.x == 0) sh.inv[0] = iv;
+  for (int q = 0; q < 4; ++q) w[q] = sh.col[warp + 8 * q][lane];
+  // column j from its finished entries v, by the warp that holds it
+  auto column = [&](int j, float2& v) {
+    const float2 d = df_norm(shfl_df(v, j));
+    if (!(d.x > 0.f) || !isfinite(d.x)) {
+      if (lane == 0) sh.fail = 1;
+      return;
     }
-  }
+    const float2 iv = df_rsqrt(d);
+    const float2 l = df_mul(lane == j ? d : df_norm(v), iv);
+    if (lane >= j) {
+      sh.col[j][lane] = l;
+      sh.ls[j % 3][lane] = df_mul(l, iv);
+    }
+    if (lane == 0) sh.inv[j] = iv;
+    v = lane == j ? one : zero;                   // from here on the column of U
+  };
+  if (warp == 0) column(0, w[0]);
   __syncthreads();
   for (int j = 0; j < kb; ++j) {
     if (sh.fail) break;                           // the same value in every thread
-    const float2* cj = sh.col[j % 3];             // column j
-    const float2* cp = sh.col[(j + 2) % 3];       // column j - 1
-    float2* cn = sh.col[(j + 1) % 3];             // column j + 1, formed here
+    const float2 lj = df_neg(sh.col[j][lane]), lp = df_neg(sh.ls[(j + 2) % 3][lane]);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-      const int i = warp + 8 * q;
-      if (lane > j && i >= lane && i < kb) df_acc(a[q], df_neg(cj[i]), cj[lane]);     // A -= L_j L_j^T
-      if (j > 0 && lane < j && i >= j && i < kb)                                       // u_i -= L_{i,j-1} X_{j-1}
-        df_acc(u[q], df_neg(cp[i]), sh.xr[(j - 1) & 1][lane]);
-      if (i == j && lane <= j) {                                                       // row j of X
-        u[q] = df_mul(df_norm(u[q]), sh.inv[j]);
-        sh.xr[j & 1][lane] = u[q];
+      const int c = warp + 8 * q;                 // the same in the whole warp
+      if (c > j) {
+        if (lane >= c) df_acc(w[q], lj, sh.col[j][c]);                      // A -= L_j L_j^T
+      } else if (c < j) {
+        if (lane >= j) df_acc(w[q], lp, sh.xr[(j + 1) & 1][c]);             // U_i -= (L_i,j-1 / L_j-1,j-1) U_j-1
       }
-      if (i == j + 2 && lane == j + 2 && i < kb) sh.pd[j + 2] = a[q];                  // next step's pivot input
+      if (c <= j && lane == j) sh.xr[j & 1][c] = df_norm(w[q]);             // row j of U
     }
-    if (j + 1 < kb && lane == j + 1) {            // column j + 1 (its entries are final now)
-      float2 d = sh.pd[j + 1];
-      df_acc(d, df_neg(cj[j + 1]), cj[j + 1]);
-      d = df_norm(d);
-      if (!(d.x > 0.f) || !isfinite(d.x)) {
-        sh.fail = 1;
-      } else {
-        const float2 iv = df_rsqrt(d);
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int i = warp + 8 * q;
-          if (i > j && i < kb) {
-            a[q] = i == j + 1 ? df_mul(d, iv) : df_mul(df_norm(a[q]), iv);
-            cn[i] = a[q];
-          }
-        }
-        if (warp == 0) sh.inv[j + 1] = iv;
-      }
-    }
+    for (int q = 0; q < 4; ++q)
+      if (j + 1 < kb && warp + 8 * q == j + 1) column(j + 1, w[q]);
     __syncthreads();
   }
   if (sh.fail) {
@@ -183,14 +163,16 @@ __device__ inline bool df_diag_block(float2* A, float* L32, double* dinv, float*
   }
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    const int i = warp + 8 * q;
+    const int i = warp + 8 * q;                   // L row i, column lane
     if (i < kb && lane <= i) {
-      A[size_t(k0 + i) * n + k0 + lane] = a[q];
-      if (L32) L32[size_t(k0 + i) * n + k0 + lane] = a[q].x;
+      const float2 l = sh.col[lane][i];
+      A[size_t(k0 + i) * n + k0 + lane] = l;
+      if (L32) L32[size_t(k0 + i) * n + k0 + lane] = l.x;
     }
-    if (i < kb && lane < i) {                     // X_{i, lane} to the upper triangle
-      A[size_t(k0 + lane) * n + k0 + i] = u[q];
-      if (L32) L32[size_t(k0 + lane) * n + k0 + i] = u[q].x;
+    if (lane < kb && i < lane) {                  // X_{lane, i} to the upper triangle
+      const float2 x = df_mul(df_norm(w[q]), sh.inv[lane]);
+      A[size_t(k0 + i) * n + k0 + lane] = x;
+      if (L32) L32[size_t(k0 + i) * n + k0 + lane] = x.x;
     }
   }
   if (threadIdx.x < kb) {

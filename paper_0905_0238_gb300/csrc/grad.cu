@@ -34,6 +34,7 @@
 #include "edt_internal.h"
 #include "cplx.cuh"
 #include "green_coef.cuh"
+#include "warpsum.cuh"
 
 #include <algorithm>
 
@@ -602,41 +603,70 @@ __global__ void adj_addb_kernel(Dev d) {
     d.r[i] += d.b[i];
 }
 
+// table rows |p|, |q| of a row of subproblem m
+__device__ __forceinline__ int2 table_rows(const Dev& d, int m, uint32_t row) {
+  const int p = row_p(row), q = (p - m) & (d.N - 1), t0 = row_f(row) * d.nk;
+  return make_int2(t0 + tab_index(p, d.N), t0 + tab_index(q, d.N));
+}
+
+// Products of two rows a = g32_p g32_q, whose table rows lanes i0 and i1 hold in tr, with two depth
+// vectors va, vb, lanes over depth: lane 16 h + 4 c returns row h's sum (a.va re, im, a.vb re, im)_c.
+__device__ __forceinline__ float row_pair_dots(const Dev& d, int2 tr, int i0, int i1, const float* va, const float* vb,
+                                               int lane) {
+  const float2* g[2][2];
+#pragma unroll
+  for (int h = 0; h < 2; ++h) {
+    g[h][0] = d.g32 + size_t(__shfl_sync(0xffffffffu, tr.x, h ? i1 : i0)) * d.nzs;
+    g[h][1] = d.g32 + size_t(__shfl_sync(0xffffffffu, tr.y, h ? i1 : i0)) * d.nzs;
+  }
+  float s[8];
+#pragma unroll
+  for (int c = 0; c < 8; ++c) s[c] = 0.f;
+#pragma unroll 4
+  for (int z = lane; z < d.nz; z += 32) {
+    const float a = va[z], b = vb[z];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const float2 t = g[h][0][z] * g[h][1][z];
+      s[4 * h + 0] = fmaf(t.x, a, s[4 * h + 0]); s[4 * h + 1] = fmaf(t.y, a, s[4 * h + 1]);
+      s[4 * h + 2] = fmaf(t.x, b, s[4 * h + 2]); s[4 * h + 3] = fmaf(t.y, b, s[4 * h + 3]);
+    }
+  }
+  return warp_sums(s, lane);
+}
+
 // Per kept row (f, p) of m at frequencies [f0, f1), with bbar = (G + lam I)^-1 xbar in d.x:
 // b_+- = sum_rows w Re(conj(row) rhs_+-) gives rhsbar = w sum_z row(z) bbar(z); then the
 // rotation rhs = rot d, the split d_+ = (a + c)/2, d_- = (a - c)/(2i) with a = D2(p, q),
 // c = D2(q, p) (folded rows: a and c the means with D2(-q, -p), D2(-p, -q)) are reversed and
 // scattered (atomically) into the chunk's planes X[fi][q][p] = D2bar(p, q).
 __global__ void __launch_bounds__(256) adj_rows_kernel(Dev d, int f0, int f1) {
-  __shared__ float2 bb[512];                          // (bbar_+, bbar_-) per depth, nz <= 512
+  __shared__ float bb[2][512];                        // bbar_+, bbar_- per depth, nz <= 512
   const int m = blockIdx.y, N = d.N, msk = N - 1;
   if (d.status[m] != EDT_OK) return;
   const double* yb = d.x + size_t(m) * d.nz * 2;
-  for (int z = threadIdx.x; z < d.nz; z += blockDim.x) bb[z] = make_float2(float(yb[2 * z]), float(yb[2 * z + 1]));
+  for (int z = threadIdx.x; z < d.nz; z += blockDim.x) {
+    bb[0][z] = float(yb[2 * z]);
+    bb[1][z] = float(yb[2 * z + 1]);
+  }
   __syncthreads();
   const long long r0 = d.row_off_mf[size_t(m) * (d.nf + 1) + f0];
   const long long r1 = d.row_off_mf[size_t(m) * (d.nf + 1) + f1];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
   float2* X = reinterpret_cast<float2*>(d.X);
-  // one warp per row, lanes over depth
-  for (long long ri = r0 + (long long)blockIdx.x * nwarp + warp; ri < r1; ri += (long long)gridDim.x * nwarp) {
+  // two rows per warp, lanes over depth; lane 16 h ends with row h's sums
+  const long long step = 2LL * gridDim.x * nwarp;
+  for (long long rb = r0 + 2 * ((long long)blockIdx.x * nwarp + warp); rb < r1; rb += step) {
+    const bool two = rb + 1 < r1;
+    const long long ri = rb + (two ? lane >> 4 : 0);
     const uint32_t row = d.rows[ri];
     const int f = row_f(row), p = row_p(row), q = (p - m) & msk;
-    const float2* g1 = d.g32 + (size_t(f) * d.nk + tab_index(p, N)) * d.nzs;
-    const float2* g2 = d.g32 + (size_t(f) * d.nk + tab_index(q, N)) * d.nzs;
-    float2 sp = make_float2(0.f, 0.f), sm = sp;
-    for (int z = lane; z < d.nz; z += 32) {
-      const float2 t = g1[z] * g2[z], b2 = bb[z];
-      sp.x = fmaf(t.x, b2.x, sp.x); sp.y = fmaf(t.y, b2.x, sp.y);
-      sm.x = fmaf(t.x, b2.y, sm.x); sm.y = fmaf(t.y, b2.y, sm.y);
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      sp.x += __shfl_xor_sync(0xffffffffu, sp.x, o);
-      sp.y += __shfl_xor_sync(0xffffffffu, sp.y, o);
-      sm.x += __shfl_xor_sync(0xffffffffu, sm.x, o);
-      sm.y += __shfl_xor_sync(0xffffffffu, sm.y, o);
-    }
-    if (lane != 0) continue;
+    const int2 tr = table_rows(d, m, row);
+    const float s = row_pair_dots(d, tr, 0, 16, bb[0], bb[1], lane);
+    const int l0 = lane & 16;
+    const float2 sp = make_float2(__shfl_sync(0xffffffffu, s, l0), __shfl_sync(0xffffffffu, s, l0 + 4));
+    const float2 sm = make_float2(__shfl_sync(0xffffffffu, s, l0 + 8), __shfl_sync(0xffffffffu, s, l0 + 12));
+    if (lane != 0 && !(lane == 16 && two)) continue;
     const bool w2 = row_w2(row);
     const FreqConst fc = d.fc[f];
     const float2 crot = make_float2(float(fc.rot_re), float(-fc.rot_im));   // conj(rot)
@@ -683,7 +713,7 @@ constexpr int IG_WARPS = 8, IG_RPW = 16;             // 128 rows per CTA of the 
 __global__ void __launch_bounds__(IG_WARPS * 32) ig_rowdot_kernel(Dev d, int mode) {
   __shared__ float vs[2][512];
   __shared__ double red[IG_WARPS];
-  const int m = blockIdx.y, nz = d.nz, N = d.N, msk = N - 1;
+  const int m = blockIdx.y, nz = d.nz;
   const bool ok = d.status[m] == EDT_OK;
   const long long r0 = d.row_off[m], nr = d.row_off[m + 1] - r0;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -720,41 +750,26 @@ __global__ void __launch_bounds__(IG_WARPS * 32) ig_rowdot_kernel(Dev d, int mod
   __syncthreads();
   const long long wb = (long long)blockIdx.x * IG_WARPS * IG_RPW + warp * IG_RPW;
   const long long we = min(nr, wb + IG_RPW);
-  const float2* rhs = reinterpret_cast<const float2*>(d.rhs);
-  for (long long i = wb; i < we; ++i) {
-    const long long ri = r0 + i;
-    const uint32_t row = d.rows[ri];
-    const int f = row_f(row), p = row_p(row), q = (p - m) & msk;
-    const float2* gp = d.g32 + (size_t(f) * d.nk + tab_index(p, N)) * d.nzs;
-    const float2* gq = d.g32 + (size_t(f) * d.nk + tab_index(q, N)) * d.nzs;
-    float2 sp = make_float2(0.f, 0.f), sm = sp;
-    for (int z = lane; z < nz; z += 32) {
-      const float2 t = gp[z] * gq[z];
-      const float a = vs[0][z], b = vs[1][z];
-      sp.x = fmaf(t.x, a, sp.x); sp.y = fmaf(t.y, a, sp.y);
-      sm.x = fmaf(t.x, b, sm.x); sm.y = fmaf(t.y, b, sm.y);
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      sp.x += __shfl_xor_sync(0xffffffffu, sp.x, o); sp.y += __shfl_xor_sync(0xffffffffu, sp.y, o);
-      sm.x += __shfl_xor_sync(0xffffffffu, sm.x, o); sm.y += __shfl_xor_sync(0xffffffffu, sm.y, o);
-    }
-    if (lane == 0) {
-      float4 o = make_float4(0.f, 0.f, 0.f, 0.f);
-      if (ok) {
-        if (mode) {
-          o = make_float4(-sp.x, -sp.y, -sm.x, -sm.y);
-        } else {
-          const float2 dp = rhs[2 * ri], dm = rhs[2 * ri + 1];
-          o = make_float4(dp.x - sp.x, dp.y - sp.y, dm.x - sm.x, dm.y - sm.y);
-        }
-      }
-      d.rowc[2 * ri + mode] = o;
+  const int cnt = int(max(0LL, we - wb));
+  const float* rhs = reinterpret_cast<const float*>(d.rhs);    // [row][+ re, + im, - re, - im]
+  // lane i holds row i's table rows, so that a pair's loads wait for no metadata
+  const int2 tr = lane < cnt ? table_rows(d, m, d.rows[r0 + wb + lane]) : make_int2(0, 0);
+  for (int i = 0; i < cnt; i += 2) {
+    const float s = row_pair_dots(d, tr, i, min(i + 1, cnt - 1), vs[0], vs[1], lane);
+    const int c = lane >> 2, row = i + (c >> 2);
+    if ((lane & 3) == 0 && row < cnt) {
+      const size_t at = size_t(r0 + wb + row);
+      float* o = reinterpret_cast<float*>(d.rowc + 2 * at + mode) + (c & 3);
+      *o = !ok ? 0.f : mode ? -s : rhs[4 * at + (c & 3)] - s;
     }
   }
 }
 
 // One warp per table row (f, n), n = 0 .. N/2, lanes over depth (NZL per lane): gbar of that
-// row from every row that reads it, in row order; 32 rows summed in FP32, then into FP64.
+// row from every row that reads it, in row order; 32 rows summed in FP32, then into FP64.  Lane l
+// reads the metadata of the 32 rows' l-th and hands it round by shuffles, so the depth loads of
+// successive rows wait for nothing but their turn (each row's chain of three dependent loads
+// before its depths made the kernel 21 % of an inversion with its vector-Jacobian products).
 template <int NZL>
 __global__ void __launch_bounds__(256) ig_gather_kernel(Dev d) {
   const long long te = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
@@ -772,31 +787,44 @@ __global__ void __launch_bounds__(256) ig_gather_kernel(Dev d) {
     acc[t] = make_double2(0.0, 0.0);
   }
   const long long b0 = d.tref_off[te], b1 = d.tref_off[te + 1];
-  for (long long i = b0; i < b1; ++i) {
-    const int2 rf = d.tref[i];
-    const int m = rf.y >> 1, side = rf.y & 1;
-    const uint32_t row = d.rows[rf.x];
-    const int p = row_p(row), q = (p - m) & msk;
-    const float2* go = d.g32 + (size_t(f) * d.nk + tab_index(side ? p : q, N)) * d.nzs;
-    const float4 u = d.rowc[2 * size_t(rf.x)], v = d.rowc[2 * size_t(rf.x) + 1];
-    const float w = row_w2(row) ? 2.f : 1.f, gam = float(d.gam[m]);
-    const float4* xm = d.xmu + size_t(m) * nz;
+  for (long long base = b0; base < b1; base += 32) {
+    const int cnt = int(min(32LL, b1 - base));
+    int li = 0, lg = 0, lm = 0;                          // row, other table row, m (w2 in the sign)
+    float lgam = 0.f;
+    if (lane < cnt) {
+      const int2 rf = d.tref[base + lane];
+      const uint32_t row = d.rows[rf.x];
+      const int m = rf.y >> 1, p = row_p(row), q = (p - m) & msk;
+      li = rf.x;
+      lg = f * d.nk + tab_index(rf.y & 1 ? p : q, N);
+      lm = row_w2(row) ? ~m : m;
+      lgam = float(d.gam[m]);
+    }
+#pragma unroll 2
+    for (int k = 0; k < cnt; ++k) {
+      const int ri = __shfl_sync(0xffffffffu, li, k), mw = __shfl_sync(0xffffffffu, lm, k);
+      const float2* go = d.g32 + size_t(__shfl_sync(0xffffffffu, lg, k)) * d.nzs;
+      const float gam = __shfl_sync(0xffffffffu, lgam, k);
+      const float4 u = d.rowc[2 * size_t(ri)], v = d.rowc[2 * size_t(ri) + 1];
+      const float w = mw < 0 ? 2.f : 1.f;
+      const float4* xm = d.xmu + size_t(mw < 0 ? ~mw : mw) * nz;
 #pragma unroll
-    for (int t = 0; t < NZL; ++t) {
-      const int z = lane + 32 * t;
-      if (z < nz) {
-        const float2 g2 = go[z];
-        const float4 xv = xm[z];                       // (x_+, x_-, mu_+, mu_-)
-        const float2 A = self[t] * g2;
-        float2 ab;
-        ab.x = fmaf(u.x, xv.z, fmaf(u.z, xv.w, fmaf(v.x, xv.x, fmaf(v.z, xv.y, gam * A.x))));
-        ab.y = fmaf(u.y, xv.z, fmaf(u.w, xv.w, fmaf(v.y, xv.x, fmaf(v.w, xv.y, gam * A.y))));
-        ab.x *= w; ab.y *= w;
-        part[t].x = fmaf(g2.x, ab.x, fmaf(g2.y, ab.y, part[t].x));      // g2 conj(ab)
-        part[t].y = fmaf(g2.y, ab.x, fmaf(-g2.x, ab.y, part[t].y));
+      for (int t = 0; t < NZL; ++t) {
+        const int z = lane + 32 * t;
+        if (z < nz) {
+          const float2 g2 = go[z];
+          const float4 xv = xm[z];                       // (x_+, x_-, mu_+, mu_-)
+          const float2 A = self[t] * g2;
+          float2 ab;
+          ab.x = fmaf(u.x, xv.z, fmaf(u.z, xv.w, fmaf(v.x, xv.x, fmaf(v.z, xv.y, gam * A.x))));
+          ab.y = fmaf(u.y, xv.z, fmaf(u.w, xv.w, fmaf(v.y, xv.x, fmaf(v.w, xv.y, gam * A.y))));
+          ab.x *= w; ab.y *= w;
+          part[t].x = fmaf(g2.x, ab.x, fmaf(g2.y, ab.y, part[t].x));      // g2 conj(ab)
+          part[t].y = fmaf(g2.y, ab.x, fmaf(-g2.x, ab.y, part[t].y));
+        }
       }
     }
-    if (((i - b0) & 31) == 31) {
+    if (cnt == 32) {
 #pragma unroll
       for (int t = 0; t < NZL; ++t) {
         acc[t].x += double(part[t].x); acc[t].y += double(part[t].y);

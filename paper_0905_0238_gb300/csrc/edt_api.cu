@@ -729,7 +729,7 @@ void layout(edt_ctx* c) {
   take(c->r_vfull, (c->win ? nxy : N) * nz * sizeof(double2));
   // misfit gradients: line geometry, mixed path (their dJ/dg buffer aliases r_g64)
   const bool grad = !c->win && mixed && c->nlayer <= GRAD_MAX_LAYERS && N >= 64;
-  take(c->r_gscr, grad ? nf * size_t(c->nlayer) * 8 * nk * sizeof(double2) : 0);
+  take(c->r_gscr, grad ? nf * size_t(c->nlayer) * GS_SLOTS * nk * sizeof(double2) : 0);
   take(c->r_adj, grad ? size_t(N) * nz * sizeof(double2) : 0);
   take(c->r_gacc, grad ? size_t(1 + c->nlayer) * sizeof(double) : 0);
   take(c->r_bexp, mixed && !c->win ? (nf * nk + N) * sizeof(int) : 0);
@@ -1597,10 +1597,10 @@ int edt_get_stats(edt_ctx* c, edt_stats* o) {
   }
   o->freq_chunk = c->band_mode ? c->band_maxplanes : c->fchunk;
   // misfit gradient: green, zero, lateral DFT and its FP32 copy, per chunk transform (2), the
-  // residual (2) and two contractions, depth march forward / field / reversed (3), inverse
+  // residual (2) and two contractions, depth march states / field / recursions / layer sums (4), inverse
   // lateral DFT, finalize
   o->launches_per_grad = grad_supported(c->dev) && c->fchunk > 0
-                             ? green_launches(c->dev, GREEN_G32) + 3 + 6 * ((c->nf + c->fchunk - 1) / c->fchunk) + 5 : 0;
+                             ? green_launches(c->dev, GREEN_G32) + 3 + 6 * ((c->nf + c->fchunk - 1) / c->fchunk) + 6 : 0;
   o->gram_rows_padded = 0;
   for (long long n : c->seg_nrow) o->gram_rows_padded += (n + TC_KC - 1) / TC_KC * TC_KC;
   if (c->ws) {

@@ -159,7 +159,7 @@ struct Dev {
   double2* vhat;                // [nsub][nz]
   double2* vfull;               // [N][nz] scratch for the forward model (Vhat of V)
   // misfit gradients (line geometry, mixed path)
-  double2* gscr;                // [nf][nlayer][8][nk] depth-march states and cotangents
+  double2* gscr;                // [nf][nlayer][GS_SLOTS][nk] depth-march states and cotangents
   double2* adj;                 // [N][nz] Ahat = F^H R2 summed over frequencies
   double* gacc;                 // [1 + nlayer] sum |R2|^2
   double* gcpart;               // [warps of the reverse march][nlayer] partial dJ/dc_l
@@ -209,6 +209,7 @@ int record_cuda_error(cudaError_t e);
 
 // ---- launchers (each returns cudaGetLastError()) ---------------------------------------
 constexpr int GREEN_G64 = 1, GREEN_G32 = 2, GREEN_G32DF = 4;   // tables launch_green writes
+constexpr int GS_SLOTS = 12;    // of gscr (csrc/grad.cu)
 constexpr int GREEN_G32F = 8, GREEN_COEF = 16;
 // GREEN_G32 alone: the fast FP32 evaluation for the mixed path (no FP64 table);
 // GREEN_G32F: the same table from coefficients formed in FP32 (green_coef32; about the number

@@ -411,15 +411,25 @@ cudaError_t gbar_launch(const Dev& d, int f0, int nfc, cudaStream_t s) {
 // is the sum over its uses of (output cotangent) x (complex partial derivative).  Reverse
 // order: the field, the downward recursion (l descending), the upward one (l ascending),
 // finally d kappa_l/d c_l = -omega~^2/(c_l^3 kappa_l).
-constexpr int GS_KAP = 0, GS_RHO = 1, GS_R = 2, GS_A = 3, GS_BKAP = 4, GS_BRHO = 5, GS_BA = 6, GS_BR = 7;
-constexpr int GS_SLOTS = 8;
+// Reversed, with b(x) the cotangent of x, the two recursions are linear ones along l,
+//   b(A_l) += b(A_{l+1}) F_l,
+//   b(rho_l) += b(A_{l+1}) P_l + b(r_l) E_l,   b(r_{l+1}) = b(rho_l) X_l - b(A_{l+1}) Q_l,
+//   P_l = A_l dF_l/drho_l,  Q_l = -A_l dF_l/dr_{l+1},  X_l = (drho_l/dy)(dy/dr_{l+1}),
+// and the kappa_l collect b(A_{l+1}) A_l dF_l/dkappa_l, b(r_l) dr_l/dkappa_l, b(rho_l) U_l and
+// b(rho_{l-1}) W_{l-1}, U_l = drho_l/dkappa_l, W_l = (drho_l/dy)(dy/dkappa_{l+1}).  All coefficients
+// and collections are formed per layer in parallel; only the recursions themselves, a
+// multiply-add or two per layer, run one layer after the other (with everything inside them, two
+// reciprocals per layer, they took 0.40 ms for the 512-point line, 128 frequencies and 20 layers).
+constexpr int GS_KAP = 0, GS_RHO = 1, GS_A = 2, GS_BKAP = 3, GS_BRHO = 4, GS_BA = 5, GS_F = 6, GS_X = 7, GS_P = 8,
+              GS_Q = 9, GS_U = 10, GS_W = 11;
+constexpr int GS_BR = GS_X;              // takes X's place as the recursion passes
 
 __device__ __forceinline__ double2& gs_at(const Dev& d, int f, int l, int slot, int k) {
   return d.gscr[((size_t(f) * d.nlayer + l) * GS_SLOTS + slot) * d.nk + k];
 }
 
-// kappa_l, rho_l, r_l, A_l per (f, k, l) from the depth march's FP64 coefficients (launch_green ran
-// with the same reference), the cotangent slot of r cleared
+// kappa_l, rho_l, A_l per (f, k, l) from the depth march's FP64 coefficients (launch_green ran with the
+// same reference), and the reversed recursions' coefficients
 __global__ void __launch_bounds__(128) grad_state_kernel(Dev d) {
   const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
   const int J = d.nlayer;
@@ -428,12 +438,21 @@ __global__ void __launch_bounds__(128) grad_state_kernel(Dev d) {
   const long long fl = gid / d.nk;
   const int l = int(fl % J), f = int(fl / J);
   const GreenLayer q = green_layer_state(d, f, k, l);
-  const double2 zero = cmk(0.0, 0.0);
+  const double2 one = cmk(1.0, 0.0);
   gs_at(d, f, l, GS_KAP, k) = q.kappa;
   gs_at(d, f, l, GS_RHO, k) = q.rho;
-  gs_at(d, f, l, GS_R, k) = l < J - 1 ? q.rho * (q.eh * q.eh) : zero;
   gs_at(d, f, l, GS_A, k) = q.amp;
-  gs_at(d, f, l, GS_BR, k) = zero;
+  if (l == J - 1) return;
+  const GreenLayer n = green_layer_state(d, f, k, l + 1);
+  const double2 rn = l + 1 < J - 1 ? n.rho * (n.eh * n.eh) : cmk(0.0, 0.0);        // r_{l+1}
+  const double2 ir = crcp(one + rn), dy = (one - rn) * ir, y = n.kappa * dy, sm = q.kappa + y, is2 = crcp(sm * sm);
+  const double2 P = q.amp * q.eh * ir, up = (one + q.rho) * ir;
+  gs_at(d, f, l, GS_F, k) = q.eh * up;
+  gs_at(d, f, l, GS_X, k) = (4.0 * q.kappa) * n.kappa * is2 * (ir * ir);
+  gs_at(d, f, l, GS_P, k) = P;
+  gs_at(d, f, l, GS_Q, k) = P * up;
+  gs_at(d, f, l, GS_U, k) = (2.0 * y) * is2;
+  gs_at(d, f, l, GS_W, k) = (-2.0 * q.kappa) * is2 * dy;
 }
 
 // field, reversed, per (f, k, l): the depths z_j of layer l (a contiguous index range, dz apart)
@@ -503,69 +522,69 @@ __global__ void __launch_bounds__(128) grad_field_kernel(Dev d, const double2* g
   gs_at(d, f, l, GS_BKAP, k) = bK;
 }
 
-// the two recursions reversed per (f, k), then dJ/dc_l = Re(kappabar_l dkappa_l/dc_l)
-// summed over (f, k): warp sums, one partial per warp and layer (added in warp order by the
-// finalize kernel, so the result does not depend on the order the warps ran in)
-__global__ void __launch_bounds__(128) grad_reverse_kernel(Dev d) {
-  const int k = blockIdx.x * blockDim.x + threadIdx.x;
-  const int f = blockIdx.y;
+// the reversed recursions per (f, k), each layer's operands loaded while the one before it is
+// worked on
+__global__ void __launch_bounds__(32) grad_reverse_kernel(Dev d) {
+  const int gid = blockIdx.x * 32 + threadIdx.x, J = d.nlayer;
+  if (gid >= d.nf * d.nk) return;
+  const int f = gid / d.nk, k = gid - f * d.nk;
+  // downward recursion: A_{l+1} = A_l F_l
+  double2 bA = gs_at(d, f, J - 1, GS_BA, k);
+  double2 F, B;
+  auto fetch_a = [&](int l) { F = gs_at(d, f, l, GS_F, k); B = gs_at(d, f, l, GS_BA, k); };
+  if (J > 1) fetch_a(J - 2);
+  for (int l = J - 2; l >= 0; --l) {
+    bA = B + bA * F;
+    if (l > 0) fetch_a(l - 1);
+    gs_at(d, f, l, GS_BA, k) = bA;
+  }
+  // upward recursion (l ascending: r_l's cotangent is complete when l is reached)
+  double2 bR = cmk(0.0, 0.0), rho, P, Q, X, eh, A1;
+  auto fetch_r = [&](int l) {
+    rho = gs_at(d, f, l, GS_BRHO, k);
+    P = gs_at(d, f, l, GS_P, k);
+    Q = gs_at(d, f, l, GS_Q, k);
+    X = gs_at(d, f, l, GS_X, k);
+    eh = green_layer_eh(d, f, k, l);
+    A1 = gs_at(d, f, l + 1, GS_BA, k);
+  };
+  if (J > 1) fetch_r(0);
+  for (int l = 0; l <= J - 2; ++l) {
+    const double2 bRho = rho + A1 * P + bR * (eh * eh), next = bRho * X - A1 * Q;
+    if (l < J - 2) fetch_r(l + 1);
+    gs_at(d, f, l, GS_BRHO, k) = bRho;
+    gs_at(d, f, l, GS_BR, k) = bR;
+    bR = next;
+  }
+}
+
+// dJ/dc_l = Re(kappabar_l dkappa_l/dc_l) summed over (f, k): warp sums, one partial per warp and layer
+// (added in warp order by the finalize kernel, so the result does not depend on the order the
+// warps ran in)
+__global__ void __launch_bounds__(128) grad_layer_kernel(Dev d) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x, l = blockIdx.y, f = blockIdx.z;
   const int J = d.nlayer;
-  const bool live = k < d.nk;
-  const int kk = live ? k : 0;
-  const double2 one = cmk(1.0, 0.0);
-  const FreqConst fc = d.fc[f];
-  const double2 om = cmk(fc.om_re, fc.om_im), om2 = om * om;
-  if (live) {
-    // downward recursion, reversed: A_{l+1} = A_l F_l
-    double2 bA1 = gs_at(d, f, J - 1, GS_BA, kk);
-    for (int l = J - 2; l >= 0; --l) {
+  double v = 0.0;
+  if (k < d.nk) {
+    const double2 kl = gs_at(d, f, l, GS_KAP, k);
+    double2 b = gs_at(d, f, l, GS_BKAP, k);
+    if (l < J - 1) {
       const double h = d.layer_top[l + 1] - d.layer_top[l];
-      const double2 rho = gs_at(d, f, l, GS_RHO, kk);
-      const double2 rn = gs_at(d, f, l + 1, GS_R, kk), Al = gs_at(d, f, l, GS_A, kk);
-      const double2 e1 = green_layer_eh(d, f, kk, l);
-      const double2 inv1r = crcp(one + rn);
-      const double2 F = e1 * (one + rho) * inv1r;
-      const double2 bF = bA1 * Al;
-      const double2 bA = gs_at(d, f, l, GS_BA, kk) + bA1 * F;
-      gs_at(d, f, l, GS_BKAP, kk) = gs_at(d, f, l, GS_BKAP, kk) + bF * F * cmk(0.0, h);
-      gs_at(d, f, l, GS_BRHO, kk) = gs_at(d, f, l, GS_BRHO, kk) + bF * e1 * inv1r;
-      gs_at(d, f, l + 1, GS_BR, kk) = gs_at(d, f, l + 1, GS_BR, kk) - bF * F * inv1r;
-      bA1 = bA;
+      const double2 eh = green_layer_eh(d, f, k, l);
+      b = b + gs_at(d, f, l + 1, GS_BA, k) * gs_at(d, f, l, GS_A, k) * gs_at(d, f, l, GS_F, k) * cmk(0.0, h);
+      b = b + gs_at(d, f, l, GS_BR, k) * gs_at(d, f, l, GS_RHO, k) * (eh * eh) * cmk(0.0, 2.0 * h);
+      b = b + gs_at(d, f, l, GS_BRHO, k) * gs_at(d, f, l, GS_U, k);
     }
-    {
-      const double2 k0 = gs_at(d, f, 0, GS_KAP, kk);
-      gs_at(d, f, 0, GS_BKAP, kk) = gs_at(d, f, 0, GS_BKAP, kk) + bA1 * cmk(0.0, -0.5) * crcp(k0 * k0);
-    }
-    // upward recursion, reversed (l ascending: r_l's cotangent is complete when l is reached)
-    for (int l = 0; l <= J - 2; ++l) {
-      const double h = d.layer_top[l + 1] - d.layer_top[l];
-      const double2 kl = gs_at(d, f, l, GS_KAP, kk), kn = gs_at(d, f, l + 1, GS_KAP, kk);
-      const double2 rn = gs_at(d, f, l + 1, GS_R, kk), rho = gs_at(d, f, l, GS_RHO, kk);
-      const double2 e1 = green_layer_eh(d, f, kk, l), E = e1 * e1;
-      const double2 bR = gs_at(d, f, l, GS_BR, kk);
-      const double2 bRho = gs_at(d, f, l, GS_BRHO, kk) + bR * E;
-      double2 bK = gs_at(d, f, l, GS_BKAP, kk) + bR * rho * E * cmk(0.0, 2.0 * h);
-      const double2 iopr = crcp(one + rn);
-      const double2 y = kn * (one - rn) * iopr;
-      const double2 sm = kl + y, is2 = crcp(sm * sm);
-      bK = bK + bRho * (2.0 * y) * is2;
-      const double2 bY = bRho * (-2.0 * kl) * is2;
-      gs_at(d, f, l, GS_BKAP, kk) = bK;
-      gs_at(d, f, l + 1, GS_BKAP, kk) = gs_at(d, f, l + 1, GS_BKAP, kk) + bY * (one - rn) * iopr;
-      gs_at(d, f, l + 1, GS_BR, kk) = gs_at(d, f, l + 1, GS_BR, kk) + bY * kn * (-2.0 * (iopr * iopr));
-    }
+    if (l > 0) b = b + gs_at(d, f, l - 1, GS_BRHO, k) * gs_at(d, f, l - 1, GS_W, k);
+    else b = b + gs_at(d, f, 0, GS_BA, k) * cmk(0.0, -0.5) * crcp(kl * kl);
+    const FreqConst fc = d.fc[f];
+    const double2 om = cmk(fc.om_re, fc.om_im);
+    const double c = d.layer_vel[l];
+    v = (b * ((-1.0 / (c * c * c)) * (om * om) * crcp(kl))).x;
   }
-  for (int l = 0; l < J; ++l) {
-    double v = 0.0;
-    if (live) {
-      const double c = d.layer_vel[l];
-      const double2 dk = (-1.0 / (c * c * c)) * om2 * crcp(gs_at(d, f, l, GS_KAP, kk));
-      v = (gs_at(d, f, l, GS_BKAP, kk) * dk).x;
-    }
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    const size_t wid = (size_t(blockIdx.y) * gridDim.x + blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if ((threadIdx.x & 31) == 0) d.gcpart[wid * J + l] = v;
-  }
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  const size_t wid = (size_t(f) * gridDim.x + blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
+  if ((threadIdx.x & 31) == 0) d.gcpart[wid * J + l] = v;
 }
 
 // nw: the reverse kernel's warps.  One warp per layer: lane l adds the partials l, l + 32, ... in
@@ -892,7 +911,8 @@ cudaError_t launch_invert_vjp(const Dev& d0, const void* Vbar, int Vbar_dtype, v
     const long long nfl = (long long)d.nf * d.nlayer * d.nk;
     grad_state_kernel<<<unsigned((nfl + 127) / 128), 128, 0, s>>>(d);
     grad_field_kernel<<<unsigned((nfl + 127) / 128), 128, 0, s>>>(d, d.g64);
-    grad_reverse_kernel<<<gk, 128, 0, s>>>(d);
+    grad_reverse_kernel<<<unsigned((d.nf * d.nk + 31) / 32), 32, 0, s>>>(d);
+    grad_layer_kernel<<<dim3(gk.x, d.nlayer, d.nf), 128, 0, s>>>(d);
     grad_finalize_kernel<<<d.nlayer, 32, 0, s>>>(d, nullptr, gc, int(gk.x * gk.y * 4));
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
   }
@@ -961,7 +981,8 @@ cudaError_t launch_misfit_grad(const Dev& d, const void* V, int V_dtype, const v
   const long long nfl = (long long)d.nf * d.nlayer * d.nk;
   grad_state_kernel<<<unsigned((nfl + 127) / 128), 128, 0, s>>>(d);
   grad_field_kernel<<<unsigned((nfl + 127) / 128), 128, 0, s>>>(d, nullptr);
-  grad_reverse_kernel<<<gk, 128, 0, s>>>(d);
+  grad_reverse_kernel<<<unsigned((d.nf * d.nk + 31) / 32), 32, 0, s>>>(d);
+  grad_layer_kernel<<<dim3(gk.x, d.nlayer, d.nf), 128, 0, s>>>(d);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if ((e = launch_lateral_idft_real(d, d.adj, 2.0 / (double(N) * N), gV, V_dtype, s)) != cudaSuccess) return e;
   grad_finalize_kernel<<<d.nlayer, 32, 0, s>>>(d, J, gc, int(gk.x * gk.y * 4));

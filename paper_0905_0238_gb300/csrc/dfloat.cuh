@@ -117,6 +117,8 @@ __device__ inline bool df_diag_block(float2* A, float* L32, double* dinv, float*
     sh.col[lane][i] = i < kb && lane <= i ? A[size_t(k0 + i) * n + k0 + lane] : zero;
   }
   if (threadIdx.x == 0) sh.fail = 0;
+  if (threadIdx.x < 64) sh.xr[threadIdx.x >> 5][lane] = zero;
+  if (threadIdx.x < 96) sh.ls[threadIdx.x >> 5][lane] = zero;
   __syncthreads();
   float2 w[4];
 #pragma unroll
@@ -141,16 +143,20 @@ __device__ inline bool df_diag_block(float2* A, float* L32, double* dinv, float*
   __syncthreads();
   for (int j = 0; j < kb; ++j) {
     if (sh.fail) break;                           // the same value in every thread
-    const float2 lj = df_neg(sh.col[j][lane]), lp = df_neg(sh.ls[(j + 2) % 3][lane]);
+    // columns c > j: A -= L_j L_j^T (rows above c are not used); c < j: U_i -= (L_i,j-1 / L_j-1,j-1) U_j-1
+    // for the rows i >= j, the others and column j subtract zero
+    const float2 lj = df_neg(sh.col[j][lane]);
+    const float2 lp = lane >= j ? df_neg(sh.ls[(j + 2) % 3][lane]) : zero;
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const int c = warp + 8 * q;                 // the same in the whole warp
-      if (c > j) {
-        if (lane >= c) df_acc(w[q], lj, sh.col[j][c]);                      // A -= L_j L_j^T
-      } else if (c < j) {
-        if (lane >= j) df_acc(w[q], lp, sh.xr[(j + 1) & 1][c]);             // U_i -= (L_i,j-1 / L_j-1,j-1) U_j-1
-      }
-      if (c <= j && lane == j) sh.xr[j & 1][c] = df_norm(w[q]);             // row j of U
+      const float2 o = c > j ? sh.col[j][c] : sh.xr[(j + 1) & 1][c];
+      df_acc(w[q], c > j ? lj : c < j ? lp : zero, o);
+    }
+    if (lane == j) {                              // row j of U
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (warp + 8 * q <= j) sh.xr[j & 1][warp + 8 * q] = df_norm(w[q]);
     }
 #pragma unroll
     for (int q = 0; q < 4; ++q)

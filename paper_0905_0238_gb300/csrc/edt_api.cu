@@ -71,6 +71,7 @@ struct edt_ctx {
   std::vector<int> jact, jmap, nact;   // active offset wavenumbers per frequency
   std::vector<int> q_off, q_xy;        // a grid's quadrant points with kept rows, per frequency
   std::vector<int4> q_rows;            // [q_xy] rows of the pairs (kx, ky) and (-kx, ky)
+  std::vector<int2> q_ext;             // [nf] their largest x and y
   int q_max = 0;                       // most points of a frequency
   long long rows_max_sub = 0;
   // band-limited transform of the mixed path
@@ -271,6 +272,7 @@ void plan_window(edt_ctx* c, double cmin) {
   c->q_off.assign(nf + 1, 0);
   c->q_xy.clear(); c->q_rows.clear();
   c->q_max = 0;
+  c->q_ext.assign(nf, make_int2(0, 0));
   if (ny > 1) {
     std::vector<int> pair_of(size_t(ny) * nx, -1);
     for (int p = 0; p < c->nsub; ++p) pair_of[c->pair_m[p]] = p;
@@ -286,6 +288,7 @@ void plan_window(edt_ctx* c, double cmin) {
           }
           if (r.y + r.w == 0) continue;
           c->q_xy.push_back(qy << 16 | qx);
+          c->q_ext[f] = make_int2(std::max(c->q_ext[f].x, qx), std::max(c->q_ext[f].y, qy));
           c->q_rows.push_back(r);
         }
       c->q_off[f + 1] = int(c->q_xy.size());
@@ -938,7 +941,7 @@ int transform_rhs(edt_ctx* c, const void* D, int D_dtype, cudaStream_t s) {
 int kernel_rows(edt_ctx* c, cudaStream_t s) {
   if (!c->win) return EDT_OK;
   for (int f = 0; f < c->nf; ++f) {
-    if (c->ny > 1) EDT_TRY(launch_fa_grid(c->dev, f, c->q_off[f], c->q_off[f + 1] - c->q_off[f], c->cf[f], s));
+    if (c->ny > 1) EDT_TRY(launch_fa_grid(c->dev, f, c->q_off[f], c->q_off[f + 1] - c->q_off[f], c->q_ext[f], c->cf[f], s));
     else EDT_TRY(launch_fa_line(c->dev, f, c->nact[f], c->cf[f], s));
   }
   return EDT_OK;

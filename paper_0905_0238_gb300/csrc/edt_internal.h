@@ -237,12 +237,13 @@ cudaError_t prepare_band(const Dev& d);
 // right-hand sides, the inverse transform to V[ny][nx][nz]; supported grids and windows.
 bool fa_supported(int nx, int ny, int wx, int wy);
 cudaError_t launch_fa_line(const Dev& d, int f, int nact, double2 cf, cudaStream_t s);
-// the same for a grid (csrc/fagrid.cu): the frequency's points are q_xy/q_rows[qoff .. qoff + nq)
+// the same for a grid (csrc/fagrid.cu): the frequency's points are q_xy/q_rows[qoff .. qoff + nq), their
+// largest x and y qmax
 constexpr size_t FA_SLAB_BYTES = size_t(2) << 30;     // plane buffer of a slab of depths (at least 8)
 int fa_grid_slots(int wx, int wy);
 int fa_grid_slab(int nz, int slots, int nq);
 size_t fa_grid_bytes(int nzb, int slots, int nq);
-cudaError_t launch_fa_grid(const Dev& d, int f, int qoff, int nq, double2 cf, cudaStream_t s);
+cudaError_t launch_fa_grid(const Dev& d, int f, int qoff, int nq, int2 qmax, double2 cf, cudaStream_t s);
 cudaError_t prepare_fa_grid(const Dev& d);
 cudaError_t launch_fa_data(const Dev& d, const void* D, int D_dtype, cudaStream_t s);
 cudaError_t launch_fa_inverse(const Dev& d, void* V, int V_dtype, cudaStream_t s);

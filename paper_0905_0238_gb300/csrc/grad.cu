@@ -784,23 +784,25 @@ __global__ void __launch_bounds__(IG_WARPS * 32) ig_rowdot_kernel(Dev d, int mod
   }
 }
 
-// One warp per table row (f, n), n = 0 .. N/2, lanes over depth (NZL per lane): gbar of that
+// One warp per table row (f, n), n = 0 .. N/2, and 32 NZL depths, lanes over depth (NZL per lane): gbar of that
 // row from every row that reads it, in row order; 32 rows summed in FP32, then into FP64.  Lane l
 // reads the metadata of the 32 rows' l-th and hands it round by shuffles, so the depth loads of
 // successive rows wait for nothing but their turn (each row's chain of three dependent loads
-// before its depths made the kernel 21 % of an inversion with its vector-Jacobian products).
+// before its depths made the kernel 21 % of an inversion with its vector-Jacobian products).  More than
+// 128 depths go to several warps: eight depths per lane left 16 warps per SM (dL/dc of the 512-point
+// line with 256 depths 4.70 ms, 4.03 with four).
 template <int NZL>
 __global__ void __launch_bounds__(256) ig_gather_kernel(Dev d) {
   const long long te = (long long)blockIdx.x * 8 + (threadIdx.x >> 5);
   if (te >= (long long)d.nf * d.nk) return;
-  const int lane = threadIdx.x & 31, nz = d.nz, N = d.N, msk = N - 1;
+  const int lane = threadIdx.x & 31, nz = d.nz, N = d.N, msk = N - 1, z0 = 32 * NZL * blockIdx.y + lane;
   const int f = int(te / d.nk);
   const float2* gs = d.g32 + size_t(te) * d.nzs;
   float2 self[NZL], part[NZL];
   double2 acc[NZL];
 #pragma unroll
   for (int t = 0; t < NZL; ++t) {
-    const int z = lane + 32 * t;
+    const int z = z0 + 32 * t;
     self[t] = z < nz ? gs[z] : make_float2(0.f, 0.f);
     part[t] = make_float2(0.f, 0.f);
     acc[t] = make_double2(0.0, 0.0);
@@ -829,7 +831,7 @@ __global__ void __launch_bounds__(256) ig_gather_kernel(Dev d) {
       const float4* xm = d.xmu + size_t(mw < 0 ? ~mw : mw) * nz;
 #pragma unroll
       for (int t = 0; t < NZL; ++t) {
-        const int z = lane + 32 * t;
+        const int z = z0 + 32 * t;
         if (z < nz) {
           const float2 g2 = go[z];
           const float4 xv = xm[z];                       // (x_+, x_-, mu_+, mu_-)
@@ -855,7 +857,7 @@ __global__ void __launch_bounds__(256) ig_gather_kernel(Dev d) {
   double2* out = d.g64 + size_t(te) * nz;
 #pragma unroll
   for (int t = 0; t < NZL; ++t) {
-    const int z = lane + 32 * t;
+    const int z = z0 + 32 * t;
     if (z < nz) out[z] = make_double2(sq * (acc[t].x + double(part[t].x)), sq * (acc[t].y + double(part[t].y)));
   }
 }
@@ -900,9 +902,7 @@ cudaError_t launch_invert_vjp(const Dev& d0, const void* Vbar, int Vbar_dtype, v
     ig_rowdot_kernel<<<rg, IG_WARPS * 32, 0, s>>>(d, 1);          // v = -A mu, gamma
     const unsigned gg = unsigned(((long long)d.nf * d.nk + 7) / 8);
     if (d.nz <= 64) ig_gather_kernel<2><<<gg, 256, 0, s>>>(d);
-    else if (d.nz <= 128) ig_gather_kernel<4><<<gg, 256, 0, s>>>(d);
-    else if (d.nz <= 256) ig_gather_kernel<8><<<gg, 256, 0, s>>>(d);
-    else ig_gather_kernel<16><<<gg, 256, 0, s>>>(d);
+    else ig_gather_kernel<4><<<dim3(gg, (d.nz + 127) / 128), 256, 0, s>>>(d);
     if ((e = cudaGetLastError()) != cudaSuccess) return e;
     grad_zero_kernel<<<152, 256, 0, s>>>(d);
     // the forward solve's depth march may have been the FP32 one: its FP64 coefficients

@@ -945,9 +945,10 @@ def main_grad(args, world, rank, local):
             dist.destroy_process_group()
         return
     nf, N, nz = len(wl.freq_hz), wl.nx, wl.nz
-    # four contractions over (f, p, q, z): residual, adjoint Born, and the two legs of dJ/dg,
-    # each a complex product (6 flops) and a complex multiply-add (8 flops) per term
-    flops = 56.0 * nf * N * N * nz
+    # folded contractions over (f, pair, z): the residual, N^2/8 pairs (a complex product and
+    # eight multiply-adds, 22 flops), the adjoint Born sum, N^2/4 classes, and dJ/dg, N^2/2 terms
+    # (a complex product and four multiply-adds, 14 flops each)
+    flops = (22.0 / 8 + 14.0 / 4 + 14.0 / 2) * nf * N * N * nz
     peak = 152 * 128 * 2 * 2.07 / 1e3        # FP32 FMA lanes x 2 flops x 2.07 GHz -> TFLOP/s
     achieved = flops / (ms_total / args.steps / 1e3) / 1e12
     cpu = None
@@ -970,7 +971,7 @@ def main_grad(args, world, rank, local):
                  h2d_bytes_per_step=int(D.numel() * D.element_size() + V.numel() * V.element_size()),
                  d2h_bytes_per_step=int(gV.numel() * gV.element_size() + gc.numel() * 8 + 8)),
         gpu_launches=None,
-        roofline=dict(bound="alu", kernel="grad_residual + grad_vhat + grad_gbar (whole call)",
+        roofline=dict(bound="alu", kernel="born_resid + grad_vhat + grad_gbar (whole call)",
                       achieved=achieved, peak=peak, unit="TFLOP/s", frac=achieved / peak,
                       traffic=None, peak_source="derived: 152 SMs x 128 FP32 lanes x 2 flops x 2.07 GHz",
                       flops_per_launch=flops),

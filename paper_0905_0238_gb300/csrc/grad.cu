@@ -27,9 +27,10 @@
 //   grad_vhat      (m, j) outputs: Ahat(m) + conj Ahat(-m), m = 0..N/2, accumulated across
 //                  frequencies in FP64;
 //   grad_gbar      (n, j) outputs on the table index n = 0..N/2: S1 and S2 of both signs;
-// then once, in FP64: grad_state (per (f, k, layer): the march's coefficients), grad_field (per
+// then once, in FP64: grad_state (per (f, k, layer): the march's state and the reversed recursions'
+// coefficients), grad_field (per
 // (f, k, layer): the field's depths of that layer, reversed), grad_reverse (per (f, k): the
-// two recursions reversed, then the per-layer sums); the inverse lateral DFT of Ahat and a
+// two recursions reversed), grad_layer (the per-layer sums); the inverse lateral DFT of Ahat and a
 // finalize kernel.
 #include "edt_internal.h"
 #include "cplx.cuh"

@@ -409,25 +409,32 @@ __global__ void __launch_bounds__(32) green_eval64_kernel(Dev d) {
   const int J = d.nlayer;
   const double2* c = d.coef;
   const int zc = blockIdx.y * EV_ZC;
+  // both waves carry the amplitude (and, where only sqrt|s_f| g is wanted, sqrt|s_f|) from their anchors,
+  // so a depth takes two products and a sum, 10 FP64 operations instead of 18 (256 points, 150 depths,
+  // 75 frequencies: an inversion takes 0.985 ms, 1.000 with 18)
+  const double sq_own = d.g32 ? sqrt(d.fc[f].s_abs) : 0.0;
+  const bool fold = d.g32 && !d.g64;
   {
     int cur = -1;
-    double2 e1 = cmk(0.0, 0.0), e2 = e1, E = e1, Ei = e1, amp = e1, rho = e1;
+    double2 e1 = cmk(0.0, 0.0), e2 = e1, E = e1, Ei = e1;
     for (int i = 0; i < EV_ZC && zc + i < d.nz; ++i) {
       const int z = zc + i;
       const int l = d.z_layer[z];
       if (l != cur) {             // anchor: direct evaluation at layer entry / chunk start
         cur = l;
         const double2 kap = c[cix(d, f, n, l, C_KAP)];
+        double2 amp, rho;
         layer_waves(d, f, n, l, amp, rho);
+        if (fold) amp = sq_own * amp;
         if (z + 1 < d.nz && d.z_layer[z + 1] == l) {
           E = c[cix(d, f, n, l, C_E)];
           Ei = c[cix(d, f, n, l, C_EI)];
         }
         const double off = d.z_off[z];
-        e1 = cexp(cmk(-kap.y * off, kap.x * off));
+        e1 = amp * cexp(cmk(-kap.y * off, kap.x * off));
         if (l < J - 1) {
           const double a = 2.0 * (d.layer_top[l + 1] - d.layer_top[l]) - off;
-          e2 = cexp(cmk(-kap.y * a, kap.x * a));
+          e2 = (amp * rho) * cexp(cmk(-kap.y * a, kap.x * a));
         } else {
           e2 = cmk(0.0, 0.0);
         }
@@ -435,23 +442,22 @@ __global__ void __launch_bounds__(32) green_eval64_kernel(Dev d) {
         e1 = e1 * E;
         e2 = e2 * Ei;
       }
-      tile[lane][i] = amp * (e1 + rho * e2);
+      tile[lane][i] = e1 + e2;
     }
   }
   __syncwarp();
   constexpr int RP = 32 / EV_ZC;                          // rows written together
   const int z = zc + lane % EV_ZC;
-  const double sq_lane = d.g32 ? sqrt(d.fc[f].s_abs) : 0.0;
   for (int rr = 0; rr < 32; rr += RP) {
     const int nl = rr + lane / EV_ZC;
-    const double sq = __shfl_sync(0xffffffffu, sq_lane, nl);
+    const double sq = __shfl_sync(0xffffffffu, sq_own, nl);
     const long long r = r0 + nl;
     if (r < nrow && z < d.nz) {
       const double2 v = tile[nl][lane % EV_ZC];
       if (d.g64) d.g64[size_t(r) * d.nz + z] = v;
       if (d.g32) {
         // sqrt|s_f| g rounded to FP32, and (double-float table) the FP32 rounding of the rest
-        const double sx = sq * v.x, sy = sq * v.y;
+        const double sx = fold ? v.x : sq * v.x, sy = fold ? v.y : sq * v.y;
         const float hx = float(sx), hy = float(sy);
         const size_t o32 = size_t(r) * d.nzs + z;
         d.g32[o32] = make_float2(hx, hy);

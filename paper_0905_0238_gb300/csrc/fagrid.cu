@@ -17,7 +17,7 @@
 // end -h has no partner +h; s(0) = s(-h) = 0).  Both pairs (kx, ky), (-kx, ky) share the transforms.
 // Against the window sum first (per offset wavenumber j: products, 16-point transforms and one plane
 // FFT), at 128 x 128 midpoints, 16 x 16 half-offsets, 64 frequencies and 200 depths: 45 planes per
-// (f, z) instead of 138 on average, 49 ms of kernels instead of 144; 64 x 64, 8 x 8, 12 frequencies, 100
+// (f, z) instead of 138 on average, 46 ms of kernels instead of 144; 64 x 64, 8 x 8, 12 frequencies, 100
 // depths: 0.55 ms instead of 1.36.
 // Per frequency and slab of depths (all of them unless the planes would take more than
 // FA_SLAB_BYTES; slabs that stay in L2 lost more to short launches than they saved: 134 ms per

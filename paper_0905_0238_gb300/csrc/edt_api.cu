@@ -55,7 +55,7 @@ struct edt_ctx {
   std::vector<int> z_layer;
   std::vector<double> z_off;
   std::vector<float> z_off32;      // [nz][4]
-  std::vector<float2> fc32;        // [nf] sqrt|s_f| as a pair of floats
+  std::vector<float> fc32;         // [nf] sqrt|s_f|
   std::vector<uint32_t> rows;
   std::vector<long long> row_off;
   std::vector<long long> row_off_mf;   // [nsub][nf + 1]
@@ -465,10 +465,7 @@ void plan(edt_ctx* c) {
   c->fc32.resize(c->nf);
   // line geometry: the FP32 table carries sqrt|s_f| (rows are products of two table rows);
   // window geometry: plain g (the assembly applies the prefactor)
-  for (int f = 0; f < c->nf; ++f) {
-    const double sq = c->win ? 1.0 : std::sqrt(c->fc[f].s_abs);
-    c->fc32[f] = make_float2(float(sq), float(sq - double(float(sq))));
-  }
+  for (int f = 0; f < c->nf; ++f) c->fc32[f] = c->win ? 1.f : float(std::sqrt(c->fc[f].s_abs));
   const double cmin = *std::min_element(c->vel.begin(), c->vel.end());
   if (c->win) {
     plan_window(c, cmin);
@@ -699,9 +696,9 @@ void layout(edt_ctx* c) {
   take(c->r_ctas, std::max<size_t>(c->cta_seg0.size(), 1) * sizeof(int));
   take(c->r_mslot, (ns + 1) * sizeof(int));
   take(c->r_zo32, nz * 4 * sizeof(float));
-  take(c->r_fc32, nf * sizeof(float2));
+  take(c->r_fc32, nf * sizeof(float));
   take(c->r_coef, nf * nk * c->nlayer * 7 * sizeof(double2));
-  take(c->r_coef32, mixed ? nf * nk * c->nlayer * 12 * sizeof(float) : 0);
+  take(c->r_coef32, mixed ? nf * nk * c->nlayer * 8 * sizeof(float) : 0);
   take(c->r_g64, nf * nk * nz * sizeof(double2));
   take(c->r_g32, mixed ? nf * nk * size_t((c->nz + 1) & ~1) * sizeof(float2) : 0);
   take(c->r_g32lo, c->resid_df ? nf * nk * size_t((c->nz + 1) & ~1) * sizeof(float2) : 0);
@@ -822,7 +819,7 @@ void bind(edt_ctx* c) {
   d.coef = at<double2*>(c, c->r_coef);
   d.coef32 = c->r_coef32.bytes ? at<float*>(c, c->r_coef32) : nullptr;
   d.z_off32 = at<const float*>(c, c->r_zo32);
-  d.fc32_sqrt_s = at<const float2*>(c, c->r_fc32);
+  d.fc32_sqrt_s = at<const float*>(c, c->r_fc32);
   d.g64 = at<double2*>(c, c->r_g64);
   d.g32 = c->r_g32.bytes ? at<float2*>(c, c->r_g32) : nullptr;
   d.g32lo = c->r_g32lo.bytes ? at<float2*>(c, c->r_g32lo) : nullptr;

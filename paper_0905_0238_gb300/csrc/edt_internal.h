@@ -79,7 +79,7 @@ struct Dev {
   const int* z_layer;           // [nz] layer of each sample depth
   const double* z_off;          // [nz] depth below that layer's top
   const float* z_off32;         // [nz][4] (off hi, off lo, 2h - off hi, 2h - off lo) as floats
-  const float2* fc32_sqrt_s;    // [nf] sqrt|s_f| as a pair of floats (high, low)
+  const float* fc32_sqrt_s;     // [nf] sqrt|s_f| as float
   const uint32_t* rows;         // [rows_solved], grouped by m
   const long long* row_off;     // [nsub + 1]
   long long rows_max_sub;       // most rows of any subproblem
@@ -124,8 +124,7 @@ struct Dev {
   int nseg, ncta_gram;
   // scratch
   double2* coef;                // [nf][nk][nlayer][7] recursion coefficients (FP64)
-  float* coef32;                // [nf][nk][nlayer][8] FP32 copies for the fast evaluation, then
-                                //   [nf][nk][nlayer][4] the low parts of amplitude and reflection
+  float* coef32;                // [nf][nk][nlayer][8] FP32 copies for the fast evaluation
   double2* g64;                 // [nf][nk][nz]
   float2* g32;                  // [nf][nk][nzs] sqrt|s_f| g, mixed path (padding zero)
   float2* g32lo;                // [nf][nk][nzs] its FP32 remainder: g32 + g32lo carries the

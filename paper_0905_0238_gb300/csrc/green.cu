@@ -38,7 +38,6 @@
 #include "edt_internal.h"
 #include "cplx.cuh"
 #include "green_coef.cuh"
-#include "dfloat.cuh"
 
 namespace edt {
 
@@ -46,9 +45,6 @@ namespace {
 
 // FP32 copies for the fast evaluation: kappa.x and kappa.y as (hi, lo) pairs, amp, rho
 constexpr int NCOEF32 = 8;
-__device__ __forceinline__ float4* coef32_low(const Dev& d) {
-  return reinterpret_cast<float4*>(d.coef32 + size_t(d.nf) * d.nk * d.nlayer * NCOEF32);
-}
 
 // sqrt(w) on the branch Im >= 0, FP64: the FP32 root (relative error ~1e-7) and two Newton steps
 // k + (w - k^2) / (2 k) whose residual is formed in FP64 and whose divisor is the FP32 root's (it
@@ -313,13 +309,7 @@ __global__ void __launch_bounds__(128) green_coef32_kernel(Dev d) {
   split_ff(kap.y, k4.z, k4.w);
   float4* o = reinterpret_cast<float4*>(d.coef32 + ((size_t(f) * d.nk + n) * J + j) * NCOEF32);
   o[0] = k4;
-  float4 hi, lo;
-  split_ff(a.x, hi.x, lo.x);
-  split_ff(a.y, hi.y, lo.y);
-  split_ff(r.x, hi.z, lo.z);
-  split_ff(r.y, hi.w, lo.w);
-  o[1] = hi;
-  coef32_low(d)[((size_t(f) * d.nk + n) * J + j)] = lo;
+  o[1] = make_float4(float(a.x), float(a.y), float(r.x), float(r.y));
 }
 
 // The FP32 recursion's rounding errors (and those of its FP32 exponentials) compound over the
@@ -467,66 +457,27 @@ __global__ void __launch_bounds__(32) green_eval64_kernel(Dev d) {
   }
 }
 
-// e^{i kappa x} as expi_ff, with what that rounds away before sincos and exp put back to first order:
-// the reduced phase is kept as a pair (its rounding, up to 1.2e-7 near pi, is an error of the entry), and
-// the decay's exponent likewise (kappa's low imaginary part and the product's error)
-__device__ __forceinline__ float2 expi_fine(float4 k4, float xh, float xl) {
-  const float C1 = 6.28125f, C2 = 0.0019353071693331003f, C3 = 1.0253131677018246e-11f;
-  const float p = __fmul_rn(k4.x, xh);
-  const float q = fmaf(k4.x, xh, -p) + fmaf(k4.x, xl, k4.y * xh);
-  const float k = rintf(p * 0.15915493667125702f);
-  const float k2 = __fmul_rn(-k, C2);
-  const float2 s = two_sum(fmaf(-k, C1, p), k2);
-  const float2 r = two_sum(s.x, (s.y + fmaf(-k, C2, -k2)) + fmaf(-k, C3, q));
-  float sn, cs;
-  sincosf(r.x, &sn, &cs);
-  const float y = __fmul_rn(k4.z, xh);
-  const float rest = fmaf(k4.z, xh, -y) + fmaf(k4.z, xl, k4.w * xh);
-  const float mag = expf(-y);
-  return make_float2(mag * fmaf(-rest, cs, fmaf(-r.y, sn, cs)), mag * fmaf(-rest, sn, fmaf(r.y, cs, sn)));
-}
-// (h + l) v
-__device__ __forceinline__ float2 cmul_pair(float2 h, float2 l, float2 v) {
-  return make_float2(fmaf(h.x, v.x, fmaf(-h.y, v.y, fmaf(l.x, v.x, -l.y * v.y))),
-                     fmaf(h.x, v.y, fmaf(h.y, v.x, fmaf(l.x, v.y, l.y * v.x))));
-}
-
-// FINE (the line's table of the gradients): what is common to many depths (decay rates, amplitudes,
-// reflections, sqrt|s_f|) as pairs, so that an entry's error is its own few roundings.  The misfit's
-// layer gradients are small sums of large terms and keep a common error: at 512 points, 128
-// frequencies and 256 depths they were 2.3e-6 off 64 bits with the factors rounded to FP32 (mean of
-// 14 draws), 0.75e-6 with the pairs, for 25 us of a 5.2 ms gradient; the FP64 table rounded takes 0.3 ms.
 // One CTA per table row (f, n), threads over depth; the row's largest |value| goes to rowmax
 // (when present) for the FP16 operand scales of the Gram, so that no pass re-reads the table.
-template <bool FINE>
 __global__ void __launch_bounds__(256) green_eval32_kernel(Dev d) {
   __shared__ float red[8];
   const long long fn = blockIdx.x;
   const int J = d.nlayer;
   const int f = int(fn / d.nk);
-  const float2 sq = d.fc32_sqrt_s[f];
+  const float sq = d.fc32_sqrt_s[f];
   float mx = 0.f;
   for (int z = threadIdx.x; z < d.nz; z += blockDim.x) {
     const int l = d.z_layer[z];
     const float4 zo = reinterpret_cast<const float4*>(d.z_off32)[z];   // off (hi, lo), 2h - off (hi, lo)
     const float4* c4 = reinterpret_cast<const float4*>(d.coef32 + (fn * J + l) * NCOEF32);
     const float4 k4 = c4[0], ar = c4[1];
-    float2 v;
-    if constexpr (FINE) {
-      const float4 lo = coef32_low(d)[fn * J + l];
-      float2 e = expi_fine(k4, zo.x, zo.y);
-      if (l < J - 1) e = e + cmul_pair(make_float2(ar.z, ar.w), make_float2(lo.z, lo.w), expi_fine(k4, zo.z, zo.w));
-      const float2 g = cmul_pair(make_float2(ar.x, ar.y), make_float2(lo.x, lo.y), e);
-      v = make_float2(fmaf(sq.x, g.x, sq.y * g.x), fmaf(sq.x, g.y, sq.y * g.y));
-    } else {
-      float2 e = expi_ff(k4.x, k4.y, k4.z, zo.x, zo.y);
-      if (l < J - 1) {
-        const float2 e2 = expi_ff(k4.x, k4.y, k4.z, zo.z, zo.w);
-        e = e + make_float2(ar.z, ar.w) * e2;
-      }
-      const float2 g = make_float2(ar.x, ar.y) * e;
-      v = make_float2(sq.x * g.x, sq.x * g.y);
+    float2 e = expi_ff(k4.x, k4.y, k4.z, zo.x, zo.y);
+    if (l < J - 1) {
+      const float2 e2 = expi_ff(k4.x, k4.y, k4.z, zo.z, zo.w);
+      e = e + make_float2(ar.z, ar.w) * e2;
     }
+    const float2 g = make_float2(ar.x, ar.y) * e;
+    const float2 v = make_float2(sq * g.x, sq * g.y);
     d.g32[size_t(fn) * d.nzs + z] = v;
     mx = fmaxf(mx, sqrtf(v.x * v.x + v.y * v.y));
   }
@@ -569,8 +520,7 @@ cudaError_t launch_green(const Dev& d, cudaStream_t s, int tables) {
   }
   if (tables == GREEN_COEF) return cudaGetLastError();
   if (fast32) {
-    if (tables == GREEN_G32 && d.geom != EDT_GEOM_WINDOW) green_eval32_kernel<true><<<unsigned((long long)d.nf * d.nk), 256, 0, s>>>(d);
-    else green_eval32_kernel<false><<<unsigned((long long)d.nf * d.nk), 256, 0, s>>>(d);
+    green_eval32_kernel<<<unsigned((long long)d.nf * d.nk), 256, 0, s>>>(d);
   } else {
     Dev e = d;
     if (!(tables & (GREEN_G32 | GREEN_G32DF))) e.g32 = nullptr;

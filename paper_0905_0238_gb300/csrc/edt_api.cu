@@ -766,7 +766,8 @@ template <typename P> P at(edt_ctx* c, const Region& r) {
   return reinterpret_cast<P>(static_cast<char*>(c->ws) + r.off);
 }
 
-void bind(edt_ctx* c) {
+// The plan's numbers in the device structure, which launch counts read before there is a workspace.
+void bind_plan(edt_ctx* c) {
   Dev& d = c->dev;
   d.N = c->N; d.nk = c->nk; d.nz = c->nz; d.nf = c->nf; d.nsub = c->nsub; d.nlayer = c->nlayer;
   d.nzs = (c->nz + 1) & ~1;
@@ -775,6 +776,27 @@ void bind(edt_ctx* c) {
   d.chol_df = c->cfg.precision == EDT_MIXED && c->cfg.chol_df != 2 ? 1 : 0;
   d.chol_tc = d.chol_df && c->cfg.chol_df == 3 ? 1 : 0;
   d.alpha = c->cfg.alpha; d.dx = c->cfg.dx; d.dz = c->cfg.dz;
+  d.fchunk = c->fchunk;
+  d.rows_max_sub = c->rows_max_sub;
+  d.tune_bc = c->tune_bc; d.tune_rf = c->tune_rf; d.tune_zc = c->tune_zc;
+  d.geom = c->win ? EDT_GEOM_WINDOW : EDT_GEOM_LINE;
+  d.ny = c->ny; d.wx = c->wx; d.wy = c->wy; d.W = c->W; d.nxy = c->nxy; d.dy = c->cfg.dy;
+  d.fa_slab = c->win && c->ny > 1 ? fa_grid_slab(c->nz, fa_grid_slots(c->wx, c->wy), c->q_max) : 0;
+  d.ones_row = (long long)c->rows.size();
+  d.nseg = c->nslot; d.ncta_gram = c->ncta_gram;
+  d.f16 = c->r_gscale.bytes > 0;
+  d.resid_df = c->resid_df ? 1 : 0;
+  d.rf_stride = refine_stride(c->rows_max_sub);
+  d.refine_nodata = 0;
+  d.solver = c->cfg.solver;
+  d.tsvd_tol = c->cfg.tsvd_tol;
+  d.g64_split = c->cfg.precision == EDT_MIXED ? 1 : gram_f64_split(c->nz, c->nsub);
+  d.tlog_stride = c->r_tlog.bytes ? tsvd_log_doubles(c->nz) : 0;
+}
+
+void bind(edt_ctx* c) {
+  bind_plan(c);
+  Dev& d = c->dev;
   d.fc = at<const FreqConst*>(c, c->r_fc);
   d.layer_top = at<const double*>(c, c->r_ltop);
   d.layer_vel = at<const double*>(c, c->r_lvel);
@@ -783,11 +805,6 @@ void bind(edt_ctx* c) {
   d.rows = at<const uint32_t*>(c, c->r_rows);
   d.row_off = at<const long long*>(c, c->r_roff);
   d.row_off_mf = at<const long long*>(c, c->r_roffmf);
-  d.fchunk = c->fchunk;
-  d.rows_max_sub = c->rows_max_sub;
-  d.tune_bc = c->tune_bc; d.tune_rf = c->tune_rf; d.tune_zc = c->tune_zc;
-  d.geom = c->win ? EDT_GEOM_WINDOW : EDT_GEOM_LINE;
-  d.ny = c->ny; d.wx = c->wx; d.wy = c->wy; d.W = c->W; d.nxy = c->nxy; d.dy = c->cfg.dy;
   d.kval = c->win ? at<const double*>(c, c->r_kval) : nullptr;
   d.pair_m = at<const int*>(c, c->r_pairm);
   d.fj_off = at<const int*>(c, c->r_fjoff);
@@ -796,12 +813,10 @@ void bind(edt_ctx* c) {
   d.jmap = at<const int*>(c, c->r_jmap);
   d.q_xy = at<const int*>(c, c->r_qxy);
   d.q_rows = at<const int4*>(c, c->r_qrows);
-  d.fa_slab = c->win && c->ny > 1 ? fa_grid_slab(c->nz, fa_grid_slots(c->wx, c->wy), c->q_max) : 0;
   d.Gs = c->r_Gs.bytes ? at<float2*>(c, c->r_Gs) : nullptr;
   d.U = c->r_U.bytes ? at<float2*>(c, c->r_U) : nullptr;
   d.Dw = c->r_Dw.bytes ? at<float2*>(c, c->r_Dw) : nullptr;
   d.A32 = c->r_A32.bytes ? at<float2*>(c, c->r_A32) : nullptr;
-  d.ones_row = (long long)c->rows.size();
   d.band = at<const BandInfo*>(c, c->r_band);
   d.bcol = at<const int2*>(c, c->r_bcol);
   d.cpre = at<const long long*>(c, c->r_cpre);
@@ -815,7 +830,6 @@ void bind(edt_ctx* c) {
   d.seg_nrow = at<const long long*>(c, c->r_segn);
   d.cta_seg0 = at<const int*>(c, c->r_ctas);
   d.m_slot0 = at<const int*>(c, c->r_mslot);
-  d.nseg = c->nslot; d.ncta_gram = c->ncta_gram;
   d.coef = at<double2*>(c, c->r_coef);
   d.coef32 = c->r_coef32.bytes ? at<float*>(c, c->r_coef32) : nullptr;
   d.z_off32 = at<const float*>(c, c->r_zo32);
@@ -825,8 +839,6 @@ void bind(edt_ctx* c) {
   d.g32lo = c->r_g32lo.bytes ? at<float2*>(c, c->r_g32lo) : nullptr;
   d.rowmax = c->r_rowmax.bytes ? at<float*>(c, c->r_rowmax) : nullptr;
   d.gscale = c->r_gscale.bytes ? at<int2*>(c, c->r_gscale) : nullptr;
-  d.f16 = d.gscale != nullptr;
-  d.resid_df = c->resid_df ? 1 : 0;
   d.rowtab32 = c->win ? d.A32 : d.g32;
   d.X = at<void*>(c, c->r_X);
   d.Dstage = at<void*>(c, c->r_Dst);
@@ -844,7 +856,6 @@ void bind(edt_ctx* c) {
   d.x = at<double*>(c, c->r_x);
   d.r = at<double*>(c, c->r_r);
   d.rpart = c->r_rpart.bytes ? at<double*>(c, c->r_rpart) : nullptr;
-  d.rf_stride = refine_stride(c->rows_max_sub);
   d.vhat = at<double2*>(c, c->r_vhat);
   d.vfull = at<double2*>(c, c->r_vfull);
   d.gscr = c->r_gscr.bytes ? at<double2*>(c, c->r_gscr) : nullptr;
@@ -859,16 +870,11 @@ void bind(edt_ctx* c) {
   d.gam = c->r_gam.bytes ? at<double*>(c, c->r_gam) : nullptr;
   d.tref = c->r_tref.bytes ? at<const int2*>(c, c->r_tref) : nullptr;
   d.tref_off = c->r_treoff.bytes ? at<const long long*>(c, c->r_treoff) : nullptr;
-  d.refine_nodata = 0;
   d.status = at<int*>(c, c->r_status);
   d.flags = at<unsigned*>(c, c->r_flags);
-  d.solver = c->cfg.solver;
-  d.tsvd_tol = c->cfg.tsvd_tol;
-  d.g64_split = c->cfg.precision == EDT_MIXED ? 1 : gram_f64_split(c->nz, c->nsub);
   d.g64part = c->r_g64part.bytes ? at<double*>(c, c->r_g64part) : nullptr;
   d.b64part = c->r_b64part.bytes ? at<double*>(c, c->r_b64part) : nullptr;
   d.tlog = c->r_tlog.bytes ? at<double*>(c, c->r_tlog) : nullptr;
-  d.tlog_stride = c->r_tlog.bytes ? tsvd_log_doubles(c->nz) : 0;
   const bool disk = c->r_kzP.bytes > 0;
   d.kz_P = disk ? at<const double*>(c, c->r_kzP) : nullptr;
   d.kz_p = disk ? at<const int*>(c, c->r_kzp) : nullptr;
@@ -1040,6 +1046,7 @@ int edt_create(edt_ctx** out, const edt_config* cfg, size_t* workspace_bytes) {
                 (c->cfg.resid == 2 || (c->cfg.resid == 0 && c->cfg.alpha < kResidDfAlpha));
   plan(c);
   layout(c);
+  bind_plan(c);
   if (workspace_bytes) *workspace_bytes = c->ws_bytes;
   *out = c;
   return EDT_OK;
@@ -1143,6 +1150,7 @@ static int apply_tuning(edt_ctx* c) {
     const double cmin = *std::min_element(c->vel.begin(), c->vel.end());
     plan_band(c, cmin);
   }
+  bind_plan(c);
   if (!c->ws) return EDT_OK;
   bind(c);
   if (c->band_mode) {
@@ -1602,7 +1610,7 @@ int edt_get_stats(edt_ctx* c, edt_stats* o) {
   // misfit gradient: green, zero, lateral DFT and its FP32 copy, per chunk transform (2), the
   // residual (2) and two contractions, depth march states / field / recursions / layer sums (4), inverse
   // lateral DFT, finalize
-  o->launches_per_grad = grad_supported(c->dev) && c->fchunk > 0
+  o->launches_per_grad = c->r_gscr.bytes > 0 && c->fchunk > 0
                              ? green_launches(c->dev, GREEN_G32) + 3 + 6 * ((c->nf + c->fchunk - 1) / c->fchunk) + 6 : 0;
   o->gram_rows_padded = 0;
   for (long long n : c->seg_nrow) o->gram_rows_padded += (n + TC_KC - 1) / TC_KC * TC_KC;

@@ -274,3 +274,34 @@ def test_ranged_and_sharded_row_plans_without_gpu():
         with pytest.raises(edt.EdtError) as ei:
             edt.edt_create(c)
         assert ei.value.code == edt.EDT_EINVAL
+
+
+def _launches(**kw):
+    import numpy as np
+    from paper_0905_0238_gb300 import edt, Config
+    n = kw.pop("nlayer", 3)
+    cfg = Config(**{**dict(nx=64, dx=10.0, nz=40, dz=10.0, z0=0.0, freq_hz=np.array([8.0, 15.0, 25.0]), eps=0.15,
+                           layer_top=np.arange(n) * (400.0 / n), layer_vel=np.linspace(1500.0, 3000.0, n),
+                           alpha=1e-2, cutoff=1.0), **kw})
+    ctx, _ = edt.edt_create(cfg.c_config()[0])
+    try:
+        st = edt.edt_get_stats(ctx)
+        return st.launches_per_invert, st.launches_per_grad
+    finally:
+        edt.edt_destroy(ctx)
+
+
+def test_launch_counts_before_there_is_a_workspace():
+    """edt_get_stats on a context without a workspace counts what the plan launches: the march's
+    kernels follow the layers (three up to 32 layers with FP32 coefficients, four above), the
+    gradients exist where they are planned, and a window grid has three kernels per frequency."""
+    from paper_0905_0238_gb300 import edt
+    few, few_grad = _launches(precision=edt.EDT_MIXED, nlayer=32)
+    many, _ = _launches(precision=edt.EDT_MIXED, nlayer=33)
+    assert many == few + 1
+    assert few_grad > 0 and _launches(precision=edt.EDT_FP64)[1] == 0
+    win = dict(geometry=edt.EDT_GEOM_WINDOW, precision=edt.EDT_MIXED, fold=0, wx=4, dy=10.0, refine=0)
+    line = _launches(ny=1, wy=1, **win)[0]
+    grid = _launches(ny=64, wy=4, **win)[0]
+    assert grid == line + 1                  # three kernels per frequency each; one more inverse pass
+    assert _launches(ny=64, wy=4, **{**win, "refine": 1})[0] == grid + 3

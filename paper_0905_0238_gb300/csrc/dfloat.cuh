@@ -89,7 +89,7 @@ struct DfDiagScratch {
   float2 ls[3][32];                               // column j of L over L_jj (three in use at a time)
   float2 xr[2][32];                               // finished rows of U (below)
   float2 inv[32];                                 // 1 / L_jj
-  int fail;
+  int fail[2];                                    // column j failed: slot j & 1
 };
 
 // Diagonal block of step k0 of one subproblem (kb = min(32, n - k0) columns), factored and
@@ -116,7 +116,7 @@ __device__ inline bool df_diag_block(float2* A, float* L32, double* dinv, float*
     const int i = warp + 8 * q;
     sh.col[lane][i] = i < kb && lane <= i ? A[size_t(k0 + i) * n + k0 + lane] : zero;
   }
-  if (threadIdx.x == 0) sh.fail = 0;
+  if (threadIdx.x < 2) sh.fail[threadIdx.x] = 0;
   if (threadIdx.x < 64) sh.xr[threadIdx.x >> 5][lane] = zero;
   if (threadIdx.x < 96) sh.ls[threadIdx.x >> 5][lane] = zero;
   __syncthreads();
@@ -127,7 +127,7 @@ __device__ inline bool df_diag_block(float2* A, float* L32, double* dinv, float*
   auto column = [&](int j, float2& v) {
     const float2 d = df_norm(shfl_df(v, j));
     if (!(d.x > 0.f) || !isfinite(d.x)) {
-      if (lane == 0) sh.fail = 1;
+      if (lane == 0) sh.fail[j & 1] = 1;
       return;
     }
     const float2 iv = df_rsqrt(d);
@@ -142,7 +142,9 @@ __device__ inline bool df_diag_block(float2* A, float* L32, double* dinv, float*
   if (warp == 0) column(0, w[0]);
   __syncthreads();
   for (int j = 0; j < kb; ++j) {
-    if (sh.fail) break;                           // the same value in every thread
+    // published before the last barrier; column j + 1, which another warp may be working on
+    // already, has the other slot: every thread leaves at the same step
+    if (sh.fail[j & 1]) break;
     // columns c > j: A -= L_j L_j^T (rows above c are not used); c < j: U_i -= (L_i,j-1 / L_j-1,j-1) U_j-1
     // for the rows i >= j, the others and column j subtract zero
     const float2 lj = df_neg(sh.col[j][lane]);
@@ -163,7 +165,7 @@ __device__ inline bool df_diag_block(float2* A, float* L32, double* dinv, float*
       if (j + 1 < kb && warp + 8 * q == j + 1) column(j + 1, w[q]);
     __syncthreads();
   }
-  if (sh.fail) {
+  if (sh.fail[0] | sh.fail[1]) {                  // uniform: no column was formed since the last barrier
     if (threadIdx.x == 0) *status = EDT_ENOTPD;
     return false;
   }

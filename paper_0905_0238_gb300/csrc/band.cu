@@ -221,12 +221,11 @@ cudaError_t run_chunk(const Dev& d, const BandChunk& ch, const void* D, int D_dt
 
 template <class F>
 cudaError_t prepare_policy() {
-  cudaError_t e = cudaFuncSetAttribute(band_cols_kernel<F, 4>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       int(cols_smem<F>(4)));
+  cudaError_t e = allow_smem(band_cols_kernel<F, 4>, int(cols_smem<F>(4)));
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(band_cols_kernel<F, 8>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(cols_smem<F>(8)));
+    e = allow_smem(band_cols_kernel<F, 8>, int(cols_smem<F>(8)));
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(band_cols_kernel<F, 16>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(cols_smem<F>(16)));
+    e = allow_smem(band_cols_kernel<F, 16>, int(cols_smem<F>(16)));
   return e;
 }
 

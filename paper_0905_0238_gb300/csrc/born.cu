@@ -556,10 +556,9 @@ __global__ void __launch_bounds__(256) born_resid_edge_kernel(Dev d, int f0) {
 }  // namespace
 
 cudaError_t prepare_born() {
-  const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
-  cudaError_t e = cudaFuncSetAttribute(born_fwd_df_kernel, attr, int(tile_smem<float4>()));
+  cudaError_t e = allow_smem(born_fwd_df_kernel, int(tile_smem<float4>()));
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(born_fwd_f64_kernel, attr, int(tile_smem<double2>()));
+  return allow_smem(born_fwd_f64_kernel, int(tile_smem<double2>()));
 }
 
 cudaError_t launch_born_prep(const Dev& d, cudaStream_t s) {

@@ -701,8 +701,7 @@ int chol_launches(int nz) { return 1; }
 static size_t chol_smem(int nz) { return (size_t(nz) * LDP + NB * LDP + 2 * nz + 40) * sizeof(double); }
 
 cudaError_t prepare_chol(const Dev& d) {
-  cudaError_t e = cudaFuncSetAttribute(chol_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       int(chol_smem(d.nz)));
+  cudaError_t e = allow_smem(chol_kernel<false>, int(chol_smem(d.nz)));
   if (e != cudaSuccess) return e;
   return prepare_chol_dfloat(d);
 }
@@ -731,8 +730,7 @@ cudaError_t launch_refine_update(const Dev& d, cudaStream_t s) {
 // Streaming batches: subproblem m has size sub_n[m] <= nmax; lam = trace[m] (trace_mode 1
 // with alpha = 1: the caller accumulates alpha * trace).
 cudaError_t prepare_chol_var(int nmax) {
-  return cudaFuncSetAttribute(chol_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              int(chol_smem(nmax)));
+  return allow_smem(chol_kernel<true>, int(chol_smem(nmax)));
 }
 
 int chol_block_cols() { return NB; }

@@ -501,13 +501,11 @@ int chol_dfloat_launches(int n) {
 }
 
 cudaError_t prepare_chol_dfloat(const Dev& d) {
-  cudaError_t e = cudaFuncSetAttribute(cdf_final_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       int(cdf_final_smem(d.nz)));
+  cudaError_t e = allow_smem(cdf_final_kernel, int(cdf_final_smem(d.nz)));
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(cdf_update_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, TCU_SMEM);
+  e = allow_smem(cdf_update_tc_kernel, TCU_SMEM);
   if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(cdf_resolve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              int(cdf_final_smem(d.nz)));
+  return allow_smem(cdf_resolve_kernel, int(cdf_final_smem(d.nz)));
 }
 
 cudaError_t launch_chol_dfloat_resolve(const Dev& d, cudaStream_t s) {

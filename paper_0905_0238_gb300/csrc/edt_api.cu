@@ -30,6 +30,15 @@ struct Region { size_t off = 0, bytes = 0; };
 
 int record_cuda_error(cudaError_t e) { return cuda_fail(e); }
 
+cudaError_t allow_smem(const void* f, size_t bytes) {
+  static std::mutex mu;
+  std::lock_guard<std::mutex> lk(mu);
+  cudaFuncAttributes a;
+  const cudaError_t e = cudaFuncGetAttributes(&a, f);
+  if (e != cudaSuccess || size_t(a.maxDynamicSharedSizeBytes) >= bytes) return e;
+  return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
+}
+
 // Most complex rows one FP32 tensor-memory accumulation of the Gram covers (a segment);
 // longer runs are split into several segments, each flushed to its own partial tile.
 // Damping below which the automatic residual mode switches to double-float: with FP32

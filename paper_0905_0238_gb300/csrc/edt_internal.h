@@ -207,6 +207,15 @@ struct Dev {
 // Record a CUDA error for edt_last_cuda_error; returns EDT_ECUDA.
 int record_cuda_error(cudaError_t e);
 
+// Dynamic shared memory of at least `bytes` for kernel f on the current device.  The limit belongs
+// to the kernel, for every context of the process, so it is only ever raised: a context with fewer
+// depths leaves the launches of a larger one alone.  May be called by several threads at once.
+cudaError_t allow_smem(const void* f, size_t bytes);
+template <class... A>
+inline cudaError_t allow_smem(void (*kernel)(A...), size_t bytes) {
+  return allow_smem(reinterpret_cast<const void*>(kernel), bytes);
+}
+
 // ---- launchers (each returns cudaGetLastError()) ---------------------------------------
 constexpr int GREEN_G64 = 1, GREEN_G32 = 2, GREEN_G32DF = 4;   // tables launch_green writes
 constexpr int GS_SLOTS = 12;    // of gscr (csrc/grad.cu)

@@ -443,15 +443,14 @@ cudaError_t dwin_for(const Dev& d, const TIN* D, cudaStream_t s) {
 template <int PX, int PY>
 cudaError_t prepare_plane() {
   const int sm = int(plane_smem<PX, PY>());
-  const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e;
   if constexpr (PY == 0) {
-    if ((e = cudaFuncSetAttribute(fa_gspace_kernel<PX>, attr, sm)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(fa_mrows_kernel<PX, 2>, attr, sm)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(fa_mrows_kernel<PX, 4>, attr, sm)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(fa_mrows_kernel<PX, 8>, attr, sm)) != cudaSuccess) return e;
+    if ((e = allow_smem(fa_gspace_kernel<PX>, sm)) != cudaSuccess) return e;
+    if ((e = allow_smem(fa_mrows_kernel<PX, 2>, sm)) != cudaSuccess) return e;
+    if ((e = allow_smem(fa_mrows_kernel<PX, 4>, sm)) != cudaSuccess) return e;
+    if ((e = allow_smem(fa_mrows_kernel<PX, 8>, sm)) != cudaSuccess) return e;
   }
-  return cudaFuncSetAttribute(fa_drhs_kernel<PX, PY>, attr, sm);
+  return allow_smem(fa_drhs_kernel<PX, PY>, sm);
 }
 
 // plane shapes: (nx, ny) = (32 PX, 32 PY), PY = 0 for a line
@@ -519,8 +518,8 @@ cudaError_t prepare_fa(const Dev& d) {
   cudaError_t e = cudaSuccess;
   switch (d.wx * 32 + d.wy) {
 #define FA_A(WX, WY) case WX * 32 + WY: \
-    e = cudaFuncSetAttribute(fa_dwin_kernel<WX, WY, float2>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(ExLayout<WX, WY>::SIZE * sizeof(float2))); \
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(fa_dwin_kernel<WX, WY, double2>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(ExLayout<WX, WY>::SIZE * sizeof(float2))); \
+    e = allow_smem(fa_dwin_kernel<WX, WY, float2>, int(ExLayout<WX, WY>::SIZE * sizeof(float2))); \
+    if (e == cudaSuccess) e = allow_smem(fa_dwin_kernel<WX, WY, double2>, int(ExLayout<WX, WY>::SIZE * sizeof(float2))); \
     break;
     FA_A(1, 1) FA_A(2, 1) FA_A(4, 1) FA_A(8, 1) FA_A(16, 1)
     FA_A(2, 2) FA_A(4, 4) FA_A(8, 8) FA_A(16, 16) FA_A(4, 2) FA_A(8, 4) FA_A(16, 8)

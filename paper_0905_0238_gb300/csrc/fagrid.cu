@@ -458,8 +458,8 @@ cudaError_t planes_for(const Dev& d, const int* qxy, int nq, int2 qmax, int z0, 
 
 template <int N>
 cudaError_t prepare_n() {
-  cudaError_t e = cudaFuncSetAttribute(grid_gspace_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, Half<N>::SMEM);
-  return e != cudaSuccess ? e : cudaFuncSetAttribute(grid_planes_kernel<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, Half<N>::SMEM);
+  cudaError_t e = allow_smem(grid_gspace_kernel<N>, Half<N>::SMEM);
+  return e != cudaSuccess ? e : allow_smem(grid_planes_kernel<N>, Half<N>::SMEM);
 }
 
 }  // namespace
@@ -508,7 +508,7 @@ cudaError_t prepare_fa_grid(const Dev& d) {
   if (e != cudaSuccess) return e;
   switch (d.wx * 32 + d.wy) {
 #define GA(WX, WY) case WX * 32 + WY: \
-    return cudaFuncSetAttribute(grid_rows_kernel<WX, WY>, cudaFuncAttributeMaxDynamicSharedMemorySize, rows_smem<WX, WY>());
+    return allow_smem(grid_rows_kernel<WX, WY>, rows_smem<WX, WY>());
     GRID_WINDOWS(GA)
 #undef GA
     default: return cudaErrorInvalidValue;

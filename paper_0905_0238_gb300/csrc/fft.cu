@@ -225,7 +225,7 @@ template <int P>
 cudaError_t wfft_cols_prepare() {
   constexpr int N = 32 * P, WC = P >= 32 ? 8 : 16;
   const size_t smem = size_t(WC) * (N + N / 16 + 1) * sizeof(float2);
-  return cudaFuncSetAttribute(wfft_cols_kernel<P, WC>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem));
+  return allow_smem(wfft_cols_kernel<P, WC>, int(smem));
 }
 
 // FP32 row / column transforms for N >= 32 (warp FFT); false if N is outside that range
@@ -386,30 +386,21 @@ cudaError_t launch_transform(const Dev& d, const void* D, int D_dtype, int f0, i
 template cudaError_t launch_transform<float>(const Dev&, const void*, int, int, int, cudaStream_t);
 template cudaError_t launch_transform<double>(const Dev&, const void*, int, int, int, cudaStream_t);
 
-// Opt-in shared-memory sizes of this file's kernels, set once per context (outside any
-// stream capture).
+// Opt-in shared-memory sizes of this file's kernels, allowed when a context gets its workspace
+// (outside any stream capture).
 cudaError_t prepare_fft(const Dev& d) {
   const int N = d.N;
   const int rpb32 = std::max(1, 4096 / N), rpb64 = std::max(1, 2048 / N);
   const int cpb32 = std::min(N, 16), cpb64 = std::min(N, 8);
   const size_t inv = size_t(INV_ZT) * (padded_len(N) + 1) * sizeof(double2);
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(fft_rows_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                int(size_t(rpb32) * padded_len(N) * sizeof(float2)))) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(fft_rows_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                int(size_t(rpb64) * padded_len(N) * sizeof(double2)))) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(fft_cols_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                int(size_t(cpb32) * (padded_len(N) + 1) * sizeof(float2)))) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(fft_cols_kernel<double>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                int(size_t(cpb64) * (padded_len(N) + 1) * sizeof(double2)))) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(inverse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(inv))) != cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(lateral_dft_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(inv))) !=
-      cudaSuccess)
-    return e;
-  if ((e = cudaFuncSetAttribute(lateral_idft_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(inv))) !=
-      cudaSuccess)
-    return e;
+  if ((e = allow_smem(fft_rows_kernel<float>, int(size_t(rpb32) * padded_len(N) * sizeof(float2)))) != cudaSuccess) return e;
+  if ((e = allow_smem(fft_rows_kernel<double>, int(size_t(rpb64) * padded_len(N) * sizeof(double2)))) != cudaSuccess) return e;
+  if ((e = allow_smem(fft_cols_kernel<float>, int(size_t(cpb32) * (padded_len(N) + 1) * sizeof(float2)))) != cudaSuccess) return e;
+  if ((e = allow_smem(fft_cols_kernel<double>, int(size_t(cpb64) * (padded_len(N) + 1) * sizeof(double2)))) != cudaSuccess) return e;
+  if ((e = allow_smem(inverse_kernel, int(inv))) != cudaSuccess) return e;
+  if ((e = allow_smem(lateral_dft_kernel, int(inv))) != cudaSuccess) return e;
+  if ((e = allow_smem(lateral_idft_kernel, int(inv))) != cudaSuccess) return e;
   switch (N) {
     case 32: return wfft_cols_prepare<1>();
     case 64: return wfft_cols_prepare<2>();

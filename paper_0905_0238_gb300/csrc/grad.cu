@@ -921,12 +921,11 @@ cudaError_t launch_invert_vjp(const Dev& d0, const void* Vbar, int Vbar_dtype, v
 }
 
 cudaError_t prepare_grad() {
-  const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
   cudaError_t e;
-  if ((e = cudaFuncSetAttribute(grad_vhat_kernel<1>, attr, VhatShape<1>::SMEM)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(grad_vhat_kernel<2>, attr, VhatShape<2>::SMEM)) != cudaSuccess) return e;
-  if ((e = cudaFuncSetAttribute(grad_gbar_kernel<1>, attr, GbarShape<1>::SMEM)) != cudaSuccess) return e;
-  return cudaFuncSetAttribute(grad_gbar_kernel<2>, attr, GbarShape<2>::SMEM);
+  if ((e = allow_smem(grad_vhat_kernel<1>, VhatShape<1>::SMEM)) != cudaSuccess) return e;
+  if ((e = allow_smem(grad_vhat_kernel<2>, VhatShape<2>::SMEM)) != cudaSuccess) return e;
+  if ((e = allow_smem(grad_gbar_kernel<1>, GbarShape<1>::SMEM)) != cudaSuccess) return e;
+  return allow_smem(grad_gbar_kernel<2>, GbarShape<2>::SMEM);
 }
 
 bool grad_supported(const Dev& d) {

@@ -197,7 +197,7 @@ size_t gram_f64_part_doubles(int nz, int nsub) {
 }
 
 cudaError_t prepare_gram_f64(const Dev& d) {
-  return cudaFuncSetAttribute(gram_f64_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(gram_smem(d.nz)));
+  return allow_smem(gram_f64_kernel, int(gram_smem(d.nz)));
 }
 
 cudaError_t launch_gram_f64(const Dev& d, cudaStream_t s) {

@@ -629,12 +629,9 @@ static int tc_smem_bytes(const Dev& d) {
 
 cudaError_t prepare_gram_tc(const Dev& d) {
   const int smem = tc_smem_bytes(d);
-  const auto attr = cudaFuncAttributeMaxDynamicSharedMemorySize;
   if (d.f16)
-    return d.passes == 3 ? cudaFuncSetAttribute(gram_tc_kernel<3, true>, attr, smem)
-                         : cudaFuncSetAttribute(gram_tc_kernel<1, true>, attr, smem);
-  return d.passes == 3 ? cudaFuncSetAttribute(gram_tc_kernel<3, false>, attr, smem)
-                       : cudaFuncSetAttribute(gram_tc_kernel<1, false>, attr, smem);
+    return d.passes == 3 ? allow_smem(gram_tc_kernel<3, true>, smem) : allow_smem(gram_tc_kernel<1, true>, smem);
+  return d.passes == 3 ? allow_smem(gram_tc_kernel<3, false>, smem) : allow_smem(gram_tc_kernel<1, false>, smem);
 }
 
 int gram_scale_launches(const Dev& d, bool rowmax_ready) {

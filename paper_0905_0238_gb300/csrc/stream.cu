@@ -514,8 +514,7 @@ __global__ void __launch_bounds__(256) st_rsum_kernel(StBatch b) {
 int st_gram_smem_bytes() { return GS_STAGES * GS_STAGE + 1024 + 128; }
 
 cudaError_t prepare_stream() {
-  cudaError_t e = cudaFuncSetAttribute(st_gram_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       st_gram_smem_bytes());
+  cudaError_t e = allow_smem(st_gram_kernel, st_gram_smem_bytes());
   if (e != cudaSuccess) return e;
   return prepare_chol_var(ST_MAX_NZ);
 }

@@ -347,8 +347,7 @@ size_t tsvd_log_doubles(int p) {
 
 cudaError_t prepare_variants(int nz) {
   if (nz > TSVD_MAX_NZ) return cudaSuccess;
-  return cudaFuncSetAttribute(tsvd_jacobi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              int(tsvd_smem_bytes(nz)));
+  return allow_smem(tsvd_jacobi_kernel, int(tsvd_smem_bytes(nz)));
 }
 
 cudaError_t launch_solve_variant(const Dev& d, cudaStream_t s) {

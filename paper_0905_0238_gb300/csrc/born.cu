@@ -227,8 +227,29 @@ __global__ void __launch_bounds__(PREP_THREADS) born_prep_kernel(Dev d, double2*
   if (threadIdx.x == 0) exps[row] = e;
 }
 
-// Vhat rows rounded to FP32 in place (row m's float2 values at the start of its FP64 row)
-__global__ void __launch_bounds__(PREP_THREADS) born_v32_kernel(Dev d) {
+// exponent e with |v| < 2^e (both components), by their bits; non-finite: above any finite one
+__device__ __forceinline__ int exp_above(double2 v) {
+  return max((__double2hiint(v.x) >> 20) & 0x7ff, (__double2hiint(v.y) >> 20) & 0x7ff) - 1022;
+}
+
+// Vhat for the misfit: FP32 in place (row m's float2 values at the start of its FP64 row), all of it
+// times one power of two 2^-e with the largest component just under 1, e in exps[0].  The products
+// residual x Vhat x table then neither vanish nor overflow where their sum does not: with Vhat as it
+// is, dJ/dc lost digits for models and data 1e-17 of the usual size and was not finite at 1e20 times.
+__global__ void __launch_bounds__(PREP_THREADS) born_vexp_kernel(Dev d, int* rowe) {
+  const double2* r = d.vfull + size_t(blockIdx.x) * d.nz;
+  int e = -1022;
+  for (int z = threadIdx.x; z < d.nz; z += PREP_THREADS) e = max(e, exp_above(r[z]));
+  __shared__ int red[PREP_THREADS / 32];
+  e = __reduce_max_sync(0xffffffffu, e);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e;
+  __syncthreads();
+  if (threadIdx.x == 0) rowe[blockIdx.x] = max(max(red[0], red[1]), max(red[2], red[3]));
+}
+
+__global__ void __launch_bounds__(PREP_THREADS) born_v32_kernel(Dev d, const int* rowe, int* exps) {
+  static_assert(PREP_THREADS == 128, "four warps");
+  __shared__ int red[PREP_THREADS / 32];
   double2* r = d.vfull + size_t(blockIdx.x) * d.nz;
   double2 v[PREP_Q];
 #pragma unroll
@@ -236,12 +257,20 @@ __global__ void __launch_bounds__(PREP_THREADS) born_v32_kernel(Dev d) {
     const int z = threadIdx.x + PREP_THREADS * i;
     v[i] = z < d.nz ? r[z] : make_double2(0.0, 0.0);
   }
-  __syncthreads();
+  int e = -1022;
+  for (int m = threadIdx.x; m < d.N; m += PREP_THREADS) e = max(e, rowe[m]);
+  e = __reduce_max_sync(0xffffffffu, e);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e;
+  __syncthreads();                      // and every element of the row has been read
+  // a factor that stays normal in FP32 on either side; values beyond it have their own rounding
+  e = max(-100, min(100, max(max(red[0], red[1]), max(red[2], red[3]))));
+  const double sc = __hiloint2double((1023 - e) << 20, 0);                  // 2^-e
 #pragma unroll
   for (int i = 0; i < PREP_Q; ++i) {
     const int z = threadIdx.x + PREP_THREADS * i;
-    if (z < d.nz) reinterpret_cast<float2*>(r)[z] = make_float2(float(v[i].x), float(v[i].y));
+    if (z < d.nz) reinterpret_cast<float2*>(r)[z] = make_float2(float(sc * v[i].x), float(sc * v[i].y));
   }
+  if (blockIdx.x == 0 && threadIdx.x == 0) exps[0] = e;
 }
 
 // ---- forward model -----------------------------------------------------------------------
@@ -425,10 +454,37 @@ __global__ void __launch_bounds__(256) born_fwd_edge_f64_kernel(Dev d, int f0) {
 // ---- residual and folding ----------------------------------------------------------------
 __device__ __forceinline__ float4 pack2(float2 a, float2 b) { return make_float4(a.x, a.y, b.x, b.y); }
 
-__device__ __forceinline__ void add_sq(float2& acc, float2 r, float w) {
-  df_acc(acc, make_float2(w * r.x, 0.f), make_float2(r.x, 0.f));     // w a power of two
-  df_acc(acc, make_float2(w * r.y, 0.f), make_float2(r.y, 0.f));
-}
+// Sum of squares as a float pair times 2^(2 e), e the largest exponent met: the squares of FP32 values
+// leave the FP32 range long before their FP64 sum would.
+struct SumSq {
+  float2 acc = make_float2(0.f, 0.f);
+  int e = -126;
+  __device__ __forceinline__ static float pow2(int n) { return __int_as_float((127 + n) << 23); }   // |n| <= 126
+  // w1 times the squares of the first half of r, w2 times those of the second (powers of two)
+  template <int K>
+  __device__ __forceinline__ void add(const float2 (&r)[K], float w1, float w2) {
+    float m = 0.f;
+#pragma unroll
+    for (int i = 0; i < K; ++i) m = fmaxf(m, fmaxf(fabsf(r[i].x), fabsf(r[i].y)));
+    const int en = min(126, (__float_as_int(m) >> 23) - 126);
+    if (en > e) {
+      const float k = pow2(max(e - en, -126));
+      acc = k * (k * acc);
+      e = en;
+    }
+    const float sc = pow2(-e);
+#pragma unroll
+    for (int i = 0; i < K; ++i) {
+      const float w = i < K / 2 ? w1 : w2, x = sc * r[i].x, y = sc * r[i].y;
+      df_acc(acc, make_float2(w * x, 0.f), make_float2(x, 0.f));
+      df_acc(acc, make_float2(w * y, 0.f), make_float2(y, 0.f));
+    }
+  }
+  __device__ __forceinline__ double value() const {
+    // (an infinite sum: its error terms are NaN)
+    return (isfinite(acc.x) ? df_val(acc) : double(acc.x)) * __hiloint2double((1023 + 2 * e) << 20, 0);
+  }
+};
 
 __device__ __forceinline__ double block_sum(double v, double* red) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
@@ -466,7 +522,8 @@ __global__ void __launch_bounds__(BTHREADS, 3) born_resid_kernel(Dev d, int f0) 
   float4* T = E + size_t(nk) * nk;
   const FreqConst fc = d.fc[f];
   const float2 rot = make_float2(float(fc.rot_re), float(fc.rot_im));   // conj(s_f) / |s_f|
-  float2 jp = make_float2(0.f, 0.f);
+  const float ve = RES ? __int_as_float((127 + d.born_exp[0]) << 23) : 1.f;      // the scale of Vhat
+  SumSq jp;
 #pragma unroll
   for (int a = 0; a < 2; ++a)
 #pragma unroll
@@ -479,14 +536,15 @@ __global__ void __launch_bounds__(BTHREADS, 3) born_resid_kernel(Dev d, int f0) 
       if (RES) {
         const float2 ph = cconj(rot);
         const float* s = acc[a][b].s;
-        const float2 f1 = ph * make_float2(s[0] - s[3], s[1] + s[2]), f2 = ph * make_float2(s[0] + s[3], s[1] - s[2]);
-        const float2 h1 = ph * make_float2(s[4] - s[7], s[5] + s[6]), h2 = ph * make_float2(s[4] + s[7], s[5] - s[6]);
+        const float2 f1 = ve * (ph * make_float2(s[0] - s[3], s[1] + s[2]));
+        const float2 f2 = ve * (ph * make_float2(s[0] + s[3], s[1] - s[2]));
+        const float2 h1 = ve * (ph * make_float2(s[4] - s[7], s[5] + s[6]));
+        const float2 h2 = ve * (ph * make_float2(s[4] + s[7], s[5] - s[6]));
         r[0] = f1 - r[0]; r[1] = f1 - r[1]; r[2] = f2 - r[2]; r[3] = f2 - r[3];
         r[4] = h1 - r[4]; r[5] = h1 - r[5]; r[6] = h2 - r[6]; r[7] = h2 - r[7];
         // every distinct entry once: l = 0 names its entries twice, k = l the two of each kind
         const float w1 = k == l ? (l == 0 ? 0.25f : 0.5f) : 1.f, w2 = l == 0 ? 0.f : w1;
-#pragma unroll
-        for (int i = 0; i < 4; ++i) { add_sq(jp, r[i], w1); add_sq(jp, r[4 + i], w2); }
+        jp.add(r, w1, w2);
       }
       const float2 S = rot * (r[0] + r[1]), S2 = rot * (r[2] + r[3]);
       const float2 U = rot * (r[4] + r[5]), U2 = rot * (r[6] + r[7]);
@@ -496,7 +554,7 @@ __global__ void __launch_bounds__(BTHREADS, 3) born_resid_kernel(Dev d, int f0) 
       T[size_t(l) * nk + k] = pack2(U, U2);
     }
   if (RES) {
-    const double t = block_sum(df_val(jp), red);
+    const double t = block_sum(jp.value(), red);
     if (threadIdx.x == 0) atomicAdd(d.gacc, t);
   }
 }
@@ -531,13 +589,14 @@ __global__ void __launch_bounds__(256) born_resid_edge_kernel(Dev d, int f0) {
       float2 r[4] = {X[size_t(l) * N + H], X[size_t(H) * N + nl_], X[size_t(H) * N + l], X[size_t(nl_) * N + H]};
       if (RES) {
         const float2 ph = cconj(rot);
-        const float2 f1 = ph * make_float2(p.x - q.y, p.y + q.x), f2 = ph * make_float2(p.x + q.y, p.y - q.x);
+        const float ve = __int_as_float((127 + d.born_exp[0]) << 23);            // the scale of Vhat
+        const float2 f1 = ve * (ph * make_float2(p.x - q.y, p.y + q.x));
+        const float2 f2 = ve * (ph * make_float2(p.x + q.y, p.y - q.x));
         r[0] = f1 - r[0]; r[1] = f1 - r[1]; r[2] = f2 - r[2]; r[3] = f2 - r[3];
-        float2 j2 = make_float2(0.f, 0.f);
         const float w = l == 0 ? 0.5f : (l == H ? 0.25f : 1.f);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) add_sq(j2, r[i], w);
-        jp = df_val(j2);
+        SumSq sq;
+        sq.add(r, w, w);
+        jp = sq.value();
       }
       float4* E = d.born_fold + size_t(fi) * 2 * nk * nk;
       float4* T = E + size_t(nk) * nk;
@@ -568,7 +627,9 @@ cudaError_t launch_born_prep(const Dev& d, cudaStream_t s) {
 }
 
 cudaError_t launch_born_v32(const Dev& d, cudaStream_t s) {
-  born_v32_kernel<<<d.N, PREP_THREADS, 0, s>>>(d);
+  int* rowe = d.born_exp + size_t(d.nf) * d.nk;
+  born_vexp_kernel<<<d.N, PREP_THREADS, 0, s>>>(d, rowe);
+  born_v32_kernel<<<d.N, PREP_THREADS, 0, s>>>(d, rowe, d.born_exp);
   return cudaGetLastError();
 }
 

@@ -1616,11 +1616,11 @@ int edt_get_stats(edt_ctx* c, edt_stats* o) {
                              (c->ny > 1 ? 4 : 3);
   }
   o->freq_chunk = c->band_mode ? c->band_maxplanes : c->fchunk;
-  // misfit gradient: green, zero, lateral DFT and its FP32 copy, per chunk transform (2), the
+  // misfit gradient: green, zero, lateral DFT and its scaled FP32 copy (2), per chunk transform (2), the
   // residual (2) and two contractions, depth march states / field / recursions / layer sums (4), inverse
   // lateral DFT, finalize
   o->launches_per_grad = c->r_gscr.bytes > 0 && c->fchunk > 0
-                             ? green_launches(c->dev, GREEN_G32) + 3 + 6 * ((c->nf + c->fchunk - 1) / c->fchunk) + 6 : 0;
+                             ? green_launches(c->dev, GREEN_G32) + 4 + 6 * ((c->nf + c->fchunk - 1) / c->fchunk) + 6 : 0;
   o->gram_rows_padded = 0;
   for (long long n : c->seg_nrow) o->gram_rows_padded += (n + TC_KC - 1) / TC_KC * TC_KC;
   if (c->ws) {

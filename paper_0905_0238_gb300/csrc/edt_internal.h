@@ -165,7 +165,8 @@ struct Dev {
   double* gcpart;               // [warps of the reverse march][nlayer] partial dJ/dc_l
   float2* gbar;                 // [nf][nk][nz] dJ/dg per table row (aliases g64)
   // spectral Born operator on the folded table index (csrc/born.cu)
-  int* born_exp;                // [nf * nk + N] power-of-two exponents of the forward model's
+  int* born_exp;                // [nf * nk + N] power-of-two exponents of the forward model's (the
+                                //   misfit: [0] that of Vhat, the last N its rows')
                                 //   scaled Green's-table rows and Vhat rows
   float4* born_fold;            // [fchunk][2][nk][nk] folded residual (or data) planes E, T
   // dL/dc through the damped solve (line geometry, mixed path)
@@ -295,8 +296,8 @@ cudaError_t launch_refine_update(const Dev& d, cudaStream_t s);   // x += (LL^T)
 cudaError_t launch_inverse(const Dev& d, void* V, int V_dtype, cudaStream_t s);
 // Spectral Born operator (csrc/born.cu): the chunk's planes X[fi][q][p] = F(p, q) from the FP64
 // table and vfull (mixed path: after launch_born_prep, which scales and splits both in place);
-// the folded planes of R2 = F - X (model; vfull as FP32 by launch_born_v32, sum |R2|^2 added to
-// gacc[0]) or of X itself.
+// the folded planes of R2 = F - X (model; vfull as FP32 times 2^-born_exp[0] by launch_born_v32, sum
+// |R2|^2 added to gacc[0]) or of X itself.
 cudaError_t prepare_born();
 cudaError_t launch_born_prep(const Dev& d, cudaStream_t s);
 cudaError_t launch_born_v32(const Dev& d, cudaStream_t s);

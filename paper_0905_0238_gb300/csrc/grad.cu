@@ -362,7 +362,8 @@ __global__ void __launch_bounds__(256, 2) grad_gbar_kernel(Dev d, int f0) {
     }
     if (more) store_coef(cf + (buf ^ 1) * S::NC);
   }
-  const float sc = float(2.0 / (double(N) * N) * sqrt(d.fc[f].s_abs));
+  // times the scale of Vhat (launch_born_v32)
+  const float sc = float(scalbn(2.0 / (double(N) * N) * sqrt(d.fc[f].s_abs), d.born_exp[0]));
   float2* G = d.gbar + size_t(f) * nk * d.nz;
 #pragma unroll
   for (int k = 0; k < GN; ++k) {

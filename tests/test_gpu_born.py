@@ -60,3 +60,17 @@ def test_gradient_edges(nx, nz, nf):
     assert rel_l2(gc.cpu().numpy(), grad2d.grad_c(wl, V, D)) < 1e-5
     Vt = _solver(wl, EDT_MIXED).adjoint(dev(D)).cpu().numpy()
     assert rel_l2(Vt, edt2d.adjoint(wl, D)) < 1e-5
+
+
+@pytest.mark.parametrize("scale", [1e-18, 1e-12, 1e12, 1e18, 1e20])
+def test_misfit_does_not_depend_on_the_unit_of_the_data(scale):
+    """Model and data times a factor: J and dJ/dc change by its square and dJ/dV by the factor, to
+    the same 1e-5, although the squares of the residual, and its products with the model, leave the FP32
+    range."""
+    from paper_0905_0238_gb300 import EDT_MIXED
+    wl = _workload(64, 40, 3)
+    V, D = _model(wl, 2), edt2d.forward(wl, _model(wl, 3))
+    J, gV, gc = _solver(wl, EDT_MIXED).misfit_grad(dev(scale * V), dev(scale * D))
+    assert abs(float(J.cpu()) / scale / scale / grad2d.misfit(wl, V, D) - 1) < 1e-5
+    assert rel_l2(gV.cpu().numpy() / scale, grad2d.grad_V(wl, V, D)) < 1e-5
+    assert rel_l2(gc.cpu().numpy() / scale / scale, grad2d.grad_c(wl, V, D)) < 1e-5

@@ -17,17 +17,28 @@
 //   F32   the misfit's residual (the FP32 table sqrt|s_f| g);
 //   F64   the forward model of the FP64 path, bound by the FP64 unit;
 //   DF    the forward model of the mixed path, FP64 table and sums carried as float pairs on
-//         the FP32 pipes (an FP64 multiply-add costs 64 FP32 ones here).  Table and Vhat rows
-//         are scaled by powers of two to at most 1, so a sum of nz products stays below nz and
-//         is accumulated on a bias C = 4 nz (rounded up to a power of two): s stays within a
-//         binade or two of C, the rounding error of s' = fma(a, v, s) is then exactly
-//         fma(a, v, s - s'), and one multiply-add of pairs takes 6 FP32 operations instead of
-//         the 12 of an unordered TwoSum.  The result is rounded to FP32 once.
+//         the FP32 pipes (an FP64 multiply-add costs 64 FP32 ones here).  Table rows are scaled by
+//         powers of two to a 2-norm of at most 1 and Vhat rows to components of at most 1, so every
+//         sum stays within 1 (Cauchy-Schwarz) and is accumulated on a bias C = 4: s keeps to [3, 5],
+//         s - s' is exact for s' = fma(a, v, s), and fma(a, v, s - s') is the rounding error of s'
+//         up to its own rounding to 24 bits; one multiply-add of pairs takes 6 FP32 operations
+//         instead of the 12 of an unordered TwoSum.  The captured errors are summed in FP32 and carried
+//         back into s after every 32 depths (3 operations), so that this sum stays within a few units
+//         of C's last place, 2^-21.  The error of a sum is then that of some 3 nz roundings to 2^-45 or
+//         finer: sqrt(nz) 2^-43 of the bound 1 is taken for it, whatever the sum itself comes to.
 //
-// Measured at N = 512, 128 frequencies, 256 depths (GB300): the forward contraction 3.55 ms in
-// DF, where the 512^2 entries one by one in FP64 took 153 ms (FP64-bound); the operation count
-// (86 FP32 operations per pair and depth) allows 2.3 ms.  Against a 64-bit restatement the
-// data are 1.6e-7 off either way: the FP32 transforms behind it set the error.
+// The depth sums of a smooth model, or of a deep one under strong decay, come to far less than their
+// bound.  The mixed forward model holds a plane's error to 2^-27 of its 2-norm, below the 1.2e-7 of
+// the FP32 transforms behind it: every tile leaves the squares of its sums and of their bounds, and the planes
+// whose ratio falls short (born_pick_kernel) are formed again in FP64 from the same pairs (49 bits of the
+// FP64 table, as many as the march's rounding leaves right).  A Gaussian perturbation of 120 m in a
+// homogeneous reference, 20 to 60 Hz: up to 1.1e-2 off by pairs alone, at most 1.9e-7 so.
+//
+// Measured at N = 512, 128 frequencies, 256 depths (GB300): the forward contraction 3.61 ms in DF, where
+// the 512^2 entries one by one in FP64 took 153 ms (FP64-bound); the operation count (87 FP32
+// operations per pair and depth) allows 2.3 ms.  The planes formed again take 0.23 ms each (30 ms for
+// all 128); finding none takes 9 us.  Against a 64-bit restatement the data are 1.2e-7 to 1.6e-7 off: the
+// FP32 transforms set the error.
 //
 // The gradients read the residual plane R2 (or the data plane) only through the sums over the
 // entries of a class, so the residual kernel leaves, per pair, the folded values
@@ -45,10 +56,13 @@ namespace {
 constexpr int BT = 32, BZ = 8;              // pairs per tile side, depths per staged chunk
 constexpr int BKS = BT + 1, BVS = 2 * BT + 1;   // odd rows: the transposing stores spread over banks
 constexpr int BTHREADS = 256;
+constexpr int BSETTLE = 4;                  // chunks after which the DF form's low sums are carried up
 
 // ---- arithmetics -------------------------------------------------------------------------
 struct ArF32 {
-  using E = float2;
+  using E = float2;                        // as staged
+  using S = float2;                        // as stored
+  __device__ __forceinline__ static E of(S v) { return v; }
   float s[8];
   __device__ __forceinline__ void init(float) {
 #pragma unroll
@@ -61,10 +75,16 @@ struct ArF32 {
     s[4] = fmaf(a.x, w.x, s[4]); s[5] = fmaf(a.y, w.x, s[5]);
     s[6] = fmaf(a.x, w.y, s[6]); s[7] = fmaf(a.y, w.y, s[7]);
   }
+  __device__ __forceinline__ void settle() {}
 };
 
-struct ArF64 {
+template <class Src> struct ArF64 {
   using E = double2;
+  using S = Src;                           // doubles, or the pairs of the DF form
+  __device__ __forceinline__ static E of(double2 v) { return v; }
+  __device__ __forceinline__ static E of(float4 v) {
+    return make_double2(double(v.x) + double(v.z), double(v.y) + double(v.w));
+  }
   double s[8];
   __device__ __forceinline__ void init(float) {
 #pragma unroll
@@ -77,19 +97,32 @@ struct ArF64 {
     s[4] = fma(a.x, w.x, s[4]); s[5] = fma(a.y, w.x, s[5]);
     s[6] = fma(a.x, w.y, s[6]); s[7] = fma(a.y, w.y, s[7]);
   }
+  __device__ __forceinline__ void settle() {}
 };
 
-// complex pairs (re hi, im hi, re lo, im lo), |re|, |im| <= 1
+// complex pairs (re hi, im hi, re lo, im lo), scaled as above
+constexpr float DF_BIAS = 4.f;
 struct ArDF {
   using E = float4;
+  using S = float4;
+  __device__ __forceinline__ static E of(S v) { return v; }
   float s[8], lo[8];
-  __device__ __forceinline__ void init(float bias) {
+  __device__ __forceinline__ void init(float) {
 #pragma unroll
-    for (int i = 0; i < 8; ++i) { s[i] = bias; lo[i] = 0.f; }
+    for (int i = 0; i < 8; ++i) { s[i] = DF_BIAS; lo[i] = 0.f; }
+  }
+  // the low sums' high parts into s
+  __device__ __forceinline__ void settle() {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float t = __fadd_rn(s[i], lo[i]);
+      lo[i] = __fsub_rn(lo[i], __fsub_rn(t, s[i]));
+      s[i] = t;
+    }
   }
   __device__ __forceinline__ void acc(int i, float ah, float al, float vh, float vl) {
     const float t = fmaf(ah, vh, s[i]);
-    const float e = fmaf(ah, vh, __fsub_rn(s[i], t));      // the rounding error of t, exactly
+    const float e = fmaf(ah, vh, __fsub_rn(s[i], t));      // the rounding error of t, rounded
     s[i] = t;
     lo[i] = fmaf(al, vh, fmaf(ah, vl, __fadd_rn(lo[i], e)));
   }
@@ -130,7 +163,7 @@ template <class E> constexpr size_t tile_smem() { return size_t(BZ) * (2 * BKS +
 // Sums of the tile's pairs over the depths.  g: table row n at g + n gs; v: Vhat row m at
 // v + m vs.  Rows k, l >= H are not part of the tile (their pairs are not used).
 template <class Ar>
-__device__ __forceinline__ void fold_tile(const typename Ar::E* g, size_t gs, const typename Ar::E* v, size_t vs,
+__device__ __forceinline__ void fold_tile(const typename Ar::S* g, size_t gs, const typename Ar::S* v, size_t vs,
                                           int nz, int N, int k0, int l0, typename Ar::E* sm, Ar (&acc)[2][2]) {
   using E = typename Ar::E;
   E* sk = sm;                       // [BZ][BKS] rows k0 + i
@@ -145,14 +178,14 @@ __device__ __forceinline__ void fold_tile(const typename Ar::E* g, size_t gs, co
     for (int e = threadIdx.x; e < BT * BZ; e += BTHREADS) {
       const int i = e / BZ, zz = e - i * BZ;
       const bool in = z0 + zz < nz;
-      sk[zz * BKS + i] = in && k0 + i < H ? g[size_t(k0 + i) * gs + z0 + zz] : zero_of<E>();
-      sl[zz * BKS + i] = in && l0 + i < H ? g[size_t(l0 + i) * gs + z0 + zz] : zero_of<E>();
+      sk[zz * BKS + i] = in && k0 + i < H ? Ar::of(g[size_t(k0 + i) * gs + z0 + zz]) : zero_of<E>();
+      sl[zz * BKS + i] = in && l0 + i < H ? Ar::of(g[size_t(l0 + i) * gs + z0 + zz]) : zero_of<E>();
     }
     for (int e = threadIdx.x; e < 2 * BT * BZ; e += BTHREADS) {
       const int i = e / BZ, zz = e - i * BZ;
       const bool in = z0 + zz < nz;
-      s1[zz * BVS + i] = in ? v[size_t((k0 - l0 - (BT - 1) + i) & msk) * vs + z0 + zz] : zero_of<E>();
-      s2[zz * BVS + i] = in ? v[size_t((k0 + l0 + i) & msk) * vs + z0 + zz] : zero_of<E>();
+      s1[zz * BVS + i] = in ? Ar::of(v[size_t((k0 - l0 - (BT - 1) + i) & msk) * vs + z0 + zz]) : zero_of<E>();
+      s2[zz * BVS + i] = in ? Ar::of(v[size_t((k0 + l0 + i) & msk) * vs + z0 + zz]) : zero_of<E>();
     }
     __syncthreads();
 #pragma unroll 2
@@ -174,62 +207,75 @@ __device__ __forceinline__ void fold_tile(const typename Ar::E* g, size_t gs, co
         for (int b = 0; b < 2; ++b)
           if (!(diag && a < b)) acc[a][b].mac(gk[a], gl[b], v1[a - b + 1], v2[a + b]);   // a < b: k < l
     }
+    if ((z0 / BZ) % BSETTLE == BSETTLE - 1) {
+#pragma unroll
+      for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) acc[a][b].settle();
+    }
     __syncthreads();
   }
 }
 
 // ---- preparation of the double-float forward model ---------------------------------------
-__device__ __forceinline__ float block_max(float m, float* red) {
-  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
-  __syncthreads();
-  m = red[0];
-  for (int w = 1; w < int(blockDim.x >> 5); ++w) m = fmaxf(m, red[w]);
-  return m;
+// exponent e with |v| < 2^e (both components), by their bits; non-finite: above any finite one
+__device__ __forceinline__ int exp_above(double2 v) {
+  return max((__double2hiint(v.x) >> 20) & 0x7ff, (__double2hiint(v.y) >> 20) & 0x7ff) - 1022;
 }
 
-// One row of nz <= 512 FP64 complex values per CTA, replaced in place by float pairs of
-// value * c * 2^-e with the largest component just under 1; e goes to exps[row].  c is
-// sqrt(s_f) = omega~ sqrt(dz/dx) for the Green's table (so the products carry s_f) and 1 for Vhat.
-constexpr int PREP_THREADS = 128, PREP_Q = 4;
-__global__ void __launch_bounds__(PREP_THREADS) born_prep_kernel(Dev d, double2* rows, int per_f, int* exps) {
-  __shared__ float red[PREP_THREADS / 32];
-  const size_t row = blockIdx.x;
+// One row of nz <= 256 FP64 complex values per warp, replaced in place by float pairs of
+// value * c * 2^-e; e goes to exps[row].  Green's table (per_f rows to a frequency): the row's 2-norm in
+// [1/2, 1), c = sqrt(s_f) = omega~ sqrt(dz/dx), so the products carry s_f.  Vhat (per_f = 0): the largest
+// component in [1/2, 1), c = 1.
+constexpr int PREP_THREADS = 128, PREP_Q = 8;
+__global__ void __launch_bounds__(PREP_THREADS) born_prep_kernel(Dev d, double2* rows, long long nrow, int per_f, int* exps) {
+  const int lane = threadIdx.x & 31;
+  const long long row = (long long)blockIdx.x * (PREP_THREADS / 32) + (threadIdx.x >> 5);
+  if (row >= nrow) return;
   double2 c = make_double2(1.0, 0.0);
   if (per_f) {
     const FreqConst fc = d.fc[row / per_f];
     const double q = sqrt(d.dz / d.dx);
     c = make_double2(q * fc.om_re, q * fc.om_im);
   }
-  double2* r = rows + row * d.nz;
+  double2* r = rows + size_t(row) * d.nz;
   double2 v[PREP_Q];
-  float m = 0.f;
+  int e = -1022;
 #pragma unroll
   for (int i = 0; i < PREP_Q; ++i) {
-    const int z = threadIdx.x + PREP_THREADS * i;
+    const int z = lane + 32 * i;
     v[i] = z < d.nz ? r[z] : make_double2(0.0, 0.0);
-    if (per_f) v[i] = c * v[i];
-    m = fmaxf(m, fmaxf(fabsf(float(v[i].x)), fabsf(float(v[i].y))));
   }
-  m = block_max(m, red);
-  int e = 0;
-  if (m > 0.f && isfinite(m)) frexpf(m, &e);
-  e = max(-126, min(126, e));
-  const double sc = __longlong_as_double((long long)(1023 - e) << 52);      // 2^-e
 #pragma unroll
   for (int i = 0; i < PREP_Q; ++i) {
-    const int z = threadIdx.x + PREP_THREADS * i;
-    if (z >= d.nz) continue;
+    if (per_f) v[i] = c * v[i];
+    e = max(e, exp_above(v[i]));
+  }
+  e = max(-1000, min(1000, __reduce_max_sync(0xffffffffu, e)));
+  const double sc = __hiloint2double((1023 - e) << 20, 0);                  // 2^-e
+  float4 o[PREP_Q];
+  float q = 0.f;
+#pragma unroll
+  for (int i = 0; i < PREP_Q; ++i) {
     const double x = v[i].x * sc, y = v[i].y * sc;
     const float xh = float(x), yh = float(y);
-    reinterpret_cast<float4*>(r)[z] = make_float4(xh, yh, float(x - double(xh)), float(y - double(yh)));
+    o[i] = make_float4(xh, yh, float(x - double(xh)), float(y - double(yh)));
+    q = fmaf(xh, xh, fmaf(yh, yh, q));
   }
-  if (threadIdx.x == 0) exps[row] = e;
-}
-
-// exponent e with |v| < 2^e (both components), by their bits; non-finite: above any finite one
-__device__ __forceinline__ int exp_above(double2 v) {
-  return max((__double2hiint(v.x) >> 20) & 0x7ff, (__double2hiint(v.y) >> 20) & 0x7ff) - 1022;
+  float un = 1.f;
+  if (per_f) {
+    for (int w = 16; w > 0; w >>= 1) q += __shfl_xor_sync(0xffffffffu, q, w);
+    int en = 0;
+    if (q > 0.f && isfinite(q)) frexpf(sqrtf(q), &en);
+    e += en;
+    un = __int_as_float((127 - en) << 23);                                  // 2^-en
+  }
+#pragma unroll
+  for (int i = 0; i < PREP_Q; ++i) {
+    const int z = lane + 32 * i;
+    if (z < d.nz) reinterpret_cast<float4*>(r)[z] = make_float4(un * o[i].x, un * o[i].y, un * o[i].z, un * o[i].w);
+  }
+  if (lane == 0) exps[row] = e;
 }
 
 // Vhat for the misfit: FP32 in place (row m's float2 values at the start of its FP64 row), all of it
@@ -250,10 +296,11 @@ __global__ void __launch_bounds__(PREP_THREADS) born_vexp_kernel(Dev d, int* row
 __global__ void __launch_bounds__(PREP_THREADS) born_v32_kernel(Dev d, const int* rowe, int* exps) {
   static_assert(PREP_THREADS == 128, "four warps");
   __shared__ int red[PREP_THREADS / 32];
+  constexpr int Q = 2;                  // nz <= 256
   double2* r = d.vfull + size_t(blockIdx.x) * d.nz;
-  double2 v[PREP_Q];
+  double2 v[Q];
 #pragma unroll
-  for (int i = 0; i < PREP_Q; ++i) {
+  for (int i = 0; i < Q; ++i) {
     const int z = threadIdx.x + PREP_THREADS * i;
     v[i] = z < d.nz ? r[z] : make_double2(0.0, 0.0);
   }
@@ -266,7 +313,7 @@ __global__ void __launch_bounds__(PREP_THREADS) born_v32_kernel(Dev d, const int
   e = max(-100, min(100, max(max(red[0], red[1]), max(red[2], red[3]))));
   const double sc = __hiloint2double((1023 - e) << 20, 0);                  // 2^-e
 #pragma unroll
-  for (int i = 0; i < PREP_Q; ++i) {
+  for (int i = 0; i < Q; ++i) {
     const int z = threadIdx.x + PREP_THREADS * i;
     if (z < d.nz) reinterpret_cast<float2*>(r)[z] = make_float2(float(sc * v[i].x), float(sc * v[i].y));
   }
@@ -274,37 +321,67 @@ __global__ void __launch_bounds__(PREP_THREADS) born_v32_kernel(Dev d, const int
 }
 
 // ---- forward model -----------------------------------------------------------------------
-__host__ __device__ inline float df_bias(int nz) {
-  float c = 4.f;
-  for (int n = 1; n < nz; n <<= 1) c *= 2.f;
-  return c;
-}
-
 // one rounding of (xh + xl) + sg (yh + yl), scaled by 2^e
 __device__ __forceinline__ float df_comb(float xh, float xl, float yh, float yl, float sg, int e) {
   const float2 t = two_sum(xh, sg * yh);
   return ldexpf(t.x + (t.y + (xl + sg * yl)), e);
 }
 // f1 = A + iB, f2 = A - iB for A = (s[o], s[o+1]), B = (s[o+2], s[o+3])
-__device__ __forceinline__ void df_result(const ArDF& a, int o, float bias, int e, float2& f1, float2& f2) {
-  const float a0 = a.s[o] - bias, a1 = a.s[o + 1] - bias, b0 = a.s[o + 2] - bias, b1 = a.s[o + 3] - bias;
+__device__ __forceinline__ void df_result(const ArDF& a, int o, int e, float2& f1, float2& f2) {
+  const float a0 = a.s[o] - DF_BIAS, a1 = a.s[o + 1] - DF_BIAS, b0 = a.s[o + 2] - DF_BIAS, b1 = a.s[o + 3] - DF_BIAS;
   f1 = make_float2(df_comb(a0, a.lo[o], b1, a.lo[o + 3], -1.f, e), df_comb(a1, a.lo[o + 1], b0, a.lo[o + 2], 1.f, e));
   f2 = make_float2(df_comb(a0, a.lo[o], b1, a.lo[o + 3], 1.f, e), df_comb(a1, a.lo[o + 1], b0, a.lo[o + 2], -1.f, e));
 }
 
-// X[fi][q][p] = F(p, q) for the pairs of one tile (mixed path: FP32 planes)
+__device__ __forceinline__ double block_sum(double v, double* red) {
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+  const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if ((threadIdx.x & 31) == 0) red[w] = v;
+  __syncthreads();
+  double t = 0.0;
+  if (threadIdx.x == 0)
+    for (int i = 0; i < nw; ++i) t += red[i];
+  return t;
+}
+
+// the eight entries of pair (k, l): f1, f2 of k - l, h1, h2 of k + l
+template <class T2>
+__device__ __forceinline__ void put_pair(T2* X, int N, int k, int l, T2 f1, T2 f2, T2 h1, T2 h2) {
+  const int msk = N - 1, nk_ = (N - k) & msk, nl_ = (N - l) & msk;
+  X[size_t(l) * N + k] = f1;
+  X[size_t(nk_) * N + nl_] = f1;
+  X[size_t(k) * N + l] = f2;
+  X[size_t(nl_) * N + nk_] = f2;
+  X[size_t(nl_) * N + k] = h1;
+  X[size_t(nk_) * N + l] = h1;
+  X[size_t(l) * N + nk_] = h2;
+  X[size_t(k) * N + nl_] = h2;
+}
+// the four of (H, l)
+template <class T2>
+__device__ __forceinline__ void put_edge(T2* X, int N, int l, T2 f1, T2 f2) {
+  const int H = N / 2, nl_ = (N - l) & (N - 1);
+  X[size_t(l) * N + H] = f1;
+  X[size_t(H) * N + nl_] = f1;
+  X[size_t(H) * N + l] = f2;
+  X[size_t(nl_) * N + H] = f2;
+}
+
+// X[fi][q][p] = F(p, q) for the pairs of one tile (mixed path: FP32 planes), and into born_part[fi][tile]
+// the sums over its entries of |F|^2 and of the squared bounds 2^e of F
 __global__ void __launch_bounds__(BTHREADS, 2) born_fwd_df_kernel(Dev d, int f0) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ float2 red[BTHREADS / 32];
+  __shared__ int emax[BTHREADS / 32];
   const int N = d.N, H = N / 2, msk = N - 1, fi = blockIdx.y, f = f0 + fi;
   int tk, tl;
   tile_of(blockIdx.x, tk, tl);
   const int k0 = tk * BT, l0 = tl * BT;
-  const float bias = df_bias(d.nz);
   ArDF acc[2][2];
 #pragma unroll
   for (int a = 0; a < 2; ++a)
 #pragma unroll
-    for (int b = 0; b < 2; ++b) acc[a][b].init(bias);
+    for (int b = 0; b < 2; ++b) acc[a][b].init(0.f);
   fold_tile<ArDF>(reinterpret_cast<const float4*>(d.g64) + size_t(f) * d.nk * d.nz, d.nz,
                   reinterpret_cast<const float4*>(d.vfull), d.nz, d.nz, N, k0, l0,
                   reinterpret_cast<float4*>(smem_raw), acc);
@@ -313,39 +390,67 @@ __global__ void __launch_bounds__(BTHREADS, 2) born_fwd_df_kernel(Dev d, int f0)
   float2* X = reinterpret_cast<float2*>(d.X) + size_t(fi) * N * N;
   const int* eg = d.born_exp + size_t(f) * d.nk;
   const int* ev = d.born_exp + size_t(d.nf) * d.nk;
+  // the tile's largest exponent, to which its squares are scaled
+  int em = -4000;
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const int k = k0 + tx + 16 * a, l = l0 + ty + 16 * b;
+      if (k < H && l <= k) em = max(em, eg[k] + eg[l] + max(ev[(k - l) & msk], ev[(k + l) & msk]));
+    }
+  em = __reduce_max_sync(0xffffffffu, em);
+  if ((threadIdx.x & 31) == 0) emax[threadIdx.x >> 5] = em;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < BTHREADS / 32; ++w) em = max(em, emax[w]);
+  float sf = 0.f, sb = 0.f;
 #pragma unroll
   for (int a = 0; a < 2; ++a)
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
       const int k = k0 + tx + 16 * a, l = l0 + ty + 16 * b;
       if (k >= H || l > k) continue;
-      const int e = eg[k] + eg[l], nk_ = (N - k) & msk, nl_ = (N - l) & msk;
+      const int e = eg[k] + eg[l], e1 = e + ev[(k - l) & msk], e2 = e + ev[(k + l) & msk];
+      const float w1 = exp2f(float(max(-120, 2 * (e1 - em)))), w2 = exp2f(float(max(-120, 2 * (e2 - em))));
+      float q[2] = {0.f, 0.f};
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const float x = acc[a][b].s[i] - DF_BIAS + acc[a][b].lo[i];
+        q[i / 4] = fmaf(x, x, q[i / 4]);
+      }
+      sf = fmaf(w1, q[0], fmaf(w2, q[1], sf));
+      sb += w1 + w2;
       float2 f1, f2, h1, h2;
-      df_result(acc[a][b], 0, bias, e + ev[(k - l) & msk], f1, f2);
-      df_result(acc[a][b], 4, bias, e + ev[(k + l) & msk], h1, h2);
-      X[size_t(l) * N + k] = f1;
-      X[size_t(nk_) * N + nl_] = f1;
-      X[size_t(k) * N + l] = f2;
-      X[size_t(nl_) * N + nk_] = f2;
-      X[size_t(nl_) * N + k] = h1;
-      X[size_t(nk_) * N + l] = h1;
-      X[size_t(l) * N + nk_] = h2;
-      X[size_t(k) * N + nl_] = h2;
+      df_result(acc[a][b], 0, e1, f1, f2);
+      df_result(acc[a][b], 4, e2, h1, h2);
+      put_pair(X, N, k, l, f1, f2, h1, h2);
     }
+  for (int o = 16; o > 0; o >>= 1) {
+    sf += __shfl_down_sync(0xffffffffu, sf, o);
+    sb += __shfl_down_sync(0xffffffffu, sb, o);
+  }
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = make_float2(sf, sb);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+#pragma unroll
+    for (int w = 1; w < BTHREADS / 32; ++w) { sf += red[w].x; sb += red[w].y; }
+    d.born_part[size_t(fi) * gridDim.x + blockIdx.x] = make_float4(sf, sb, __int_as_float(em), 0.f);
+  }
 }
 
 __global__ void __launch_bounds__(BTHREADS, 2) born_fwd_f64_kernel(Dev d, int f0) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int N = d.N, H = N / 2, msk = N - 1, fi = blockIdx.y, f = f0 + fi;
+  const int N = d.N, H = N / 2, fi = blockIdx.y, f = f0 + fi;
   int tk, tl;
   tile_of(blockIdx.x, tk, tl);
   const int k0 = tk * BT, l0 = tl * BT;
-  ArF64 acc[2][2];
+  ArF64<double2> acc[2][2];
 #pragma unroll
   for (int a = 0; a < 2; ++a)
 #pragma unroll
     for (int b = 0; b < 2; ++b) acc[a][b].init(0.f);
-  fold_tile<ArF64>(d.g64 + size_t(f) * d.nk * d.nz, d.nz, d.vfull, d.nz, d.nz, N, k0, l0,
+  fold_tile<ArF64<double2>>(d.g64 + size_t(f) * d.nk * d.nz, d.nz, d.vfull, d.nz, d.nz, N, k0, l0,
                    reinterpret_cast<double2*>(smem_raw), acc);
   int tx, ty;
   thread_xy(tx, ty);
@@ -358,18 +463,9 @@ __global__ void __launch_bounds__(BTHREADS, 2) born_fwd_f64_kernel(Dev d, int f0
     for (int b = 0; b < 2; ++b) {
       const int k = k0 + tx + 16 * a, l = l0 + ty + 16 * b;
       if (k >= H || l > k) continue;
-      const int nk_ = (N - k) & msk, nl_ = (N - l) & msk;
       const double* s = acc[a][b].s;
-      const double2 f1 = sf * make_double2(s[0] - s[3], s[1] + s[2]), f2 = sf * make_double2(s[0] + s[3], s[1] - s[2]);
-      const double2 h1 = sf * make_double2(s[4] - s[7], s[5] + s[6]), h2 = sf * make_double2(s[4] + s[7], s[5] - s[6]);
-      X[size_t(l) * N + k] = f1;
-      X[size_t(nk_) * N + nl_] = f1;
-      X[size_t(k) * N + l] = f2;
-      X[size_t(nl_) * N + nk_] = f2;
-      X[size_t(nl_) * N + k] = h1;
-      X[size_t(nk_) * N + l] = h1;
-      X[size_t(l) * N + nk_] = h2;
-      X[size_t(k) * N + nl_] = h2;
+      put_pair(X, N, k, l, sf * make_double2(s[0] - s[3], s[1] + s[2]), sf * make_double2(s[0] + s[3], s[1] - s[2]),
+               sf * make_double2(s[4] - s[7], s[5] + s[6]), sf * make_double2(s[4] + s[7], s[5] - s[6]));
     }
 }
 
@@ -400,7 +496,7 @@ template <> struct EdgeSum<float> {                       // double-float partia
 };
 
 __global__ void __launch_bounds__(256) born_fwd_edge_df_kernel(Dev d, int f0) {
-  const int N = d.N, H = N / 2, msk = N - 1, lane = threadIdx.x & 31;
+  const int N = d.N, H = N / 2, lane = threadIdx.x & 31;
   const int l = blockIdx.x * 8 + (threadIdx.x >> 5), fi = blockIdx.y, f = f0 + fi;
   if (l > H) return;
   const float4* g = reinterpret_cast<const float4*>(d.g64) + size_t(f) * d.nk * d.nz;
@@ -415,40 +511,115 @@ __global__ void __launch_bounds__(256) born_fwd_edge_df_kernel(Dev d, int f0) {
   auto out = [&](float2 x, float2 y, float sg) { return df_comb(x.x, x.y, y.x, y.y, sg, e); };
   const float2 f1 = make_float2(out(a.s[0], a.s[3], -1.f), out(a.s[1], a.s[2], 1.f));
   const float2 f2 = make_float2(out(a.s[0], a.s[3], 1.f), out(a.s[1], a.s[2], -1.f));
-  float2* X = reinterpret_cast<float2*>(d.X) + size_t(fi) * N * N;
-  const int nl_ = (N - l) & msk;
-  X[size_t(l) * N + H] = f1;
-  X[size_t(H) * N + nl_] = f1;
-  X[size_t(H) * N + l] = f2;
-  X[size_t(nl_) * N + H] = f2;
+  put_edge(reinterpret_cast<float2*>(d.X) + size_t(fi) * N * N, N, l, f1, f2);
 }
 
-__global__ void __launch_bounds__(256) born_fwd_edge_f64_kernel(Dev d, int f0) {
-  const int N = d.N, H = N / 2, msk = N - 1, lane = threadIdx.x & 31;
-  const int l = blockIdx.x * 8 + (threadIdx.x >> 5), fi = blockIdx.y, f = f0 + fi;
-  if (l > H) return;
-  const double2* g = d.g64 + size_t(f) * d.nk * d.nz;
-  const double2* v = d.vfull + size_t(H - l) * d.nz;
-  double2 p = make_double2(0.0, 0.0), q = p;
-  for (int z = lane; z < d.nz; z += 32) {
-    const double2 a = g[size_t(H) * d.nz + z] * g[size_t(l) * d.nz + z];
-    p = p + v[z].x * a;
-    q = q + v[z].y * a;
+// sums over the depths of a (H, l) pair by a warp: (P, Q) in every lane
+template <class Src>
+__device__ __forceinline__ void edge_sums(const Src* gh, const Src* gl, const Src* v, int nz, int lane, double2& p, double2& q) {
+  using A = ArF64<Src>;
+  p = q = make_double2(0.0, 0.0);
+  for (int z = lane; z < nz; z += 32) {
+    const double2 a = A::of(gh[z]) * A::of(gl[z]), b = A::of(v[z]);
+    p = p + b.x * a;
+    q = q + b.y * a;
   }
   for (int o = 16; o > 0; o >>= 1) {
     p.x += __shfl_xor_sync(0xffffffffu, p.x, o); p.y += __shfl_xor_sync(0xffffffffu, p.y, o);
     q.x += __shfl_xor_sync(0xffffffffu, q.x, o); q.y += __shfl_xor_sync(0xffffffffu, q.y, o);
   }
+}
+
+__global__ void __launch_bounds__(256) born_fwd_edge_f64_kernel(Dev d, int f0) {
+  const int N = d.N, H = N / 2, lane = threadIdx.x & 31;
+  const int l = blockIdx.x * 8 + (threadIdx.x >> 5), fi = blockIdx.y, f = f0 + fi;
+  if (l > H) return;
+  const double2* g = d.g64 + size_t(f) * d.nk * d.nz;
+  double2 p, q;
+  edge_sums(g + size_t(H) * d.nz, g + size_t(l) * d.nz, d.vfull + size_t(H - l) * d.nz, d.nz, lane, p, q);
   if (lane != 0) return;
   const FreqConst fc = d.fc[f];
   const double2 om = make_double2(fc.om_re, fc.om_im), sf = (d.dz / d.dx) * (om * om);
-  const double2 f1 = sf * make_double2(p.x - q.y, p.y + q.x), f2 = sf * make_double2(p.x + q.y, p.y - q.x);
-  double2* X = reinterpret_cast<double2*>(d.X) + size_t(fi) * N * N;
-  const int nl_ = (N - l) & msk;
-  X[size_t(l) * N + H] = f1;
-  X[size_t(H) * N + nl_] = f1;
-  X[size_t(H) * N + l] = f2;
-  X[size_t(nl_) * N + H] = f2;
+  put_edge(reinterpret_cast<double2*>(d.X) + size_t(fi) * N * N, N, l, sf * make_double2(p.x - q.y, p.y + q.x),
+           sf * make_double2(p.x + q.y, p.y - q.x));
+}
+
+// born_redo[fi]: the plane's sums by pairs are not 2^-27 of the plane accurate: their sum of squares falls
+// below (sqrt(nz) 2^-43 2^27)^2 times that of the bounds.  One warp per plane.
+__global__ void __launch_bounds__(32) born_pick_kernel(Dev d, int ntile) {
+  const int fi = blockIdx.x, lane = threadIdx.x;
+  const float4* part = d.born_part + size_t(fi) * ntile;
+  int em = -4000;
+  for (int i = lane; i < ntile; i += 32) em = max(em, __float_as_int(part[i].z));
+  em = __reduce_max_sync(0xffffffffu, em);
+  float sf = 0.f, sb = 0.f;
+  for (int i = lane; i < ntile; i += 32) {
+    const float4 p = part[i];
+    const float w = exp2f(float(max(-120, 2 * (__float_as_int(p.z) - em))));
+    sf = fmaf(w, p.x, sf);
+    sb = fmaf(w, p.y, sb);
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    sf += __shfl_xor_sync(0xffffffffu, sf, o);
+    sb += __shfl_xor_sync(0xffffffffu, sb, o);
+  }
+  if (lane == 0) d.born_redo[fi] = !(sf >= float(d.nz) * 0x1p-32f * sb);
+}
+
+// These planes in FP64.  CTAs below ntile take a tile, the others eight edge pairs, of every
+// gridDim.y-th of the planes.
+__device__ __forceinline__ void redo_part(const Dev& d, int f0, int fi, int ntile, double2* sm) {
+  const int N = d.N, H = N / 2, msk = N - 1, f = f0 + fi;
+  const float4* g = reinterpret_cast<const float4*>(d.g64) + size_t(f) * d.nk * d.nz;
+  const float4* v = reinterpret_cast<const float4*>(d.vfull);
+  const int* eg = d.born_exp + size_t(f) * d.nk;
+  const int* ev = d.born_exp + size_t(d.nf) * d.nk;
+  float2* X = reinterpret_cast<float2*>(d.X) + size_t(fi) * N * N;
+  auto out = [](double x, double y, int e) { return make_float2(float(scalbn(x, e)), float(scalbn(y, e))); };
+  if (int(blockIdx.x) >= ntile) {
+    const int l = (int(blockIdx.x) - ntile) * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (l > H) return;
+    double2 p, q;
+    edge_sums(g + size_t(H) * d.nz, g + size_t(l) * d.nz, v + size_t(H - l) * d.nz, d.nz, lane, p, q);
+    if (lane != 0) return;
+    const int e = eg[H] + eg[l] + ev[H - l];
+    put_edge(X, N, l, out(p.x - q.y, p.y + q.x, e), out(p.x + q.y, p.y - q.x, e));
+    return;
+  }
+  int tk, tl;
+  tile_of(blockIdx.x, tk, tl);
+  const int k0 = tk * BT, l0 = tl * BT;
+  ArF64<float4> acc[2][2];
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int b = 0; b < 2; ++b) acc[a][b].init(0.f);
+  fold_tile<ArF64<float4>>(g, d.nz, v, d.nz, d.nz, N, k0, l0, sm, acc);
+  int tx, ty;
+  thread_xy(tx, ty);
+#pragma unroll
+  for (int a = 0; a < 2; ++a)
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const int k = k0 + tx + 16 * a, l = l0 + ty + 16 * b;
+      if (k >= H || l > k) continue;
+      const int e = eg[k] + eg[l], e1 = e + ev[(k - l) & msk], e2 = e + ev[(k + l) & msk];
+      const double* s = acc[a][b].s;
+      put_pair(X, N, k, l, out(s[0] - s[3], s[1] + s[2], e1), out(s[0] + s[3], s[1] - s[2], e1),
+               out(s[4] - s[7], s[5] + s[6], e2), out(s[4] + s[7], s[5] - s[6], e2));
+    }
+}
+
+constexpr int REDO_Y = 8;
+__global__ void __launch_bounds__(BTHREADS, 2) born_redo_kernel(Dev d, int f0, int nfc, int ntile) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int lane = threadIdx.x & 31;
+  int n = 0;                                 // planes met so far
+  for (int b = 0; b < nfc; b += 32) {
+    unsigned m = __ballot_sync(0xffffffffu, b + lane < nfc && d.born_redo[b + lane]);
+    for (; m; m &= m - 1, ++n)
+      if (n % REDO_Y == int(blockIdx.y)) redo_part(d, f0, b + __ffs(m) - 1, ntile, reinterpret_cast<double2*>(smem_raw));
+  }
 }
 
 // ---- residual and folding ----------------------------------------------------------------
@@ -485,17 +656,6 @@ struct SumSq {
     return (isfinite(acc.x) ? df_val(acc) : double(acc.x)) * __hiloint2double((1023 + 2 * e) << 20, 0);
   }
 };
-
-__device__ __forceinline__ double block_sum(double v, double* red) {
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  if ((threadIdx.x & 31) == 0) red[w] = v;
-  __syncthreads();
-  double t = 0.0;
-  if (threadIdx.x == 0)
-    for (int i = 0; i < nw; ++i) t += red[i];
-  return t;
-}
 
 // RES: R = F - D2 with the FP32 table and Vhat, sum |R|^2 into gacc[0] and R folded;
 // else R = D2 (the adjoint operator).  X[fi][q][p] = D2(p, q) is only read.
@@ -614,15 +774,21 @@ __global__ void __launch_bounds__(256) born_resid_edge_kernel(Dev d, int f0) {
 
 }  // namespace
 
+// elements of one plane in born_part
+int born_tiles(int N) { return tile_count(N / 2); }
+
 cudaError_t prepare_born() {
   cudaError_t e = allow_smem(born_fwd_df_kernel, int(tile_smem<float4>()));
   if (e != cudaSuccess) return e;
-  return allow_smem(born_fwd_f64_kernel, int(tile_smem<double2>()));
+  if ((e = allow_smem(born_fwd_f64_kernel, int(tile_smem<double2>()))) != cudaSuccess) return e;
+  return allow_smem(born_redo_kernel, int(tile_smem<double2>()));
 }
 
 cudaError_t launch_born_prep(const Dev& d, cudaStream_t s) {
-  born_prep_kernel<<<unsigned(size_t(d.nf) * d.nk), PREP_THREADS, 0, s>>>(d, d.g64, d.nk, d.born_exp);
-  born_prep_kernel<<<d.N, PREP_THREADS, 0, s>>>(d, d.vfull, 0, d.born_exp + size_t(d.nf) * d.nk);
+  constexpr int W = PREP_THREADS / 32;
+  const long long rows = (long long)d.nf * d.nk;
+  born_prep_kernel<<<unsigned((rows + W - 1) / W), PREP_THREADS, 0, s>>>(d, d.g64, rows, d.nk, d.born_exp);
+  born_prep_kernel<<<(d.N + W - 1) / W, PREP_THREADS, 0, s>>>(d, d.vfull, d.N, 0, d.born_exp + rows);
   return cudaGetLastError();
 }
 
@@ -641,6 +807,8 @@ cudaError_t launch_born_forward(const Dev& d, int f0, int nfc, cudaStream_t s) {
   } else {
     born_fwd_df_kernel<<<g, BTHREADS, tile_smem<float4>(), s>>>(d, f0);
     born_fwd_edge_df_kernel<<<ge, 256, 0, s>>>(d, f0);
+    born_pick_kernel<<<nfc, 32, 0, s>>>(d, int(g.x));
+    born_redo_kernel<<<dim3(g.x + ge.x, REDO_Y), BTHREADS, tile_smem<double2>(), s>>>(d, f0, nfc, int(g.x));
   }
   return cudaGetLastError();
 }

@@ -168,6 +168,9 @@ struct Dev {
   int* born_exp;                // [nf * nk + N] power-of-two exponents of the forward model's (the
                                 //   misfit: [0] that of Vhat, the last N its rows')
                                 //   scaled Green's-table rows and Vhat rows
+  float4* born_part;            // [fchunk][tiles] a tile's sums of |F|^2 and of their bounds' squares, times
+                                //   2^(-2 e), and e
+  int* born_redo;               // [fchunk] planes to form again in FP64
   float4* born_fold;            // [fchunk][2][nk][nk] folded residual (or data) planes E, T
   // dL/dc through the damped solve (line geometry, mixed path)
   float4* rowc;                 // [rows_solved][2] per row (u_+, u_-) = d - A x, (v_+, v_-) = -A mu
@@ -295,9 +298,11 @@ int refine_stride(long long rows_max_sub);                      // refinement CT
 cudaError_t launch_refine_update(const Dev& d, cudaStream_t s);   // x += (LL^T)^-1 (r - lam x)
 cudaError_t launch_inverse(const Dev& d, void* V, int V_dtype, cudaStream_t s);
 // Spectral Born operator (csrc/born.cu): the chunk's planes X[fi][q][p] = F(p, q) from the FP64
-// table and vfull (mixed path: after launch_born_prep, which scales and splits both in place);
+// table and vfull (mixed path: after launch_born_prep, which scales and splits both in place; by
+// float pairs, planes that these do not hold to the FP32 transforms' accuracy in FP64);
 // the folded planes of R2 = F - X (model; vfull as FP32 times 2^-born_exp[0] by launch_born_v32, sum
 // |R2|^2 added to gacc[0]) or of X itself.
+int born_tiles(int N);
 cudaError_t prepare_born();
 cudaError_t launch_born_prep(const Dev& d, cudaStream_t s);
 cudaError_t launch_born_v32(const Dev& d, cudaStream_t s);

@@ -7,9 +7,10 @@ pair, four with the edge N/2, fewer distinct ones at 0 and on the diagonal): N =
 a 32-wide tile empty, N = 64 fills one, N = 128 takes off-diagonal tiles.  Depths come in chunks
 of 8 in the forward model and 32 to 128 in the gradients.
 
-Tolerances: the mixed forward model carries its sums in about 48 bits and rounds once, so its
-error is that of the two FP32 transforms, at most about 3 u per radix-2 stage (u = 2^-24) in the
-2-norm, 2 * 7 * 3 u = 2.5e-6 for N = 128; FP64 1e-11 as elsewhere.  The misfit's sums are FP32
+Tolerances: the mixed forward model holds each plane's sums to 2^-27 of the plane (float pairs, or FP64
+where the sums cancel too far for those), so its error is that of the two FP32 transforms, at most
+about 3 u per radix-2 stage (u = 2^-24) in the 2-norm, 2 * 7 * 3 u = 2.5e-6 for N = 128; FP64 1e-11 as
+elsewhere.  The misfit's sums are FP32
 over the depths and one lateral axis: 1e-5 as in test_gpu_grad."""
 import numpy as np
 import pytest
@@ -47,6 +48,23 @@ def test_forward_edges(precision, tol, nx, nz, nf):
     s = _solver(wl, EDT_FP64 if precision == "fp64" else EDT_MIXED)
     D = s.forward(dev(V)).cpu().numpy()
     assert rel_l2(D, edt2d.forward(wl, V)) < tol
+
+
+@pytest.mark.parametrize("nx,nz,eps,depth,sigma", [
+    (64, 200, 0.15, 800.0, 60.0), (128, 200, 0.15, 800.0, 120.0), (128, 200, 0.15, 800.0, 160.0),
+    (64, 255, 5.0, 1200.0, 30.0), (64, 256, 10.0, 1600.0, 10.0),
+])
+def test_forward_of_models_whose_sums_cancel(nx, nz, eps, depth, sigma):
+    """Smooth perturbations of a homogeneous reference, and deep ones under strong decay: the depth sums come
+    to 1e-4 to 1e-10 of their terms, and every frequency keeps the accuracy of the transforms."""
+    from paper_0905_0238_gb300 import EDT_MIXED
+    wl = small_workload(nx=nx, nz=nz, nf=4, fmin=20.0, fmax=60.0, dx=12.5, dz=8.0, cutoff=0.0, eps=eps,
+                        layers=(np.array([0.0]), np.array([2000.0])))
+    x, z = np.arange(nx) * 12.5, (np.arange(nz) + 0.5) * 8.0
+    V = 1e-8 * np.exp(-((x[:, None] - nx * 6.25) ** 2 + (z[None, :] - depth) ** 2) / (2 * sigma ** 2))
+    D, want = _solver(wl, EDT_MIXED).forward(dev(V)).cpu().numpy(), edt2d.forward(wl, V)
+    for f in range(4):
+        assert rel_l2(D[f], want[f]) < 2.5e-6
 
 
 @pytest.mark.parametrize("nx,nz,nf", [(64, 1, 2), (64, 65, 1), (64, 129, 1), (128, 7, 2), (256, 34, 1)])

@@ -641,36 +641,35 @@ class Solver:
 _SUB1D = struct.Struct("@i5diPPiPiPiPP0d")
 
 
-def _pointer(a, dtype, keep):
-    """Address of a C-contiguous array of `dtype` holding `a`; a converted copy is kept in `keep`."""
-    if type(a) is not np.ndarray or a.dtype != dtype or not a.flags.c_contiguous:
-        a = np.ascontiguousarray(a, dtype=dtype)
-        keep.append(a)
-    return a.__array_interface__["data"][0]
+def _array(a, dtype):
+    """`a` itself if it is a C-contiguous array of `dtype`, else a copy that is one."""
+    if type(a) is np.ndarray and a.dtype == dtype and a.flags.c_contiguous:
+        return a
+    return np.ascontiguousarray(a, dtype=dtype)
 
 
 def _sub1d_array(subs):
     """Array of edt_sub1d for objects with the fields of synth.stream.Sub1D, plus what it points
-    into (kept alive by the caller until the submit returns).  The records are packed with
-    struct: setting the fields of a ctypes structure one by one took 20 us per request, as long
-    as the device takes to solve it."""
+    into (kept alive by the caller until the submit returns).  The fields may be anything that
+    numpy makes arrays of.  The records are packed with struct: setting the fields of a ctypes
+    structure one by one took 20 us per request, as long as the device takes to solve it."""
     if _SUB1D.size != C.sizeof(edt_sub1d):
         raise RuntimeError("edt_sub1d layout mismatch")
     buf = bytearray(max(len(subs), 1) * _SUB1D.size)
-    keep = [subs]
+    keep = []
     f8, i4, c8 = np.dtype(np.float64), np.dtype(np.int32), np.dtype(np.complex64)
     for i, s in enumerate(subs):
-        tops, freq, kval, rows, data = s.layer_top, s.freq_hz, s.kval, s.rows, s.data
+        arrays = (_array(s.layer_top, f8), _array(s.layer_vel, f8), _array(s.freq_hz, f8), _array(s.kval, f8),
+                  _array(s.rows, i4), _array(s.data, c8))
         # the arrays themselves, not only the request, so that a field replaced meanwhile is safe
-        keep.append((tops, s.layer_vel, freq, kval, rows, data))
-        tp, vp = _pointer(tops, f8, keep), _pointer(s.layer_vel, f8, keep)
-        fp, kp = _pointer(freq, f8, keep), _pointer(kval, f8, keep)
-        rp, dp = _pointer(rows, i4, keep), _pointer(data, c8, keep)
-        nrow, odd = divmod(np.size(rows), 3)
-        if odd or np.size(data) % 2:
+        keep.append(arrays)
+        tops, _, freq, kval, rows, data = arrays
+        tp, vp, fp, kp, rp, dp = [a.__array_interface__["data"][0] for a in arrays]
+        nrow, odd = divmod(rows.size, 3)
+        if odd or data.size % 2:
             raise ValueError("rows are (f, p, q) triples and data (d_+, d_-) pairs")
-        _SUB1D.pack_into(buf, i * _SUB1D.size, int(s.nz), s.dz, s.z0, s.eps, s.alpha, s.dx, len(tops), tp, vp,
-                         len(freq), fp, len(kval), kp, nrow, rp, dp)
+        _SUB1D.pack_into(buf, i * _SUB1D.size, int(s.nz), float(s.dz), float(s.z0), float(s.eps), float(s.alpha),
+                         float(s.dx), len(tops), tp, vp, len(freq), fp, len(kval), kp, nrow, rp, dp)
     return (edt_sub1d * max(len(subs), 1)).from_buffer(buf), keep
 
 

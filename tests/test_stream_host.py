@@ -91,3 +91,32 @@ def test_request_marshalling_round_trips():
         d = np.ctypeslib.as_array(e.data, (e.nrow, 4))
         np.testing.assert_array_equal(d[:, 0] + 1j * d[:, 1], s.data[:, 0])
         np.testing.assert_array_equal(d[:, 2] + 1j * d[:, 3], s.data[:, 1])
+
+
+@pytest.mark.parametrize("form", ["lists", "tensors", "strided", "wider types", "text scalars"])
+def test_request_fields_of_any_form_are_marshalled(form):
+    """Whatever numpy makes arrays of (and float a number of) is accepted and carries the same values."""
+    s = stream.stream_requests(1, salt=24)[0]
+    names = ("layer_top", "layer_vel", "freq_hz", "kval", "rows", "data")
+    t = copy.copy(s)
+    for k in names:
+        a = np.array(getattr(s, k))
+        if form == "lists":
+            a = a.tolist()
+        elif form == "tensors":
+            a = pytest.importorskip("torch").from_numpy(a)
+        elif form == "strided":
+            a = np.repeat(a, 2, axis=0)[::2]
+        elif form == "wider types":
+            a = a.astype({"f": np.longdouble, "i": np.int64, "c": np.complex128}[a.dtype.kind])
+        setattr(t, k, a)
+    if form == "text scalars":
+        t.dz, t.dx = str(s.dz), str(s.dx)
+    (want,), k0 = edt._sub1d_array([s])
+    (got,), k1 = edt._sub1d_array([t])
+    for field in ("nz", "dz", "z0", "eps", "alpha", "dx", "nlayer", "nfreq", "nk", "nrow"):
+        assert getattr(got, field) == getattr(want, field), field
+    for field, n in (("layer_top_m", s.layer_top.size), ("layer_vel_mps", s.layer_vel.size), ("freq_hz", s.freq_hz.size),
+                     ("kval", s.kval.size), ("rows", s.rows.size), ("data", 2 * s.data.size)):
+        np.testing.assert_array_equal(np.ctypeslib.as_array(getattr(got, field), (n,)),
+                                      np.ctypeslib.as_array(getattr(want, field), (n,)))

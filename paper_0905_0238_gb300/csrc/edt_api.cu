@@ -693,7 +693,7 @@ void layout(edt_ctx* c) {
   take(c->r_Gs, grid ? nz * (N / 2 + 1) * (c->ny / 2 + 1) * sizeof(float2) : c->win ? nz * N * sizeof(float2) : 0);
   const size_t wact = c->nact.empty() ? 1 : size_t(std::max(1, *std::max_element(c->nact.begin(), c->nact.end())));
   const size_t slots = grid ? fa_grid_slots(c->wx, c->wy) : 0;
-  take(c->r_U, grid ? fa_grid_bytes(fa_grid_slab(c->nz, int(slots), c->q_max), int(slots), c->q_max)
+  take(c->r_U, grid ? fa_grid_bytes(c->nz, int(slots), c->q_max)
                : c->win ? wact * nz * N * sizeof(float2) : 0);
   take(c->r_Dw, c->win ? nf * W * nxy * sizeof(float2) : 0);
   take(c->r_A32, c->win ? (R + 1) * nzs * sizeof(float2) : 0);
@@ -792,7 +792,6 @@ void bind_plan(edt_ctx* c) {
   d.tune_bc = c->tune_bc; d.tune_rf = c->tune_rf; d.tune_zc = c->tune_zc;
   d.geom = c->win ? EDT_GEOM_WINDOW : EDT_GEOM_LINE;
   d.ny = c->ny; d.wx = c->wx; d.wy = c->wy; d.W = c->W; d.nxy = c->nxy; d.dy = c->cfg.dy;
-  d.fa_slab = c->win && c->ny > 1 ? fa_grid_slab(c->nz, fa_grid_slots(c->wx, c->wy), c->q_max) : 0;
   d.ones_row = (long long)c->rows.size();
   d.nseg = c->nslot; d.ncta_gram = c->ncta_gram;
   d.f16 = c->r_gscale.bytes > 0;
@@ -1610,13 +1609,11 @@ int edt_get_stats(edt_ctx* c, edt_stats* o) {
   // or Jacobi), the back-projection with the disk; the Jacobi kernel alone without it
   if (c->variant) o->launches_per_invert += (c->kz_p.empty() ? 1 : 5) - chol_launches(c->nz);
   if (c->win) {
-    // green (3), rows per frequency that keeps any (a line: 3; a grid: 1 and 2 per slab of
-    // depths), data (2), Gram (2), Cholesky,
+    // green (3 or 4), rows (3) per frequency that keeps any, data (2), Gram (2), Cholesky,
     // refinement (3 per step), inverse (completion, FP64 row and column transforms, output: 3 or 4)
     int fk = 0;
     for (int n : c->nact) fk += n > 0;
-    const int per_f = c->ny > 1 ? 1 + 2 * ((c->nz + c->dev.fa_slab - 1) / c->dev.fa_slab) : 3;
-    o->launches_per_invert = green_launches(c->dev, green_tables(c)) + per_f * fk + 2 + 2 + chol_n + 3 * c->cfg.refine +
+    o->launches_per_invert = green_launches(c->dev, green_tables(c)) + 3 * fk + 2 + 2 + chol_n + 3 * c->cfg.refine +
                              (c->ny > 1 ? 4 : 3);
   }
   o->freq_chunk = c->band_mode ? c->band_maxplanes : c->fchunk;

@@ -108,11 +108,10 @@ struct Dev {
   const int* jmap;              // [nf][W] position of j among the active ones, or -1
   const int* q_xy;              // a grid's quadrant points (y << 16 | x) with kept rows, per frequency
   const int4* q_rows;           // their rows: (first, count) of the pair (kx, ky), then of (-kx, ky)
-  int fa_slab;                  // depths whose planes of one frequency are held at a time (grid)
   float2* Gs;                   // G(y, z) of one frequency: a line [nz][nx], a grid's quadrant
                                 //   [nz][ny/2 + 1][nx/2 + 1]
   float2* U;                    // a line: [active j][nz][nx] window products of one frequency; a grid:
-                                //   tiles of the slab's planes (csrc/fagrid.cu)
+                                //   tiles of its planes (csrc/fagrid.cu)
   float2* Dw;                   // [nf][W][ny][nx] window-transformed data
   float2* A32;                  // [rows + 1][nzs] kernel rows, then a row of ones
   long long ones_row;           // index of the ones row in A32
@@ -251,10 +250,8 @@ bool fa_supported(int nx, int ny, int wx, int wy);
 cudaError_t launch_fa_line(const Dev& d, int f, int nact, double2 cf, cudaStream_t s);
 // the same for a grid (csrc/fagrid.cu): the frequency's points are q_xy/q_rows[qoff .. qoff + nq), their
 // largest x and y qmax
-constexpr size_t FA_SLAB_BYTES = size_t(2) << 30;     // plane buffer of a slab of depths (at least 8)
 int fa_grid_slots(int wx, int wy);
-int fa_grid_slab(int nz, int slots, int nq);
-size_t fa_grid_bytes(int nzb, int slots, int nq);
+size_t fa_grid_bytes(int nz, int slots, int nq);        // plane buffer for at most nq points
 cudaError_t launch_fa_grid(const Dev& d, int f, int qoff, int nq, int2 qmax, double2 cf, cudaStream_t s);
 cudaError_t prepare_fa_grid(const Dev& d);
 cudaError_t launch_fa_data(const Dev& d, const void* D, int D_dtype, cudaStream_t s);

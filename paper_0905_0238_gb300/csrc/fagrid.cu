@@ -19,9 +19,9 @@
 // FFT), at 128 x 128 midpoints, 16 x 16 half-offsets, 64 frequencies and 200 depths: 45 planes per
 // (f, z) instead of 138 on average, 46 ms of kernels instead of 144; 64 x 64, 8 x 8, 12 frequencies, 100
 // depths: 0.55 ms instead of 1.36.
-// Per frequency and slab of depths (all of them unless the planes would take more than
-// FA_SLAB_BYTES; slabs that stay in L2 lost more to short launches than they saved: 134 ms per
-// inversion at 80 MB, 123 at 240 MB, 115 with one slab):
+// Per frequency, for all depths at once (slabs of depths whose planes stay in L2 lost more to short
+// launches than they saved: 134 ms per inversion at 80 MB, 123 at 240 MB, 115 with none; the largest
+// accepted grid, window and depth count have 1.3 GB of planes):
 //   grid_gspace  G on the quadrant, by a half-plane inverse FFT of the |k| table;
 //   grid_planes  P_ab from G in shared memory, its half-plane FFT, E and O at the quadrant points q
 //                = (kx, ky) that have kept rows, as tiles of 8 q x 8 z: F[q / 8][z / 8][slot][z % 8][q % 8];
@@ -187,25 +187,25 @@ __global__ void __launch_bounds__(Half<N>::THREADS) grid_gspace_kernel(Dev d, in
 }
 
 // ---- products and planes --------------------------------------------------------------------
-// CTA per (z of the slab, every gridDim.x-th plane).  swap: only a >= b, the other half of the
+// CTA per (z, every gridDim.x-th plane).  swap: only a >= b, the other half of the
 // windows from the transposed points.  cmax: the largest column among the points (transposed ones
 // included); at low frequencies the cut keeps no point beyond it, and the rest is not transformed (128 x
 // 128 midpoints, 4-50 Hz: 84.6 ms per inversion, 85.4 with all columns).
 template <int N>
 __global__ void __launch_bounds__(Half<N>::THREADS, N == 128 ? 2 : 3)
-grid_planes_kernel(Dev d, const int* qxy, int nq, int z0, int hx, int hy, int swap, int nplane, int cmax) {
+grid_planes_kernel(Dev d, const int* qxy, int nq, int hx, int hy, int swap, int nplane, int cmax) {
   using S = Half<N>;
   constexpr int H = S::H, V = S::V, QD = S::QD;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* s = reinterpret_cast<float2*>(smem_raw);
   float2* tw = s + S::PLANE;
   float2* gq = tw + S::TW;
-  const float2* G = d.Gs + size_t(z0 + blockIdx.y) * S::QUAD;
+  const float2* G = d.Gs + size_t(blockIdx.y) * S::QUAD;
   half_twiddles<N>(tw, d.tw32);
   for (int e = threadIdx.x; e < S::QUAD; e += blockDim.x) gq[e] = G[e];
   const int nE = (hx + 1) * (hy + 1);
-  // slot stride GT_P within a tile, gridDim.y depths per slab
-  const size_t ns = size_t(nE + hx * hy), zt = (gridDim.y + GT_Z - 1) / GT_Z;
+  // slot stride GT_P within a tile
+  const size_t ns = size_t(nE + hx * hy), zt = (d.nz + GT_Z - 1) / GT_Z;
   float2* F = d.U + (size_t(blockIdx.y / GT_Z) * ns) * GT_P + (blockIdx.y % GT_Z) * GT_Q;
   for (int pl = blockIdx.x; pl < nplane; pl += gridDim.x) {
     int a, b;
@@ -322,7 +322,7 @@ __device__ __forceinline__ int rt_at(int q, int z) { return 32 * (z >> 2) + ((4 
 
 template <int WX, int WY>
 __global__ void __launch_bounds__(RT_THREADS, 3)
-grid_rows_kernel(Dev d, const int4* qrows, int nq, int z0, int nzb, float2 cf) {
+grid_rows_kernel(Dev d, const int4* qrows, int nq, float2 cf) {
   constexpr int HX = WX / 2, HY = WY / 2, NE = (HX + 1) * (HY + 1), NS = NE + HX * HY;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float2* v = reinterpret_cast<float2*>(smem_raw);
@@ -396,10 +396,10 @@ grid_rows_kernel(Dev d, const int4* qrows, int nq, int z0, int nzb, float2 cf) {
   __syncthreads();
   // the kept rows of both pairs of every point, 8 lanes (depths) per row, four groups per point
   const int z = lane & 7, g = warp * 4 + (lane >> 3), q = g & 7;
-  if (q0 + q >= nq || zb + z >= nzb) return;
+  if (q0 + q >= nq || zb + z >= d.nz) return;
   const int4 R = qrows[q0 + q];
   const int n = R.y + R.w;
-  float2* A = d.A32 + z0 + zb + z;
+  float2* A = d.A32 + zb + z;
   const float2* p = v + rt_at(q, z);
   const float2 ohh = p[(NS - 1) * GT_P];
   constexpr int STEP = RT_THREADS / 64, AHEAD = 4;        // rows' j read ahead
@@ -446,13 +446,13 @@ constexpr int rows_smem() { return ((WX / 2 + 1) * (WY / 2 + 1) + (WX / 2) * (WY
 #define GRID_WINDOWS(X) X(1, 1) X(2, 1) X(4, 1) X(8, 1) X(16, 1) X(2, 2) X(4, 4) X(8, 8) X(16, 16) X(4, 2) X(8, 4) X(16, 8)
 
 template <int N>
-cudaError_t planes_for(const Dev& d, const int* qxy, int nq, int2 qmax, int z0, int nzb, cudaStream_t s) {
+cudaError_t planes_for(const Dev& d, const int* qxy, int nq, int2 qmax, cudaStream_t s) {
   const int hx = d.wx / 2, hy = d.wy / 2, swap = d.wx == d.wy && d.dx == d.dy;
   const int npl = swap ? (hx + 1) * (hx + 2) / 2 : (hx + 1) * (hy + 1);
   // about four rounds of CTAs where there are planes enough; each loads its depth's quadrant once
-  const int nx = std::min(npl, std::max(1, (4 * 304 + nzb - 1) / nzb));
-  grid_planes_kernel<N><<<dim3(nx, nzb), Half<N>::THREADS, Half<N>::SMEM, s>>>(d, qxy, nq, z0, hx, hy, swap, npl,
-                                                                                        swap ? std::max(qmax.x, qmax.y) : qmax.x);
+  const int nx = std::min(npl, std::max(1, (4 * 304 + d.nz - 1) / d.nz));
+  grid_planes_kernel<N><<<dim3(nx, d.nz), Half<N>::THREADS, Half<N>::SMEM, s>>>(
+      d, qxy, nq, hx, hy, swap, npl, swap ? std::max(qmax.x, qmax.y) : qmax.x);
   return cudaGetLastError();
 }
 
@@ -466,13 +466,8 @@ cudaError_t prepare_n() {
 
 int fa_grid_slots(int wx, int wy) { return (wx / 2 + 1) * (wy / 2 + 1) + (wx / 2) * (wy / 2); }
 
-int fa_grid_slab(int nz, int slots, int nq) {
-  const size_t n = std::max<size_t>(1, FA_SLAB_BYTES / fa_grid_bytes(GT_Z, slots, nq));
-  return int(std::min<size_t>(size_t(nz), n * GT_Z));
-}
-
-size_t fa_grid_bytes(int nzb, int slots, int nq) {
-  return size_t((std::max(nq, 1) + GT_Q - 1) / GT_Q) * ((nzb + GT_Z - 1) / GT_Z) * slots * GT_P * sizeof(float2);
+size_t fa_grid_bytes(int nz, int slots, int nq) {
+  return size_t((std::max(nq, 1) + GT_Q - 1) / GT_Q) * ((nz + GT_Z - 1) / GT_Z) * slots * GT_P * sizeof(float2);
 }
 
 cudaError_t launch_fa_grid(const Dev& d, int f, int qoff, int nq, int2 qmax, double2 cf, cudaStream_t s) {
@@ -483,24 +478,20 @@ cudaError_t launch_fa_grid(const Dev& d, int f, int qoff, int nq, int2 qmax, dou
   else grid_gspace_kernel<128><<<d.nz, Half<128>::THREADS, Half<128>::SMEM, s>>>(d, f);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   const float2 c = make_float2(float(0.5 * cf.x), float(0.5 * cf.y));
-  for (int z0 = 0; z0 < d.nz; z0 += d.fa_slab) {
-    const int nzb = std::min(d.fa_slab, d.nz - z0);
-    e = d.N == 32 ? planes_for<32>(d, d.q_xy + qoff, nq, qmax, z0, nzb, s)
-        : d.N == 64 ? planes_for<64>(d, d.q_xy + qoff, nq, qmax, z0, nzb, s)
-                    : planes_for<128>(d, d.q_xy + qoff, nq, qmax, z0, nzb, s);
-    if (e != cudaSuccess) return e;
-    // the depth tiles of a point side by side: its rows' neighbouring 64-byte pieces meet in L2
-    const dim3 g((nzb + GT_Z - 1) / GT_Z, (nq + GT_Q - 1) / GT_Q);
-    switch (d.wx * 32 + d.wy) {
+  e = d.N == 32 ? planes_for<32>(d, d.q_xy + qoff, nq, qmax, s)
+      : d.N == 64 ? planes_for<64>(d, d.q_xy + qoff, nq, qmax, s)
+                  : planes_for<128>(d, d.q_xy + qoff, nq, qmax, s);
+  if (e != cudaSuccess) return e;
+  // the depth tiles of a point side by side: its rows' neighbouring 64-byte pieces meet in L2
+  const dim3 g((d.nz + GT_Z - 1) / GT_Z, (nq + GT_Q - 1) / GT_Q);
+  switch (d.wx * 32 + d.wy) {
 #define GR(WX, WY) case WX * 32 + WY: \
-      grid_rows_kernel<WX, WY><<<g, RT_THREADS, rows_smem<WX, WY>(), s>>>(d, d.q_rows + qoff, nq, z0, nzb, c); break;
-      GRID_WINDOWS(GR)
+    grid_rows_kernel<WX, WY><<<g, RT_THREADS, rows_smem<WX, WY>(), s>>>(d, d.q_rows + qoff, nq, c); break;
+    GRID_WINDOWS(GR)
 #undef GR
-      default: return cudaErrorInvalidValue;
-    }
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    default: return cudaErrorInvalidValue;
   }
-  return cudaSuccess;
+  return cudaGetLastError();
 }
 
 cudaError_t prepare_fa_grid(const Dev& d) {

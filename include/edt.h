@@ -225,7 +225,8 @@ typedef struct {
                                    chose them (0 if never tuned)                           */
 } edt_tuning;
 
-/* Create a context for `cfg` and report the device workspace it needs.
+/* Create a context for `cfg` and report the device workspace it needs (a size of this version of the
+ * library: query it, a buffer sized for another version may be too small).
  * Returns EDT_OK, EDT_EINVAL or EDT_EUNSUPPORTED.  *out is NULL on failure. */
 int edt_create(edt_ctx** out, const edt_config* cfg, size_t* workspace_bytes);
 

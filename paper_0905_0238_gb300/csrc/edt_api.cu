@@ -714,10 +714,19 @@ void layout(edt_ctx* c) {
   take(c->r_rowmax, mixed && !c->win ? nf * nk * sizeof(float) : 0);
   take(c->r_gscale, mixed && !c->win ? std::max<size_t>(c->nslot, 1) * sizeof(int2) : 0);
   // full planes of the forward model (and of the FP64 transform), or the band spectra of
-  // one chunk (Y, then Xc at a 256-byte boundary); one call uses one of the two
-  take(c->r_X, std::max(size_t(c->fchunk) * N * N * (mixed ? sizeof(float2) : sizeof(double2)),
-                        std::max(align_up(c->band_ymax * sizeof(float2), 256) + c->band_xmax * sizeof(float2),
-                                 c->ws_band_elems * sizeof(float2))));
+  // one chunk (Y, then Xc at a 256-byte boundary); one call uses one of the two.  The FP64 path's
+  // spectra are read before its Gram runs and its partial Gram before the solve, so the sums of the
+  // Gram's parts and the truncated SVD's log take their place
+  const size_t gsp = mixed ? 1 : gram_f64_split(c->nz, c->nsub);
+  const size_t g64part = gsp > 1 ? gram_f64_part_doubles(c->nz, c->nsub) * sizeof(double) : 0;
+  const size_t b64part = gsp > 1 ? ns * gsp * nz * 2 * sizeof(double) : 0;
+  const size_t tlog = c->cfg.solver == EDT_SOLVE_TSVD ? ns * tsvd_log_floats(c->nz) * sizeof(float) : 0;
+  take(c->r_X, std::max({size_t(c->fchunk) * N * N * (mixed ? sizeof(float2) : sizeof(double2)),
+                         align_up(c->band_ymax * sizeof(float2), 256) + c->band_xmax * sizeof(float2),
+                         c->ws_band_elems * sizeof(float2), align_up(g64part, 256) + b64part, tlog}));
+  c->r_g64part = {c->r_X.off, g64part};
+  c->r_b64part = {c->r_X.off + align_up(g64part, 256), b64part};
+  c->r_tlog = {c->r_X.off, tlog};
   c->dst_half = align_up((c->win ? nf * nxy * W : nf * N * N) * sizeof(double2), 256);
   take(c->r_Dst, 2 * c->dst_half);                 // two staging buffers
   take(c->r_Vst, (c->win ? nxy : N) * nz * sizeof(double));
@@ -725,7 +734,15 @@ void layout(edt_ctx* c) {
   // so its array (like the row metadata) carries 32 rows of padding
   take(c->r_rhs, (mixed ? R + 32 : std::max<size_t>(R, 1)) * 2 * (mixed ? sizeof(float2) : sizeof(double2)));
   take(c->r_gent, mixed ? (R + 32) * sizeof(GramRow) : 0);
-  take(c->r_gpart, mixed ? size_t(c->nslot) * TC_M * tc_cols(c->nz) * sizeof(float) : 0);
+  // the tensor-core Gram's partial tiles; misfit gradients (line geometry, mixed path): the folded
+  // planes, then, when the last chunk of them has been read, the reversed depth march's states
+  const bool grad = !c->win && mixed && c->nlayer <= GRAD_MAX_LAYERS && N >= 64;
+  const size_t gpart = mixed ? size_t(c->nslot) * TC_M * tc_cols(c->nz) * sizeof(float) : 0;
+  const size_t gscr = grad ? nf * size_t(c->nlayer) * GS_SLOTS * nk * sizeof(double2) : 0;
+  const size_t bfold = grad ? size_t(c->fchunk) * 2 * nk * nk * sizeof(float4) : 0;
+  take(c->r_gpart, std::max({gpart, gscr, bfold}));
+  c->r_gscr = {c->r_gpart.off, gscr};
+  c->r_bfold = {c->r_gpart.off, bfold};
   take(c->r_G, ns * nz * nz * sizeof(double));
   take(c->r_dinv, ns * nz * sizeof(double));
   take(c->r_L32, mixed && c->cfg.refine > 0 ? ns * nz * nz * sizeof(float) : 0);
@@ -739,15 +756,12 @@ void layout(edt_ctx* c) {
                        ? ns * size_t(refine_stride(c->rows_max_sub)) * nz * 2 * sizeof(double) : 0);
   take(c->r_vhat, ns * nz * sizeof(double2));
   take(c->r_vfull, (c->win ? nxy : N) * nz * sizeof(double2));
-  // misfit gradients: line geometry, mixed path (their dJ/dg buffer aliases r_g64)
-  const bool grad = !c->win && mixed && c->nlayer <= GRAD_MAX_LAYERS && N >= 64;
-  take(c->r_gscr, grad ? nf * size_t(c->nlayer) * GS_SLOTS * nk * sizeof(double2) : 0);
+  // misfit gradients (their dJ/dg buffer aliases r_g64)
   take(c->r_adj, grad ? size_t(N) * nz * sizeof(double2) : 0);
   take(c->r_gacc, grad ? size_t(1 + c->nlayer) * sizeof(double) : 0);
   take(c->r_bexp, mixed && !c->win ? (nf * nk + N) * sizeof(int) : 0);
   take(c->r_bpart, mixed && !c->win ? size_t(c->fchunk) * born_tiles(c->N) * sizeof(float4) : 0);
   take(c->r_bredo, mixed && !c->win ? size_t(c->fchunk) * sizeof(int) : 0);
-  take(c->r_bfold, grad ? size_t(c->fchunk) * 2 * nk * nk * sizeof(float4) : 0);
   take(c->r_gcpart, grad ? size_t(nf) * ((nk + 127) / 128) * 4 * c->nlayer * sizeof(double) : 0);
   const bool rg = ref_grad_planned(c);
   take(c->r_rowc, rg ? std::max<size_t>(R, 1) * 2 * sizeof(float4) : 0);
@@ -758,10 +772,6 @@ void layout(edt_ctx* c) {
   take(c->r_status, ns * sizeof(int));
   take(c->r_flags, 8 * sizeof(unsigned));
   const bool disk = !c->kz_p.empty();
-  const size_t gsp = mixed ? 1 : gram_f64_split(c->nz, c->nsub);
-  take(c->r_g64part, gsp > 1 ? gram_f64_part_doubles(c->nz, c->nsub) * sizeof(double) : 0);
-  take(c->r_b64part, gsp > 1 ? ns * gsp * nz * 2 * sizeof(double) : 0);
-  take(c->r_tlog, c->cfg.solver == EDT_SOLVE_TSVD ? ns * tsvd_log_doubles(c->nz) * sizeof(double) : 0);
   take(c->r_kzP, disk ? size_t(nz) * nz * sizeof(double) : 0);
   take(c->r_kzp, disk ? ns * sizeof(int) : 0);
   take(c->r_kzgoff, disk ? ns * sizeof(long long) : 0);
@@ -801,7 +811,7 @@ void bind_plan(edt_ctx* c) {
   d.solver = c->cfg.solver;
   d.tsvd_tol = c->cfg.tsvd_tol;
   d.g64_split = c->cfg.precision == EDT_MIXED ? 1 : gram_f64_split(c->nz, c->nsub);
-  d.tlog_stride = c->r_tlog.bytes ? tsvd_log_doubles(c->nz) : 0;
+  d.tlog_stride = c->r_tlog.bytes ? tsvd_log_floats(c->nz) : 0;
 }
 
 void bind(edt_ctx* c) {
@@ -886,7 +896,7 @@ void bind(edt_ctx* c) {
   d.flags = at<unsigned*>(c, c->r_flags);
   d.g64part = c->r_g64part.bytes ? at<double*>(c, c->r_g64part) : nullptr;
   d.b64part = c->r_b64part.bytes ? at<double*>(c, c->r_b64part) : nullptr;
-  d.tlog = c->r_tlog.bytes ? at<double*>(c, c->r_tlog) : nullptr;
+  d.tlog = c->r_tlog.bytes ? at<float*>(c, c->r_tlog) : nullptr;
   const bool disk = c->r_kzP.bytes > 0;
   d.kz_P = disk ? at<const double*>(c, c->r_kzP) : nullptr;
   d.kz_p = disk ? at<const int*>(c, c->r_kzp) : nullptr;

@@ -170,7 +170,8 @@ struct Dev {
   float4* born_part;            // [fchunk][tiles] a tile's sums of |F|^2 and of their bounds' squares, times
                                 //   2^(-2 e), and e
   int* born_redo;               // [fchunk] planes to form again in FP64
-  float4* born_fold;            // [fchunk][2][nk][nk] folded residual (or data) planes E, T
+  float4* born_fold;            // [fchunk][2][nk][nk] folded residual (or data) planes E, T (over gpart,
+                                //   as is gscr)
   // dL/dc through the damped solve (line geometry, mixed path)
   float4* rowc;                 // [rows_solved][2] per row (u_+, u_-) = d - A x, (v_+, v_-) = -A mu
   float4* xmu;                  // [nsub][nz] (x_+, x_-, mu_+, mu_-) in FP32
@@ -201,9 +202,10 @@ struct Dev {
   double* kz_x;                 // [nsub][nz][2] restricted solutions
   // FP64 Gram: parts a subproblem's rows are added in, at most, and their sums
   int g64_split;
-  double* g64part;              // [nsub][groups][g64_split] tile sums (csrc/gram_f64.cu)
+  double* g64part;              // [nsub][groups][g64_split] tile sums (csrc/gram_f64.cu; over X, as is
+                                //   tlog)
   double* b64part;              // [nsub][g64_split][nz][2]
-  double* tlog;                 // [nsub][tlog_stride] tangents of the truncated SVD's rotations
+  float* tlog;                  // [nsub][tlog_stride] tangents of the truncated SVD's rotations
   size_t tlog_stride;
 };
 
@@ -357,7 +359,7 @@ int chol_block_cols();
 // vertical-wavenumber disk, in place of the Cholesky stage of the FP64 line path.
 constexpr int TSVD_MAX_NZ = 96;
 size_t tsvd_smem_bytes(int p);
-size_t tsvd_log_doubles(int p);                                 // rotation log of one subproblem
+size_t tsvd_log_floats(int p);                                  // rotation log of one subproblem
 cudaError_t prepare_variants(int nz);
 cudaError_t launch_solve_variant(const Dev& d, cudaStream_t s);
 

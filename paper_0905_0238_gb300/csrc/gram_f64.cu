@@ -37,6 +37,11 @@ __host__ __device__ inline int tile_groups(int nz) {
   const int mr = micro_rows(nz), n = mr * (mr + 1) / 2;
   return (n + G_TILES - 1) / G_TILES;
 }
+// sums one part of a group leaves: whole rounds of the CTA's threads over the most tiles a group has
+__host__ __device__ inline int part_doubles(int nz) {
+  const int mr = micro_rows(nz), n = mr * (mr + 1) / 2;
+  return 4 * G_THREADS * ((min(n, G_TILES) + G_THREADS - 1) / G_THREADS);
+}
 __device__ __forceinline__ void tri_of(int t, int& r, int& c) {      // tile (r >= c), row-major
   r = int((sqrtf(8.0f * t + 1.0f) - 1.0f) * 0.5f);
   while (r * (r + 1) / 2 > t) --r;
@@ -141,7 +146,7 @@ __global__ void __launch_bounds__(G_THREADS, 2) gram_f64_kernel(Dev d, int kc) {
     for (int q = 0; q < G_MT; ++q)
       if (q < nq) put_tile(d, m, tr[q], tc[q], acc[q]);
   } else {
-    double* P = d.g64part + ((size_t(m) * gridDim.x + grp) * d.g64_split + part) * (4 * G_TILES) + threadIdx.x;
+    double* P = d.g64part + ((size_t(m) * gridDim.x + grp) * d.g64_split + part) * part_doubles(nz) + threadIdx.x;
 #pragma unroll
     for (int q = 0; q < G_MT; ++q)
       if (q < nq)
@@ -164,14 +169,14 @@ __global__ void __launch_bounds__(G_THREADS) gram_f64_sum_kernel(Dev d) {
   const int np = parts_of(d.row_off[m + 1] - d.row_off[m], d.g64_split);
   if (np == 1) return;
   const int mr = micro_rows(nz), ntile = mr * (mr + 1) / 2;
-  const double* P = d.g64part + (size_t(m) * gridDim.x + grp) * d.g64_split * (4 * G_TILES) + threadIdx.x;
+  const double* P = d.g64part + (size_t(m) * gridDim.x + grp) * d.g64_split * part_doubles(nz) + threadIdx.x;
   for (int q = 0; q < G_MT; ++q) {
     const int t = grp * G_TILES + q * G_THREADS + int(threadIdx.x);
     if (t >= ntile) break;
     double v[4] = {};
     for (int s = 0; s < np; ++s)
 #pragma unroll
-      for (int i = 0; i < 4; ++i) v[i] += P[size_t(s) * (4 * G_TILES) + size_t(4 * q + i) * G_THREADS];
+      for (int i = 0; i < 4; ++i) v[i] += P[size_t(s) * part_doubles(nz) + size_t(4 * q + i) * G_THREADS];
     int r, c;
     tri_of(t, r, c);
     put_tile(d, m, r, c, v);
@@ -193,7 +198,7 @@ int gram_f64_split(int nz, int nsub) {
 }
 
 size_t gram_f64_part_doubles(int nz, int nsub) {
-  return size_t(nsub) * tile_groups(nz) * gram_f64_split(nz, nsub) * 4 * G_TILES;
+  return size_t(nsub) * tile_groups(nz) * gram_f64_split(nz, nsub) * part_doubles(nz);
 }
 
 cudaError_t prepare_gram_f64(const Dev& d) {

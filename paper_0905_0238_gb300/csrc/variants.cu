@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(JAC_THREADS) tsvd_jacobi_kernel(Dev d, const d
     bL[q] = e < nblk ? L : -1;
     bK[q] = e - L * (L + 1) / 2;
   }
-  double* tl = d.tlog + size_t(m) * d.tlog_stride;
+  float* tl = d.tlog + size_t(m) * d.tlog_stride;
   // Which pairs to rotate.  Without a threshold: while |a_ij| > 1e-14 sqrt(a_ii a_jj) (relative to
   // its own diagonal, which keeps small eigenvalues of the positive semi-definite matrix accurate;
   // well above the FP64 rounding of a rotation, so the sweeps end).  With one, only the
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(JAC_THREADS) tsvd_jacobi_kernel(Dev d, const d
           if (!(fabsf(t) <= 2.f)) t = 0.f;     // outside the estimates' range: nothing to rotate
         }
         pj[k] = a; pj[npair + k] = b;
-        tl[size_t(nround) * npair + k] = double(t);
+        tl[size_t(nround) * npair + k] = t;
         double alpha = 0.0, beta = 0.0;
         if (t != 0.f) {
           *rotated = 1;
@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(JAC_THREADS) tsvd_jacobi_kernel(Dev d, const d
     double* ls = lc + cnt;
     __syncthreads();
     for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
-      const double t = tl[size_t(r0) * npair + e];
+      const double t = double(tl[size_t(r0) * npair + e]);
       const double c = t != 0.0 ? cos_of(t) : 1.0;
       lc[e] = c;
       ls[e] = t * c;
@@ -339,8 +339,9 @@ size_t tsvd_smem_bytes(int p) {
   return (size_t(p) * (p + 1) + 4 * p + 2 * P2 + 32) * sizeof(double) + (P2 + 1) * sizeof(int);
 }
 
-// doubles of one subproblem's rotation log: every pair of every round of the most sweeps
-size_t tsvd_log_doubles(int p) {
+// one subproblem's rotation log: the tangent, which is chosen in FP32, of every pair of every round of the
+// most sweeps
+size_t tsvd_log_floats(int p) {
   const size_t P2 = (p + 1) & ~1;
   return size_t(JAC_MAX_SWEEPS) * (P2 - 1) * (P2 / 2);
 }

@@ -305,3 +305,27 @@ def test_launch_counts_before_there_is_a_workspace():
     grid = _launches(ny=64, wy=4, **win)[0]
     assert grid == line + 1                  # three kernels per frequency each; one more inverse pass
     assert _launches(ny=64, wy=4, **{**win, "refine": 1})[0] == grid + 3
+
+
+@pytest.mark.parametrize("kind,limit_mb", [("production", 2450), ("gradient line", 320), ("paper tsvd", 60),
+                                           ("largest tsvd", 570), ("small line", 21)])
+def test_workspace_sizes(kind, limit_mb):
+    """Scratch that one call uses at a time shares its memory, so that a context pays for the largest
+    of its calls and not for all of them (limits in MiB, 1 to 5 % above the present sizes)."""
+    import numpy as np
+    from paper_0905_0238_gb300 import edt, Config
+    kw = dict(nx=512, dx=12.5, nz=256, dz=8.0, z0=0.0, freq_hz=np.linspace(3, 60, 128), eps=0.15,
+              layer_top=np.arange(20) * 100.0, layer_vel=np.linspace(1500.0, 4000.0, 20), alpha=1e-2, cutoff=1.0,
+              precision=edt.EDT_MIXED)
+    if kind == "gradient line":
+        kw.update(nx=256, nz=128, freq_hz=np.linspace(3, 60, 64))
+    elif kind == "small line":
+        kw.update(nx=64, nz=64, dx=10.0, dz=10.0, freq_hz=np.linspace(5, 40, 32))
+    elif kind.endswith("tsvd"):
+        kw.update(nx=256, nz=65, dx=50.0, dz=50.0, z0=775.0, freq_hz=np.linspace(1, 10, 10), precision=edt.EDT_FP64,
+                  solver=edt.EDT_SOLVE_TSVD, tsvd_tol=-1e-2, layer_top=np.array([0.0, 1000.0]),
+                  layer_vel=np.array([1500.0, 4000.0]))
+        kw.update(dict(nx=1024, nz=96) if kind == "largest tsvd" else dict(kz_disk=2.2))
+    ctx, nbytes = edt.edt_create(Config(**kw).c_config()[0])
+    edt.edt_destroy(ctx)
+    assert nbytes <= limit_mb * 2 ** 20

@@ -39,3 +39,33 @@ def test_a_smaller_context_leaves_a_larger_one_alone(kind, small):
     V2 = other.invert(_data(kind, wl2, 2))
     assert torch.isfinite(V2).all()
     assert np.array_equal(big.invert(D).cpu().numpy(), want)
+
+
+def test_calls_that_share_scratch_do_not_disturb_one_another():
+    """The Gram's partial tiles, the folded residual planes and the reversed march's states share memory, as
+    do the FP64 spectra, the Gram's parts and the truncated SVD's log: every call on a context that has
+    made the others gives what it gives on a new context, bit for bit."""
+    layers = (np.array([0.0, 60.0, 150.0, 250.0]), np.array([1500.0, 1800.0, 2300.0, 2900.0]))
+    wl = small_workload(nx=64, nz=40, nf=4, alpha=1e-2, cutoff=0.0, layers=layers)
+    from paper_0905_0238_gb300 import Config, Solver, EDT_MIXED
+    new = lambda: Solver(Config.from_workload(wl, precision=EDT_MIXED))
+    rng = synth.rng_for(2, salt=7)
+    D = dev((rng.standard_normal((4, 64, 64)) + 1j * rng.standard_normal((4, 64, 64))).astype(np.complex64))
+    V = dev(1e-8 * rng.standard_normal((64, 40)))
+
+    def calls(solver):
+        return dict(invert=lambda: [solver().invert(D)],
+                    vjp=lambda: (lambda s: [s.invert(D), *s.invert_vjp(V, out_dtype=torch.complex64)][2:])(solver()),
+                    misfit=lambda: [solver().misfit_grad(V, D)[2]],        # dJ/dc: no atomic sums
+                    forward=lambda: [solver().forward(V)], gram=lambda: list(solver().gram(D)))
+
+    want = {k: [a.cpu().numpy() for a in f()] for k, f in calls(new).items()}
+    one = new()
+    order = ["invert", "misfit", "vjp", "forward", "gram", "misfit", "invert", "vjp"]
+    for k in order:
+        for a, b in zip(calls(lambda: one)[k](), want[k]):
+            assert np.array_equal(a.cpu().numpy(), b), k
+    tsvd, wl2 = _solver("tsvd", 64, 96)
+    D2 = _data("tsvd", wl2, 1)
+    first, G = tsvd.invert(D2).cpu().numpy(), tsvd.gram(D2)[0].cpu().numpy()
+    assert np.array_equal(tsvd.invert(D2).cpu().numpy(), first) and np.array_equal(tsvd.gram(D2)[0].cpu().numpy(), G)

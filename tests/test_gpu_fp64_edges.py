@@ -43,3 +43,26 @@ def test_jacobi_without_truncation():
     _, vh_or = edt2d.invert(wl, D, solver="tsvd", tsvd_tol=1e-30)
     _, vh = solve_gpu(wl, D, solver=1, tsvd_tol=1e-30)
     assert rel_l2(vh, vh_or) < 1e-8
+
+
+@pytest.mark.parametrize("nz,dz", [(3, 60.0), (8, 60.0), (13, 60.0), (33, 40.0)])
+def test_jacobi_with_a_threshold_of_zero(nz, dz):
+    """tsvd_tol = 0 keeps every positive singular value, and every pair is rotated to its own diagonal:
+    the least-squares solution.  Compared where the system's condition is below 1e3: its square, which
+    the normal matrix has, times the FP64 rounding of nz sums gives 1e-8."""
+    from paper_0905_0238_gb300 import Config, Solver, EDT_FP64
+    wl = small_workload(nx=32, nz=nz, nf=12, dz=dz, alpha=1e-3)
+    D = data(wl, 24)
+    s = Solver(Config.from_workload(wl, precision=EDT_FP64, solver=1, tsvd_tol=0.0))
+    s.invert(torch.from_numpy(D).cuda())
+    vh, D2, seen = s.vhat().cpu().numpy(), edt2d.data_transform(D), 0
+    for m in range(wl.nx // 2 + 1):
+        want, system = edt2d.solve_wavenumber(wl, D2, m, return_system=True, solver="tsvd", tsvd_tol=0.0)
+        if "Ahat" not in system:             # no row is kept
+            assert not vh[m].any()
+            continue
+        sv = np.linalg.svd(system["Ahat"], compute_uv=False)
+        if sv[-1] * 1e3 > sv[0]:
+            assert rel_l2(vh[m], want) < 1e-8, m
+            seen += 1
+    assert seen >= 6

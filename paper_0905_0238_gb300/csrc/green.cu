@@ -513,7 +513,8 @@ cudaError_t launch_green(const Dev& d, cudaStream_t s, int tables) {
     if (run == 4) green_layer_kernel<4><<<lb, LBLOCK, 0, s>>>(d, steps);
     else green_layer_kernel<1><<<lb, LBLOCK, 0, s>>>(d, steps);
     // the split walks every layer twice (2 x 2 matrices, then the run): only for stacks of at
-    // least four layers per run over too few (f, n) to fill the SMs' quarters
+    // least four layers per run over too few (f, n) to fill the SMs' quarters (257 layers over 1056: an
+    // inversion takes 0.37 ms, 0.70 with one lane; one and 16 lanes are what was measured)
     if (d.nlayer > 4 * 16 && rows < 32 * 304) green_recursion_kernel<16><<<unsigned((rows + 1) / 2), 32, 0, s>>>(d);
     else green_recursion_kernel<1><<<unsigned((rows + 31) / 32), 32, 0, s>>>(d);
     if (fast32) green_coef32_kernel<<<unsigned((nl + 127) / 128), 128, 0, s>>>(d);

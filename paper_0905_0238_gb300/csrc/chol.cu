@@ -700,10 +700,10 @@ int chol_launches(int nz) { return 1; }
 
 static size_t chol_smem(int nz) { return (size_t(nz) * LDP + NB * LDP + 2 * nz + 40) * sizeof(double); }
 
-cudaError_t prepare_chol(const Dev& d) {
-  cudaError_t e = allow_smem(chol_kernel<false>, int(chol_smem(d.nz)));
+cudaError_t prepare_chol() {
+  cudaError_t e = allow_smem(chol_kernel<false>, chol_smem(MAX_NZ));
   if (e != cudaSuccess) return e;
-  return prepare_chol_dfloat(d);
+  return prepare_chol_dfloat();
 }
 
 cudaError_t launch_chol_solve(const Dev& d, int trace_mode, cudaStream_t s, const CholLookahead* la) {
@@ -729,8 +729,8 @@ cudaError_t launch_refine_update(const Dev& d, cudaStream_t s) {
 
 // Streaming batches: subproblem m has size sub_n[m] <= nmax; lam = trace[m] (trace_mode 1
 // with alpha = 1: the caller accumulates alpha * trace).
-cudaError_t prepare_chol_var(int nmax) {
-  return allow_smem(chol_kernel<true>, int(chol_smem(nmax)));
+cudaError_t prepare_chol_var() {
+  return allow_smem(chol_kernel<true>, chol_smem(MAX_NZ));
 }
 
 int chol_block_cols() { return NB; }

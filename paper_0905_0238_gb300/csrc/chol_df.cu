@@ -500,12 +500,12 @@ int chol_dfloat_launches(int n) {
   return k;
 }
 
-cudaError_t prepare_chol_dfloat(const Dev& d) {
-  cudaError_t e = allow_smem(cdf_final_kernel, int(cdf_final_smem(d.nz)));
+cudaError_t prepare_chol_dfloat() {
+  cudaError_t e = allow_smem(cdf_final_kernel, cdf_final_smem(MIXED_MAX_NZ));
   if (e != cudaSuccess) return e;
   e = allow_smem(cdf_update_tc_kernel, TCU_SMEM);
   if (e != cudaSuccess) return e;
-  return allow_smem(cdf_resolve_kernel, int(cdf_final_smem(d.nz)));
+  return allow_smem(cdf_resolve_kernel, cdf_final_smem(MIXED_MAX_NZ));
 }
 
 cudaError_t launch_chol_dfloat_resolve(const Dev& d, cudaStream_t s) {

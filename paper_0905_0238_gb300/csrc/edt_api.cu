@@ -30,15 +30,6 @@ struct Region { size_t off = 0, bytes = 0; };
 
 int record_cuda_error(cudaError_t e) { return cuda_fail(e); }
 
-cudaError_t allow_smem(const void* f, size_t bytes) {
-  static std::mutex mu;
-  std::lock_guard<std::mutex> lk(mu);
-  cudaFuncAttributes a;
-  const cudaError_t e = cudaFuncGetAttributes(&a, f);
-  if (e != cudaSuccess || size_t(a.maxDynamicSharedSizeBytes) >= bytes) return e;
-  return cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, int(bytes));
-}
-
 // Most complex rows one FP32 tensor-memory accumulation of the Gram covers (a segment);
 // longer runs are split into several segments, each flushed to its own partial tile.
 // Damping below which the automatic residual mode switches to double-float: with FP32
@@ -159,9 +150,9 @@ const char* kStageNames[edt_ctx::NSTAGE] = {"green", "kernel_rows", "transform_r
 
 int validate(const edt_config* c) {
   if (!c) return EDT_EINVAL;
-  if (!is_pow2(c->nx) || c->nx < 16 || c->nx > 1024) return EDT_EUNSUPPORTED;
+  if (!is_pow2(c->nx) || c->nx < 16 || c->nx > MAX_NX) return EDT_EUNSUPPORTED;
   if (!(c->dx > 0) || !(c->dz > 0) || !(c->z0 >= 0) || !(c->eps >= 0)) return EDT_EINVAL;
-  if (c->nz < 1 || c->nz > 512) return EDT_EUNSUPPORTED;
+  if (c->nz < 1 || c->nz > MAX_NZ) return EDT_EUNSUPPORTED;
   if (c->nfreq < 1 || c->nfreq > 32767 || !c->freq_hz) return EDT_EINVAL;
   if (c->nlayer < 1 || c->nlayer > 4096 || !c->layer_top_m || !c->layer_vel_mps) return EDT_EINVAL;
   if (c->layer_top_m[0] != 0.0) return EDT_EINVAL;
@@ -175,7 +166,7 @@ int validate(const edt_config* c) {
   if (c->precision == EDT_MIXED) {
     if (c->passes != 1 && c->passes != 3) return EDT_EINVAL;
     if (c->refine < 0 || c->refine > 8) return EDT_EINVAL;
-    if (c->nz > 256) return EDT_EUNSUPPORTED;
+    if (c->nz > MIXED_MAX_NZ) return EDT_EUNSUPPORTED;
     // the tensor-core producer addresses the FP32 table with 32-bit element offsets
     if (double(c->nfreq) * (c->nx / 2 + 1) * c->nz >= 4294967295.0) return EDT_EUNSUPPORTED;
   }
@@ -1132,15 +1123,15 @@ int edt_set_workspace(edt_ctx* c, void* ws, size_t bytes) {
     EDT_TRYI(upload(c, c->r_kzp, c->kz_p));
     EDT_TRYI(upload(c, c->r_kzgoff, c->kz_goff));
     EDT_TRYI(upload(c, c->r_kzvoff, c->kz_voff));
-    EDT_TRY(prepare_chol_var(c->nz));
+    EDT_TRY(prepare_chol_var());
   }
-  if (c->variant) EDT_TRY(prepare_variants(c->nz));
+  if (c->variant) EDT_TRY(prepare_variants());
   EDT_TRY(prepare_fft(c->dev));
   EDT_TRY(prepare_born());
   EDT_TRY(prepare_grad());
-  EDT_TRY(prepare_chol(c->dev));
+  EDT_TRY(prepare_chol());
   if (c->cfg.precision == EDT_MIXED) EDT_TRY(prepare_gram_tc(c->dev));
-  else EDT_TRY(prepare_gram_f64(c->dev));
+  else EDT_TRY(prepare_gram_f64());
   if (c->band_mode) EDT_TRY(prepare_band(c->dev));
   if (c->win) EDT_TRY(prepare_fa(c->dev));
   if (!c->aux) {

@@ -212,13 +212,16 @@ struct Dev {
 // Record a CUDA error for edt_last_cuda_error; returns EDT_ECUDA.
 int record_cuda_error(cudaError_t e);
 
-// Dynamic shared memory of at least `bytes` for kernel f on the current device.  The limit belongs
-// to the kernel, for every context of the process, so it is only ever raised: a context with fewer
-// depths leaves the launches of a larger one alone.  May be called by several threads at once.
-cudaError_t allow_smem(const void* f, size_t bytes);
+// Largest accepted plans (edt_create, edt_stream_create).
+constexpr int MAX_NX = 1024, MAX_NZ = 512, MIXED_MAX_NZ = 256;
+
+// Dynamic shared memory of kernel f on the current device.  The limit belongs to the kernel, for every
+// context of the process and every thread, so `bytes` is always what the largest accepted plan needs,
+// never a context's own size: a context with fewer depths would take it away from a larger one.
 template <class... A>
 inline cudaError_t allow_smem(void (*kernel)(A...), size_t bytes) {
-  return allow_smem(reinterpret_cast<const void*>(kernel), bytes);
+  return cudaFuncSetAttribute(reinterpret_cast<const void*>(kernel), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              int(bytes));
 }
 
 // ---- launchers (each returns cudaGetLastError()) ---------------------------------------
@@ -286,7 +289,7 @@ struct CholLookahead {
 };
 cudaError_t launch_chol_solve(const Dev& d, int trace_mode, cudaStream_t s, const CholLookahead* la = nullptr);
 // The double-float factorisation and solve (csrc/chol_df.cu), used when d.chol_df is set.
-cudaError_t prepare_chol_dfloat(const Dev& d);
+cudaError_t prepare_chol_dfloat();
 int chol_dfloat_launches(int nz);
 cudaError_t launch_chol_dfloat_resolve(const Dev& d, cudaStream_t s);           // x = (LL^T)^-1 b
 cudaError_t launch_chol_dfloat_export(const Dev& d, double* out, cudaStream_t s); // factor as FP64
@@ -340,7 +343,7 @@ cudaError_t launch_adjoint(const Dev& d, const void* D, int D_dtype, void* V, in
 cudaError_t launch_adjoint64_chunk(const Dev& d, const void* D, int D_dtype, int f0, int nfc, cudaStream_t s);
 
 // Streaming batches: Cholesky and refinement update with per-subproblem sizes (<= nmax).
-cudaError_t prepare_chol_var(int nmax);
+cudaError_t prepare_chol_var();
 cudaError_t launch_chol_var(const Dev& d, int nmax, cudaStream_t s);
 cudaError_t launch_refine_update_var(const Dev& d, int nmax, cudaStream_t s);
 // Blocked Cholesky over several launches (panel + tile update per 32-column step, then the
@@ -360,14 +363,14 @@ int chol_block_cols();
 constexpr int TSVD_MAX_NZ = 96;
 size_t tsvd_smem_bytes(int p);
 size_t tsvd_log_floats(int p);                                  // rotation log of one subproblem
-cudaError_t prepare_variants(int nz);
+cudaError_t prepare_variants();
 cudaError_t launch_solve_variant(const Dev& d, cudaStream_t s);
 
 // One-time kernel attribute setup (opt-in shared memory), done outside any stream capture.
 cudaError_t prepare_fft(const Dev& d);
-cudaError_t prepare_chol(const Dev& d);
+cudaError_t prepare_chol();
 cudaError_t prepare_gram_tc(const Dev& d);
-cudaError_t prepare_gram_f64(const Dev& d);
+cudaError_t prepare_gram_f64();
 cudaError_t prepare_grad();
 
 // Tensor-core Gram tiling (shared by host planning and the kernel).

@@ -389,19 +389,17 @@ template cudaError_t launch_transform<double>(const Dev&, const void*, int, int,
 // Opt-in shared-memory sizes of this file's kernels, allowed when a context gets its workspace
 // (outside any stream capture).
 cudaError_t prepare_fft(const Dev& d) {
-  const int N = d.N;
-  const int rpb32 = std::max(1, 4096 / N), rpb64 = std::max(1, 2048 / N);
-  const int cpb32 = std::min(N, 16), cpb64 = std::min(N, 8);
-  const size_t inv = size_t(INV_ZT) * (padded_len(N) + 1) * sizeof(double2);
+  // rows: 4096 or 2048 elements and their padding whatever the length; the others grow with it
+  const size_t row = padded_len(MAX_NX), col = row + 1, inv = INV_ZT * col * sizeof(double2);
   cudaError_t e;
-  if ((e = allow_smem(fft_rows_kernel<float>, int(size_t(rpb32) * padded_len(N) * sizeof(float2)))) != cudaSuccess) return e;
-  if ((e = allow_smem(fft_rows_kernel<double>, int(size_t(rpb64) * padded_len(N) * sizeof(double2)))) != cudaSuccess) return e;
-  if ((e = allow_smem(fft_cols_kernel<float>, int(size_t(cpb32) * (padded_len(N) + 1) * sizeof(float2)))) != cudaSuccess) return e;
-  if ((e = allow_smem(fft_cols_kernel<double>, int(size_t(cpb64) * (padded_len(N) + 1) * sizeof(double2)))) != cudaSuccess) return e;
-  if ((e = allow_smem(inverse_kernel, int(inv))) != cudaSuccess) return e;
-  if ((e = allow_smem(lateral_dft_kernel, int(inv))) != cudaSuccess) return e;
-  if ((e = allow_smem(lateral_idft_kernel, int(inv))) != cudaSuccess) return e;
-  switch (N) {
+  if ((e = allow_smem(fft_rows_kernel<float>, 4096 / MAX_NX * row * sizeof(float2))) != cudaSuccess) return e;
+  if ((e = allow_smem(fft_rows_kernel<double>, 2048 / MAX_NX * row * sizeof(double2))) != cudaSuccess) return e;
+  if ((e = allow_smem(fft_cols_kernel<float>, 128 / sizeof(float2) * col * sizeof(float2))) != cudaSuccess) return e;
+  if ((e = allow_smem(fft_cols_kernel<double>, 128 / sizeof(double2) * col * sizeof(double2))) != cudaSuccess) return e;
+  if ((e = allow_smem(inverse_kernel, inv)) != cudaSuccess) return e;
+  if ((e = allow_smem(lateral_dft_kernel, inv)) != cudaSuccess) return e;
+  if ((e = allow_smem(lateral_idft_kernel, inv)) != cudaSuccess) return e;
+  switch (d.N) {
     case 32: return wfft_cols_prepare<1>();
     case 64: return wfft_cols_prepare<2>();
     case 128: return wfft_cols_prepare<4>();

@@ -201,8 +201,10 @@ size_t gram_f64_part_doubles(int nz, int nsub) {
   return size_t(nsub) * tile_groups(nz) * gram_f64_split(nz, nsub) * part_doubles(nz);
 }
 
-cudaError_t prepare_gram_f64(const Dev& d) {
-  return allow_smem(gram_f64_kernel, int(gram_smem(d.nz)));
+cudaError_t prepare_gram_f64() {
+  size_t most = 0;
+  for (int nz = 1; nz <= MAX_NZ; ++nz) most = std::max(most, gram_smem(nz));
+  return allow_smem(gram_f64_kernel, most);
 }
 
 cudaError_t launch_gram_f64(const Dev& d, cudaStream_t s) {

@@ -621,14 +621,15 @@ int tc_cols(int nz) { return cols_of(nzp_of(nz)); }
 
 int gram_trace_parts() { return PRODUCER_WARPS; }
 
-static int tc_smem_bytes(const Dev& d) {
-  const int zr = zrows_of(nzp_of(d.nz));
-  const int stages = stages_of(d.passes, d.f16), ncomp = d.passes == 1 ? 1 : 2;
-  return 1024 + stages * ncomp * zr * ROWB + 2 * TAB_BYTES + raw_bytes(d.nzs, d.f16) + (2 * stages + 6 + 2 * RAW_PARTS) * 8 + 16;
+static int tc_smem_bytes(int nz, int passes, bool f16) {
+  const int zr = zrows_of(nzp_of(nz));
+  const int stages = stages_of(passes, f16), ncomp = passes == 1 ? 1 : 2;
+  return 1024 + stages * ncomp * zr * ROWB + 2 * TAB_BYTES + raw_bytes((nz + 1) & ~1, f16) +
+         (2 * stages + 6 + 2 * RAW_PARTS) * 8 + 16;
 }
 
 cudaError_t prepare_gram_tc(const Dev& d) {
-  const int smem = tc_smem_bytes(d);
+  const int smem = tc_smem_bytes(MIXED_MAX_NZ, d.passes, d.f16);
   if (d.f16)
     return d.passes == 3 ? allow_smem(gram_tc_kernel<3, true>, smem) : allow_smem(gram_tc_kernel<1, true>, smem);
   return d.passes == 3 ? allow_smem(gram_tc_kernel<3, false>, smem) : allow_smem(gram_tc_kernel<1, false>, smem);
@@ -647,7 +648,7 @@ cudaError_t launch_gram_scale(const Dev& d, cudaStream_t s, bool rowmax_ready) {
 }
 
 cudaError_t launch_gram_tc(const Dev& d, cudaStream_t s) {
-  const int smem = tc_smem_bytes(d);
+  const int smem = tc_smem_bytes(d.nz, d.passes, d.f16);
   cudaError_t e;
   if (d.ncta_gram > 0) {
     if (d.f16) {

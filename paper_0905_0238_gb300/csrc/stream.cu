@@ -516,7 +516,7 @@ int st_gram_smem_bytes() { return GS_STAGES * GS_STAGE + 1024 + 128; }
 cudaError_t prepare_stream() {
   cudaError_t e = allow_smem(st_gram_kernel, st_gram_smem_bytes());
   if (e != cudaSuccess) return e;
-  return prepare_chol_var(ST_MAX_NZ);
+  return prepare_chol_var();
 }
 
 static unsigned blocks_for(long long n, int per) { return unsigned((n + per - 1) / per); }

@@ -346,9 +346,8 @@ size_t tsvd_log_floats(int p) {
   return size_t(JAC_MAX_SWEEPS) * (P2 - 1) * (P2 / 2);
 }
 
-cudaError_t prepare_variants(int nz) {
-  if (nz > TSVD_MAX_NZ) return cudaSuccess;
-  return allow_smem(tsvd_jacobi_kernel, int(tsvd_smem_bytes(nz)));
+cudaError_t prepare_variants() {
+  return allow_smem(tsvd_jacobi_kernel, tsvd_smem_bytes(TSVD_MAX_NZ));
 }
 
 cudaError_t launch_solve_variant(const Dev& d, cudaStream_t s) {

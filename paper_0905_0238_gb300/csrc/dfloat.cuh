@@ -89,7 +89,7 @@ struct DfDiagScratch {
   float2 ls[3][32];                               // column j of L over L_jj (three in use at a time)
   float2 xr[2][32];                               // finished rows of U (below)
   float2 inv[32];                                 // 1 / L_jj
-  int fail[2];                                    // column j failed: slot j & 1
+  int fail;                                       // a pivot failed; read after the last column only
 };
 
 // Diagonal block of step k0 of one subproblem (kb = min(32, n - k0) columns), factored and
@@ -104,8 +104,9 @@ struct DfDiagScratch {
 // first blocks of the 2050 systems of a 64 x 64 grid: 149 us then, 107 now; its inversion 2.36 ms, 2.23).
 // Writes L_kk (lower triangle) and its FP32 copy (L32, may be null; X goes there too), X to the strict
 // upper triangle (X_il at (l, i)), and the reciprocal pivots (dinv FP64; dinv32 FP32, may be null).  A
-// non-positive or non-finite pivot sets EDT_ENOTPD and returns false (in every thread).  Every thread
-// of the CTA calls it; A's block must be final and visible to the CTA.
+// non-positive or non-finite pivot sets EDT_ENOTPD and returns false (in every thread), after all columns:
+// a thread that left the loop by itself would miss barriers that the others wait at, and what follows a
+// failed pivot is not written.  Every thread of the CTA calls it; A's block must be final and visible to the CTA.
 __device__ inline bool df_diag_block(float2* A, float* L32, double* dinv, float* dinv32, int* status, int n,
                                      int k0, DfDiagScratch& sh) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -116,7 +117,7 @@ __device__ inline bool df_diag_block(float2* A, float* L32, double* dinv, float*
     const int i = warp + 8 * q;
     sh.col[lane][i] = i < kb && lane <= i ? A[size_t(k0 + i) * n + k0 + lane] : zero;
   }
-  if (threadIdx.x < 2) sh.fail[threadIdx.x] = 0;
+  if (threadIdx.x == 0) sh.fail = 0;
   if (threadIdx.x < 64) sh.xr[threadIdx.x >> 5][lane] = zero;
   if (threadIdx.x < 96) sh.ls[threadIdx.x >> 5][lane] = zero;
   __syncthreads();
@@ -126,10 +127,7 @@ __device__ inline bool df_diag_block(float2* A, float* L32, double* dinv, float*
   // column j from its finished entries v, by the warp that holds it
   auto column = [&](int j, float2& v) {
     const float2 d = df_norm(shfl_df(v, j));
-    if (!(d.x > 0.f) || !isfinite(d.x)) {
-      if (lane == 0) sh.fail[j & 1] = 1;
-      return;
-    }
+    if ((!(d.x > 0.f) || !isfinite(d.x)) && lane == 0) sh.fail = 1;
     const float2 iv = df_rsqrt(d);
     const float2 l = df_mul(lane == j ? d : df_norm(v), iv);
     if (lane >= j) {
@@ -142,9 +140,6 @@ __device__ inline bool df_diag_block(float2* A, float* L32, double* dinv, float*
   if (warp == 0) column(0, w[0]);
   __syncthreads();
   for (int j = 0; j < kb; ++j) {
-    // published before the last barrier; column j + 1, which another warp may be working on
-    // already, has the other slot: every thread leaves at the same step
-    if (sh.fail[j & 1]) break;
     // columns c > j: A -= L_j L_j^T (rows above c are not used); c < j: U_i -= (L_i,j-1 / L_j-1,j-1) U_j-1
     // for the rows i >= j, the others and column j subtract zero
     const float2 lj = df_neg(sh.col[j][lane]);
@@ -165,7 +160,7 @@ __device__ inline bool df_diag_block(float2* A, float* L32, double* dinv, float*
       if (j + 1 < kb && warp + 8 * q == j + 1) column(j + 1, w[q]);
     __syncthreads();
   }
-  if (sh.fail[0] | sh.fail[1]) {                  // uniform: no column was formed since the last barrier
+  if (sh.fail) {                                  // not written since the last barrier
     if (threadIdx.x == 0) *status = EDT_ENOTPD;
     return false;
   }

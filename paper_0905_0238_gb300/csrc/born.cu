@@ -218,11 +218,6 @@ __device__ __forceinline__ void fold_tile(const typename Ar::S* g, size_t gs, co
 }
 
 // ---- preparation of the double-float forward model ---------------------------------------
-// exponent e with |v| < 2^e (both components), by their bits; non-finite: above any finite one
-__device__ __forceinline__ int exp_above(double2 v) {
-  return max((__double2hiint(v.x) >> 20) & 0x7ff, (__double2hiint(v.y) >> 20) & 0x7ff) - 1022;
-}
-
 // One row of nz <= 256 FP64 complex values per warp, replaced in place by float pairs of
 // value * c * 2^-e; e goes to exps[row].  Green's table (per_f rows to a frequency): the row's 2-norm in
 // [1/2, 1), c = sqrt(s_f) = omega~ sqrt(dz/dx), so the products carry s_f.  Vhat (per_f = 0): the largest
@@ -282,18 +277,7 @@ __global__ void __launch_bounds__(PREP_THREADS) born_prep_kernel(Dev d, double2*
 // times one power of two 2^-e with the largest component just under 1, e in exps[0].  The products
 // residual x Vhat x table then neither vanish nor overflow where their sum does not: with Vhat as it
 // is, dJ/dc lost digits for models and data 1e-17 of the usual size and was not finite at 1e20 times.
-__global__ void __launch_bounds__(PREP_THREADS) born_vexp_kernel(Dev d, int* rowe) {
-  const double2* r = d.vfull + size_t(blockIdx.x) * d.nz;
-  int e = -1022;
-  for (int z = threadIdx.x; z < d.nz; z += PREP_THREADS) e = max(e, exp_above(r[z]));
-  __shared__ int red[PREP_THREADS / 32];
-  e = __reduce_max_sync(0xffffffffu, e);
-  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e;
-  __syncthreads();
-  if (threadIdx.x == 0) rowe[blockIdx.x] = max(max(red[0], red[1]), max(red[2], red[3]));
-}
-
-__global__ void __launch_bounds__(PREP_THREADS) born_v32_kernel(Dev d, const int* rowe, int* exps) {
+__global__ void __launch_bounds__(PREP_THREADS) born_v32_kernel(Dev d, const int* tile, int ntile, int* exps) {
   static_assert(PREP_THREADS == 128, "four warps");
   __shared__ int red[PREP_THREADS / 32];
   constexpr int Q = 2;                  // nz <= 256
@@ -305,7 +289,7 @@ __global__ void __launch_bounds__(PREP_THREADS) born_v32_kernel(Dev d, const int
     v[i] = z < d.nz ? r[z] : make_double2(0.0, 0.0);
   }
   int e = -1022;
-  for (int m = threadIdx.x; m < d.N; m += PREP_THREADS) e = max(e, rowe[m]);
+  for (int i = threadIdx.x; i < ntile; i += PREP_THREADS) e = max(e, tile[i]);
   e = __reduce_max_sync(0xffffffffu, e);
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = e;
   __syncthreads();                      // and every element of the row has been read
@@ -544,7 +528,12 @@ __global__ void __launch_bounds__(256) born_fwd_edge_f64_kernel(Dev d, int f0) {
            sf * make_double2(p.x + q.y, p.y - q.x));
 }
 
-// born_redo[fi]: the plane's sums by pairs are not 2^-27 of the plane accurate: their sum of squares falls
+// flags of the planes to form again, behind the partial sums
+__device__ __forceinline__ int* redo_flags(const Dev& d, int ntile) {
+  return reinterpret_cast<int*>(d.born_part + size_t(d.fchunk) * ntile);
+}
+
+// Flags plane fi if its sums by pairs are not 2^-27 of the plane accurate: their sum of squares falls
 // below (sqrt(nz) 2^-43 2^27)^2 times that of the bounds.  One warp per plane.
 __global__ void __launch_bounds__(32) born_pick_kernel(Dev d, int ntile) {
   const int fi = blockIdx.x, lane = threadIdx.x;
@@ -563,7 +552,7 @@ __global__ void __launch_bounds__(32) born_pick_kernel(Dev d, int ntile) {
     sf += __shfl_xor_sync(0xffffffffu, sf, o);
     sb += __shfl_xor_sync(0xffffffffu, sb, o);
   }
-  if (lane == 0) d.born_redo[fi] = !(sf >= float(d.nz) * 0x1p-32f * sb);
+  if (lane == 0) redo_flags(d, ntile)[fi] = !(sf >= float(d.nz) * 0x1p-32f * sb);
 }
 
 // These planes in FP64.  CTAs below ntile take a tile, the others eight edge pairs, of every
@@ -614,9 +603,10 @@ constexpr int REDO_Y = 8;
 __global__ void __launch_bounds__(BTHREADS, 2) born_redo_kernel(Dev d, int f0, int nfc, int ntile) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int lane = threadIdx.x & 31;
+  const int* flag = redo_flags(d, ntile);
   int n = 0;                                 // planes met so far
   for (int b = 0; b < nfc; b += 32) {
-    unsigned m = __ballot_sync(0xffffffffu, b + lane < nfc && d.born_redo[b + lane]);
+    unsigned m = __ballot_sync(0xffffffffu, b + lane < nfc && flag[b + lane]);
     for (; m; m &= m - 1, ++n)
       if (n % REDO_Y == int(blockIdx.y)) redo_part(d, f0, b + __ffs(m) - 1, ntile, reinterpret_cast<double2*>(smem_raw));
   }
@@ -792,10 +782,10 @@ cudaError_t launch_born_prep(const Dev& d, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+int* born_v32_exps(const Dev& d) { return d.born_exp + 1; }
+
 cudaError_t launch_born_v32(const Dev& d, cudaStream_t s) {
-  int* rowe = d.born_exp + size_t(d.nf) * d.nk;
-  born_vexp_kernel<<<d.N, PREP_THREADS, 0, s>>>(d, rowe);
-  born_v32_kernel<<<d.N, PREP_THREADS, 0, s>>>(d, rowe, d.born_exp);
+  born_v32_kernel<<<d.N, PREP_THREADS, 0, s>>>(d, born_v32_exps(d), lateral_tiles(d.nz), d.born_exp);
   return cudaGetLastError();
 }
 

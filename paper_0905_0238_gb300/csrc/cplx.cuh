@@ -88,6 +88,11 @@ __device__ __forceinline__ float2 cinv32(float2 b) {
   return make_float2(b.x * r, -b.y * r);
 }
 
+// exponent e with |v| < 2^e (both components), by their bits; non-finite: above any finite one
+__device__ __forceinline__ int exp_above(double2 v) {
+  return max((__double2hiint(v.x) >> 20) & 0x7ff, (__double2hiint(v.y) >> 20) & 0x7ff) - 1022;
+}
+
 // principal square root in FP32, then the branch with non-negative imaginary part
 __device__ __forceinline__ float2 csqrt_upper32(float2 w) {
   const float r = hypotf(w.x, w.y);

@@ -108,7 +108,7 @@ struct edt_ctx {
   void* ws = nullptr;
   Region r_fc, r_ltop, r_lvel, r_zl, r_zo, r_rows, r_roff, r_roffmf, r_band, r_bcol, r_cpre, r_kval, r_pairm, r_fjoff, r_fjent, r_jact, r_jmap, r_qxy, r_qrows, r_Gs, r_U, r_Dw, r_A32, r_tw64, r_tw32, r_segm, r_segr0,
       r_segn, r_ctas, r_mslot, r_zo32, r_fc32, r_coef, r_coef32, r_g64, r_g32, r_g32lo, r_rowmax, r_gscale, r_X, r_Dst, r_Vst, r_rhs, r_gent, r_gpart, r_G,
-      r_dinv, r_L32, r_dinv32, r_b, r_tr, r_tpart, r_x, r_r, r_rpart, r_rowc, r_xmu, r_gam, r_tref, r_treoff, r_vhat, r_vfull, r_gscr, r_adj, r_gacc, r_gcpart, r_bexp, r_bpart, r_bredo, r_bfold, r_status, r_flags,
+      r_dinv, r_L32, r_dinv32, r_b, r_tr, r_tpart, r_x, r_r, r_rpart, r_rowc, r_xmu, r_gam, r_tref, r_treoff, r_vhat, r_vfull, r_gscr, r_adj, r_gacc, r_gcpart, r_bexp, r_bpart, r_bfold, r_status, r_flags,
       r_g64part, r_b64part, r_tlog, r_kzP, r_kzp, r_kzgoff, r_kzvoff, r_kzG, r_kzT, r_kzb, r_kzx;
   Dev dev{};
   cudaStream_t last_stream = nullptr;
@@ -750,9 +750,8 @@ void layout(edt_ctx* c) {
   // misfit gradients (their dJ/dg buffer aliases r_g64)
   take(c->r_adj, grad ? size_t(N) * nz * sizeof(double2) : 0);
   take(c->r_gacc, grad ? size_t(1 + c->nlayer) * sizeof(double) : 0);
-  take(c->r_bexp, mixed && !c->win ? (nf * nk + N) * sizeof(int) : 0);
-  take(c->r_bpart, mixed && !c->win ? size_t(c->fchunk) * born_tiles(c->N) * sizeof(float4) : 0);
-  take(c->r_bredo, mixed && !c->win ? size_t(c->fchunk) * sizeof(int) : 0);
+  take(c->r_bexp, mixed && !c->win ? (nf * nk + N + nz) * sizeof(int) : 0);
+  take(c->r_bpart, mixed && !c->win ? size_t(c->fchunk) * (born_tiles(c->N) * sizeof(float4) + sizeof(int)) : 0);
   take(c->r_gcpart, grad ? size_t(nf) * ((nk + 127) / 128) * 4 * c->nlayer * sizeof(double) : 0);
   const bool rg = ref_grad_planned(c);
   take(c->r_rowc, rg ? std::max<size_t>(R, 1) * 2 * sizeof(float4) : 0);
@@ -875,7 +874,6 @@ void bind(edt_ctx* c) {
   d.gcpart = c->r_gcpart.bytes ? at<double*>(c, c->r_gcpart) : nullptr;
   d.born_exp = c->r_bexp.bytes ? at<int*>(c, c->r_bexp) : nullptr;
   d.born_part = c->r_bpart.bytes ? at<float4*>(c, c->r_bpart) : nullptr;
-  d.born_redo = c->r_bredo.bytes ? at<int*>(c, c->r_bredo) : nullptr;
   d.born_fold = c->r_bfold.bytes ? at<float4*>(c, c->r_bfold) : nullptr;
   d.gbar = c->r_gscr.bytes ? reinterpret_cast<float2*>(d.g64) : nullptr;
   d.rowc = c->r_rowc.bytes ? at<float4*>(c, c->r_rowc) : nullptr;
@@ -1618,11 +1616,11 @@ int edt_get_stats(edt_ctx* c, edt_stats* o) {
                              (c->ny > 1 ? 4 : 3);
   }
   o->freq_chunk = c->band_mode ? c->band_maxplanes : c->fchunk;
-  // misfit gradient: green, zero, lateral DFT and its scaled FP32 copy (2), per chunk transform (2), the
+  // misfit gradient: green, zero, lateral DFT and its scaled FP32 copy, per chunk transform (2), the
   // residual (2) and two contractions, depth march states / field / recursions / layer sums (4), inverse
   // lateral DFT, finalize
   o->launches_per_grad = c->r_gscr.bytes > 0 && c->fchunk > 0
-                             ? green_launches(c->dev, GREEN_G32) + 4 + 6 * ((c->nf + c->fchunk - 1) / c->fchunk) + 6 : 0;
+                             ? green_launches(c->dev, GREEN_G32) + 3 + 6 * ((c->nf + c->fchunk - 1) / c->fchunk) + 6 : 0;
   o->gram_rows_padded = 0;
   for (long long n : c->seg_nrow) o->gram_rows_padded += (n + TC_KC - 1) / TC_KC * TC_KC;
   if (c->ws) {

@@ -320,8 +320,9 @@ __global__ void inverse_kernel(Dev d, void* V, int V_dtype) {
 }
 
 // ---- forward model -------------------------------------------------------------------------
-// Vhat(k_m, z) = sum_x V(x, z) e^{-i k_m x} for all m: one block per z tile.
-__global__ void lateral_dft_kernel(Dev d, const void* V, int V_dtype) {
+// Vhat(k_m, z) = sum_x V(x, z) e^{-i k_m x} for all m: one block per z tile.  exps (may be null): the
+// tile's exponent, |components| < 2^exps[tile].
+__global__ void lateral_dft_kernel(Dev d, const void* V, int V_dtype, int* exps) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   double2* s = reinterpret_cast<double2*>(smem_raw);
   const int N = d.N, logn = ilog2(N), ld = padded_len(N) + 1;
@@ -336,9 +337,21 @@ __global__ void lateral_dft_kernel(Dev d, const void* V, int V_dtype) {
   }
   __syncthreads();
   block_fft<double, double2>(s, N, logn, nzt, ld, d.tw64, -1);
+  int ex = -1022;
   for (int e = threadIdx.x; e < N * nzt; e += blockDim.x) {
     int m = e / nzt, t = e - m * nzt;
-    d.vfull[size_t(m) * d.nz + z0 + t] = s[t * ld + pd(m)];
+    const double2 v = s[t * ld + pd(m)];
+    d.vfull[size_t(m) * d.nz + z0 + t] = v;
+    ex = max(ex, exp_above(v));
+  }
+  if (!exps) return;
+  __shared__ int red[8];
+  ex = __reduce_max_sync(0xffffffffu, ex);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = ex;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < int(blockDim.x >> 5); ++w) ex = max(ex, red[w]);
+    exps[blockIdx.x] = ex;
   }
 }
 
@@ -416,9 +429,11 @@ cudaError_t launch_inverse(const Dev& d, void* V, int V_dtype, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-cudaError_t launch_lateral_dft(const Dev& d, const void* V, int V_dtype, cudaStream_t s) {
+int lateral_tiles(int nz) { return (nz + INV_ZT - 1) / INV_ZT; }
+
+cudaError_t launch_lateral_dft(const Dev& d, const void* V, int V_dtype, cudaStream_t s, int* exps) {
   size_t smem = size_t(INV_ZT) * (padded_len(d.N) + 1) * sizeof(double2);
-  lateral_dft_kernel<<<(d.nz + INV_ZT - 1) / INV_ZT, 256, smem, s>>>(d, V, V_dtype);
+  lateral_dft_kernel<<<lateral_tiles(d.nz), 256, smem, s>>>(d, V, V_dtype, exps);
   return cudaGetLastError();
 }
 
@@ -502,7 +517,7 @@ cudaError_t launch_adjoint64_chunk(const Dev& d, const void* D, int D_dtype, int
 cudaError_t launch_forward(const Dev& d, const void* V, int V_dtype, void* D, int D_dtype,
                            cudaStream_t s) {
   size_t smem = size_t(INV_ZT) * (padded_len(d.N) + 1) * sizeof(double2);
-  lateral_dft_kernel<<<(d.nz + INV_ZT - 1) / INV_ZT, 256, smem, s>>>(d, V, V_dtype);
+  lateral_dft_kernel<<<(d.nz + INV_ZT - 1) / INV_ZT, 256, smem, s>>>(d, V, V_dtype, nullptr);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   if (d.precision != EDT_FP64 && (e = launch_born_prep(d, s)) != cudaSuccess) return e;

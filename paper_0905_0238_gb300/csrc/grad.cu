@@ -968,7 +968,7 @@ cudaError_t launch_misfit_grad(const Dev& d, const void* V, int V_dtype, const v
   cudaError_t e;
   grad_zero_kernel<<<152, 256, 0, s>>>(d);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  if ((e = launch_lateral_dft(d, V, V_dtype, s)) != cudaSuccess) return e;
+  if ((e = launch_lateral_dft(d, V, V_dtype, s, born_v32_exps(d))) != cudaSuccess) return e;
   if ((e = launch_born_v32(d, s)) != cudaSuccess) return e;
   const int N = d.N;
   for (int f0 = 0; f0 < d.nf; f0 += d.fchunk) {

@@ -164,9 +164,9 @@ struct Dev {
   double* gcpart;               // [warps of the reverse march][nlayer] partial dJ/dc_l
   float2* gbar;                 // [nf][nk][nz] dJ/dg per table row (aliases g64)
   // spectral Born operator on the folded table index (csrc/born.cu)
-  int* born_exp;                // [nf * nk + N + nz] power-of-two exponents of the forward model's (the
-                                //   misfit: [0] that of Vhat, then its depth tiles')
-                                //   scaled Green's-table rows and Vhat rows
+  int* born_exp;                // [nf * nk + N + nz] power-of-two exponents of the forward model's scaled
+                                //   Green's-table rows and Vhat rows (the misfit: [0] that of Vhat, then
+                                //   its depth tiles')
   float4* born_part;            // [fchunk][tiles] a tile's sums of |F|^2 and of their bounds' squares, times
                                 //   2^(-2 e), and e; then [fchunk] planes to form again in FP64
   float4* born_fold;            // [fchunk][2][nk][nk] folded residual (or data) planes E, T (over gpart,
@@ -306,14 +306,14 @@ cudaError_t launch_inverse(const Dev& d, void* V, int V_dtype, cudaStream_t s);
 int born_tiles(int N);
 cudaError_t prepare_born();
 cudaError_t launch_born_prep(const Dev& d, cudaStream_t s);
-cudaError_t launch_born_v32(const Dev& d, cudaStream_t s);       // after launch_lateral_dft into born_v32_exps
+cudaError_t launch_born_v32(const Dev& d, cudaStream_t s);       // after launch_lateral_dft(.., born_v32_exps(d))
 int* born_v32_exps(const Dev& d);
 cudaError_t launch_born_forward(const Dev& d, int f0, int nfc, cudaStream_t s);
 cudaError_t launch_born_residual(const Dev& d, int f0, int nfc, bool model, cudaStream_t s);
 cudaError_t launch_forward(const Dev& d, const void* V, int V_dtype, void* D, int D_dtype,
                            cudaStream_t s);
-// vfull[m][z] = sum_x V[x][z] e^{-i k_m x} (FP64)
-// (exps: per depth tile, an exponent above its components; lateral_tiles of them)
+// vfull[m][z] = sum_x V[x][z] e^{-i k_m x} (FP64); exps, if given: for each of the lateral_tiles(nz)
+// depth tiles, e with |components| < 2^e
 cudaError_t launch_lateral_dft(const Dev& d, const void* V, int V_dtype, cudaStream_t s, int* exps = nullptr);
 int lateral_tiles(int nz);
 // out[x][z] = scale Re sum_m in[m][z] e^{+i k_m x} over every m (FP64 transform)

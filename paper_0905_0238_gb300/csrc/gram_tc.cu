@@ -19,7 +19,7 @@
 //     store them K-major with the 128-byte swizzle; (Re a, Im a) of one complex row are two
 //     adjacent K elements.  The data rows d_+, d_- occupy two extra operand rows;
 //   * window geometry: a stage's rows are consecutive rows of the assembled table (its second
-//     factor is the row of ones, its weights are one), so warp 17 copies them to shared memory in
+//     factor is the row of ones, its weights are one), so warp 18 copies them to shared memory in
 //     two parts by bulk copies a stage ahead and the producers convert from there; one operand
 //     stage pays for the buffer.  Read row by row by the producers, the 35.5 GB table of the 128 x 128
 //     grid with 200 depths came at 1.8 TB/s, bound by its loads' latency: 19.6 ms for the kernel, and
@@ -50,8 +50,9 @@ namespace edt {
 namespace {
 
 constexpr int PRODUCER_WARPS = 16;
-// producers, the MMA warp and, in the window geometry, a warp that copies table rows
-__host__ __device__ constexpr int nthreads(bool f16) { return (PRODUCER_WARPS + (f16 ? 1 : 2)) * 32; }
+// producers, the MMA warp, a warp that copies the stages' row metadata and data and, in the window
+// geometry, one that copies table rows
+__host__ __device__ constexpr int nthreads(bool f16) { return (PRODUCER_WARPS + (f16 ? 2 : 3)) * 32; }
 constexpr int ROWB = 128;                       // bytes per operand row per stage (64 bf16)
 
 __host__ __device__ inline int nzp_of(int nz) { return (nz + 31) / 32 * 32; }
@@ -137,7 +138,8 @@ __global__ void __launch_bounds__(nthreads(F16), 1) gram_tc_kernel(Dev d) {
   uint64_t* never = tbar + 2;              // never completed: the wait-test stall
   uint64_t* raw_full = never + 1;          // [RAW_PARTS] table-row copies (window)
   uint64_t* raw_empty = raw_full + RAW_PARTS;   // [RAW_PARTS] producers -> copies
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(raw_empty + RAW_PARTS);
+  uint64_t* tfree = raw_empty + RAW_PARTS;      // [2] producers -> row-table bulk copies
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(tfree + 2);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -159,6 +161,8 @@ __global__ void __launch_bounds__(nthreads(F16), 1) gram_tc_kernel(Dev d) {
     mbar_init(drain, 1);
     mbar_init(&tbar[0], 1);
     mbar_init(&tbar[1], 1);
+    mbar_init(&tfree[0], PRODUCER_WARPS);
+    mbar_init(&tfree[1], PRODUCER_WARPS);
     mbar_init(never, 1);
     for (int h = 0; h < RAW_PARTS; ++h) { mbar_init(&raw_full[h], 1); mbar_init(&raw_empty[h], PRODUCER_WARPS); }
     *abort_flag = 0;
@@ -230,7 +234,34 @@ __global__ void __launch_bounds__(nthreads(F16), 1) gram_tc_kernel(Dev d) {
       mbar_drain(drain, 0u);
     }
     __syncwarp();
-  } else if (!F16 && warp == PRODUCER_WARPS + 1) {
+  } else if (warp == PRODUCER_WARPS + 1) {
+    // ------------------------------------------------------------ row tables
+    // The row table of each stage (32 GramRow entries, 1 KB, and the rows' data) arrives by bulk copies
+    // issued one stage ahead into a double buffer, as soon as every producer warp has read the last
+    // stage's.  Only bounded waits connect the producers with one another and with this warp: with a
+    // barrier among them, waits that end in one warp and succeed in another (a phase that completes
+    // while the abort flag is being raised) would leave the others at the next barrier for good.
+    if (lane == 0) {
+      long long it = 0;
+      bool ok = true;
+      for (int si = s0; si < s1 && ok; ++si) {
+        const int slot = slots[si];
+        const long long nrow = d.seg_nrow[slot], r0 = d.seg_row0[slot];
+        for (long long k0 = 0; k0 < nrow; k0 += TC_KC, ++it) {
+          const int b = int(it & 1);
+          if (it >= 2 && !mbar_wait(&tfree[b], unsigned(((it - 2) >> 1) & 1), abort_flag, budget)) { ok = false; break; }
+          unsigned char* tb = rowtab + b * TAB_BYTES;
+          mbar_expect_tx(&tbar[b], TAB_BYTES);
+          bulk_g2s(tb, d.gent + r0 + k0, TC_KC * sizeof(GramRow), &tbar[b]);
+          bulk_g2s(tb + TC_KC * sizeof(GramRow), reinterpret_cast<const float4*>(d.rhs) + r0 + k0,
+                   TC_KC * sizeof(float4), &tbar[b]);
+        }
+      }
+      // copies still in flight must land before the CTA leaves
+      for (long long k = it > 2 ? it - 2 : 0; k < it; ++k) mbar_drain(&tbar[k & 1], unsigned((k >> 1) & 1));
+    }
+    __syncwarp();
+  } else if (!F16 && warp == PRODUCER_WARPS + 2) {
     // ------------------------------------------------------------ table rows of the window geometry
     // A part is refilled with the next stage's rows as soon as every producer has read it, so one
     // part is always in flight while the other is converted.
@@ -260,37 +291,10 @@ __global__ void __launch_bounds__(nthreads(F16), 1) gram_tc_kernel(Dev d) {
     __syncwarp();
   } else {
     // ------------------------------------------------------------ producers + epilogue
-    const int ptid = threadIdx.x;                 // 0..255
     const int nunits = (nzp / 32) * 8;            // (32-depth group, 16-byte K chunk)
     const float2* g32 = d.rowtab32;
     long long it = 0;
     bool ok = true;
-    // The row table of each stage (32 GramRow entries, 1 KB) arrives by a bulk copy issued
-    // one stage ahead into a double buffer, so it is off the producers' critical path.
-    int nsi = s0;                        // (segment, stage) of the next table copy to issue
-    long long nst_next = 0;
-    long long tb_issued = 0, tb_done = 0;   // table copies issued (thread 0) and waited for
-    auto issue_table = [&](long long it_next) {
-      while (nsi < s1) {
-        const int sl = slots[nsi];
-        const long long n = (d.seg_nrow[sl] + TC_KC - 1) / TC_KC;
-        if (nst_next < n) {
-          const int b = int(it_next & 1);
-          const long long r = d.seg_row0[sl] + nst_next * TC_KC;
-          unsigned char* tb = rowtab + b * TAB_BYTES;
-          mbar_expect_tx(&tbar[b], TAB_BYTES);
-          bulk_g2s(tb, d.gent + r, TC_KC * sizeof(GramRow), &tbar[b]);
-          bulk_g2s(tb + TC_KC * sizeof(GramRow), reinterpret_cast<const float4*>(d.rhs) + r,
-                   TC_KC * sizeof(float4), &tbar[b]);
-          ++nst_next;
-          ++tb_issued;
-          return;
-        }
-        ++nsi;
-        nst_next = 0;
-      }
-    };
-    if (ptid == 0) issue_table(0);
     float tr_hi = 0.f, tr_lo = 0.f;      // Kahan-compensated FP32 trace of the segment
     for (int si = s0; si < s1 && ok; ++si) {
       const int slot = slots[si];
@@ -306,12 +310,9 @@ __global__ void __launch_bounds__(nthreads(F16), 1) gram_tc_kernel(Dev d) {
           if (!mbar_wait(&empty[s], unsigned(((it / STAGES) - 1) & 1), abort_flag, budget)) { ok = false; break; }
         }
         if (!mbar_wait(&tbar[it & 1], unsigned((it >> 1) & 1), abort_flag, budget)) { ok = false; break; }
-        tb_done = it + 1;
         const GramRow* rt = reinterpret_cast<const GramRow*>(rowtab + (it & 1) * TAB_BYTES);
         const float4* rdat = reinterpret_cast<const float4*>(rt + TC_KC);
         const int nvalid = int(min((long long)TC_KC, nrow - st * TC_KC));   // rows past it: padding
-        asm volatile("bar.sync 1, %0;" ::"n"(PRODUCER_WARPS * 32) : "memory");
-        if (ptid == 0) issue_table(it + 1);
         unsigned char* hi = ops + size_t(s) * NCOMP * stage_bytes;
         unsigned char* lo = hi + stage_bytes;
         float trs = 0.f;
@@ -422,6 +423,8 @@ __global__ void __launch_bounds__(nthreads(F16), 1) gram_tc_kernel(Dev d) {
             *reinterpret_cast<uint4*>(hi + off) = h;
           }
         }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&tfree[it & 1]);
         {   // Kahan: tr_hi + tr_lo carries the segment's trace without FP64 arithmetic
           const float yk = trs - tr_lo, tk = tr_hi + yk;
           tr_lo = (tk - tr_hi) - yk;
@@ -453,9 +456,6 @@ __global__ void __launch_bounds__(nthreads(F16), 1) gram_tc_kernel(Dev d) {
       for (int o = 16; o > 0; o >>= 1) tr += __shfl_xor_sync(0xffffffffu, tr, o);
       if (lane == 0) d.tpart[size_t(slot) * PRODUCER_WARPS + warp] = tr;
     }
-    // a table copy still in flight after an early exit must land before the CTA leaves
-    if (ptid == 0)
-      for (long long k = tb_done; k < tb_issued; ++k) mbar_drain(&tbar[k & 1], unsigned((k >> 1) & 1));
   }
 
   __syncthreads();
@@ -625,7 +625,7 @@ static int tc_smem_bytes(int nz, int passes, bool f16) {
   const int zr = zrows_of(nzp_of(nz));
   const int stages = stages_of(passes, f16), ncomp = passes == 1 ? 1 : 2;
   return 1024 + stages * ncomp * zr * ROWB + 2 * TAB_BYTES + raw_bytes((nz + 1) & ~1, f16) +
-         (2 * stages + 6 + 2 * RAW_PARTS) * 8 + 16;
+         (2 * stages + 8 + 2 * RAW_PARTS) * 8 + 16;
 }
 
 cudaError_t prepare_gram_tc(const Dev& d) {

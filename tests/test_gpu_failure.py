@@ -62,3 +62,34 @@ def test_stream_gram_timeout_surfaces_per_request_and_later_batches_run():
     assert list(status) == [0] * len(subs)
     for sub, got in zip(subs, v):
         assert rel_l2(got, stream1d.solve(sub)) < 1e-5
+
+
+@pytest.mark.parametrize("kind", ["line", "window line", "window grid"])
+def test_waits_that_run_out_at_any_time_end_the_kernel(kind):
+    """Budgets from one clock cycle on, with and without the stall, so that waits run out while the
+    producers are at different stages, some of whose barriers complete at that moment: the call always
+    returns, reports the timeout unless every wait was in time (the result is then the usual one, bit
+    for bit), and the next call is right."""
+    from paper_0905_0238_gb300 import Config, Solver, EDT_ETIMEOUT, EDT_GEOM_WINDOW, EDT_MIXED, EDT_OK
+    wl = small_workload(nx=32, nz=70, nf=6, alpha=1e-2, dz=8.0)
+    kw, shape = {}, (6, 32, 32)
+    if kind != "line":
+        ny, wy = (32, 2) if kind == "window grid" else (1, 1)
+        kw, shape = dict(geometry=EDT_GEOM_WINDOW, fold=0, ny=ny, dy=wl.dx, wx=4, wy=wy), (6, ny, 32, wy, 4)
+    s = Solver(Config.from_workload(wl, precision=EDT_MIXED, passes=3, refine=1, **kw))
+    rng = synth.rng_for(0, salt=211)
+    D = dev((rng.standard_normal(shape) + 1j * rng.standard_normal(shape)).astype(np.complex64))
+    want = s.invert(D).cpu().numpy()
+    for cycles in (1, 30, 100, 300, 1000, 2000, 4000, 8000, 20_000, 100_000):
+        for stall in (False, True):
+            s.set_wait_test(cycles, stall)
+            V = s.invert(D).cpu().numpy()
+            st = s.stats()
+            if stall or st.gram_timeouts:
+                assert st.gram_timeouts == 1 and st.last_status == EDT_ETIMEOUT
+            else:
+                assert np.array_equal(V, want)
+    s.set_wait_test(0, False)
+    assert np.array_equal(s.invert(D).cpu().numpy(), want)
+    st = s.stats()
+    assert st.gram_timeouts == 0 and st.last_status == EDT_OK

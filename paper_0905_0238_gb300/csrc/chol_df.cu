@@ -364,7 +364,7 @@ __global__ void __launch_bounds__(256) cdf_update_tc_kernel(Dev d, int k0, int p
     mma_commit(&done);
   }
   __syncwarp();
-  const bool ok = mbar_wait(&done, 0u, &abort_flag);
+  const bool ok = __syncthreads_and(mbar_wait(&done, 0u, &abort_flag));   // one outcome for the CTA
   tc_fence_after();
   if (ok) {
     const int qd = warp & 3, h = warp >> 2;

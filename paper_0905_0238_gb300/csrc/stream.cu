@@ -381,7 +381,7 @@ __global__ void __launch_bounds__(GS_THREADS, 1) st_gram_kernel(StBatch b) {
     // epilogue: warp w reads tensor-memory lanes 32 (w % 4) .. + 31 = rows of the 128-row tile
     const int qd = warp & 3;
     for (int k = k0; k < k1; ++k) {
-      if (!mbar_wait(acc_full, unsigned((k - k0) & 1), abort_flag, budget)) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(acc_full, unsigned((k - k0) & 1), abort_flag, budget))) break;
       tc_fence_after();
       const StItem itm = b.items[k];
       const StSub S = b.sub[itm.req];

@@ -93,3 +93,28 @@ def test_waits_that_run_out_at_any_time_end_the_kernel(kind):
     assert np.array_equal(s.invert(D).cpu().numpy(), want)
     st = s.stats()
     assert st.gram_timeouts == 0 and st.last_status == EDT_OK
+
+
+def test_stream_waits_that_run_out_at_any_time_end_the_kernel():
+    """The same budgets for the streaming Gram: every request of a batch is reported timed out, or all of
+    them come out as usual."""
+    from paper_0905_0238_gb300 import Stream, EDT_ETIMEOUT
+    rng = synth.rng_for(4, salt=951)
+    subs = [stream.sub1d_random(rng, nz_range=(nz, nz), rows_range=(nr, nr), layers_range=(nl, nl))
+            for nz, nr, nl in ((96, 300, 6), (300, 1200, 14), (70, 2000, 9))]
+    for sub in subs:
+        sub.data = (stream1d.kernel_rows(sub) @ rng.standard_normal((sub.nz, 2))).astype(np.complex64)
+    st = Stream(max_batch=8)
+    want, status = st.solve(subs)
+    assert not np.any(status)
+    for cycles in (1, 30, 100, 300, 1000, 2000, 4000, 8000, 20_000, 100_000):
+        for stall in (False, True):
+            st.set_wait_test(cycles, stall)
+            v, status = st.solve(subs)
+            if stall or np.any(status):
+                assert list(status) == [EDT_ETIMEOUT] * len(subs)
+            else:
+                assert all(np.array_equal(a, b) for a, b in zip(v, want))
+    st.set_wait_test(0, False)
+    v, status = st.solve(subs)
+    assert not np.any(status) and all(np.array_equal(a, b) for a, b in zip(v, want))
